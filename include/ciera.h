@@ -290,6 +290,21 @@ CIERA_API int ciera_decode(const ciera_plan* plan, const void* messages_dev, voi
                  void* weights_out_dev, const uint64_t* wire_bytes_dev, void* workspace_dev, int32_t* status_dev,
                  void* stream);
 
+/* ---- whole step ---------------------------------------------------------------------------- */
+
+/*
+ * ciera_encode, ciera_transport and ciera_decode of one table in one kernel launch, with the same results: the
+ * messages in both buffers, lengths, counts, both caches and the reconstructed weights.  For sender and receiver on
+ * one GPU: every byte of a message is stored to both buffers as it is made, and the receiver's part works on it
+ * before it leaves the chip, so nothing that the step itself has written is fetched again.  The receiver's weights
+ * come from its own cache and the message's contents, as in ciera_decode.
+ * Arguments as for the three calls; msg_send_dev and msg_recv_dev are different buffers, weights_out_dev may be
+ * weights_dev.
+ */
+CIERA_API int ciera_step(const ciera_plan* plan, const void* weights_dev, void* sender_cache_dev, void* msg_send_dev,
+                         void* msg_recv_dev, void* receiver_cache_dev, void* weights_out_dev, uint64_t* wire_bytes_dev,
+                         uint32_t* changed_blocks_dev, void* workspace_dev, int32_t* status_dev, void* stream);
+
 /* ---- whole step with host buffers ---------------------------------------------------------- */
 
 /* Device buffers one ciera_roundtrip_host call works in; all caller-owned, sized as for the

@@ -83,6 +83,7 @@ _SIGS = {
     "ciera_entropy_decode": ([_vp] * 6, _i32),
     "ciera_transport": ([_vp] * 7, _i32),
     "ciera_decode": ([_vp] * 8, _i32),
+    "ciera_step": ([_vp] * 12, _i32),
     "ciera_roundtrip_host": ([_vp, _vp, _sz, _vp, _vp, _vp, _vp], _i32),
     "ciera_should_compress": ([ctypes.POINTER(GainIn), ctypes.POINTER(_dbl), ctypes.POINTER(_i32)], _i32),
     "ciera_select_shards": ([ctypes.POINTER(GainIn), _u32, _u64, _i32, _vp, _vp, _vp, _vp, _vp], _i32),
@@ -291,6 +292,15 @@ def decode(plan: Plan, messages, receiver_cache, weights_out, wire_bytes=None, w
     _check("ciera_decode",
            _lib.ciera_decode(plan.handle, _ptr(messages), _ptr(receiver_cache), _ptr(weights_out), _ptr(wire_bytes),
                              _ptr(workspace), _ptr(status), _stream(stream)))
+
+
+def step(plan: Plan, weights, sender_cache, msg_send, msg_recv, receiver_cache, weights_out, wire_bytes, changed_blocks,
+         workspace, status=None, stream=None) -> None:
+    """``encode``, ``transport`` and ``decode`` of one table in one launch (sender and receiver on this GPU)."""
+    _check("ciera_step",
+           _lib.ciera_step(plan.handle, _ptr(weights), _ptr(sender_cache), _ptr(msg_send), _ptr(msg_recv),
+                           _ptr(receiver_cache), _ptr(weights_out), _ptr(wire_bytes), _ptr(changed_blocks),
+                           _ptr(workspace), _ptr(status), _stream(stream)))
 
 
 class DeviceBuffers(ctypes.Structure):

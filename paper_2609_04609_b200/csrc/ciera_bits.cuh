@@ -165,6 +165,14 @@ __device__ __forceinline__ uint32_t word_block_flags(uint32_t d, uint32_t log2b)
     return d != 0u ? 1u : 0u;
 }
 
+// The inverse for fine blocks: `flags` = one flag per block of a piece, lowest block first; all bits of the byte
+// of every value of a flagged block, for the four values 4 i .. 4 i + 3 of the piece.
+__device__ __forceinline__ uint32_t flagged_bytes(uint32_t flags, uint32_t log2b, uint32_t i) {
+    if (log2b == 0) return ((((flags >> (4u * i)) & 0xFu) * 0x00204081u) & 0x01010101u) * 0xFFu;
+    if (log2b == 1) return (((flags >> (2u * i)) & 1u) * 0xFFFFu) | (((flags >> (2u * i + 1u)) & 1u) * 0xFFFF0000u);
+    return ((flags >> (log2b == 2 ? i : i >> 1)) & 1u) * 0xFFFFFFFFu;
+}
+
 // ---- pieces --------------------------------------------------------------------------------
 template <int DT>
 struct Piece;

@@ -42,6 +42,14 @@
 // into hash terms and add them up over the lanes that share a block, and the aggregator finishes
 // the hashes, compares them with the cached ones, refreshes HashCache and derives the block flags
 // from the comparison.
+//
+// And it serves the whole step (template flag STEP, ciera_step): sender, transport and receiver of a table on one GPU.
+// Bound by HBM, a step in three kernels writes each message, reads it, writes its copy and reads that: at q = 0.22
+// 11.1 bytes per bf16 value move.  Here every byte of a message is stored to both buffers as it is made, and the
+// consumers reconstruct a tile's weights from what travels (sign-plus-mantissa, exponents of changed blocks) and
+// the receiver's cached exponents while the tile is still in shared memory: 8.9 bytes.  Measured per OLMoE-shaped
+// layer, B = 512, q = 0.22: bf16 0.711 -> 0.579 ms (0.95 of the copy peak), fp32 1.500 -> 1.108 (0.94); every block
+// changed, bf16: 0.941 -> 0.719.
 #include <cstddef>
 #include <type_traits>
 
@@ -151,13 +159,67 @@ constexpr uint32_t kHashShortRingsLog2 = 6;  // blocks of up to 2^6 values take 
 // With 256 and more blocks in a tile (16 and 32 values per block) the consumers finish the blocks' hashes
 // themselves: kernel instance HASH == 3 (see finish_hash_groups; blocks of at least two lanes' pieces).
 constexpr uint32_t kHashByConsumersLog2 = 5;
-template <int DT, bool FINE, int HASH>
+// The whole-step kernel (STEP) also stages the receiver's cached exponents, behind each weights tile.  With coarse
+// blocks the weights stage is held until the tile's block flags are there, one slot later, so that a third stage
+// counts: bf16 with 3 + 4 stages 0.571 ms per OLMoE-shaped layer, with 2 + 6 0.628.  fp32 has room for it only with one
+// thread block per SM: 1.080 ms with 4 + 5 stages, 1.459 with two blocks of 2 + 3.  (Reconstructing at once from
+// the votes of the own warp, for blocks that lie in one warp's pieces: bf16 0.582, fp32 1.084 ms.)
+template <int DT, bool FINE>
+struct EncodeStepCfg;
+template <>
+struct EncodeStepCfg<CIERA_BF16, false> {
+    static constexpr int kWStages = 3;  // 3 x (16 + 8) KB
+    static constexpr int kEStages = 4;
+    static constexpr int kDefer = 2;
+    static constexpr int kBmWords = kBitmapWords;
+};
+template <>
+struct EncodeStepCfg<CIERA_FP32, false> {
+    static constexpr int kWStages = 4;  // 4 x (32 + 8) KB
+    static constexpr int kEStages = 5;
+    static constexpr int kDefer = 2;
+    static constexpr int kBmWords = kBitmapWords;
+};
+template <>
+struct EncodeStepCfg<CIERA_FP16, false> : EncodeStepCfg<CIERA_BF16, false> {};
+template <>
+struct EncodeStepCfg<CIERA_BF16, true> {
+    static constexpr int kWStages = 2;
+    static constexpr int kEStages = 5;
+    static constexpr int kDefer = 2;
+    static constexpr int kBmWords = kFineBitmapWords;
+};
+template <>
+struct EncodeStepCfg<CIERA_FP16, true> : EncodeStepCfg<CIERA_BF16, true> {};
+template <>
+struct EncodeStepCfg<CIERA_FP32, true> {
+    static constexpr int kWStages = 3;
+    static constexpr int kEStages = 5;
+    static constexpr int kDefer = 2;
+    static constexpr int kBmWords = kFineBitmapWords;
+};
+template <int DT, bool STEP>
+constexpr int kEncodeBlocksPerSM = STEP && DT == CIERA_FP32 ? 1 : 2;
+constexpr uint32_t kDenseValues = (uint32_t)kTileValues / 8u * 7u;  // values of changed blocks from which a tile counts as dense
+template <int DT, bool FINE, int HASH, bool STEP>
 struct EncodeCfgOf {
     using type = EncodeHashCfg<DT, HASH>;
 };
 template <int DT, bool FINE>
-struct EncodeCfgOf<DT, FINE, 0> {
+struct EncodeCfgOf<DT, FINE, 0, false> {
     using type = EncodeCfg<DT, FINE>;
+};
+template <int DT, bool FINE>
+struct EncodeCfgOf<DT, FINE, 0, true> {
+    using type = EncodeStepCfg<DT, FINE>;
+};
+
+// Distances, in bytes, from the sender's buffers to their counterparts on the receiver's side (STEP; else unused):
+// unit layouts are the same on both sides, so one distance serves a whole buffer.
+struct StepTwins {
+    int64_t msg;      // sent messages -> received messages
+    int64_t cache;    // sender's exponent cache -> receiver's
+    int64_t weights;  // weights -> reconstructed weights
 };
 
 // Shared-memory bytes of the cached hashes (`hold`) and of the partial sums (`part`) of one tile:
@@ -182,7 +244,8 @@ struct __align__(16) EncodeTileInfo {
     uint8_t* c_ptr;        // the tile's cached exponents (with HashCache: the cached hash of the tile's first block)
     const uint8_t* w_src;  // the tile's weights
     uint32_t nv;           // values in the tile
-    uint32_t pad[3];
+    uint32_t r_staged;     // STEP: the receiver's cached exponents are staged (else the few needed are read where they lie)
+    uint32_t pad[2];
 };
 
 template <int SW, int SE, int BW>
@@ -506,10 +569,11 @@ struct HashTile {
     ulonglong2* dst;
 };
 
-template <int DT, bool FINE, int HASH>
+template <int DT, bool FINE, int HASH, bool STEP>
 __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, bool publish,
                                                    const uint32_t* ballot, uint32_t* bm, uint16_t* pre, uint8_t* msgs,
-                                                   unsigned long long* tile_status, const HashTile& ht, uint32_t lane) {
+                                                   const StepTwins& tw, unsigned long long* tile_status, const HashTile& ht,
+                                                   uint32_t lane) {
     const uint64_t N = td.n_unit;
     const uint32_t B = 1u << log2b;
     const uint32_t nbt = kTileValues >> log2b;
@@ -545,14 +609,24 @@ __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t 
         uint32_t* dst32 = reinterpret_cast<uint32_t*>(msg + byte0);
         // 16 bytes at a time, then the last words, then the last bytes
         const uint32_t quads = nbytes >> 4;
-        for (uint32_t c = lane; c < quads; c += 32) reinterpret_cast<uint4*>(dst32)[c] = reinterpret_cast<const uint4*>(bm)[c];
-        for (uint32_t w = 4u * quads + lane; w < (nbytes >> 2); w += 32) dst32[w] = bm[w];
+        auto twin32 = reinterpret_cast<uint32_t*>(msg + byte0 + tw.msg);
+        for (uint32_t c = lane; c < quads; c += 32) {
+            const uint4 v = reinterpret_cast<const uint4*>(bm)[c];
+            reinterpret_cast<uint4*>(dst32)[c] = v;
+            if (STEP) reinterpret_cast<uint4*>(twin32)[c] = v;
+        }
+        for (uint32_t w = 4u * quads + lane; w < (nbytes >> 2); w += 32) {
+            dst32[w] = bm[w];
+            if (STEP) twin32[w] = bm[w];
+        }
         const uint32_t done = nbytes & ~3u;
-        if (lane < nbytes - done) msg[byte0 + done + lane] = (uint8_t)(bm[done >> 2] >> (lane * 8u));
+        if (lane < nbytes - done)
+            put_byte<STEP>(msg + byte0 + done + lane, (uint8_t)(bm[done >> 2] >> (lane * 8u)), tw.msg);
     } else if (nbt >= 8) {
         const uint64_t byte0 = (uint64_t)td.tile_in_unit * (nbt >> 3);
         const uint32_t nbytes = (((nv + B - 1u) >> log2b) + 7u) >> 3;
-        for (uint32_t b = lane; b < nbytes; b += 32) msg[byte0 + b] = (uint8_t)(bm[b >> 2] >> ((b & 3u) * 8u));
+        for (uint32_t b = lane; b < nbytes; b += 32)
+            put_byte<STEP>(msg + byte0 + b, (uint8_t)(bm[b >> 2] >> ((b & 3u) * 8u)), tw.msg);
     }
     return agg;
 }
@@ -562,9 +636,11 @@ __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t 
 // tile) if their block changed; `base` is the tile's exclusive offset in the unit's payload.
 // (CACHE = false, the sender with HashCache: payload only.)
 // (FULL: the tile is a full one, every piece complete.)
-template <int DT, bool CACHE, bool FULL>
+// (STEP: the same bytes also go to the received message and to the receiver's cache.)
+template <int DT, bool CACHE, bool FULL, bool STEP>
 __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm,
-                                              const uint16_t* pre, uint64_t base, const uint8_t* s_exp, uint32_t tid) {
+                                              const uint16_t* pre, uint64_t base, const uint8_t* s_exp, const StepTwins& tw,
+                                              uint32_t tid) {
     using P = Piece<DT>;
 #pragma unroll
     for (int p = 0; p < P::kPerThread; ++p) {
@@ -587,43 +663,115 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
             const int nbytes = (5 * nvalid + 7) >> 3;
 #pragma unroll
             for (int i = 0; i < 5; ++i)
-                if (i < nbytes) pdst[i] = (uint8_t)(i < 4 ? lo >> (8 * i) : hi);
+                if (i < nbytes) put_byte<STEP>(pdst + i, (uint8_t)(i < 4 ? lo >> (8 * i) : hi), tw.msg);
             if (!CACHE) continue;
-            if (nvalid == P::kValues)
+            if (nvalid == P::kValues) {
                 x.template store_exp_full<Global>(cdst);
-            else
+                if (STEP) x.template store_exp_full<Global>(cdst + tw.cache);
+            } else {
                 x.store_exp_partial(cdst, nvalid);
+                if (STEP) x.store_exp_partial(cdst + tw.cache, nvalid);
+            }
             continue;
         }
         uint8_t* pdst = ti.pay_dst + base + ((uint64_t)rank << log2b) + (t0 & ((1u << log2b) - 1u));
         if (nvalid == P::kValues) {
             x.template store_exp_full<Global>(pdst);
             if (CACHE) x.template store_exp_full<Global>(cdst);
+            if (STEP) {
+                x.template store_exp_full<Global>(pdst + tw.msg);
+                x.template store_exp_full<Global>(cdst + tw.cache);
+            }
         } else {
             x.store_exp_partial(pdst, nvalid);
             if (CACHE) x.store_exp_partial(cdst, nvalid);
+            if (STEP) {
+                x.store_exp_partial(pdst + tw.msg, nvalid);
+                x.store_exp_partial(cdst + tw.cache, nvalid);
+            }
+        }
+    }
+}
+
+// STEP, fp32: one warp's 2 KB of reconstructed weights from the stage to global memory (one thread).
+__device__ __forceinline__ void bulk_store_tile_part(const EncodeTileInfo& ti, const StepTwins& tw, const uint8_t* s_w,
+                                                     uint32_t warp) {
+    constexpr uint32_t kPart = (uint32_t)kTileValues * 4u / (uint32_t)kWarps;
+    bulk_store(const_cast<uint8_t*>(ti.w_src) + tw.weights + (size_t)warp * kPart, s_w + (size_t)warp * kPart, kPart);
+    bulk_commit();
+}
+
+// STEP, coarse blocks: the receiver's part of one tile.  Every consumer thread splits its pieces of the tile once
+// more (the stage still holds the weights), takes the exponents of an unchanged block from the receiver's cache and
+// those of a changed one as they travel in the payload, merges them with the sign-plus-mantissa as it travels and
+// stores the reconstructed weights.  (The receiver's cache of changed blocks is refreshed by write_changed.)
+// BULK: the thread's weights are left in their place of the stage instead.
+template <int DT, bool FULL, bool BULK>
+__device__ __forceinline__ void reconstruct(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm, uint8_t* s_w,
+                                            const uint8_t* s_r, const StepTwins& tw, uint32_t tid) {
+    using P = Piece<DT>;
+    constexpr int VB = Traits<DT>::kValueBytes;
+#pragma unroll
+    for (int p = 0; p < P::kPerThread; ++p) {
+        const uint32_t t0 = P::start(tid, p);
+        const int nvalid = FULL ? (int)P::kValues : piece_valid<DT>(t0, ti.nv);
+        if (nvalid == 0) continue;
+        const uint32_t kb = t0 >> log2b;
+        const bool changed = (bm[kb >> 5] >> (kb & 31u)) & 1u;
+        const uint8_t* const w = ti.w_src + (size_t)t0 * VB;
+        uint8_t* const out = const_cast<uint8_t*>(w) + tw.weights;
+        P x;
+        if (FULL) {
+            x.template split_full<Shared>(s_w + (size_t)t0 * VB);
+            if (!changed) {
+                if (ti.r_staged)
+                    x.template load_exp_full<Shared>(s_r + t0);
+                else
+                    x.template load_exp_full<Global>(ti.c_ptr + tw.cache + t0);
+            }
+            if (BULK)
+                x.template merge_store_full<Shared>(s_w + (size_t)t0 * VB);
+            else
+                x.template merge_store_full<Global>(out);
+        } else {
+            const uint8_t* const r = ti.c_ptr + tw.cache + t0;
+            if (nvalid == P::kValues) {
+                x.template split_full<Global>(w);
+                if (!changed) x.template load_exp_full<Global>(r);
+                x.template merge_store_full<Global>(out);
+            } else {
+                x.split_partial(w, nvalid);
+                if (!changed) x.load_exp_partial(r, nvalid);
+                x.merge_store_partial(out, nvalid);
+            }
         }
     }
 }
 
 // One block of B = 2^LB (fine) exponent bytes from shared memory to global memory; both addresses are B-aligned.
-template <int LB>
-__device__ __forceinline__ void copy_block(uint8_t* dst, const uint8_t* s_src) {
+// (TWICE: and to the address `twin` bytes further on.)
+template <int LB, bool TWICE>
+__device__ __forceinline__ void copy_block(uint8_t* dst, const uint8_t* s_src, int64_t twin) {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(s_src);
     if (LB == 0) {
         uint32_t v;
         asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
         __stcs(dst, (uint8_t)v);
+        if (TWICE) __stcs(dst + twin, (uint8_t)v);
     } else if (LB == 1) {
         uint16_t v;
         asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
         __stcs(reinterpret_cast<uint16_t*>(dst), v);
+        if (TWICE) __stcs(reinterpret_cast<uint16_t*>(dst + twin), v);
     } else if (LB == 2) {
         uint32_t v;
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
         __stcs(reinterpret_cast<uint32_t*>(dst), v);
+        if (TWICE) __stcs(reinterpret_cast<uint32_t*>(dst + twin), v);
     } else {
-        st_stream8(dst, ld_shared8(s_src));
+        const uint2 v = ld_shared8(s_src);
+        st_stream8(dst, v);
+        if (TWICE) st_stream8(dst + twin, v);
     }
 }
 
@@ -638,9 +786,10 @@ __device__ __forceinline__ void copy_block(uint8_t* dst, const uint8_t* s_src) {
 // the same DRAM traffic and one store instruction per thread instead of one per changed value.
 // (fp16: a changed block's exponents go out five bits each, the block rounded up to whole bytes -- 1, 2, 3 or 5
 // bytes for 1, 2, 4 or 8 values -- and byte by byte, since such blocks start on any byte.)
-template <int DT, int LB>
+// (STEP: the payload bytes also go to the received message.)
+template <int DT, int LB, bool STEP>
 __device__ __forceinline__ void write_changed_fine(const EncodeTileInfo& ti, const uint32_t* bm, const uint16_t* pre,
-                                                   uint64_t base, const uint8_t* s_exp, uint32_t tid) {
+                                                   uint64_t base, const uint8_t* s_exp, const StepTwins& tw, uint32_t tid) {
     constexpr uint32_t B = 1u << LB;
     constexpr uint32_t kFlags = 16u >> LB;  // flags per thread
     const uint32_t bit0 = tid * kFlags;
@@ -672,7 +821,7 @@ __device__ __forceinline__ void write_changed_fine(const EncodeTileInfo& ti, con
             const uint32_t nbytes = (5u * len + 7u) >> 3;
 #pragma unroll
             for (uint32_t k = 0; k < kBlockBytes; ++k)
-                if (k < nbytes) pdst[k] = (uint8_t)(packed >> (8u * k));
+                if (k < nbytes) put_byte<STEP>(pdst + k, (uint8_t)(packed >> (8u * k)), tw.msg);
             pdst += kBlockBytes;
         }
         return;
@@ -683,9 +832,9 @@ __device__ __forceinline__ void write_changed_fine(const EncodeTileInfo& ti, con
         bits &= bits - 1u;
         const uint32_t v = (bit0 + j) << LB;  // the block's first value; < nv, since blocks past the end are never flagged
         if (ti.nv - v >= B) {
-            copy_block<LB>(pdst, s_exp + v);
+            copy_block<LB, STEP>(pdst, s_exp + v, tw.msg);
         } else {
-            for (uint32_t i = 0; i < ti.nv - v; ++i) pdst[i] = s_exp[v + i];  // the unit's short last block
+            for (uint32_t i = 0; i < ti.nv - v; ++i) put_byte<STEP>(pdst + i, s_exp[v + i], tw.msg);  // the unit's short last block
         }
         pdst += B;
     }
@@ -706,10 +855,10 @@ constexpr uint32_t kGatherDensity = 4;
 // shared memory -- every thread walks its set flags as before, but stores into the warp's gather space -- and
 // then writes it out in whole 16-byte pieces, one per lane, with single bytes only at the two ragged ends.
 // The cache is refreshed by whole sectors as in write_changed_fine.
-template <int LB>
+template <int LB, bool STEP>
 __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti, const uint32_t* bm, const uint16_t* pre,
                                                         uint64_t base, const uint8_t* s_exp, uint8_t* s_gather,
-                                                        uint32_t tid) {
+                                                        const StepTwins& tw, uint32_t tid) {
     constexpr uint32_t kFlags = 16u >> LB;  // flags per thread
     const uint32_t lane = tid & 31u;
     const uint32_t bit0 = tid * kFlags;
@@ -748,66 +897,77 @@ __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti
     uint8_t* const g16 = gdst - skew;
     const uint32_t head_end = min((skew + 15u) & ~15u, end);  // first 16-byte boundary at or after the run's start
     const uint32_t tail_start = max(head_end, end & ~15u);     // last 16-byte boundary at or before its end
-    if (skew + lane < head_end) g16[skew + lane] = s_gather[skew + lane];
-    for (uint32_t c = ((skew + 15u) >> 4) + lane; 16u * c + 16u <= end; c += 32u)
-        st_stream16(g16 + 16u * c, ld_shared16(s_gather + 16u * c));
-    if (tail_start + lane < end) g16[tail_start + lane] = s_gather[tail_start + lane];
+    if (skew + lane < head_end) put_byte<STEP>(g16 + skew + lane, s_gather[skew + lane], tw.msg);
+    for (uint32_t c = ((skew + 15u) >> 4) + lane; 16u * c + 16u <= end; c += 32u) {
+        const uint4 v = ld_shared16(s_gather + 16u * c);
+        st_stream16(g16 + 16u * c, v);
+        if (STEP) st_stream16(g16 + tw.msg + 16u * c, v);  // (the buffers lie a multiple of 16 bytes apart)
+    }
+    if (tail_start + lane < end) put_byte<STEP>(g16 + tail_start + lane, s_gather[tail_start + lane], tw.msg);
     __syncwarp();  // the gather space is free again
 }
 
-template <int DT, bool FINE, int HASH>
+template <int DT, bool FINE, int HASH, bool STEP>
 __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm,
                                              const uint16_t* pre, uint64_t base, uint32_t tile_payload_bytes,
-                                             const uint8_t* s_exp, uint8_t* s_gather, uint32_t tid) {
+                                             const uint8_t* s_exp, uint8_t* s_gather, const StepTwins& tw,
+                                             uint32_t tid) {
     if (!FINE) {
         // (as in the consumers' main loop: the two instances named there keep the one form that tests as it goes)
-        constexpr bool kOneBody = (DT == CIERA_BF16 && HASH == 0) || (DT == CIERA_FP32 && HASH != 0);
+        constexpr bool kOneBody = (DT == CIERA_BF16 && HASH == 0 && !STEP) || (DT == CIERA_FP32 && HASH != 0);
         if (!kOneBody && ti.nv == (uint32_t)kTileValues)
-            write_changed<DT, HASH == 0, true>(ti, log2b, bm, pre, base, s_exp, tid);
+            write_changed<DT, HASH == 0, true, STEP>(ti, log2b, bm, pre, base, s_exp, tw, tid);
         else
-            write_changed<DT, HASH == 0, false>(ti, log2b, bm, pre, base, s_exp, tid);
+            write_changed<DT, HASH == 0, false, STEP>(ti, log2b, bm, pre, base, s_exp, tw, tid);
     } else if (DT != CIERA_FP16 && ti.nv == (uint32_t)kTileValues &&
                tile_payload_bytes >= (uint32_t)kTileValues / kGatherDensity) {
         // a full tile in which many exponents changed: gathered in shared memory, written out in whole pieces
         switch (log2b) {
-            case 0: write_changed_fine_full<0>(ti, bm, pre, base, s_exp, s_gather, tid); break;
-            case 1: write_changed_fine_full<1>(ti, bm, pre, base, s_exp, s_gather, tid); break;
-            case 2: write_changed_fine_full<2>(ti, bm, pre, base, s_exp, s_gather, tid); break;
-            default: write_changed_fine_full<3>(ti, bm, pre, base, s_exp, s_gather, tid); break;
+            case 0: write_changed_fine_full<0, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            case 1: write_changed_fine_full<1, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            case 2: write_changed_fine_full<2, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            default: write_changed_fine_full<3, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
         }
     } else {  // few changes (a store per changed block is cheaper than the gathering), a unit's last, short tile, or fp16
         switch (log2b) {
-            case 0: write_changed_fine<DT, 0>(ti, bm, pre, base, s_exp, tid); break;
-            case 1: write_changed_fine<DT, 1>(ti, bm, pre, base, s_exp, tid); break;
-            case 2: write_changed_fine<DT, 2>(ti, bm, pre, base, s_exp, tid); break;
-            default: write_changed_fine<DT, 3>(ti, bm, pre, base, s_exp, tid); break;
+            case 0: write_changed_fine<DT, 0, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
+            case 1: write_changed_fine<DT, 1, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
+            case 2: write_changed_fine<DT, 2, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
+            default: write_changed_fine<DT, 3, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
         }
     }
 }
 
 // `cache` is the sender's exponent cache or, with HASH, its HashCache; `tile_hash` (HASH only) gives
 // the index of every tile's first block in it.
-template <int DT, bool FINE, int HASH>
-__global__ void __launch_bounds__(kEncodeThreads, 2)
+template <int DT, bool FINE, int HASH, bool STEP>
+__global__ void __launch_bounds__(kEncodeThreads, kEncodeBlocksPerSM<DT, STEP>)
 encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
               uint32_t spread_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
               unsigned int* unit_ticket, unsigned int* blocks_done, int32_t* status,
-              const unsigned long long* __restrict__ tile_hash) {
+              const unsigned long long* __restrict__ tile_hash, StepTwins tw) {
     static_assert(!(HASH && FINE), "HashCache: blocks of 16 values and more");
+    static_assert(!(HASH && STEP), "the whole step compares with the exponent cache");
     using P = Piece<DT>;
     constexpr int VB = Traits<DT>::kValueBytes;
     constexpr int SMB = Traits<DT>::kSmBytes;
-    using Cfg = typename EncodeCfgOf<DT, FINE, HASH>::type;
+    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
     constexpr int SW = Cfg::kWStages;
     constexpr int SE = Cfg::kEStages;
     constexpr int kDefer = Cfg::kDefer;
+    // coarse blocks: a tile's weights are reconstructed one slot after its votes, when its block flags are there
+    constexpr bool kRebuild = STEP && !FINE;
+    // fp32: the reconstructed weights of a full tile leave the stage by one bulk store per warp (64 bytes per lane
+    // scatter over the stores of a warp)
+    constexpr bool kBulkOut = STEP && DT == CIERA_FP32;
     static_assert(kDescRing > SE + 2 && SE > kDefer, "ring depths");
     constexpr uint32_t kWBytes = kTileValues * VB;
     constexpr uint32_t kEBytes = kTileValues;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* const ring_w = smem;
-    uint8_t* const ring_e = smem + (size_t)SW * kWBytes;
+    constexpr uint32_t kWStage = kWBytes + (STEP ? kEBytes : 0u);  // STEP: then the receiver's cached exponents
+    uint8_t* const ring_e = smem + (size_t)SW * kWStage;
     using Ctl = EncodeCtl<SW, SE, Cfg::kBmWords>;
     Ctl* ctl = reinterpret_cast<Ctl*>(ring_e + (size_t)SE * kEBytes);
     // HASH: per stage of the exponent ring, the tile's cached hashes and then the partial sums
@@ -883,6 +1043,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 ctl->seq[k % kDescRing] = seq;
                 const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
                 const uint64_t left = td.n_unit - v0;
+                bool r_staged = true;
                 {
                     const uint64_t smoff = sm_offset(td.n_unit, log2b);
                     EncodeTileInfo ti;
@@ -891,13 +1052,18 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     ti.c_ptr = HASH ? cache + hb * 16ull : cache + td.c_off;
                     ti.w_src = weights + td.w_off;
                     ti.nv = (uint32_t)min((uint64_t)kTileValues, left);
+                    // Only unchanged blocks need the receiver's cached exponents.  Where nearly all blocks changed in
+                    // the tile that this stage held before, they are not staged: with every block changed that is
+                    // 1 byte of 12 per value that need not be read.
+                    r_staged = FINE || k < (uint32_t)SE || ctl->agg[se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
+                    ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
                 }
                 if constexpr (HASH) {
                     // the cached hashes of the tile's blocks (16 bytes each) come in for every tile
                     if (left >= (uint64_t)kTileValues) {
                         mbar_arrive_expect_tx(&ctl->full_w[sw], kWBytes);
-                        bulk_load(ring_w + (size_t)sw * kWBytes, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
+                        bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
                     } else {
                         mbar_arrive(&ctl->full_w[sw]);
                     }
@@ -905,10 +1071,13 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     mbar_arrive_expect_tx(&ctl->full_e[se], nblk * 16u);
                     bulk_load(ring_h + (size_t)se * kHStage, cache + hb * 16ull, nblk * 16u, &ctl->full_e[se]);
                 } else if (left >= (uint64_t)kTileValues) {
-                    // both copies of the tile complete on the one barrier the consumers wait for
-                    mbar_arrive_expect_tx(&ctl->full_w[sw], kWBytes + kEBytes);
-                    bulk_load(ring_w + (size_t)sw * kWBytes, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
+                    // all copies of the tile complete on the one barrier the consumers wait for
+                    mbar_arrive_expect_tx(&ctl->full_w[sw], kWBytes + kEBytes + (STEP && r_staged ? kEBytes : 0u));
+                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
                     bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, kEBytes, &ctl->full_w[sw]);
+                    if (STEP && r_staged)
+                        bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, kEBytes,
+                                  &ctl->full_w[sw]);
                 } else {
                     // short tile: consumers read global memory themselves
                     mbar_arrive(&ctl->full_w[sw]);
@@ -941,8 +1110,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 ht.part = reinterpret_cast<const ulonglong2*>(ring_h + (size_t)se * kHStage + kHoldBytes);
                 ht.dst = reinterpret_cast<ulonglong2*>(ctl->info[k % kDescRing].c_ptr);
             }
-            const uint64_t agg = aggregate_tile<DT, FINE, HASH>(td, tile, log2b, !seq, ctl->ballot[se], ctl->bm[se],
-                                                                ctl->pre[se], msgs, tile_status, ht, lane);
+            const uint64_t agg = aggregate_tile<DT, FINE, HASH, STEP>(td, tile, log2b, !seq, ctl->ballot[se], ctl->bm[se],
+                                                                      ctl->pre[se], msgs, tw, tile_status, ht, lane);
             if (seq) {
                 // the run is this block's: the tile's offset is the running sum; a run that does not start its
                 // unit carries on from the inclusive offset that the run before it left in its last tile's
@@ -964,9 +1133,10 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if (nbt < 8) {
                     const uint32_t tpb = 8u / nbt, p = td.tile_in_unit & (tpb - 1u);
                     byte_acc = (p == 0 ? 0u : byte_acc) | (ctl->bm[se][0] << (p * nbt));
-                    if ((p == tpb - 1u || last) && lane == 0) msgs[td.msg_off + td.tile_in_unit / tpb] = (uint8_t)byte_acc;
+                    if ((p == tpb - 1u || last) && lane == 0)
+                        put_byte<STEP>(msgs + td.msg_off + td.tile_in_unit / tpb, (uint8_t)byte_acc, tw.msg);
                 }
-                if (last) finish_unit<DT>(td, log2b, run_incl, msgs, wire_bytes, changed_blocks, lane);
+                if (last) finish_unit<DT, STEP>(td, log2b, run_incl, msgs, tw.msg, wire_bytes, changed_blocks, lane);
                 if (lane == 0) {
                     ctl->base[se] = excl;
                     ctl->agg[se] = agg;
@@ -989,8 +1159,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             if (tile == kNoTile) break;
             if (ctl->seq[k % kDescRing] != 0) continue;  // the aggregator has done it all
             const TileDesc td = ctl->desc[k % kDescRing];
-            const uint64_t excl = resolve_tile<DT>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, wire_bytes,
-                                                   changed_blocks, tile_status, status, lane);
+            const uint64_t excl = resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, tw.msg, wire_bytes,
+                                                         changed_blocks, tile_status, status, lane);
             if (lane == 0) {
                 ctl->base[se] = excl;
                 mbar_arrive(&ctl->resolved[se]);
@@ -1003,6 +1173,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         // stage and phase of slot k in the two rings, and of slot k - kDefer in the exponent ring, kept
         // as running counters (the ring depths are no powers of two)
         uint32_t sw = 0, pw = 0, se = 0, pe = 0, je = 0, pj = 0;
+        uint32_t rw = 0, re = 0, pr = 0;  // kRebuild: stages of slot k - 1 in the two rings, phase in the exponent ring
         // HASH: the lanes of a warp that share a block (a power of two, at most the warp) add up their terms
         const uint32_t hash_lanes_l2 = min(5u, log2b - (uint32_t)P::kLog2Values);
         for (;; ++k) {
@@ -1023,7 +1194,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             } else {
                 const EncodeTileInfo ti = ctl->info[k % kDescRing];
                 const uint32_t nv = ti.nv;
-                const uint8_t* const s_w = ring_w + (size_t)sw * kWBytes;
+                uint8_t* const s_w = ring_w + (size_t)sw * kWStage;
+                const uint8_t* const s_r = s_w + kWBytes;  // STEP: the receiver's cached exponents
                 uint8_t* const s_e = ring_e + (size_t)se * kEBytes;
                 uint64_t hash_a[P::kPerThread], hash_b[P::kPerThread];  // HASH: the pieces' sums of terms
                 // The pieces of this thread.  Most instances compile the loop twice: for full tiles (staged
@@ -1031,7 +1203,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 // tile; that measured 2-12 % faster (fp16 most).  Two instances keep one loop that tests as it
                 // goes, which measured faster for them: bf16 with coarse blocks and the exponent cache (1 %),
                 // fp32 with HashCache (5 %).
-                constexpr bool kOneBody = (DT == CIERA_BF16 && !FINE && HASH == 0) || (DT == CIERA_FP32 && HASH != 0);
+                constexpr bool kOneBody = (DT == CIERA_BF16 && !FINE && HASH == 0 && !STEP) || (DT == CIERA_FP32 && HASH != 0);
                 if constexpr (kOneBody) {
                     // a plain loop that tests as it goes
 #define CIERA_PIECES_FULL false
@@ -1067,10 +1239,46 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                                                          (P::start(tid, P::kPerThread - 1) >> P::kLog2Values) >> hash_lanes_l2, part, lane);
                     }
                 }
+                if (kBulkOut && !kRebuild) fence_async_shared();
                 __syncwarp();  // the warp's shared-memory accesses above are ordered before lane 0's arrives
                 if (lane == 0) {
-                    mbar_arrive(&ctl->empty_w[sw]);
                     mbar_arrive(&ctl->voted[se]);
+                    if (!kRebuild) {
+                        if (kBulkOut && nv == (uint32_t)kTileValues) {
+                            bulk_store_tile_part(ti, tw, s_w, warp);
+                            bulk_wait_read<0>();
+                        }
+                        mbar_arrive(&ctl->empty_w[sw]);
+                    }
+                }
+            }
+            if constexpr (kRebuild) {
+                // the receiver's part of the tile before this one: its block flags are there by now
+                if (k != 0 && k - 1u < k_end) {
+                    if (!mbar_wait(&ctl->summed[re], pr, abort, status)) break;
+                    const EncodeTileInfo ti = ctl->info[(k - 1u) % kDescRing];
+                    uint8_t* const s_w = ring_w + (size_t)rw * kWStage;
+                    const bool full = ti.nv == (uint32_t)kTileValues;
+                    if (full)
+                        reconstruct<DT, true, kBulkOut>(ti, log2b, ctl->bm[re], s_w, s_w + kWBytes, tw, tid);
+                    else
+                        reconstruct<DT, false, false>(ti, log2b, ctl->bm[re], s_w, s_w + kWBytes, tw, tid);
+                    if (kBulkOut) fence_async_shared();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (kBulkOut && full) {
+                            bulk_store_tile_part(ti, tw, s_w, warp);
+                            bulk_wait_read<0>();
+                        }
+                        mbar_arrive(&ctl->empty_w[rw]);
+                    }
+                }
+                if (k != 0) {
+                    if (++rw == (uint32_t)SW) rw = 0;
+                    if (++re == (uint32_t)SE) {
+                        re = 0;
+                        pr ^= 1u;
+                    }
                 }
             }
 
@@ -1078,9 +1286,9 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             if (k >= (uint32_t)kDefer) {
                 if (k - kDefer < k_end) {
                     if (!mbar_wait(&ctl->resolved[je], pj, abort, status)) break;
-                    send_changed<DT, FINE, HASH>(ctl->info[(k - kDefer) % kDescRing], log2b, ctl->bm[je], ctl->pre[je],
+                    send_changed<DT, FINE, HASH, STEP>(ctl->info[(k - kDefer) % kDescRing], log2b, ctl->bm[je], ctl->pre[je],
                                                  ctl->base[je], (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes,
-                                                 s_gather, tid);
+                                                 s_gather, tw, tid);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->empty_e[je]);
                 }
@@ -1104,14 +1312,15 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             for (uint32_t j = k + 1u >= (uint32_t)kDefer ? k + 1u - kDefer : 0u; j < k_end; ++j) {
                 const uint32_t je = j % SE;
                 if (!mbar_wait(&ctl->resolved[je], (j / SE) & 1u, abort, status)) break;
-                send_changed<DT, FINE, HASH>(ctl->info[j % kDescRing], log2b, ctl->bm[je], ctl->pre[je], ctl->base[je],
-                                             (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes, s_gather, tid);
+                send_changed<DT, FINE, HASH, STEP>(ctl->info[j % kDescRing], log2b, ctl->bm[je], ctl->pre[je], ctl->base[je],
+                                             (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes, s_gather, tw, tid);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctl->empty_e[je]);
             }
         }
     }
 
+    if (kBulkOut) bulk_wait_all<0>();  // this thread's bulk stores are complete before the block ends
     // leave together; after an aborted run wait (bounded) for bulk copies that are still in flight
     __syncthreads();
     if (tid == 0 && ctl->abort) {
@@ -1141,17 +1350,17 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
 }
 
 // (with HashCache the size depends on the block size: see hash_hold_bytes, hash_part_bytes)
-template <int DT, bool FINE, int HASH>
+template <int DT, bool FINE, int HASH, bool STEP>
 static size_t encode_smem_bytes(uint32_t log2b) {
-    using Cfg = typename EncodeCfgOf<DT, FINE, HASH>::type;
+    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
     constexpr int SW = Cfg::kWStages, SE = Cfg::kEStages;
     const size_t hash_stage = HASH ? (size_t)hash_hold_bytes<DT>(log2b) + hash_part_bytes<DT>(log2b) : 0;
-    return (size_t)SW * kTileValues * Traits<DT>::kValueBytes + (size_t)SE * kTileValues +
+    return (size_t)SW * kTileValues * (Traits<DT>::kValueBytes + (STEP ? 1 : 0)) + (size_t)SE * kTileValues +
            sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)SE * hash_stage + (FINE ? (size_t)kWarps * kWarpGatherBytes : 0);
 }
 
 // Largest grid whose blocks are all resident at once, per device and block size (0 = not yet known).
-template <int DT, bool FINE, int HASH>
+template <int DT, bool FINE, int HASH, bool STEP>
 static int encode_grid_limit(uint32_t log2b, int* out) {
     static std::atomic<int> cached[64][16];  // (zero-initialised; any host thread may be the first to fill an entry)
     int dev = 0;
@@ -1159,13 +1368,13 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
     if (e != cudaSuccess) return record_cuda_error(e);
     if (dev < 0 || dev >= 64 || log2b >= 16) return CIERA_ERR_UNSUPPORTED;
     if (cached[dev][log2b].load(std::memory_order_acquire) == 0) {
-        const size_t smem = encode_smem_bytes<DT, FINE, HASH>(log2b);
+        const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
         // (the limit set here is the largest any block size asks for: the smallest block of the class)
-        e = cudaFuncSetAttribute(encode_kernel<DT, FINE, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)encode_smem_bytes<DT, FINE, HASH>(FINE ? 0u : HASH == 1 ? kHashShortRingsLog2 + 1u : kFineLog2));
+        e = cudaFuncSetAttribute(encode_kernel<DT, FINE, HASH, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)encode_smem_bytes<DT, FINE, HASH, STEP>(FINE ? 0u : HASH == 1 ? kHashShortRingsLog2 + 1u : kFineLog2));
         if (e != cudaSuccess) return record_cuda_error(e);
         int per_sm = 0, sms = 0, coop = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH>, kEncodeThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH, STEP>, kEncodeThreads, smem);
         if (e != cudaSuccess) return record_cuda_error(e);
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return record_cuda_error(e);
@@ -1180,12 +1389,12 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
 
 // `scratch`: one status word per tile, then the run counter and the counter of finished blocks; all zero when
 // the kernel starts, and all zero again when it has finished without a device-side error.
-template <int DT, bool FINE, int HASH = 0>
+template <int DT, bool FINE, int HASH = 0, bool STEP = false>
 static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
-                         cudaStream_t s) {
+                         cudaStream_t s, StepTwins tw = StepTwins{0, 0, 0}) {
     int limit = 0;
-    const int rc = encode_grid_limit<DT, FINE, HASH>(p->log2b, &limit);
+    const int rc = encode_grid_limit<DT, FINE, HASH, STEP>(p->log2b, &limit);
     if (rc) return rc;
     const TileDesc* tiles = p->tiles_dev;
     uint32_t nt = (uint32_t)p->tiles.size();
@@ -1202,20 +1411,20 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     unsigned int* ticket = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(nt));
     unsigned int* done = ticket + 1;
     const unsigned long long* tile_hash = HASH ? p->tile_hash_dev : nullptr;
-    const size_t smem = encode_smem_bytes<DT, FINE, HASH>(log2b);
+    const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
     const bool has_spread = p->seq_first.back() < nt;  // tiles of longer units: look-back between blocks
     cudaError_t e;
     if (has_spread) {
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
         void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &log2b, &w, &c, &m, &wb, &changed_blocks_dev, &ts,
-                        &ticket, &done, &status_dev, &tile_hash};
-        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH>, dim3(grid), dim3(kEncodeThreads), args,
+                        &ticket, &done, &status_dev, &tile_hash, &tw};
+        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads), args,
                                         smem, s);
     } else {
-        encode_kernel<DT, FINE, HASH><<<grid, kEncodeThreads, smem, s>>>(
+        encode_kernel<DT, FINE, HASH, STEP><<<grid, kEncodeThreads, smem, s>>>(
             tiles, nt, seq_runs, n_runs, spread_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
-            tile_hash);
+            tile_hash, tw);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return record_cuda_error(e);
@@ -1224,24 +1433,27 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
 }
 
 // picks the kernel for the plan's precision and block class
+template <int DT>
+static int launch_encode_of(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
+                            uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
+                            cudaStream_t s, const StepTwins* tw) {
+    auto launch = [&](auto fine, auto step) {
+        return launch_encode<DT, decltype(fine)::value, 0, decltype(step)::value>(
+            p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev, scratch, status_dev, s,
+            tw ? *tw : StepTwins{0, 0, 0});
+    };
+    if (is_fine(p->log2b)) return tw ? launch(std::true_type{}, std::true_type{}) : launch(std::true_type{}, std::false_type{});
+    return tw ? launch(std::false_type{}, std::true_type{}) : launch(std::false_type{}, std::false_type{});
+}
+// (tw: the whole step; null: the sender's part alone)
 static int launch_encode_any(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                              uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
-                             cudaStream_t s) {
-    const bool fine = is_fine(p->log2b);
-    if (p->dtype == CIERA_FP16)
-        return fine ? launch_encode<CIERA_FP16, true>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                      changed_blocks_dev, scratch, status_dev, s)
-                    : launch_encode<CIERA_FP16, false>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                       changed_blocks_dev, scratch, status_dev, s);
-    if (p->dtype == CIERA_BF16)
-        return fine ? launch_encode<CIERA_BF16, true>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                      changed_blocks_dev, scratch, status_dev, s)
-                    : launch_encode<CIERA_BF16, false>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                       changed_blocks_dev, scratch, status_dev, s);
-    return fine ? launch_encode<CIERA_FP32, true>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                  changed_blocks_dev, scratch, status_dev, s)
-                : launch_encode<CIERA_FP32, false>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev,
-                                                   changed_blocks_dev, scratch, status_dev, s);
+                             cudaStream_t s, const StepTwins* tw = nullptr) {
+    auto* launch = p->dtype == CIERA_FP16   ? launch_encode_of<CIERA_FP16>
+                   : p->dtype == CIERA_BF16 ? launch_encode_of<CIERA_BF16>
+                                            : launch_encode_of<CIERA_FP32>;
+    return launch(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev, scratch, status_dev, s,
+                  tw);
 }
 
 // the sender with HashCache: blocks of 16 values and more (checked by the caller)
@@ -1305,6 +1517,35 @@ extern "C" int ciera_encode(const ciera_plan* p, const void* weights_dev, void* 
     // or left so by the previous call), and the kernel hands it back all zero
     return launch_encode_any(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev,
                              workspace_dev, status_dev, s);
+}
+
+extern "C" int ciera_step(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* msg_send_dev,
+                          void* msg_recv_dev, void* receiver_cache_dev, void* weights_out_dev, uint64_t* wire_bytes_dev,
+                          uint32_t* changed_blocks_dev, void* workspace_dev, int32_t* status_dev, void* stream) {
+    if (!p) return CIERA_ERR_INVALID_ARG;
+    if (!p->tiles.empty() && !p->tiles_dev) return CIERA_ERR_NOT_BOUND;
+    if (p->n_units == 0) return CIERA_OK;
+    if (!wire_bytes_dev || !changed_blocks_dev) return CIERA_ERR_INVALID_ARG;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (p->has_empty_units) {  // units without tiles: their outputs are written here
+        cudaError_t e = cudaMemsetAsync(wire_bytes_dev, 0, sizeof(uint64_t) * p->n_units, s);
+        if (e != cudaSuccess) return record_cuda_error(e);
+        e = cudaMemsetAsync(changed_blocks_dev, 0, sizeof(uint32_t) * p->n_units, s);
+        if (e != cudaSuccess) return record_cuda_error(e);
+    }
+    if (p->tiles.empty()) return CIERA_OK;
+    if (!weights_dev || !sender_cache_dev || !msg_send_dev || !msg_recv_dev || !receiver_cache_dev || !weights_out_dev ||
+        !workspace_dev)
+        return CIERA_ERR_INVALID_ARG;
+    if (misaligned16(weights_dev) || misaligned16(sender_cache_dev) || misaligned16(msg_send_dev) ||
+        misaligned16(msg_recv_dev) || misaligned16(receiver_cache_dev) || misaligned16(weights_out_dev) ||
+        misaligned16(workspace_dev) || ((uintptr_t)wire_bytes_dev & 7u) || ((uintptr_t)changed_blocks_dev & 3u))
+        return CIERA_ERR_MISALIGNED;
+    const StepTwins tw{(int64_t)((intptr_t)msg_recv_dev - (intptr_t)msg_send_dev),
+                       (int64_t)((intptr_t)receiver_cache_dev - (intptr_t)sender_cache_dev),
+                       (int64_t)((intptr_t)weights_out_dev - (intptr_t)weights_dev)};
+    return launch_encode_any(p, weights_dev, sender_cache_dev, msg_send_dev, wire_bytes_dev, changed_blocks_dev,
+                             workspace_dev, status_dev, s, &tw);
 }
 
 // ------------------------------------------------------------------------------------------

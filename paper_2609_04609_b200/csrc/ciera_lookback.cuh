@@ -43,9 +43,17 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
     return v;
 }
 
+// One byte of a message; with TWICE also `twin` bytes further on (the whole-step kernel writes a message into the
+// sender's and the receiver's buffer alike).
+template <bool TWICE>
+__device__ __forceinline__ void put_byte(uint8_t* p, uint8_t v, int64_t twin) {
+    p[0] = v;
+    if (TWICE) p[twin] = v;
+}
+
 // The unit's last tile reports the totals and zeroes the two pads (one warp).
-template <int DT>
-__device__ __forceinline__ void finish_unit(const TileDesc& td, uint32_t log2b, uint64_t total, uint8_t* msgs,
+template <int DT, bool TWICE>
+__device__ __forceinline__ void finish_unit(const TileDesc& td, uint32_t log2b, uint64_t total, uint8_t* msgs, int64_t twin,
                                             unsigned long long* wire_bytes, uint32_t* changed_blocks, uint32_t lane) {
     const uint64_t N = td.n_unit;
     uint8_t* msg = msgs + td.msg_off;
@@ -62,17 +70,17 @@ __device__ __forceinline__ void finish_unit(const TileDesc& td, uint32_t log2b, 
             changed_blocks[td.unit] = (uint32_t)((total + (1ull << log2b) - 1u) >> log2b);
         }
     }
-    for (uint64_t b = bitmap_bytes(N, log2b) + lane; b < smoff; b += 32) msg[b] = 0;
-    for (uint64_t b = smoff + sm_bytes + lane; b < payoff; b += 32) msg[b] = 0;
+    for (uint64_t b = bitmap_bytes(N, log2b) + lane; b < smoff; b += 32) put_byte<TWICE>(msg + b, 0, twin);
+    for (uint64_t b = smoff + sm_bytes + lane; b < payoff; b += 32) put_byte<TWICE>(msg + b, 0, twin);
 }
 
 // Resolver warp, one spread tile: exclusive prefix of the payload bytes over the earlier tiles of
 // the same unit by a single-pass look-back over the status words, then the duties that need it.
 // Returns the tile's exclusive payload offset inside its unit.
-template <int DT>
+template <int DT, bool TWICE>
 __device__ __forceinline__ uint64_t resolve_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, uint64_t agg,
-                                                 const uint32_t* bm, uint8_t* msgs, unsigned long long* wire_bytes,
-                                                 uint32_t* changed_blocks, unsigned long long* tile_status,
+                                                 const uint32_t* bm, uint8_t* msgs, int64_t twin,
+                                                 unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
                                                  int32_t* status, uint32_t lane) {
     const uint32_t nbt = kTileValues >> log2b;
     uint8_t* msg = msgs + td.msg_off;
@@ -109,11 +117,11 @@ __device__ __forceinline__ uint64_t resolve_tile(const TileDesc& td, uint32_t ti
             }
             __syncwarp();
             part = __reduce_or_sync(0xffffffffu, part);
-            if (lane == 0) msg[td.tile_in_unit / tpb] = (uint8_t)(part | (mybits << (p * nbt)));
+            if (lane == 0) put_byte<TWICE>(msg + td.tile_in_unit / tpb, (uint8_t)(part | (mybits << (p * nbt))), twin);
         }
     }
     if (td.tile_in_unit == td.n_tiles_unit - 1u)
-        finish_unit<DT>(td, log2b, excl + agg, msgs, wire_bytes, changed_blocks, lane);
+        finish_unit<DT, TWICE>(td, log2b, excl + agg, msgs, twin, wire_bytes, changed_blocks, lane);
     return excl;
 }
 

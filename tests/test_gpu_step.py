@@ -1,0 +1,89 @@
+"""The whole step in one launch (``ciera_step``) against the three calls it stands for, and those three against the
+oracle: tolerance 0.  Units end at the edges of pieces, warps, blocks and tiles; one is long enough for the look-back
+between thread blocks; the block changes from hardly any to every block, so that the receiver's cached exponents come
+both staged and straight from memory.  In a second pass the receiver's cache holds other exponents than the sender's:
+what comes out then shows that the receiver's part uses its own cache and not the sender's weights."""
+import numpy as np
+import pytest
+import torch
+
+from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes
+from paper_2609_04609_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+NAME = {0: "bf16", 1: "fp32", 2: "fp16"}
+SIZES = [1, 7, 8, 9, 255, 256, 257, 0, 511, 513, 4096, 8191, 8192, 8193, 8192 * 5, 8192 * 12 + 4097, 8192 * 40 + 3]
+STATE = ("sender_cache", "receiver_cache", "weights_out", "wire_bytes", "changed_blocks")
+
+
+def _three_calls(codec, w):
+    codec.encode(w)
+    codec.transport()
+    codec.decode()
+
+
+@pytest.mark.parametrize("block", [1, 2, 4, 8, 16, 32, 256, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_one_launch_equals_three_calls_equals_the_oracle(dtype, block):
+    from paper_2609_04609_b200 import ciera, runtime
+
+    one, three = (guard(runtime.LayerCodec.from_tensors(SIZES, 1, NAME[dtype], block, DEV, slack=256)) for _ in range(2))
+    table = OracleTable(one.units, dtype, block, one.cache_bytes, one.msg_bytes)
+    gen = wl.make_generator(31 * block + dtype)
+    w = [wl.init_weights(one.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    for model, kw in (("clustered", {"f": 0.1}), ("inject", {"c": 0.9}), ("inject", {"c": 0.0})):
+        step = wl.step_clustered if model == "clustered" else wl.inject_exponent_changes
+        w.append(step(w[-1], gen, **kw))
+    bits = [wl.as_bits(x) for x in w]
+    dev = [to_dev_bytes(b, DEV) for b in bits]
+    table.init_caches(bits[0])
+    for codec in (one, three):
+        codec.init_caches(dev[0])
+    for t in (1, 2, 3):
+        exp = table.step(bits[t])
+        launches0 = ciera.kernel_launch_count()
+        one.step(dev[t])
+        assert ciera.kernel_launch_count() - launches0 == 1
+        _three_calls(three, dev[t])
+        torch.cuda.synchronize()
+        for codec in (one, three):
+            codec.check_status()
+            compare_step(codec, exp, bits[t], f"t={t}")
+            compare_caches(codec, table, f"t={t}")
+            compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+    # the receiver's cache out of step with the sender's
+    other = to_dev_bytes(wl.as_bits(wl.init_weights(w[0].numel(), NAME[dtype], gen)), DEV)
+    for codec in (one, three):
+        ciera.cache_init(codec.plan, codec.receiver_cache, other)
+    one.step(dev[1])
+    _three_calls(three, dev[1])
+    torch.cuda.synchronize()
+    for codec in (one, three):
+        codec.check_status()
+        codec.canaries.check("receiver out of step")
+    for name in STATE:
+        assert torch.equal(getattr(one, name), getattr(three, name)), name
+    assert not torch.equal(one.weights_out[: dev[1].numel()], dev[1])
+    for u, n in zip(one.units, one.wire_bytes.tolist()):
+        lo = int(u["msg_off"])
+        for name in ("msg_send", "msg_recv"):
+            assert torch.equal(getattr(one, name)[lo : lo + n], three.msg_send[lo : lo + n]), name
+
+
+def test_in_place():
+    """Reconstructed weights may overwrite the weights."""
+    from paper_2609_04609_b200 import runtime
+
+    codec = runtime.LayerCodec.from_tensors(SIZES, 2, "bf16", 512, DEV)
+    gen = wl.make_generator(5)
+    w0 = wl.init_weights(codec.weights_bytes // 2, "bf16", gen)
+    w1 = wl.step_clustered(w0, gen, f=0.3)
+    codec.init_caches(to_dev_bytes(wl.as_bits(w0), DEV))
+    buf = to_dev_bytes(wl.as_bits(w1), DEV)
+    want = buf.clone()
+    codec.step(buf, buf)
+    torch.cuda.synchronize()
+    codec.check_status()
+    assert torch.equal(buf, want)
