@@ -178,6 +178,12 @@ def pipelined_step(layers: List[LayerCodec], weights: List[torch.Tensor], outs: 
 class LayerPipeline:
     """A stack of layers stepped repeatedly on two streams (see ``pipelined_step``).
 
+    A step that needs neither timers nor a stage between sender and receiver (entropy, hashed sender) runs
+    every layer in one launch (``LayerCodec.step``): both sides of a layer then share one pass over memory, which
+    is worth more than two layers' kernels side by side, each of them bound by memory (four OLMoE-shaped bf16
+    layers: 2.79 ms on two streams, 2.26 ms like this).  The launches go to the receiver's stream, between what
+    either stream held before and what it is given next.
+
     Across iterations it keeps the dependency that the layers' buffers impose: the sender side of
     layer l in iteration i+1 (it overwrites the layer's messages, lengths and scratch) starts only
     after the decode of layer l in iteration i has finished.  ``timers``, if given, collects six CUDA
@@ -201,6 +207,17 @@ class LayerPipeline:
     def step(self, weights: List[torch.Tensor], outs: Optional[List[Optional[torch.Tensor]]] = None,
              timers: Optional[list] = None) -> None:
         s_enc, s_dec = self.s_enc, self.s_dec
+        if self.layers and timers is None and not self.entropy and all(
+                getattr(c, "hash_cache", None) is None for c in self.layers):
+            if not self.serial:
+                self.sent[0].record(s_enc)
+                s_dec.wait_event(self.sent[0])
+            for l, (codec, w) in enumerate(zip(self.layers, weights)):
+                codec.step(w, None if outs is None else outs[l], s_dec)
+            if not self.serial:
+                self.decoded[0].record(s_dec)
+                s_enc.wait_event(self.decoded[0])
+            return
         for l, (codec, w) in enumerate(zip(self.layers, weights)):
             if not self.serial:
                 s_enc.wait_event(self.decoded[l])
