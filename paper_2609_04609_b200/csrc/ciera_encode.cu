@@ -1400,8 +1400,8 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     uint32_t nt = (uint32_t)p->tiles.size();
     const uint32_t grid = nt < (uint32_t)limit ? nt : (uint32_t)limit;
     const uint2* seq_runs = p->seq_runs_dev;
-    uint32_t n_runs = (uint32_t)p->seq_runs.size();
-    uint32_t spread_first = p->seq_first.back();
+    uint32_t n_runs = p->spread_all ? 0u : (uint32_t)p->seq_runs.size();
+    uint32_t spread_first = p->spread_all ? 0u : p->seq_first.back();
     uint32_t log2b = p->log2b;
     const uint8_t* w = (const uint8_t*)weights_dev;
     uint8_t* c = (uint8_t*)sender_cache_dev;
@@ -1412,7 +1412,7 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     unsigned int* done = ticket + 1;
     const unsigned long long* tile_hash = HASH ? p->tile_hash_dev : nullptr;
     const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
-    const bool has_spread = p->seq_first.back() < nt;  // tiles of longer units: look-back between blocks
+    const bool has_spread = spread_first < nt;  // look-back between blocks
     cudaError_t e;
     if (has_spread) {
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the

@@ -124,11 +124,18 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     // processing order: short units by descending tile count (ties in table order), then the rest
     auto tiles_of = [&](uint32_t u) { return (uint32_t)((units_host[u].n_values + kTileValues - 1) / kTileValues); };
     std::vector<uint32_t> shorts, longs;
+    uint64_t short_tiles = 0;
+    uint32_t longest_short = 0;
     for (uint32_t u = 0; u < n_units; ++u) {
         const uint32_t nt = tiles_of(u);
         if (nt == 0) continue;
         (nt <= kSeqMaxTiles ? shorts : longs).push_back(u);
+        if (nt <= kSeqMaxTiles) {
+            short_tiles += nt;
+            longest_short = std::max(longest_short, nt);
+        }
     }
+    p->spread_all = short_tiles < (uint64_t)kSpreadShare * longest_short;
     std::stable_sort(shorts.begin(), shorts.end(), [&](uint32_t a, uint32_t b) { return tiles_of(a) > tiles_of(b); });
     auto emit = [&](uint32_t u) {
         const ciera_unit& un = units_host[u];

@@ -136,6 +136,13 @@ __host__ __device__ inline size_t workspace_total_bytes(size_t nt) {
 // a short unit tile after tile (the tile's place in the payload is then a running sum inside the
 // block) and spreads everything else tile by tile over all blocks.
 constexpr uint32_t kSeqMaxTiles = 32;
+// That needs many more units than thread blocks: a table whose short units' tiles are fewer than kSpreadShare times
+// the longest of these units would leave most of the GPU idle while a few blocks work through their units, so the
+// encode kernel spreads all tiles of such a table.  197 = 2/3 of the 296 thread blocks that a B200
+// holds, where the two ways cross.  Whole step, bf16, units of 16 tiles, in runs / spread: 64 tiles 26.4 / 7.7 us,
+// 768 tiles 26.2 / 12.9, 2048 tiles 40.0 / 34.6, 3072 tiles 47.1 / 50.0, 49152 tiles 570 / 625; units of 32 tiles:
+// 1536 tiles 50.4 / 23.5, 4096 tiles 76.5 / 63.0.
+constexpr uint32_t kSpreadShare = 197;
 // A short unit is handed out in runs of this many tiles (all units' first runs, then all second runs, ...): the
 // smaller the piece of work a thread block draws, the less the blocks differ in when they finish.  A run's first
 // tile takes its payload offset from the status word that the run before it left.  A multiple of 4, so that tiles
@@ -168,6 +175,7 @@ struct ciera_plan {
     struct SeqRun {
         uint32_t lo, hi;               // tiles [lo, hi) of the table
     };
+    bool spread_all = false;           // the short units' tiles are spread too (kSpreadShare)
     std::vector<SeqRun> seq_runs;      // the short units' runs of tiles in the order they are handed out
     std::vector<uint32_t> unit_first;  // first tile of every unit (0xffffffff: a unit without values)
     std::vector<uint64_t> hash_base;   // index of every unit's first block in a per-block hash cache

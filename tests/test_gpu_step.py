@@ -87,3 +87,29 @@ def test_in_place():
     torch.cuda.synchronize()
     codec.check_status()
     assert torch.equal(buf, want)
+
+
+@pytest.mark.parametrize("block", [1, 8, 64, 512, 2048, 4096])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_runs_of_short_units(dtype, block):
+    """Enough units of five tiles (a run of four, then a run of one) that they are handed out in runs rather than
+    spread tile by tile; the three calls, then the whole step, against the oracle."""
+    from paper_2609_04609_b200 import runtime
+
+    sizes = [8192 * 5, 8192 * 4 + 1, 8192 * 5 - 1, 8192 * 4 + 4100] * 55 + [100, 8192 * 33 + 5]
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(7 * block + dtype, DEV)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    w += [wl.step_clustered(w[0], gen, f=0.3)]
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    for t, step in ((1, _three_calls), (0, lambda c, x: c.step(x))):
+        exp = table.step(bits[t])
+        step(codec, to_dev_bytes(bits[t], DEV))
+        torch.cuda.synchronize()
+        codec.check_status()
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        compare_recon(codec, exp, bits[t], dtype, f"t={t}")
