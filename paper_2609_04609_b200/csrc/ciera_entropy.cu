@@ -107,7 +107,7 @@ __device__ __forceinline__ void normalise_model(const uint32_t* h, uint64_t P, u
     {
         uint32_t v = 0;
         if (h[tid]) {
-            v = (uint32_t)((uint64_t)h[tid] * kProbScale / P);
+            v = P < (1ull << 20) ? h[tid] * kProbScale / (uint32_t)P : (uint32_t)((uint64_t)h[tid] * kProbScale / P);
             if (v == 0) v = 1;
         }
         f[tid] = (uint16_t)v;
@@ -134,112 +134,164 @@ __device__ __forceinline__ void normalise_model(const uint32_t* h, uint64_t P, u
     __syncthreads();
 }
 
-// Starts c[] and reciprocals from final frequencies.  Ends with a barrier.
-// x / f through a multiplication: rcp = ceil(2^64 / f) exceeds 2^64 / f by less than 1, so for
-// x < 2^32 the product x * rcp / 2^64 exceeds x / f by less than 2^-32 -- too little to reach the next
-// integer, because the fraction of x / f is at most 1 - 1/4096.  (f = 1 is handled apart.)
-// The coder reads one 16-byte entry per symbol: {rcp low, rcp high, f | c << 16, 0}.
-__device__ __forceinline__ void encoder_tables(const uint16_t* f, uint4* enc, uint32_t tid) {
-    const unsigned long long rcp = f[tid] > 1 ? (~0ull) / f[tid] + 1ull : 0ull;
-    enc[tid].x = (uint32_t)rcp;
-    enc[tid].y = (uint32_t)(rcp >> 32);
-    enc[tid].w = 0u;
+// The coder's tables from final frequencies.  Ends with a barrier.
+// q = x / f for x < f * 2^20 <= 2^32 is one 32-bit multiplication and a shift.  With s = floor(log2 f), P = 2^(32 + s),
+// m = floor(P / f) and e = (m + 1) * f - P:
+//   f = 1                     m = 2^32 - 1 gives x - 1 (x > 0), the missing 1 * (4096 - f) goes into c
+//   f a power of two          m = 2^31, shift s - 1
+//   f * 2^20 * e <= P         q = ((m + 1) * x) / P, the round-up reciprocal (all f < 2^11, most others)
+//   else                      q = (m * (x + 1)) / P, the round-down one: exact if f * 2^20 * (f - e) <= P, which
+//                             follows from e > P / (f * 2^20) >= 2^23 / f for 2^11 < f < 2^12
+// At most one symbol is of the last kind; whether there is one comes back (the same in all threads).  An entry of 16
+// bytes holds what a coder step needs:
+//   {multiplier, largest x below f * 2^20, c, (4096 - f) << 5 | shift, bit 31: x + 1}
+__device__ __forceinline__ bool encoder_tables(const uint16_t* f, uint4* enc, uint32_t tid) {
+    const uint32_t fs = f[tid] ? f[tid] : 1u;
+    uint32_t s = 31u - (uint32_t)__clz(fs), m = 0xFFFFFFFFu, plus = 0u;
+    if (fs & (fs - 1u)) {
+        // floor(2^(32 + s) / f) in two 32-bit divisions: s + 16 < 28 and the first remainder is below 2^12
+        const uint32_t a = 1u << (s + 16u), q1 = a / fs, r1 = (a - q1 * fs) << 16, q0 = r1 / fs;
+        m = (q1 << 16) + q0;
+        const uint32_t e = fs - (r1 - q0 * fs);  // (m + 1) * f - P
+        if (((unsigned long long)fs << 20) * e <= (1ull << (32u + s)))
+            m += 1u;
+        else
+            plus = 1u;
+    } else if (s) {
+        m = 0x80000000u;
+        s -= 1u;
+    }
+    enc[tid].x = m;
+    enc[tid].y = (uint32_t)(((unsigned long long)fs << 20) - 1ull);
+    enc[tid].w = ((kProbScale - fs) << 5) | s | (plus << 31);
     if (tid < 32) {
         uint32_t local[8], total;
         const uint32_t base = warp_prefix256(f, tid, local, total);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) enc[8 * tid + i].z = (uint32_t)f[8 * tid + i] | ((base + local[i]) << 16);
+        for (int i = 0; i < 8; ++i) enc[8 * tid + i].z = base + local[i] + (f[8 * tid + i] == 1 ? kProbScale - 1u : 0u);
     }
-    __syncthreads();
+    return __syncthreads_or((int)plus) != 0;
 }
 
 // One warp codes one segment: src[0, n) -> slot (32 states, then the words).  Returns the word count.
-__device__ __forceinline__ uint32_t encode_segment(const uint8_t* src, uint32_t n, uint8_t* stage, const uint4* enc,
-                                                   uint8_t* slot, uint32_t lane) {
-    for (uint32_t i = lane * 16; i < n; i += 32 * 16) {
-        if (i + 16 <= n) {
-            *reinterpret_cast<uint4*>(stage + i) = *reinterpret_cast<const uint4*>(src + i);
-        } else {
-            for (uint32_t k = i; k < n; ++k) stage[k] = src[k];
-        }
-    }
-    __syncwarp();
-    uint16_t* words = reinterpret_cast<uint16_t*>(slot + 4 * 32);
+// Bound by instruction issue.  A lane's symbols lie 32 bytes apart; four steps' worth of a warp (128 bytes) come in
+// with one load, a word per lane, and are turned into a word of four successive symbols per lane by a 4 x 4
+// transposition inside every quad of lanes (two exchanges, two byte permutes).  Sixteen steps are loaded ahead of the
+// sixteen in work.  (With a staged copy of the segment, a byte load per step and a 64-bit reciprocal: 0.180 ms per
+// OLMoE-shaped layer, B = 512, q = 0.22; like this 0.154.  4 / 6 thread blocks per SM instead of 5: 0.168 / 0.190.)
+// `src` is 4-byte aligned.  PLUS: the tables hold a symbol whose quotient takes x + 1.
+template <bool PLUS>
+__device__ __forceinline__ uint32_t encode_segment(const uint8_t* src, uint32_t n, const uint4* enc, uint8_t* slot,
+                                                   uint32_t lane) {
+    uint16_t* const words = reinterpret_cast<uint16_t*>(slot + 4 * 32);
     uint32_t x = kRansL, nw = 0;
     const uint32_t below = (1u << lane) - 1u;
-    const uint32_t enc_a = (uint32_t)__cvta_generic_to_shared(enc);
-    const uint32_t stage_a = (uint32_t)__cvta_generic_to_shared(stage) + lane;
-    // one coder step of this lane for the symbol at byte 32 t + lane of the segment
-    auto step = [&](uint32_t t, bool has) {
-        uint32_t s = 0;
-        if (has) asm volatile("ld.shared.u8 %0, [%1];" : "=r"(s) : "r"(stage_a + 32u * t) : "memory");
-        uint4 en;
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(en.x), "=r"(en.y), "=r"(en.z), "=r"(en.w)
-                     : "r"(enc_a + (s << 4))
-                     : "memory");
-        const uint32_t fs = en.z & 0xFFFFu, cs = en.z >> 16;
-        const bool emit = has && (x >> 20) >= fs;  // x >= f * 2^20
+    // one coder step of this lane for symbol s
+    auto step = [&](uint32_t s, bool has) {
+        const uint4 en = enc[s];
+        const bool emit = has && x > en.y;  // x >= f * 2^20
         const uint32_t votes = __ballot_sync(0xffffffffu, emit);
         if (emit) {
             words[nw + __popc(votes & below)] = (uint16_t)x;
             x >>= 16;
         }
         nw += __popc(votes);
-        if (has) {
-            const unsigned long long rcp = (unsigned long long)en.x | ((unsigned long long)en.y << 32);
-            const uint32_t q = fs > 1 ? (uint32_t)__umul64hi((unsigned long long)x, rcp) : x;
-            x = q * kProbScale + (x - q * fs) + cs;
-        }
+        // x / f (the shift takes the low 5 bits of its amount), then q * 4096 + x mod f + c
+        const uint32_t q = __funnelshift_r(__umulhi(PLUS ? x + (en.w >> 31) : x, en.x), 0u, en.w);
+        const uint32_t y = x + en.z + q * (PLUS ? (en.w >> 5) & 0x1FFFu : en.w >> 5);
+        x = has ? y : x;
     };
-    uint32_t t = (n + 31u) >> 5;
-    if (n & 31u) {  // the last, incomplete step comes first (the coder walks backwards)
-        --t;
-        step(t, lane < (n & 31u));
+    // the rows of 32 symbols behind the last whole block of 16 rows come first (the coder walks backwards)
+    const uint32_t blocks = n >> 9;
+    for (uint32_t t = (n + 31u) >> 5; t-- > 16u * blocks;) {
+        const uint32_t at = 32u * t + lane;
+        step(at < n ? src[at] : 0u, at < n);
     }
-    while (t-- > 0) step(t, true);
+    if (blocks) {
+        // lane 4 c + j loads row j of a group of four rows, columns 4 c .. 4 c + 3
+        const uint32_t* from = reinterpret_cast<const uint32_t*>(src) + 128u * (blocks - 1u) + 8u * (lane & 3u) + (lane >> 2);
+        const uint32_t sel1 = (lane & 1u) ? 0x3715u : 0x6240u, sel2 = (lane & 2u) ? 0x3276u : 0x5410u;
+        uint32_t next[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) next[i] = from[32 * i];
+        for (uint32_t b = blocks; b != 0u;) {
+            uint32_t cur[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cur[i] = next[i];
+            from -= 128;
+            if (--b) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) next[i] = from[32 * i];
+            }
+#pragma unroll
+            for (int i = 3; i >= 0; --i) {
+                uint32_t v = cur[i];
+                v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 1), sel1);
+                v = __byte_perm(v, __shfl_xor_sync(0xffffffffu, v, 2), sel2);
+                step(v >> 24, true);
+                step(__byte_perm(v, 0u, 0x4442u), true);
+                step(__byte_perm(v, 0u, 0x4441u), true);
+                step(v & 0xFFu, true);
+            }
+        }
+    }
     reinterpret_cast<uint32_t*>(slot)[lane] = x;
     if (lane == 0 && (nw & 1u)) words[nw] = 0;
     __syncwarp();
     return nw;
 }
 
-// Receiver tables from the transmitted frequencies (f[] already in shared memory and synced):
-// starts c[], then one word per slot: symbol | (f - 1) << 8 | (slot - c) << 20.  Returns false (in every
-// thread) if the table does not sum to 4096.  The owner of a slot is the last symbol that starts at or
-// below it (symbols that do not occur share their start with the next one, or start at 4096 behind the
-// last occurring one).
-__device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, uint32_t* tab, uint32_t* flag, uint32_t tid) {
+// Receiver tables from the transmitted frequencies (f[] already in shared memory and synced): one word per slot:
+// (slot - c) | symbol << 12 | (f - 1) << 20.  Returns false (in every thread) if the table does not sum to 4096.
+// The owner of a slot is the last symbol that occurs and starts at or below it.  Every symbol that occurs marks the
+// slot it starts at with its number + 1; a warp then carries the largest mark forward over its 512 slots, 128 at a
+// time.  (A search per thread and a walk over its 16 slots took three times the instructions, most of them diverged.)
+//   base[s] = symbol << 12 | (f - 1) << 20, less c, so that a slot's word is base[owner] + slot
+__device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, uint32_t* base, uint32_t* tab, uint32_t* flag,
+                                               uint32_t tid) {
+    const uint32_t lane = tid & 31u, warp = tid >> 5;
+    uint4* const tab4 = reinterpret_cast<uint4*>(tab);
+#pragma unroll
+    for (int i = 0; i < (int)(kProbScale / 4) / kEntThreads; ++i) tab4[tid + i * kEntThreads] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < 32) {
         uint32_t local[8], total;
-        const uint32_t base = warp_prefix256(f, tid, local, total);
+        const uint32_t first = warp_prefix256(f, tid, local, total);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) c[8 * tid + i] = (uint16_t)min(base + local[i], kProbScale);
+        for (int i = 0; i < 8; ++i) c[8 * tid + i] = (uint16_t)min(first + local[i], kProbScale);
         if (tid == 0) *flag = total == kProbScale ? 1u : 0u;
     }
     __syncthreads();
     if (*flag == 0) return false;
-    // thread t fills slots 16 t .. 16 t + 15: a binary search for the owner of the first, then a walk
-    {
-        uint32_t slot = tid * 16;
-        uint32_t lo = 0, hi = 255;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (c[mid] <= slot)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        uint32_t cs = c[lo], fm1 = (uint32_t)f[lo] - 1u;
-        for (uint32_t k = 0; k < 16; ++k, ++slot) {
-            if (slot - cs > fm1) {  // past the owner's last slot: on to the next symbol that occurs
-                do ++lo; while (lo < 255u && c[lo + 1] <= slot);
-                cs = c[lo];
-                fm1 = (uint32_t)f[lo] - 1u;
-            }
-            // the owner occurs (f >= 1, its slots are [c, c + f)): the sum is 4096 and every slot has one
-            tab[slot] = lo | (fm1 & 0xFFFu) << 8 | ((slot - cs) & 0xFFFu) << 20;
-        }
+    const uint32_t start = c[tid];
+    base[tid] = (tid << 12 | ((uint32_t)f[tid] - 1u) << 20) - start;
+    if (f[tid]) tab[start] = tid + 1u;  // f >= 1: the start is a slot, and no other symbol's start
+    // the owner of the slot in front of the warp's first one (mark 0: there is none)
+    const uint32_t slot0 = warp * (kProbScale / kEntWarps);
+    uint32_t carry = 0;
+#pragma unroll
+    for (uint32_t s = lane; s < 256u; s += 32u)
+        if (f[s] && c[s] < slot0) carry = s + 1u;
+    carry = __reduce_max_sync(0xffffffffu, carry);
+    __syncthreads();
+#pragma unroll
+    for (uint32_t r = 0; r < kProbScale / kEntWarps / 128u; ++r) {
+        const uint32_t slot = slot0 + 128u * r + 4u * lane;
+        uint4 v = tab4[slot >> 2];
+        v.y = max(v.x, v.y);
+        v.z = max(v.y, v.z);
+        v.w = max(v.z, v.w);
+        uint32_t incl = v.w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) incl = max(incl, __shfl_up_sync(0xffffffffu, incl, o));
+        uint32_t before = __shfl_up_sync(0xffffffffu, incl, 1);
+        before = max(lane ? before : 0u, carry);
+        carry = max(carry, __shfl_sync(0xffffffffu, incl, 31));
+        // (the sum is 4096, so every slot has an owner: slot 0 is the first occurring symbol's start)
+        v.x = base[max(v.x, before) - 1u] + slot;
+        v.y = base[max(v.y, before) - 1u] + slot + 1u;
+        v.z = base[max(v.z, before) - 1u] + slot + 2u;
+        v.w = base[max(v.w, before) - 1u] + slot + 3u;
+        tab4[slot >> 2] = v;
     }
     __syncthreads();
     return true;
@@ -251,39 +303,44 @@ __device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, u
 // next steps); without a staged copy the kernel's shared memory is the slot table, and many warps per
 // SM hide the latency of a line's first touch.
 // Returns false (in every lane) if the words run out, are left over, or a lane does not end in the
-// start state.
+// start state.  (Whether the words have run out is looked at after every four steps: they take 128 words at most, so a
+// damaged section makes a lane read at most 256 bytes in front of its words -- other parts of the same message.)
+// (Layer as above: 0.190 ms with the check in every step and a slot's owner searched for, 0.150 like this.)
 __device__ __forceinline__ bool decode_segment(const uint8_t* coded, uint32_t snw, uint32_t n, const uint32_t* tab,
                                                uint8_t* out, uint32_t lane) {
     const uint16_t* words = reinterpret_cast<const uint16_t*>(coded + 4 * 32);
     for (uint32_t i = lane * 64u; i < snw; i += 32u * 64u)  // bring the word list towards the SM, a line per lane
         asm volatile("prefetch.global.L2 [%0];" ::"l"(words + i));
-    const uint32_t tab_a = (uint32_t)__cvta_generic_to_shared(tab);
-    uint32_t x = reinterpret_cast<const uint32_t*>(coded)[lane], ptr = snw;
+    uint32_t x = reinterpret_cast<const uint32_t*>(coded)[lane];
+    int32_t ptr = (int32_t)snw;
     const uint32_t below = (1u << lane) - 1u;
-    const uint32_t full = n >> 5;  // steps in which every lane has a symbol
     uint8_t* o = out + lane;
-    bool ok = true;
-    // one step: `has` = this lane decodes a symbol in it
-    auto step = [&](bool has) -> bool {
-        bool need = false;
+    auto step = [&](uint8_t* dst, bool has) {  // `has`: this lane decodes a symbol in this step
+        const uint32_t en = tab[x & (kProbScale - 1u)];
+        const uint32_t hi = x >> kProbBits;
+        const uint32_t y = (en >> 20) * hi + hi + (en & 0xFFFu);
         if (has) {
-            uint32_t en;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(en) : "r"(tab_a + ((x & (kProbScale - 1u)) << 2)) : "memory");
-            *o = (uint8_t)en;
-            x = (((en >> 8) & 0xFFFu) + 1u) * (x >> kProbBits) + (en >> 20);
-            need = x < kRansL;
+            *dst = (uint8_t)(en >> 12);
+            x = y;
         }
-        o += 32;
+        const bool need = has && y < kRansL;
         const uint32_t votes = __ballot_sync(0xffffffffu, need);
-        const uint32_t k_need = __popc(votes);
-        if (k_need > ptr) return false;  // the words run out (the same in every lane)
-        ptr -= k_need;
-        if (need) x = (x << 16) | words[ptr + __popc(votes & below)];
-        return true;
+        ptr -= __popc(votes);
+        if (need) x = __byte_perm((uint32_t)words[ptr + (int32_t)__popc(votes & below)], x, 0x5410u);
     };
-    for (uint32_t t = 0; t < full && ok; ++t) ok = step(true);
-    if (ok && (n & 31u)) ok = step(lane < (n & 31u));
-    ok = ok && ptr == 0 && !__any_sync(0xffffffffu, x != kRansL);
+    const uint32_t full = n >> 5;  // steps in which every lane has a symbol
+    uint32_t t = 0;
+    for (; t + 4u <= full; t += 4u) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) step(o + 32 * k, true);
+        o += 128;
+        if (ptr < 0) return false;  // the words ran out (the same in every lane)
+    }
+    for (; 32u * t < n; ++t) {
+        step(o, 32u * t + lane < n);
+        o += 32;
+    }
+    const bool ok = ptr == 0 && !__any_sync(0xffffffffu, x != kRansL);
     __syncwarp();
     return ok;
 }
@@ -403,11 +460,7 @@ __global__ void __launch_bounds__(kEntThreads, 5)
 entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long long* __restrict__ seg_base,
                       int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
                       uint8_t* scratch_slots, uint32_t* scratch_nw, uint8_t* scratch_sym) {
-    __shared__ __align__(16) uint8_t s_seg[kEntWarps][kSegment];  // a warp's segment of symbols
-    // the warps' private histograms are needed before the segments are staged, the two small lists of
-    // step 4 after: all of them lie in the first part of s_seg
-    uint32_t (*const s_hist)[256] = reinterpret_cast<uint32_t (*)[256]>(&s_seg[0][0]);
-    static_assert(sizeof(uint32_t) * 256 * kEntWarps <= sizeof(uint8_t) * kSegment * kEntWarps, "histograms overlay the stages");
+    __shared__ uint32_t s_hist[kEntWarps][256];  // the warps' private histograms, then the two small lists of step 4
     __shared__ uint16_t s_f[256];
     __shared__ uint4 s_enc[256];
     __shared__ uint32_t s_scan[kEntWarps];
@@ -448,14 +501,16 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     }
     __syncthreads();
     normalise_model(s_hist[0], P, s_f, tid);
-    encoder_tables(s_f, s_enc, tid);
+    const bool plus = encoder_tables(s_f, s_enc, tid);
 
     // 3. segments: warp w codes segments w, w + 8, ... into the unit's slots of the scratch
     const unsigned long long slot0 = seg_base[unit];
     for (uint32_t g = warp; g < nseg; g += kEntWarps) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
-        const uint32_t nw = encode_segment(src + (uint64_t)g * kSegment, n, s_seg[warp], s_enc,
-                                           scratch_slots + (slot0 + g) * kSegSlot, lane);
+        const uint8_t* const seg = src + (uint64_t)g * kSegment;
+        uint8_t* const slot = scratch_slots + (slot0 + g) * kSegSlot;
+        const uint32_t nw = plus ? encode_segment<true>(seg, n, s_enc, slot, lane)
+                                 : encode_segment<false>(seg, n, s_enc, slot, lane);
         if (lane == 0) {
             scratch_nw[slot0 + g] = nw;
             atomicAdd(&s_total, (unsigned long long)segment_bytes(nw));
@@ -588,7 +643,6 @@ entropy_long_encode_kernel(const ciera_unit* __restrict__ units, const unsigned 
                            const uint4* __restrict__ chunks, int dt, uint32_t log2b, const uint8_t* msgs,
                            const unsigned long long* wire_bytes, uint8_t* recs, uint8_t* scratch_slots,
                            uint32_t* scratch_nw, const uint8_t* scratch_sym) {
-    __shared__ __align__(16) uint8_t s_seg[kEntWarps][kSegment];
     __shared__ uint16_t s_f[256];
     __shared__ uint4 s_enc[256];
     __shared__ unsigned long long s_total;
@@ -603,13 +657,15 @@ entropy_long_encode_kernel(const ciera_unit* __restrict__ units, const unsigned 
     s_f[tid] = long_model(recs, ch.z)[tid];
     if (tid == 0) s_total = 0;
     __syncthreads();
-    encoder_tables(s_f, s_enc, tid);
+    const bool plus = encoder_tables(s_f, s_enc, tid);
     const uint8_t* pay = HALF ? scratch_sym + un.cache_off : msgs + un.msg_off + payoff;  // the symbols
     const unsigned long long slot0 = seg_base[ch.x];
     for (uint32_t g = ch.y + warp; g < g_end; g += kEntWarps) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
-        const uint32_t nw = encode_segment(pay + (uint64_t)g * kSegment, n, s_seg[warp], s_enc,
-                                           scratch_slots + (slot0 + g) * kSegSlot, lane);
+        const uint8_t* const seg = pay + (uint64_t)g * kSegment;
+        uint8_t* const slot = scratch_slots + (slot0 + g) * kSegSlot;
+        const uint32_t nw = plus ? encode_segment<true>(seg, n, s_enc, slot, lane)
+                                 : encode_segment<false>(seg, n, s_enc, slot, lane);
         if (lane == 0) {
             scratch_nw[slot0 + g] = nw;
             atomicAdd(&s_total, (unsigned long long)segment_bytes(nw));
@@ -683,8 +739,9 @@ entropy_long_copy_kernel(const ciera_unit* __restrict__ units, const unsigned lo
 // units of up to kLongSegs segment slots: one thread block per unit, start to end
 
 struct DecodeShared {
-    uint32_t tab[kProbScale];      // slot -> symbol | (f - 1) << 8 | (slot - c) << 20
+    uint32_t tab[kProbScale];      // slot -> (slot - c) | symbol << 12 | (f - 1) << 20
     uint16_t f[256], c[256];
+    uint32_t base[256];            // per symbol: see decoder_tables
     uint32_t off[kEntThreads];     // per segment: byte offset in the data part
     uint32_t nw[kEntThreads];      //              word count
     uint32_t scan[kEntWarps];
@@ -727,7 +784,7 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log
     }
     sh.f[tid] = tid < hdr / 2u ? reinterpret_cast<const uint16_t*>(pay)[tid] : (uint16_t)0;
     __syncthreads();
-    if (!decoder_tables(sh.f, sh.c, sh.tab, &sh.flag, tid)) {
+    if (!decoder_tables(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
         if (tid == 0) raise_corrupt(status);
         return;
     }
@@ -855,7 +912,7 @@ entropy_long_decode_kernel(const ciera_unit* __restrict__ units, const unsigned 
     sh.f[tid] = tid < hdr / 2u ? reinterpret_cast<const uint16_t*>(pay)[tid] : (uint16_t)0;
     if (tid == 0) sh.bad = 0;
     __syncthreads();
-    if (!decoder_tables(sh.f, sh.c, sh.tab, &sh.flag, tid)) {
+    if (!decoder_tables(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
         if (tid == 0) {
             st->bad = 1;
             raise_corrupt(status);
