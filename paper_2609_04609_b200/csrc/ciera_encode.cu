@@ -943,7 +943,7 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
 template <int DT, bool FINE, int HASH, bool STEP>
 __global__ void __launch_bounds__(kEncodeThreads, kEncodeBlocksPerSM<DT, STEP>)
 encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
-              uint32_t spread_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
+              uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
               unsigned int* unit_ticket, unsigned int* blocks_done, int32_t* status,
               const unsigned long long* __restrict__ tile_hash, StepTwins tw) {
@@ -1333,6 +1333,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             }
         }
     }
+    // (clear_first: a step in parts leaves the status words to the parts that follow, and the last part empties all)
     // The scratch is handed back the way it was found, all zero: the hand-off words of the runs were emptied by
     // their readers, the run counter by its last draw; the status words of the spread tiles (read by any number
     // of later tiles) and the counter of finished blocks are emptied here by the block that finishes last.
@@ -1344,7 +1345,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (uint32_t t = spread_first + tid; t < n_tiles; t += kEncodeThreads) st_status(tile_status + t, 0ull);
+        for (uint32_t t = clear_first + tid; t < n_tiles; t += kEncodeThreads) st_status(tile_status + t, 0ull);
         if (tid == 0) atomicExch(blocks_done, 0u);
     }
 }
@@ -1389,26 +1390,36 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
 
 // `scratch`: one status word per tile, then the run counter and the counter of finished blocks; all zero when
 // the kernel starts, and all zero again when it has finished without a device-side error.
+// part of a step: the tiles [lo, hi) of `tiles`, all of them spread; the last part empties the status words
+struct EncodePart {
+    const TileDesc* tiles;
+    uint32_t lo, hi;
+    bool last;
+};
 template <int DT, bool FINE, int HASH = 0, bool STEP = false>
 static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
-                         cudaStream_t s, StepTwins tw = StepTwins{0, 0, 0}) {
+                         cudaStream_t s, StepTwins tw = StepTwins{0, 0, 0}, const EncodePart* part = nullptr) {
     int limit = 0;
     const int rc = encode_grid_limit<DT, FINE, HASH, STEP>(p->log2b, &limit);
     if (rc) return rc;
-    const TileDesc* tiles = p->tiles_dev;
-    uint32_t nt = (uint32_t)p->tiles.size();
-    const uint32_t grid = nt < (uint32_t)limit ? nt : (uint32_t)limit;
+    const TileDesc* tiles = part ? part->tiles : p->tiles_dev;
+    const uint32_t all_tiles = (uint32_t)p->tiles.size();
+    uint32_t nt = part ? part->hi : all_tiles;
+    const uint32_t to_do = part ? part->hi - part->lo : all_tiles;
+    const uint32_t grid = to_do < (uint32_t)limit ? to_do : (uint32_t)limit;
     const uint2* seq_runs = p->seq_runs_dev;
-    uint32_t n_runs = p->spread_all ? 0u : (uint32_t)p->seq_runs.size();
-    uint32_t spread_first = p->spread_all ? 0u : p->seq_first.back();
+    const bool spread_all = part || p->spread_all;
+    uint32_t n_runs = spread_all ? 0u : (uint32_t)p->seq_runs.size();
+    uint32_t spread_first = part ? part->lo : spread_all ? 0u : p->seq_first.back();
+    uint32_t clear_first = !part ? spread_first : part->last ? 0u : nt;
     uint32_t log2b = p->log2b;
     const uint8_t* w = (const uint8_t*)weights_dev;
     uint8_t* c = (uint8_t*)sender_cache_dev;
     uint8_t* m = (uint8_t*)messages_dev;
     unsigned long long* wb = (unsigned long long*)wire_bytes_dev;
     unsigned long long* ts = (unsigned long long*)scratch;
-    unsigned int* ticket = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(nt));
+    unsigned int* ticket = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(all_tiles));
     unsigned int* done = ticket + 1;
     const unsigned long long* tile_hash = HASH ? p->tile_hash_dev : nullptr;
     const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
@@ -1417,13 +1428,13 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     if (has_spread) {
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
-        void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &log2b, &w, &c, &m, &wb, &changed_blocks_dev, &ts,
+        void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb, &changed_blocks_dev, &ts,
                         &ticket, &done, &status_dev, &tile_hash, &tw};
         e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads), args,
                                         smem, s);
     } else {
         encode_kernel<DT, FINE, HASH, STEP><<<grid, kEncodeThreads, smem, s>>>(
-            tiles, nt, seq_runs, n_runs, spread_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
+            tiles, nt, seq_runs, n_runs, spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
             tile_hash, tw);
         e = cudaGetLastError();
     }
@@ -1436,11 +1447,11 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
 template <int DT>
 static int launch_encode_of(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                             uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
-                            cudaStream_t s, const StepTwins* tw) {
+                            cudaStream_t s, const StepTwins* tw, const EncodePart* part) {
     auto launch = [&](auto fine, auto step) {
         return launch_encode<DT, decltype(fine)::value, 0, decltype(step)::value>(
             p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev, scratch, status_dev, s,
-            tw ? *tw : StepTwins{0, 0, 0});
+            tw ? *tw : StepTwins{0, 0, 0}, part);
     };
     if (is_fine(p->log2b)) return tw ? launch(std::true_type{}, std::true_type{}) : launch(std::true_type{}, std::false_type{});
     return tw ? launch(std::false_type{}, std::true_type{}) : launch(std::false_type{}, std::false_type{});
@@ -1448,12 +1459,12 @@ static int launch_encode_of(const ciera_plan* p, const void* weights_dev, void* 
 // (tw: the whole step; null: the sender's part alone)
 static int launch_encode_any(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                              uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
-                             cudaStream_t s, const StepTwins* tw = nullptr) {
+                             cudaStream_t s, const StepTwins* tw = nullptr, const EncodePart* part = nullptr) {
     auto* launch = p->dtype == CIERA_FP16   ? launch_encode_of<CIERA_FP16>
                    : p->dtype == CIERA_BF16 ? launch_encode_of<CIERA_BF16>
                                             : launch_encode_of<CIERA_FP32>;
     return launch(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev, scratch, status_dev, s,
-                  tw);
+                  tw, part);
 }
 
 // the sender with HashCache: blocks of 16 values and more (checked by the caller)
@@ -1519,14 +1530,21 @@ extern "C" int ciera_encode(const ciera_plan* p, const void* weights_dev, void* 
                              workspace_dev, status_dev, s);
 }
 
-extern "C" int ciera_step(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* msg_send_dev,
-                          void* msg_recv_dev, void* receiver_cache_dev, void* weights_out_dev, uint64_t* wire_bytes_dev,
-                          uint32_t* changed_blocks_dev, void* workspace_dev, int32_t* status_dev, void* stream) {
+static StepTwins step_twins(const void* weights, const void* sender_cache, const void* msg_send, const void* msg_recv,
+                            const void* receiver_cache, const void* weights_out) {
+    return StepTwins{(int64_t)((intptr_t)msg_recv - (intptr_t)msg_send),
+                     (int64_t)((intptr_t)receiver_cache - (intptr_t)sender_cache),
+                     (int64_t)((intptr_t)weights_out - (intptr_t)weights)};
+}
+
+// The checks of a step, and the outputs of units without tiles.
+int ciera::step_begin(const ciera_plan* p, const void* weights_dev, const void* sender_cache_dev, const void* msg_send_dev,
+                            const void* msg_recv_dev, const void* receiver_cache_dev, const void* weights_out_dev,
+                            uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, const void* workspace_dev, cudaStream_t s) {
     if (!p) return CIERA_ERR_INVALID_ARG;
     if (!p->tiles.empty() && !p->tiles_dev) return CIERA_ERR_NOT_BOUND;
     if (p->n_units == 0) return CIERA_OK;
     if (!wire_bytes_dev || !changed_blocks_dev) return CIERA_ERR_INVALID_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
     if (p->has_empty_units) {  // units without tiles: their outputs are written here
         cudaError_t e = cudaMemsetAsync(wire_bytes_dev, 0, sizeof(uint64_t) * p->n_units, s);
         if (e != cudaSuccess) return record_cuda_error(e);
@@ -1541,11 +1559,28 @@ extern "C" int ciera_step(const ciera_plan* p, const void* weights_dev, void* se
         misaligned16(msg_recv_dev) || misaligned16(receiver_cache_dev) || misaligned16(weights_out_dev) ||
         misaligned16(workspace_dev) || ((uintptr_t)wire_bytes_dev & 7u) || ((uintptr_t)changed_blocks_dev & 3u))
         return CIERA_ERR_MISALIGNED;
-    const StepTwins tw{(int64_t)((intptr_t)msg_recv_dev - (intptr_t)msg_send_dev),
-                       (int64_t)((intptr_t)receiver_cache_dev - (intptr_t)sender_cache_dev),
-                       (int64_t)((intptr_t)weights_out_dev - (intptr_t)weights_dev)};
+    return CIERA_OK;
+}
+
+extern "C" int ciera_step(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* msg_send_dev,
+                          void* msg_recv_dev, void* receiver_cache_dev, void* weights_out_dev, uint64_t* wire_bytes_dev,
+                          uint32_t* changed_blocks_dev, void* workspace_dev, int32_t* status_dev, void* stream) {
+    cudaStream_t s = (cudaStream_t)stream;
+    const int rc = step_begin(p, weights_dev, sender_cache_dev, msg_send_dev, msg_recv_dev, receiver_cache_dev,
+                                    weights_out_dev, wire_bytes_dev, changed_blocks_dev, workspace_dev, s);
+    if (rc || p->tiles.empty()) return rc;
+    const StepTwins tw = step_twins(weights_dev, sender_cache_dev, msg_send_dev, msg_recv_dev, receiver_cache_dev, weights_out_dev);
     return launch_encode_any(p, weights_dev, sender_cache_dev, msg_send_dev, wire_bytes_dev, changed_blocks_dev,
                              workspace_dev, status_dev, s, &tw);
+}
+
+// (the caller has checked the buffers as ciera_step does)
+int ciera::launch_step_part(const ciera_plan* p, const ciera_device_buffers* b, uint32_t lo, uint32_t hi, cudaStream_t s) {
+    const StepTwins tw = step_twins(b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->msg_recv_dev,
+                                    b->receiver_cache_dev, b->weights_out_dev);
+    const EncodePart part{p->tiles_by_address_dev, lo, hi, hi == (uint32_t)p->tiles.size()};
+    return launch_encode_any(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->wire_bytes_dev,
+                             b->changed_blocks_dev, b->workspace_dev, b->status_dev, s, &tw, &part);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -68,7 +68,7 @@ extern "C" size_t ciera_message_bytes(uint64_t n, int dtype, uint32_t block, uin
 
 namespace {
 struct ImageLayout {
-    size_t tiles, long_off, seq_off, hash_off, first_off, seg_off, units_off, elong_off, echunk_off, thash_off, runs_off, total;
+    size_t tiles, long_off, seq_off, hash_off, first_off, seg_off, units_off, elong_off, echunk_off, byaddr_off, thash_off, runs_off, total;
 };
 size_t up16(size_t x) { return (x + 15) / 16 * 16; }
 ImageLayout image_layout(const ciera_plan* p) {
@@ -82,7 +82,8 @@ ImageLayout image_layout(const ciera_plan* p) {
     L.units_off = L.seg_off + up16((size_t)p->n_units * sizeof(uint64_t));
     L.elong_off = L.units_off + up16((size_t)p->n_units * sizeof(ciera_unit));
     L.echunk_off = L.elong_off + up16(p->ent_long_units.size() * sizeof(uint32_t));
-    L.thash_off = L.echunk_off + up16(p->ent_chunks.size() * sizeof(ciera_plan::EntChunk));
+    L.byaddr_off = L.echunk_off + up16(p->ent_chunks.size() * sizeof(ciera_plan::EntChunk));
+    L.thash_off = L.byaddr_off + p->tiles_by_address.size() * sizeof(TileDesc);
     L.runs_off = L.thash_off + up16(p->tiles.size() * sizeof(uint64_t));
     L.total = L.runs_off + p->seq_runs.size() * sizeof(ciera_plan::SeqRun) + 16;
     return L;
@@ -185,6 +186,31 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         }
     }
     for (uint32_t u : longs) emit(u);
+    // the same tiles by address, for steps on host weights
+    {
+        std::vector<uint32_t> order;
+        order.reserve(shorts.size() + longs.size());
+        for (uint32_t u = 0; u < n_units; ++u)
+            if (units_host[u].n_values) order.push_back(u);
+        auto before = [&](uint32_t a, uint32_t b) { return units_host[a].weights_off < units_host[b].weights_off; };
+        if (!std::is_sorted(order.begin(), order.end(), before)) std::stable_sort(order.begin(), order.end(), before);
+        p->by_address_ok = true;
+        for (size_t i = 0; i + 1 < order.size(); ++i)
+            p->by_address_ok &= units_host[order[i]].weights_off + units_host[order[i]].n_values * vb <= units_host[order[i + 1]].weights_off;
+        const bool same = std::equal(shorts.begin(), shorts.end(), order.begin()) &&
+                          std::equal(longs.begin(), longs.end(), order.begin() + shorts.size());
+        if (p->by_address_ok && !same) {
+            std::vector<uint32_t> first(n_units, 0);
+            for (size_t t = 0; t < p->tiles.size(); ++t)
+                if (p->tiles[t].tile_in_unit == 0) first[p->tiles[t].unit] = (uint32_t)t;
+            p->tiles_by_address.reserve(p->tiles.size());
+            for (uint32_t u : order) {
+                const uint32_t at = (uint32_t)p->tiles_by_address.size(), nt = tiles_of(u);
+                p->tiles_by_address.insert(p->tiles_by_address.end(), p->tiles.begin() + first[u], p->tiles.begin() + first[u] + nt);
+                for (uint32_t j = 0; j < nt; ++j) p->tiles_by_address[at + j].first_tile = at;
+            }
+        }
+    }
     // per unit, in table order: where its tiles start and where its blocks start in a hash cache
     p->unit_first.assign(n_units, 0xffffffffu);
     for (size_t t = 0; t < p->tiles.size(); ++t)
@@ -214,6 +240,8 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     if (L.tiles) memcpy(p->image.data(), p->tiles.data(), L.tiles);
     if (!p->long_units.empty()) memcpy(p->image.data() + L.long_off, p->long_units.data(), p->long_units.size() * 4);
     memcpy(p->image.data() + L.seq_off, p->seq_first.data(), p->seq_first.size() * 4);
+    if (!p->tiles_by_address.empty())
+        memcpy(p->image.data() + L.byaddr_off, p->tiles_by_address.data(), p->tiles_by_address.size() * sizeof(TileDesc));
     if (!p->tile_hash.empty()) memcpy(p->image.data() + L.thash_off, p->tile_hash.data(), p->tile_hash.size() * 8);
     if (!p->seq_runs.empty())
         memcpy(p->image.data() + L.runs_off, p->seq_runs.data(), p->seq_runs.size() * sizeof(ciera_plan::SeqRun));
@@ -231,7 +259,15 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     return CIERA_OK;
 }
 
-extern "C" void ciera_plan_destroy(ciera_plan* plan) { delete plan; }
+extern "C" void ciera_plan_destroy(ciera_plan* plan) {
+    if (plan)
+        for (const ciera_plan::CopyLane& lane : plan->lanes) {  // (work still queued there runs to its end)
+            cudaStreamDestroy(lane.in);
+            cudaStreamDestroy(lane.out);
+            cudaEventDestroy(lane.event);
+        }
+    delete plan;
+}
 
 extern "C" uint32_t ciera_plan_n_units(const ciera_plan* p) { return p ? p->n_units : 0; }
 extern "C" uint32_t ciera_plan_n_tiles(const ciera_plan* p) { return p ? (uint32_t)p->tiles.size() : 0; }
@@ -275,6 +311,7 @@ extern "C" int ciera_plan_bind(ciera_plan* p, void* plan_dev, size_t plan_dev_by
     p->tiles_dev = (const TileDesc*)plan_dev;
     const ImageLayout L = image_layout(p);
     const uint8_t* base = (const uint8_t*)plan_dev;
+    p->tiles_by_address_dev = p->tiles_by_address.empty() ? p->tiles_dev : (const TileDesc*)(base + L.byaddr_off);
     p->long_units_dev = (const uint32_t*)(base + L.long_off);
     p->seq_first_dev = (const uint32_t*)(base + L.seq_off);
     p->hash_base_dev = (const unsigned long long*)(base + L.hash_off);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <vector>
 
 #include "ciera.h"
@@ -180,6 +181,10 @@ struct ciera_plan {
     std::vector<uint32_t> unit_first;  // first tile of every unit (0xffffffff: a unit without values)
     std::vector<uint64_t> hash_base;   // index of every unit's first block in a per-block hash cache
     std::vector<uint64_t> tile_hash;   // the same for every tile's first block, in tile-table order
+    // the tiles of all units by ascending address of their weights, for steps on host weights; left empty where that
+    // is the order of `tiles` already.  by_address_ok: the units' weights do not overlap.
+    std::vector<ciera::TileDesc> tiles_by_address;
+    bool by_address_ok = false;
     uint64_t total_blocks = 0;
     std::vector<uint64_t> seg_base;    // index of every unit's first 4096-byte payload segment (entropy stage)
     uint64_t total_segments = 0;
@@ -194,8 +199,18 @@ struct ciera_plan {
     const uint32_t* ent_long_units_dev = nullptr;
     const uint4* ent_chunks_dev = nullptr;
     std::vector<uint8_t> image;        // device image: tiles, long_units, seq_first, hash_base, unit_first, seg_base, units,
-                                       // ent_long_units, ent_chunks, tile_hash, seq_runs
+                                       // ent_long_units, ent_chunks, tiles_by_address, tile_hash, seq_runs
     const ciera::TileDesc* tiles_dev = nullptr;
+    const ciera::TileDesc* tiles_by_address_dev = nullptr;
+    // Pairs of copy streams for steps on host weights: taken out for the length of a call, put back at its end and
+    // reused by the next; as many as calls were ever made at the same time; destroyed with the plan.
+    struct CopyLane {
+        int device;
+        cudaStream_t in, out;
+        cudaEvent_t event;
+    };
+    mutable std::mutex lanes_mutex;
+    mutable std::vector<CopyLane> lanes;
     const uint32_t* long_units_dev = nullptr;
     const uint32_t* seq_first_dev = nullptr;
     const uint2* seq_runs_dev = nullptr;
@@ -214,4 +229,10 @@ int check_launch();                            // cudaGetLastError -> status
 int launch_encode_hashed(const ciera_plan* p, const void* weights_dev, void* hash_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
                          cudaStream_t s);
+// the argument checks of ciera_step; writes the outputs of units without values
+int step_begin(const ciera_plan* p, const void* weights_dev, const void* sender_cache_dev, const void* msg_send_dev,
+               const void* msg_recv_dev, const void* receiver_cache_dev, const void* weights_out_dev, uint64_t* wire_bytes_dev,
+               uint32_t* changed_blocks_dev, const void* workspace_dev, cudaStream_t s);
+// ciera_step on the tiles [lo, hi) of the plan's tiles by address; parts of one step go to one stream in order
+int launch_step_part(const ciera_plan* p, const ciera_device_buffers* b, uint32_t lo, uint32_t hi, cudaStream_t s);
 }  // namespace ciera

@@ -361,6 +361,110 @@ extern "C" int ciera_transport(const ciera_plan* p, const void* src_messages_dev
     return check_launch();
 }
 
+// ---- a step on host weights, in parts
+//
+// Bound by the host link: copying everything in, stepping and copying everything out uses the link one direction at a
+// time.  Both directions at once carry nearly twice as much, so the step is cut into parts (ranges of the tiles by
+// address): while one part's weights come in and another's go out, the parts between them are stepped.  Units that
+// straddle parts find the offsets of their earlier tiles in the look-back words, which only the last part empties.
+// What is left of one direction at a time is the first part's way in and the last one's way out, so those two are half
+// as long as the others; but copies in pieces are slower (100 MB both ways at once on a B200 host: 2.11 ms whole, 2.21 in
+// 8 pieces, 2.73 in 32, about 20 us a piece).  Both together are least near sqrt(link time / 20 us) = sqrt(MB) parts.
+// 100 MB of bf16 weights: as a whole 3.72 ms, 8 parts 2.45, 16 equal parts 2.52, 32 equal parts 2.86; 25 MB: as a whole
+// 0.935 ms, 6 parts 0.727, 12 parts 0.811.
+constexpr uint32_t kHostPartsMax = 64;
+
+// parts to cut the step into; 1: as a whole
+static uint32_t host_step_parts(const ciera_plan* p, const void* in, const void* out, size_t bytes, cudaStream_t s) {
+    uint32_t parts = 1;
+    while (parts < kHostPartsMax && ((uint64_t)(parts + 1) * (parts + 1) << 20) <= bytes) ++parts;
+    if (parts < 2 || !p->by_address_ok) return 1;
+    // (inside a capture no streams are made; pageable memory is copied synchronously, which parts would only slow down)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return 1;
+    }
+    for (const void* q : {in, out}) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess || a.type != cudaMemoryTypeHost) {
+            cudaGetLastError();
+            return 1;
+        }
+    }
+    return parts;
+}
+
+static int take_copy_lane(const ciera_plan* p, ciera_plan::CopyLane* lane) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return record_cuda_error(e);
+    {
+        std::lock_guard<std::mutex> hold(p->lanes_mutex);
+        for (size_t i = 0; i < p->lanes.size(); ++i)
+            if (p->lanes[i].device == dev) {
+                *lane = p->lanes[i];
+                p->lanes.erase(p->lanes.begin() + i);
+                return CIERA_OK;
+            }
+    }
+    *lane = {dev, nullptr, nullptr, nullptr};
+    e = cudaStreamCreateWithFlags(&lane->in, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&lane->out, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&lane->event, cudaEventDisableTiming);
+    if (e == cudaSuccess) return CIERA_OK;
+    if (lane->in) cudaStreamDestroy(lane->in);
+    if (lane->out) cudaStreamDestroy(lane->out);
+    return record_cuda_error(e);
+}
+
+// `to` waits for what `from` holds so far (one event serves them all: a wait refers to the record before it)
+static cudaError_t join(cudaStream_t to, cudaStream_t from, cudaEvent_t event) {
+    const cudaError_t e = cudaEventRecord(event, from);
+    return e != cudaSuccess ? e : cudaStreamWaitEvent(to, event, 0);
+}
+
+static int host_step_in_parts(const ciera_plan* p, const void* weights_host, size_t weights_bytes, void* weights_out_host,
+                              const ciera_device_buffers* b, uint32_t parts, cudaStream_t s) {
+    // the checks of ciera_step, and the outputs of units without values
+    int rc = step_begin(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->msg_recv_dev, b->receiver_cache_dev,
+                              b->weights_out_dev, b->wire_bytes_dev, b->changed_blocks_dev, b->workspace_dev, s);
+    if (rc) return rc;
+    ciera_plan::CopyLane lane;
+    rc = take_copy_lane(p, &lane);
+    if (rc) return rc;
+    const std::vector<TileDesc>& tiles = p->tiles_by_address.empty() ? p->tiles : p->tiles_by_address;
+    const uint32_t nt = (uint32_t)tiles.size();
+    cudaError_t e = join(lane.in, s, lane.event);
+    uint32_t lo = 0;
+    uint64_t from = 0;  // weights up to this byte are on their way
+    for (uint32_t k = 1; k <= parts && e == cudaSuccess && rc == CIERA_OK; ++k) {
+        const uint32_t hi = k == parts ? nt : (uint32_t)((uint64_t)nt * (2u * k - 1u) / (2u * parts - 2u));
+        if (hi == lo) continue;
+        uint64_t to = hi < nt ? tiles[hi].w_off : (uint64_t)weights_bytes;
+        if (to > weights_bytes) to = weights_bytes;
+        if (to < from) to = from;
+        const uint64_t n = to - from;
+        if (n) e = cudaMemcpyAsync((uint8_t*)b->weights_dev + from, (const uint8_t*)weights_host + from, n, cudaMemcpyHostToDevice, lane.in);
+        if (e == cudaSuccess) e = join(s, lane.in, lane.event);
+        if (e == cudaSuccess) rc = launch_step_part(p, b, lo, hi, s);
+        if (e == cudaSuccess && rc == CIERA_OK) e = join(lane.out, s, lane.event);
+        if (e == cudaSuccess && rc == CIERA_OK && n)
+            e = cudaMemcpyAsync((uint8_t*)weights_out_host + from, (const uint8_t*)b->weights_out_dev + from, n, cudaMemcpyDeviceToHost, lane.out);
+        from = to;
+        lo = hi;
+    }
+    // whatever happened, the caller's stream waits for what has been queued
+    const cudaError_t e2 = join(s, lane.in, lane.event), e3 = join(s, lane.out, lane.event);
+    {
+        std::lock_guard<std::mutex> hold(p->lanes_mutex);
+        p->lanes.push_back(lane);
+    }
+    if (rc) return rc;
+    if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
+    return e != cudaSuccess ? record_cuda_error(e) : CIERA_OK;
+}
+
 extern "C" int ciera_roundtrip_host(const ciera_plan* p, const void* weights_host, size_t weights_bytes,
                                     void* weights_out_host, uint64_t* wire_bytes_host, const ciera_device_buffers* b,
                                     void* stream) {
@@ -369,20 +473,22 @@ extern "C" int ciera_roundtrip_host(const ciera_plan* p, const void* weights_hos
     if (!b || !weights_host || !weights_out_host) return CIERA_ERR_INVALID_ARG;
     if (p->tiles.empty()) return CIERA_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = cudaMemcpyAsync(b->weights_dev, weights_host, weights_bytes, cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return record_cuda_error(e);
-    rc = ciera_encode(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->wire_bytes_dev, b->changed_blocks_dev,
-                      b->workspace_dev, b->status_dev, stream);
-    if (rc) return rc;
-    rc = ciera_transport(p, b->msg_send_dev, b->msg_recv_dev, b->wire_bytes_dev, b->workspace_dev, b->status_dev, stream);
-    if (rc) return rc;
-    rc = ciera_decode(p, b->msg_recv_dev, b->receiver_cache_dev, b->weights_out_dev, b->wire_bytes_dev,
-                      b->workspace_dev, b->status_dev, stream);
-    if (rc) return rc;
-    e = cudaMemcpyAsync(weights_out_host, b->weights_out_dev, weights_bytes, cudaMemcpyDeviceToHost, s);
-    if (e != cudaSuccess) return record_cuda_error(e);
+    const uint32_t parts = host_step_parts(p, weights_host, weights_out_host, weights_bytes, s);
+    if (parts > 1) {
+        rc = host_step_in_parts(p, weights_host, weights_bytes, weights_out_host, b, parts, s);
+        if (rc) return rc;
+    } else {
+        cudaError_t e = cudaMemcpyAsync(b->weights_dev, weights_host, weights_bytes, cudaMemcpyHostToDevice, s);
+        if (e != cudaSuccess) return record_cuda_error(e);
+        rc = ciera_step(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->msg_recv_dev, b->receiver_cache_dev,
+                        b->weights_out_dev, b->wire_bytes_dev, b->changed_blocks_dev, b->workspace_dev, b->status_dev, stream);
+        if (rc) return rc;
+        e = cudaMemcpyAsync(weights_out_host, b->weights_out_dev, weights_bytes, cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess) return record_cuda_error(e);
+    }
     if (wire_bytes_host) {
-        e = cudaMemcpyAsync(wire_bytes_host, b->wire_bytes_dev, sizeof(uint64_t) * p->n_units, cudaMemcpyDeviceToHost, s);
+        const cudaError_t e =
+            cudaMemcpyAsync(wire_bytes_host, b->wire_bytes_dev, sizeof(uint64_t) * p->n_units, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return record_cuda_error(e);
     }
     return CIERA_OK;

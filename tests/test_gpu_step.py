@@ -113,3 +113,43 @@ def test_runs_of_short_units(dtype, block):
         compare_step(codec, exp, bits[t], f"t={t}")
         compare_caches(codec, table, f"t={t}")
         compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("dtype,block", [(0, 1), (0, 512), (0, 4096), (1, 64), (1, 2048), (2, 16), (2, 4096)])
+def test_host_step_in_parts(dtype, block, pinned):
+    """A step on host weights that is large enough to be cut into parts (pinned memory), with units of many sizes --
+    their order in the tile table is not that of their addresses -- and long ones that straddle parts, also in the
+    middle of a bitmap byte; twice in a row on the same plan.  Pageable memory: the step as a whole."""
+    from paper_2609_04609_b200 import runtime
+
+    sizes = [8192 * 40 + 3, 100, 0, 8192 * 200 + 4097, 8192 * 12 + 5, 1_000_000, 8192 * 3]
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(3 * block + dtype)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    for _ in range(2):
+        w.append(wl.step_clustered(w[-1], gen, f=0.3))
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    staging = torch.empty(codec.weights_bytes, dtype=torch.uint8, device=DEV)
+    wire_host = torch.zeros(codec.plan.n_units, dtype=torch.int64)
+    for t in (1, 2):
+        exp = table.step(bits[t])
+        src = torch.from_numpy(bits[t].view(np.uint8).copy())
+        out = torch.zeros(codec.weights_bytes, dtype=torch.uint8)
+        if pinned:
+            src, out, wire_host = src.pin_memory(), out.pin_memory(), wire_host.pin_memory()
+        codec.step_host(src, out, staging, wire_host)
+        torch.cuda.synchronize()
+        codec.check_status()
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+        assert np.array_equal(wire_host.numpy().astype(np.uint64), exp["wire"])
+        assert torch.equal(staging.cpu(), src)
+        host = out.numpy()
+        for u in codec.units:
+            lo, n = int(u["weights_off"]), int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]]
+            assert np.array_equal(host[lo : lo + n], src.numpy()[lo : lo + n])
