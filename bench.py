@@ -3,7 +3,8 @@
 
 One *step* = one pass of the whole path over one iterate of the synthetic weight trajectory:
 for every layer, sender-side encode, the device-to-device transport that stands where the
-Allgather would be, and receiver-side decode -- layer-pipelined on two streams.
+Allgather would be, and receiver-side decode (one launch per layer; with the entropy stage or the
+hashed sender, launches of their own on two streams).
 
 Workload at one GPU: the full OLMoE-1B-7B expert stack (16 layers x 64 experts x 3 matrices,
 bf16, 6.44 G values = 12.9 GB), 16 simulated shards per matrix, block size 512, with the
@@ -536,7 +537,7 @@ def main():
     s_enc.wait_event(ev0)
     s_dec.wait_event(ev0)
     for _ in range(args.steps):
-        pipe.step(weights_of(step_i), None, timers)
+        pipe.step(weights_of(step_i))
         step_i += 1
     cur.wait_stream(s_enc)
     cur.wait_stream(s_dec)
@@ -548,6 +549,13 @@ def main():
     ms_per_step = ms_total / args.steps
     for c in layers:
         c.check_status()
+
+    # ---- two steps with events around every kernel on the two streams (overlapped figures; with events between
+    #      them, sender, transport and receiver are launches of their own)
+    for _ in range(2):
+        pipe.step(weights_of(step_i), None, timers)
+        step_i += 1
+    barrier()
 
     # ---- the same K steps once more on ONE stream: kernels do not overlap, so the CUDA events
     #      around each launch time that kernel alone (used for the roofline entries)
@@ -591,7 +599,10 @@ def main():
     enc_gbs = a_enc / (enc_ms * 1e-3) / 1e9
     dec_gbs = a_dec / (dec_ms * 1e-3) / 1e9
     tra_gbs = a_tra / (tra_ms * 1e-3) / 1e9
-    path_gbs = len(layers) * (a_enc + a_tra + a_dec) / (ms_per_step * 1e-3) / 1e9
+    # a layer of the timed step: where it is one launch, the message is written to both buffers and not read again
+    one_launch = not args.entropy and args.detect == "compare"
+    a_step = a_enc + a_dec + (0 if one_launch else a_tra)  # (the copy's write stands for the receiver's read)
+    path_gbs = len(layers) * a_step / (ms_per_step * 1e-3) / 1e9
 
     # ---- correctness at full size: exact round trip everywhere, oracle on sampled units
     last_w = weights_of(step_i - 1)
@@ -653,7 +664,7 @@ def main():
         "kernel_ms": {"encode": enc_ms, "transport": tra_ms, "decode": dec_ms,
                       "per": "layer launch; serial re-run of the timed steps on one stream"},
         "kernel_ms_overlapped": {"encode": ovl_ms[0], "transport": ovl_ms[1], "decode": ovl_ms[2],
-                                 "per": "layer launch inside the two-stream timed region (kernels overlap)"},
+                                 "per": "layer launch of two more steps on two streams (kernels overlap)"},
         "serial_ms_per_step": serial_ms_per_step,
         "serial_step_ms_spread": step_spread,
         "kernel_ms_x_sm_mhz": ({"encode": enc_ms * clocks["sm_mhz"], "transport": tra_ms * clocks["sm_mhz"],
@@ -673,7 +684,8 @@ def main():
             "decode_kernel": {"achieved": dec_gbs, "frac": dec_gbs / peak, "algorithmic_bytes_per_launch": a_dec},
             "transport_kernel": {"achieved": tra_gbs, "frac": tra_gbs / peak, "algorithmic_bytes_per_launch": a_tra},
             "whole_step_pipelined": {"achieved": path_gbs, "frac": path_gbs / peak,
-                                     "note": "algorithmic bytes of all three kernels over the two-stream step time"},
+                                     "algorithmic_bytes_per_layer": a_step,
+                                     "note": "algorithmic bytes of a layer's launches over the timed step"},
         },
     }
 
