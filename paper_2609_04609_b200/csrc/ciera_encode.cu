@@ -272,6 +272,7 @@ struct EncodeCtl {
 };
 
 constexpr uint32_t kNoTile = 0xffffffffu;
+constexpr uint32_t kEarlyClearTiles = 4096;  // status words that one warp empties while the rest still works
 
 // How a tile relates to the run of tiles it was handed out with (a short unit's tiles go out in runs of
 // kSeqRunTiles, see ciera_internal.cuh): bit 0 = the tile belongs to a run (else: a spread tile of a longer
@@ -978,6 +979,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     const uint32_t kHStage = HASH ? kHoldBytes + hash_part_bytes<DT>(log2b) : 0u;
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const bool early_clear = spread_first < n_tiles && n_tiles - clear_first <= kEarlyClearTiles;
     volatile int* abort = &ctl->abort;
     // FINE: every consumer warp's gather space for its changed exponents (in place of the hash stages)
     uint8_t* const s_gather = ring_h + (size_t)(warp < (uint32_t)kWarps ? warp : 0u) * kWarpGatherBytes;
@@ -1156,7 +1158,22 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             const uint32_t se = k % SE;
             if (!mbar_wait(&ctl->summed[se], (k / SE) & 1u, abort, status)) break;
             const uint32_t tile = ctl->tile_idx[k % kDescRing];
-            if (tile == kNoTile) break;
+            if (tile == kNoTile) {
+                if (early_clear) {
+                    // this warp looks back no more; the last one of the grid empties the status words
+                    uint32_t last = 0;
+                    if (lane == 0) {
+                        __threadfence();
+                        last = atomicAdd(blocks_done, 1u) + 1u == gridDim.x * (uint32_t)kResolvers ? 1u : 0u;
+                    }
+                    if (__shfl_sync(0xffffffffu, last, 0)) {
+                        __threadfence();
+                        for (uint32_t t = clear_first + lane; t < n_tiles; t += 32u) st_status(tile_status + t, 0ull);
+                        if (lane == 0) atomicExch(blocks_done, 0u);
+                    }
+                }
+                break;
+            }
             if (ctl->seq[k % kDescRing] != 0) continue;  // the aggregator has done it all
             const TileDesc td = ctl->desc[k % kDescRing];
             const uint64_t excl = resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, tw.msg, wire_bytes,
@@ -1333,10 +1350,14 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             }
         }
     }
-    // (clear_first: a step in parts leaves the status words to the parts that follow, and the last part empties all)
     // The scratch is handed back the way it was found, all zero: the hand-off words of the runs were emptied by
     // their readers, the run counter by its last draw; the status words of the spread tiles (read by any number
-    // of later tiles) and the counter of finished blocks are emptied here by the block that finishes last.
+    // of later tiles) and the counter of finished blocks are emptied by whoever finishes last.  Where the words are
+    // few that is the resolver warp that looks back last, while the consumers still send (a fence and an atomic
+    // behind everything else cost the smallest tables more than a microsecond); where they are many it is the
+    // block that finishes last, with all its threads.  Without spread tiles there is nothing to empty.
+    // (clear_first: a step in parts leaves the status words to the parts that follow, and the last part empties all)
+    if (early_clear || spread_first >= n_tiles) return;
     __shared__ unsigned int s_last;
     if (tid == 0) {
         __threadfence();
