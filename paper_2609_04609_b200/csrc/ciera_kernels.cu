@@ -120,6 +120,7 @@ transport_pipe_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint
         ctl->seen = 0;
         mbar_fence_init();
     }
+    pdl_wait();
     __syncthreads();
 
     if (warp == kPipeConsumers) {
@@ -353,12 +354,14 @@ extern "C" int ciera_transport(const ciera_plan* p, const void* src_messages_dev
     if (rc) return rc;
     const uint32_t want_blocks = (nt + kPipeBatch - 1) / kPipeBatch;
     const uint32_t grid = want_blocks < (uint32_t)limit ? want_blocks : (uint32_t)limit;
-    transport_pipe_kernel<<<grid, kPipeThreads, (size_t)kPipeStages * kPipeStage + sizeof(PipeCtl), (cudaStream_t)stream>>>(
+    const cudaError_t e = launch_after(
+        transport_pipe_kernel, dim3(grid), kPipeThreads, (size_t)kPipeStages * kPipeStage + sizeof(PipeCtl), (cudaStream_t)stream,
         p->tiles_dev, nt, transport_chunk_bytes(p->dtype == CIERA_FP32 ? 3u : 1u, p->log2b), p->dtype, p->log2b,
         (const uint8_t*)src_messages_dev, (uint8_t*)dst_messages_dev, (const unsigned long long*)wire_bytes_dev, ticket,
         status_dev);
+    if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
-    return check_launch();
+    return CIERA_OK;
 }
 
 // ---- a step on host weights, in parts
