@@ -38,6 +38,11 @@ constexpr uint32_t kSegment = 4096;                              // bytes of raw
 constexpr uint32_t kSegWordsMax = kSegment * kProbBits / 16;     // 3072: a symbol adds at most 12 bits
 constexpr uint32_t kSegSlot = 4 * 32 + 2 * kSegWordsMax;         // 6272 bytes: states + words
 constexpr int kEntThreads = 256, kEntWarps = kEntThreads / 32;
+// A unit's thread block has kEntThreads threads where there are units enough to fill the GPU, else kEntWide: a segment
+// is a serial chain of 128 steps (about 8 us), and a block codes as many segments at a time as it has warps.  Four units of
+// 32 segments, sender's / receiver's stage: 66 / 92 us with 8 warps, 32 / 31 with 32; 192 units of 8 segments are better off
+// with 8 (both stages and the step: 79 us against 107).
+constexpr int kEntWide = 1024;
 constexpr uint32_t kLongSegs = 64;  // units with more segment slots than this take the chunked path
 
 __host__ __device__ inline uint64_t segments_of(uint64_t bytes) { return (bytes + kSegment - 1) / kSegment; }
@@ -48,10 +53,11 @@ __host__ __device__ inline uint32_t model_bytes(int dt) { return dt == CIERA_FP1
 // ---------------------------------------------------------------------------------- shared pieces
 
 // Adds the bytes pay[lo, hi) to the warp-private histograms (lo a multiple of 16, pay 16-byte aligned).
+template <int T>
 __device__ __forceinline__ void histogram_add(uint32_t (*hist)[256], const uint8_t* pay, uint64_t lo, uint64_t hi,
                                               uint32_t tid) {
     const uint32_t warp = tid >> 5;
-    for (uint64_t i = lo + (uint64_t)tid * 16; i < hi; i += (uint64_t)kEntThreads * 16) {
+    for (uint64_t i = lo + (uint64_t)tid * 16; i < hi; i += (uint64_t)T * 16) {
         if (i + 16 <= hi) {
             const uint4 v = *reinterpret_cast<const uint4*>(pay + i);
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -104,7 +110,7 @@ __device__ __forceinline__ uint32_t warp_argmax256(V v, uint32_t lane) {
 // Frequencies from counts (h[256] in shared memory, P = their sum): thread s owns symbol s, then the
 // first warp settles the sum.  Ends with a barrier; f is then final.
 __device__ __forceinline__ void normalise_model(const uint32_t* h, uint64_t P, uint16_t* f, uint32_t tid) {
-    {
+    if (tid < 256u) {
         uint32_t v = 0;
         if (h[tid]) {
             v = P < (1ull << 20) ? h[tid] * kProbScale / (uint32_t)P : (uint32_t)((uint64_t)h[tid] * kProbScale / P);
@@ -146,7 +152,7 @@ __device__ __forceinline__ void normalise_model(const uint32_t* h, uint64_t P, u
 // bytes holds what a coder step needs:
 //   {multiplier, largest x below f * 2^20, c, (4096 - f) << 5 | shift, bit 31: x + 1}
 __device__ __forceinline__ bool encoder_tables(const uint16_t* f, uint4* enc, uint32_t tid) {
-    const uint32_t fs = f[tid] ? f[tid] : 1u;
+    const uint32_t fs = tid < 256u && f[tid] ? f[tid] : 1u;
     uint32_t s = 31u - (uint32_t)__clz(fs), m = 0xFFFFFFFFu, plus = 0u;
     if (fs & (fs - 1u)) {
         // floor(2^(32 + s) / f) in two 32-bit divisions: s + 16 < 28 and the first remainder is below 2^12
@@ -161,9 +167,11 @@ __device__ __forceinline__ bool encoder_tables(const uint16_t* f, uint4* enc, ui
         m = 0x80000000u;
         s -= 1u;
     }
-    enc[tid].x = m;
-    enc[tid].y = (uint32_t)(((unsigned long long)fs << 20) - 1ull);
-    enc[tid].w = ((kProbScale - fs) << 5) | s | (plus << 31);
+    if (tid < 256u) {
+        enc[tid].x = m;
+        enc[tid].y = (uint32_t)(((unsigned long long)fs << 20) - 1ull);
+        enc[tid].w = ((kProbScale - fs) << 5) | s | (plus << 31);
+    }
     if (tid < 32) {
         uint32_t local[8], total;
         const uint32_t base = warp_prefix256(f, tid, local, total);
@@ -244,15 +252,16 @@ __device__ __forceinline__ uint32_t encode_segment(const uint8_t* src, uint32_t 
 // Receiver tables from the transmitted frequencies (f[] already in shared memory and synced): one word per slot:
 // (slot - c) | symbol << 12 | (f - 1) << 20.  Returns false (in every thread) if the table does not sum to 4096.
 // The owner of a slot is the last symbol that occurs and starts at or below it.  Every symbol that occurs marks the
-// slot it starts at with its number + 1; a warp then carries the largest mark forward over its 512 slots, 128 at a
+// slot it starts at with its number + 1; a warp then carries the largest mark forward over its slots, 128 at a
 // time.  (A search per thread and a walk over its 16 slots took three times the instructions, most of them diverged.)
 //   base[s] = symbol << 12 | (f - 1) << 20, less c, so that a slot's word is base[owner] + slot
+template <int T>
 __device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, uint32_t* base, uint32_t* tab, uint32_t* flag,
                                                uint32_t tid) {
     const uint32_t lane = tid & 31u, warp = tid >> 5;
     uint4* const tab4 = reinterpret_cast<uint4*>(tab);
 #pragma unroll
-    for (int i = 0; i < (int)(kProbScale / 4) / kEntThreads; ++i) tab4[tid + i * kEntThreads] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < (int)(kProbScale / 4) / T; ++i) tab4[tid + i * T] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < 32) {
         uint32_t local[8], total;
         const uint32_t first = warp_prefix256(f, tid, local, total);
@@ -262,11 +271,14 @@ __device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, u
     }
     __syncthreads();
     if (*flag == 0) return false;
-    const uint32_t start = c[tid];
-    base[tid] = (tid << 12 | ((uint32_t)f[tid] - 1u) << 20) - start;
-    if (f[tid]) tab[start] = tid + 1u;  // f >= 1: the start is a slot, and no other symbol's start
+    if (tid < 256u) {
+        const uint32_t start = c[tid];
+        base[tid] = (tid << 12 | ((uint32_t)f[tid] - 1u) << 20) - start;
+        if (f[tid]) tab[start] = tid + 1u;  // f >= 1: the start is a slot, and no other symbol's start
+    }
     // the owner of the slot in front of the warp's first one (mark 0: there is none)
-    const uint32_t slot0 = warp * (kProbScale / kEntWarps);
+    constexpr uint32_t kSlots = kProbScale * 32u / (uint32_t)T;  // slots of a warp
+    const uint32_t slot0 = warp * kSlots;
     uint32_t carry = 0;
 #pragma unroll
     for (uint32_t s = lane; s < 256u; s += 32u)
@@ -274,7 +286,7 @@ __device__ __forceinline__ bool decoder_tables(const uint16_t* f, uint16_t* c, u
     carry = __reduce_max_sync(0xffffffffu, carry);
     __syncthreads();
 #pragma unroll
-    for (uint32_t r = 0; r < kProbScale / kEntWarps / 128u; ++r) {
+    for (uint32_t r = 0; r < kSlots / 128u; ++r) {
         const uint32_t slot = slot0 + 128u * r + 4u * lane;
         uint4 v = tab4[slot >> 2];
         v.y = max(v.x, v.y);
@@ -326,7 +338,13 @@ __device__ __forceinline__ bool decode_segment(const uint8_t* coded, uint32_t sn
         const bool need = has && y < kRansL;
         const uint32_t votes = __ballot_sync(0xffffffffu, need);
         ptr -= __popc(votes);
-        if (need) x = __byte_perm((uint32_t)words[ptr + (int32_t)__popc(votes & below)], x, 0x5410u);
+        // (a predicated load: as an if it compiled to a branch with a reconvergence point, 0.147 -> 0.142 ms per layer)
+        uint32_t w;
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .u16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u16 h, 0;\n\t@p ld.global.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}"
+                     : "=r"(w)
+                     : "l"(words + (ptr + (int32_t)__popc(votes & below))), "r"((uint32_t)need)
+                     : "memory");
+        x = need ? __byte_perm(w, x, 0x5410u) : x;
     };
     const uint32_t full = n >> 5;  // steps in which every lane has a symbol
     uint32_t t = 0;
@@ -348,12 +366,13 @@ __device__ __forceinline__ bool decode_segment(const uint8_t* coded, uint32_t sn
 // Raw payload length Q in bytes and symbol count S of a unit from its bitmap (block-wide; `acc` in shared
 // memory, zeroed and synced by the caller).  The bitmap's bits past the last block and the pad behind it
 // are zero.
+template <int T>
 __device__ __forceinline__ uint64_t raw_payload_bytes(const uint8_t* msg, uint64_t N, int dt, uint32_t log2b,
                                                       unsigned long long* acc, uint32_t tid, uint64_t& S) {
     const uint64_t words = (bitmap_bytes(N, log2b) + 3) >> 2;  // inside the 16-byte padded bitmap
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msg);
     uint32_t cnt = 0;
-    for (uint64_t i = tid; i < words; i += kEntThreads) cnt += __popc(bm32[i]);
+    for (uint64_t i = tid; i < words; i += T) cnt += __popc(bm32[i]);
     cnt = __reduce_add_sync(0xffffffffu, cnt);
     if ((tid & 31u) == 0 && cnt) atomicAdd(acc, (unsigned long long)cnt);
     __syncthreads();
@@ -430,8 +449,9 @@ __device__ __forceinline__ void pack_symbols(const uint8_t* sym, uint8_t* pay, u
     }
 }
 
-// Exclusive scan of one value per thread over the block; `scan` holds kEntWarps words.  Returns
+// Exclusive scan of one value per thread over the block; `scan` holds a word per warp.  Returns
 // the thread's offset; `total` gets the block's sum.  Contains barriers.
+template <int T>
 __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* scan, uint32_t tid, uint32_t& total) {
     const uint32_t lane = tid & 31u, warp = tid >> 5;
     uint32_t incl = v;
@@ -445,7 +465,7 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* scan, uint3
     __syncthreads();
     uint32_t wbase = 0;
     total = 0;
-    for (int w = 0; w < kEntWarps; ++w) {
+    for (int w = 0; w < T / 32; ++w) {
         if (w < (int)warp) wbase += scan[w];
         total += scan[w];
     }
@@ -455,16 +475,17 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* scan, uint3
 // ------------------------------------------------------------------------------------------ sender
 // units of up to kLongSegs segment slots: one thread block per unit, start to end
 
-template <bool HALF>  // HALF: fp16, five-bit symbols (see the head of this file)
-__global__ void __launch_bounds__(kEntThreads, 5)
+template <bool HALF, int T>  // HALF: fp16, five-bit symbols (see the head of this file); T: threads of the block
+__global__ void __launch_bounds__(T, T == kEntWide ? 1 : 5)
 entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long long* __restrict__ seg_base,
                       int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
                       uint8_t* scratch_slots, uint32_t* scratch_nw, uint8_t* scratch_sym) {
-    __shared__ uint32_t s_hist[kEntWarps][256];  // the warps' private histograms, then the two small lists of step 4
+    __shared__ uint32_t s_hist[T / 32][256];  // the warps' private histograms, then the two small lists of step 4
     __shared__ uint16_t s_f[256];
     __shared__ uint4 s_enc[256];
-    __shared__ uint32_t s_scan[kEntWarps];
+    __shared__ uint32_t s_scan[T / 32];
     __shared__ unsigned long long s_total;
+    pdl_wait();
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
     if (un.n_values == 0 || segments_of(un.n_values) > kLongSegs) return;
@@ -482,7 +503,7 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     const uint8_t* src = pay;  // the symbols, one per byte
     if (HALF) {
         uint8_t* sym = scratch_sym + un.cache_off;
-        unpack_symbols(pay, sym, log2b, 0, P, tid, kEntThreads);
+        unpack_symbols(pay, sym, log2b, 0, P, tid, T);
         src = sym;
         __syncthreads();
     }
@@ -491,21 +512,22 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     for (uint32_t i = lane; i < 256; i += 32) s_hist[warp][i] = 0;
     if (tid == 0) s_total = 0;
     __syncwarp();
-    histogram_add(s_hist, src, 0, P, tid);
+    histogram_add<T>(s_hist, src, 0, P, tid);
     __syncthreads();
     {
         uint32_t h = 0;
-        for (int w = 0; w < kEntWarps; ++w) h += s_hist[w][tid];
+        if (tid < 256u)
+            for (int w = 0; w < T / 32; ++w) h += s_hist[w][tid];
         __syncthreads();
-        s_hist[0][tid] = h;
+        if (tid < 256u) s_hist[0][tid] = h;
     }
     __syncthreads();
     normalise_model(s_hist[0], P, s_f, tid);
     const bool plus = encoder_tables(s_f, s_enc, tid);
 
-    // 3. segments: warp w codes segments w, w + 8, ... into the unit's slots of the scratch
+    // 3. segments: warp w codes segments w, w + T / 32, ... into the unit's slots of the scratch
     const unsigned long long slot0 = seg_base[unit];
-    for (uint32_t g = warp; g < nseg; g += kEntWarps) {
+    for (uint32_t g = warp; g < nseg; g += T / 32) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
         const uint8_t* const seg = src + (uint64_t)g * kSegment;
         uint8_t* const slot = scratch_slots + (slot0 + g) * kSegSlot;
@@ -524,17 +546,20 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     if (tid < hdr / 2u) reinterpret_cast<uint16_t*>(pay)[tid] = s_f[tid];
     uint32_t* dir = reinterpret_cast<uint32_t*>(pay + hdr);
     uint8_t* data = pay + hdr + 4ull * nseg;
-    // nseg <= kLongSegs <= kEntThreads: one round
+    // nseg <= kLongSegs <= T: one round
     const uint32_t nw = tid < nseg ? scratch_nw[slot0 + tid] : 0u;
     const uint32_t size = tid < nseg ? segment_bytes(nw) : 0u;
     if (tid < nseg) dir[tid] = nw;
     uint32_t total;
     uint32_t* s_off = &s_hist[1][0];
     uint32_t* s_size = &s_hist[2][0];
-    s_off[tid] = block_scan(size, s_scan, tid, total);
-    s_size[tid] = size;
+    const uint32_t at = block_scan<T>(size, s_scan, tid, total);
+    if (tid < kLongSegs) {
+        s_off[tid] = at;
+        s_size[tid] = size;
+    }
     __syncthreads();
-    for (uint32_t k = warp; k < nseg; k += kEntWarps) {
+    for (uint32_t k = warp; k < nseg; k += T / 32) {
         const uint32_t* from = reinterpret_cast<const uint32_t*>(scratch_slots + (slot0 + k) * kSegSlot);
         uint32_t* to = reinterpret_cast<uint32_t*>(data + s_off[k]);
         for (uint32_t i = lane; i < (s_size[k] >> 2); i += 32) to[i] = from[i];
@@ -543,9 +568,14 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
 }
 
 // longer units: grids over chunks of kLongSegs segments.  A chunk record = {unit, first segment of
-// the chunk inside the unit, index of the unit among the long ones, 0}.  Per long unit the scratch
+// the chunk inside the unit, index of the unit among the long ones, 0}.  Where the chunks are too few to fill the GPU a
+// chunk is the work of several thread blocks (gridDim.y of them, a power of two), down to a segment per warp: 12 units of
+// 2 097 152 values, sender's / receiver's stage 137 / 205 us with a block to a chunk, 40 / 38 like this.  Per long unit the scratch
 // holds a record of 2048 bytes: 256 x u32 counts, 256 x u16 frequencies, then the words below.
 constexpr uint32_t kLongRec = 2048;
+// this block's segments of its chunk: first one inside the unit, and how many
+__device__ __forceinline__ uint32_t part_segments() { return kLongSegs / gridDim.y; }
+__device__ __forceinline__ uint32_t part_first(const uint4& chunk) { return chunk.y + blockIdx.y * part_segments(); }
 struct LongState {            // at byte 1536 of a long unit's record
     unsigned long long total;   // sender: bytes of all coded segments
     unsigned long long P;       // receiver: symbols of the raw payload
@@ -584,13 +614,14 @@ __device__ __forceinline__ const uint8_t* sender_symbols(const ciera_unit& un, i
 __global__ void __launch_bounds__(kEntThreads)
 entropy_long_unpack_kernel(const ciera_unit* __restrict__ units, const uint4* __restrict__ chunks, int dt, uint32_t log2b,
                            const uint8_t* msgs, const unsigned long long* wire_bytes, uint8_t* scratch_sym) {
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     const ciera_unit un = units[ch.x];
     uint64_t payoff, Q;
     const uint64_t P = sender_payload(un, dt, log2b, msgs, wire_bytes, ch.x, payoff, Q);
-    const uint64_t lo = (uint64_t)ch.y * kSegment;
+    const uint64_t lo = (uint64_t)part_first(ch) * kSegment;
     if (lo >= P) return;
-    const uint64_t hi = min(P, lo + (uint64_t)kLongSegs * kSegment);
+    const uint64_t hi = min(P, lo + (uint64_t)part_segments() * kSegment);
     unpack_symbols(msgs + un.msg_off + payoff, scratch_sym + un.cache_off, log2b, lo, hi, threadIdx.x, kEntThreads);
 }
 
@@ -599,17 +630,18 @@ entropy_long_hist_kernel(const ciera_unit* __restrict__ units, const uint4* __re
                          const uint8_t* msgs, const unsigned long long* wire_bytes, uint8_t* recs,
                          const uint8_t* scratch_sym) {
     __shared__ uint32_t s_hist[kEntWarps][256];
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[ch.x];
     uint64_t payoff, Q;
     const uint64_t P = sender_payload(un, dt, log2b, msgs, wire_bytes, ch.x, payoff, Q);
-    const uint64_t lo = (uint64_t)ch.y * kSegment;
+    const uint64_t lo = (uint64_t)part_first(ch) * kSegment;
     if (lo >= P) return;
-    const uint64_t hi = min(P, lo + (uint64_t)kLongSegs * kSegment);
+    const uint64_t hi = min(P, lo + (uint64_t)part_segments() * kSegment);
     for (uint32_t i = lane; i < 256; i += 32) s_hist[warp][i] = 0;
     __syncwarp();
-    histogram_add(s_hist, sender_symbols(un, dt, msgs, payoff, scratch_sym), lo, hi, tid);
+    histogram_add<kEntThreads>(s_hist, sender_symbols(un, dt, msgs, payoff, scratch_sym), lo, hi, tid);
     __syncthreads();
     uint32_t h = 0;
     for (int w = 0; w < kEntWarps; ++w) h += s_hist[w][tid];
@@ -621,6 +653,7 @@ entropy_long_model_kernel(const ciera_unit* __restrict__ units, const uint32_t* 
                           uint32_t log2b, const uint8_t* msgs, const unsigned long long* wire_bytes, uint8_t* recs) {
     __shared__ uint32_t s_h[256];
     __shared__ uint16_t s_f[256];
+    pdl_wait();
     const uint32_t li = blockIdx.x, tid = threadIdx.x, unit = long_units[li];
     uint64_t payoff, Q;
     const uint64_t P = sender_payload(units[unit], dt, log2b, msgs, wire_bytes, unit, payoff, Q);
@@ -646,21 +679,22 @@ entropy_long_encode_kernel(const ciera_unit* __restrict__ units, const unsigned 
     __shared__ uint16_t s_f[256];
     __shared__ uint4 s_enc[256];
     __shared__ unsigned long long s_total;
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[ch.x];
     uint64_t payoff, Q;
     const uint64_t P = sender_payload(un, dt, log2b, msgs, wire_bytes, ch.x, payoff, Q);
-    if ((uint64_t)ch.y * kSegment >= P) return;
+    if ((uint64_t)part_first(ch) * kSegment >= P) return;
     const uint32_t nseg = (uint32_t)segments_of(P);
-    const uint32_t g_end = min(nseg, ch.y + kLongSegs);
+    const uint32_t g_end = min(nseg, part_first(ch) + part_segments());
     s_f[tid] = long_model(recs, ch.z)[tid];
     if (tid == 0) s_total = 0;
     __syncthreads();
     const bool plus = encoder_tables(s_f, s_enc, tid);
     const uint8_t* pay = HALF ? scratch_sym + un.cache_off : msgs + un.msg_off + payoff;  // the symbols
     const unsigned long long slot0 = seg_base[ch.x];
-    for (uint32_t g = ch.y + warp; g < g_end; g += kEntWarps) {
+    for (uint32_t g = part_first(ch) + warp; g < g_end; g += kEntWarps) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
         const uint8_t* const seg = pay + (uint64_t)g * kSegment;
         uint8_t* const slot = scratch_slots + (slot0 + g) * kSegSlot;
@@ -683,6 +717,7 @@ entropy_long_layout_kernel(const ciera_unit* __restrict__ units, const unsigned 
                            unsigned long long* wire_bytes, uint8_t* recs, const uint32_t* scratch_nw,
                            uint32_t* scratch_off) {
     __shared__ uint32_t s_scan[kEntWarps];
+    pdl_wait();
     const uint32_t li = blockIdx.x, tid = threadIdx.x, unit = long_units[li];
     const ciera_unit un = units[unit];
     uint64_t payoff, Q;
@@ -703,7 +738,7 @@ entropy_long_layout_kernel(const ciera_unit* __restrict__ units, const unsigned 
         const uint32_t nw = g < nseg ? scratch_nw[slot0 + g] : 0u;
         if (g < nseg) dir[g] = nw;
         uint32_t total;
-        const uint32_t off = block_scan(g < nseg ? segment_bytes(nw) : 0u, s_scan, tid, total);
+        const uint32_t off = block_scan<kEntThreads>(g < nseg ? segment_bytes(nw) : 0u, s_scan, tid, total);
         if (g < nseg) scratch_off[slot0 + g] = carry + off;
         carry += total;
     }
@@ -718,6 +753,7 @@ __global__ void __launch_bounds__(kEntThreads)
 entropy_long_copy_kernel(const ciera_unit* __restrict__ units, const unsigned long long* __restrict__ seg_base,
                          const uint4* __restrict__ chunks, int dt, uint32_t log2b, uint8_t* msgs, uint8_t* recs,
                          const uint8_t* scratch_slots, const uint32_t* scratch_nw, const uint32_t* scratch_off) {
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     const LongState* st = long_state(recs, ch.z);
     if (st->coded == 0) return;
@@ -726,8 +762,8 @@ entropy_long_copy_kernel(const ciera_unit* __restrict__ units, const unsigned lo
     const uint32_t nseg = st->nseg;
     uint8_t* data = msgs + un.msg_off + payload_offset_of(un.n_values, dt, log2b) + model_bytes(dt) + 4ull * nseg;
     const unsigned long long slot0 = seg_base[ch.x];
-    const uint32_t g_end = min(nseg, ch.y + kLongSegs);
-    for (uint32_t g = ch.y + warp; g < g_end; g += kEntWarps) {
+    const uint32_t g_end = min(nseg, part_first(ch) + part_segments());
+    for (uint32_t g = part_first(ch) + warp; g < g_end; g += kEntWarps) {
         const uint32_t* from = reinterpret_cast<const uint32_t*>(scratch_slots + (slot0 + g) * kSegSlot);
         uint32_t* to = reinterpret_cast<uint32_t*>(data + scratch_off[slot0 + g]);
         const uint32_t words4 = segment_bytes(scratch_nw[slot0 + g]) >> 2;
@@ -742,9 +778,9 @@ struct DecodeShared {
     uint32_t tab[kProbScale];      // slot -> (slot - c) | symbol << 12 | (f - 1) << 20
     uint16_t f[256], c[256];
     uint32_t base[256];            // per symbol: see decoder_tables
-    uint32_t off[kEntThreads];     // per segment: byte offset in the data part
-    uint32_t nw[kEntThreads];      //              word count
-    uint32_t scan[kEntWarps];
+    uint32_t off[kLongSegs];       // per segment: byte offset in the data part
+    uint32_t nw[kLongSegs];        //              word count
+    uint32_t scan[kEntWide / 32];
     unsigned long long changed;    // set bits of the unit's bitmap
     uint32_t flag, bad;
 };
@@ -753,12 +789,16 @@ __device__ __forceinline__ void raise_corrupt(int32_t* status) {
     if (status) atomicCAS(status, 0, (int32_t)CIERA_ERR_CORRUPT);
 }
 
-template <bool HALF>  // HALF: fp16, five-bit symbols (see the head of this file)
-__global__ void __launch_bounds__(kEntThreads)
+// HALF: fp16, five-bit symbols (see the head of this file); T: threads of the block; BLOCKS: blocks per SM it is built for
+// (8 blocks leave 32 registers: 0.142 ms per OLMoE-shaped layer against 0.166 with 5; but where the units do not fill
+// more than 5, the 48 registers shorten the chain: 512 units 55 us against 70, 192 units 48 against 57)
+template <bool HALF, int T, int BLOCKS>
+__global__ void __launch_bounds__(T, BLOCKS)
 entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log2b, uint8_t* msgs,
                       unsigned long long* wire_bytes, uint8_t* scratch_raw, int32_t* status) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     DecodeShared& sh = *reinterpret_cast<DecodeShared*>(smem_raw);
+    pdl_wait();
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
     const uint64_t N = un.n_values;
@@ -771,7 +811,7 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log
     }
     __syncthreads();
     uint64_t P;  // symbols; Q = bytes of the raw payload
-    const uint64_t Q = raw_payload_bytes(msg, N, dt, log2b, &sh.changed, tid, P);
+    const uint64_t Q = raw_payload_bytes<T>(msg, N, dt, log2b, &sh.changed, tid, P);
     const uint64_t wire = wire_bytes[unit];
     if (Q == 0 || wire == payoff + Q) return;  // nothing travelled, or the raw form did
     const uint64_t C = wire - payoff;
@@ -782,28 +822,31 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log
         if (tid == 0) raise_corrupt(status);
         return;
     }
-    sh.f[tid] = tid < hdr / 2u ? reinterpret_cast<const uint16_t*>(pay)[tid] : (uint16_t)0;
+    if (tid < 256u) sh.f[tid] = tid < hdr / 2u ? reinterpret_cast<const uint16_t*>(pay)[tid] : (uint16_t)0;
     __syncthreads();
-    if (!decoder_tables(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
+    if (!decoder_tables<T>(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
         if (tid == 0) raise_corrupt(status);
         return;
     }
-    // where the segments lie (nseg <= kLongSegs <= kEntThreads: one round)
+    // where the segments lie (nseg <= kLongSegs <= T: one round)
     const uint32_t* dir = reinterpret_cast<const uint32_t*>(pay + hdr);
     const uint8_t* data = pay + hdr + 4ull * nseg;
     const uint64_t data_bytes = C - hdr - 4ull * nseg;
     const uint32_t nw = tid < nseg ? dir[tid] : 0u;
     if (nw > kSegWordsMax) sh.bad = 1;
     uint32_t total;
-    sh.off[tid] = block_scan(tid < nseg ? segment_bytes(min(nw, kSegWordsMax)) : 0u, sh.scan, tid, total);
-    sh.nw[tid] = min(nw, kSegWordsMax);
+    const uint32_t at = block_scan<T>(tid < nseg ? segment_bytes(min(nw, kSegWordsMax)) : 0u, sh.scan, tid, total);
+    if (tid < kLongSegs) {
+        sh.off[tid] = at;
+        sh.nw[tid] = min(nw, kSegWordsMax);
+    }
     __syncthreads();
     if (sh.bad || total != data_bytes) {
         if (tid == 0) raise_corrupt(status);
         return;
     }
     uint8_t* raw = scratch_raw + un.cache_off;  // the unit's stretch of the scratch (16-byte aligned)
-    for (uint32_t g = warp; g < nseg; g += kEntWarps) {
+    for (uint32_t g = warp; g < nseg; g += T / 32) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
         if (!decode_segment(data + sh.off[g], sh.nw[g], n, sh.tab, raw + (uint64_t)g * kSegment, lane))
             sh.bad = 1;
@@ -815,9 +858,9 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log
     }
     // the raw payload goes back into the message, which then is what the sender step had written
     if (HALF) {
-        pack_symbols(raw, pay, log2b, 0, P, tid, kEntThreads);
+        pack_symbols(raw, pay, log2b, 0, P, tid, T);
     } else {
-        for (uint64_t i = (uint64_t)tid * 16; i < P; i += (uint64_t)kEntThreads * 16) {
+        for (uint64_t i = (uint64_t)tid * 16; i < P; i += (uint64_t)T * 16) {
             if (i + 16 <= P) {
                 *reinterpret_cast<uint4*>(pay + i) = *reinterpret_cast<const uint4*>(raw + i);
             } else {
@@ -837,6 +880,7 @@ entropy_long_parse_kernel(const ciera_unit* __restrict__ units, const unsigned l
     __shared__ uint32_t s_scan[kEntWarps];
     __shared__ unsigned long long s_changed;
     __shared__ uint32_t s_bad;
+    pdl_wait();
     const uint32_t li = blockIdx.x, tid = threadIdx.x, unit = long_units[li];
     const ciera_unit un = units[unit];
     const uint64_t N = un.n_values;
@@ -851,7 +895,7 @@ entropy_long_parse_kernel(const ciera_unit* __restrict__ units, const unsigned l
     const uint8_t* msg = msgs + un.msg_off;
     const uint64_t payoff = payload_offset_of(N, dt, log2b);
     uint64_t P;  // symbols; Q = bytes of the raw payload
-    const uint64_t Q = raw_payload_bytes(msg, N, dt, log2b, &s_changed, tid, P);
+    const uint64_t Q = raw_payload_bytes<kEntThreads>(msg, N, dt, log2b, &s_changed, tid, P);
     const uint64_t wire = wire_bytes[unit];
     if (Q == 0 || wire == payoff + Q) return;
     const uint64_t C = wire - payoff;
@@ -872,7 +916,7 @@ entropy_long_parse_kernel(const ciera_unit* __restrict__ units, const unsigned l
         const uint32_t nw = g < nseg ? dir[g] : 0u;
         if (nw > kSegWordsMax) s_bad = 1;
         uint32_t total;
-        const uint32_t off = block_scan(g < nseg ? segment_bytes(min(nw, kSegWordsMax)) : 0u, s_scan, tid, total);
+        const uint32_t off = block_scan<kEntThreads>(g < nseg ? segment_bytes(min(nw, kSegWordsMax)) : 0u, s_scan, tid, total);
         if (g < nseg) {
             scratch_off[slot0 + g] = (uint32_t)(carry + off);
             scratch_nw[slot0 + g] = min(nw, kSegWordsMax);
@@ -900,9 +944,10 @@ entropy_long_decode_kernel(const ciera_unit* __restrict__ units, const unsigned 
                            int32_t* status) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     DecodeShared& sh = *reinterpret_cast<DecodeShared*>(smem_raw);
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     LongState* st = long_state(recs, ch.z);
-    if (st->coded == 0 || ch.y >= st->nseg) return;
+    if (st->coded == 0 || part_first(ch) >= st->nseg) return;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[ch.x];
     const uint64_t P = st->P;
@@ -912,7 +957,7 @@ entropy_long_decode_kernel(const ciera_unit* __restrict__ units, const unsigned 
     sh.f[tid] = tid < hdr / 2u ? reinterpret_cast<const uint16_t*>(pay)[tid] : (uint16_t)0;
     if (tid == 0) sh.bad = 0;
     __syncthreads();
-    if (!decoder_tables(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
+    if (!decoder_tables<kEntThreads>(sh.f, sh.c, sh.base, sh.tab, &sh.flag, tid)) {
         if (tid == 0) {
             st->bad = 1;
             raise_corrupt(status);
@@ -922,8 +967,8 @@ entropy_long_decode_kernel(const ciera_unit* __restrict__ units, const unsigned 
     const uint8_t* data = pay + hdr + 4ull * nseg;
     uint8_t* raw = scratch_raw + un.cache_off;
     const unsigned long long slot0 = seg_base[ch.x];
-    const uint32_t g_end = min(nseg, ch.y + kLongSegs);
-    for (uint32_t g = ch.y + warp; g < g_end; g += kEntWarps) {
+    const uint32_t g_end = min(nseg, part_first(ch) + part_segments());
+    for (uint32_t g = part_first(ch) + warp; g < g_end; g += kEntWarps) {
         const uint32_t n = (uint32_t)min((uint64_t)kSegment, P - (uint64_t)g * kSegment);
         if (!decode_segment(data + scratch_off[slot0 + g], scratch_nw[slot0 + g], n, sh.tab,
                             raw + (uint64_t)g * kSegment, lane))
@@ -940,15 +985,16 @@ __global__ void __launch_bounds__(kEntThreads)
 entropy_long_restore_kernel(const ciera_unit* __restrict__ units, const uint4* __restrict__ chunks, int dt,
                             uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes, const uint8_t* recs_c,
                             const uint8_t* scratch_raw) {
+    pdl_wait();
     const uint4 ch = chunks[blockIdx.x];
     const LongState* st = long_state(const_cast<uint8_t*>(recs_c), ch.z);
     if (st->coded == 0 || st->bad != 0) return;  // raw as received, or damaged: left as it is
     const uint32_t tid = threadIdx.x;
     const ciera_unit un = units[ch.x];
     const uint64_t P = st->P;
-    const uint64_t lo = (uint64_t)ch.y * kSegment;
+    const uint64_t lo = (uint64_t)part_first(ch) * kSegment;
     if (lo >= P) return;
-    const uint64_t hi = min(P, lo + (uint64_t)kLongSegs * kSegment);
+    const uint64_t hi = min(P, lo + (uint64_t)part_segments() * kSegment);
     const uint64_t payoff = payload_offset_of(un.n_values, dt, log2b);
     uint8_t* pay = msgs + un.msg_off + payoff;
     const uint8_t* raw = scratch_raw + un.cache_off;
@@ -963,7 +1009,7 @@ entropy_long_restore_kernel(const ciera_unit* __restrict__ units, const uint4* _
             }
         }
     }
-    if (ch.y == 0 && tid == 0) wire_bytes[ch.x] = payoff + st->Q;
+    if (lo == 0 && tid == 0) wire_bytes[ch.x] = payoff + st->Q;
 }
 
 }  // namespace ciera
@@ -1004,6 +1050,39 @@ static int check_entropy_args(const ciera_plan* p, const void* messages_dev, con
     return CIERA_OK;
 }
 
+// SMs of the current device, and the dynamic shared memory of the receiver's kernels set up once per device
+static int entropy_device(int* sms_out) {
+    static std::atomic<int> cached[64];  // (zero-initialised; any host thread may be the first to fill an entry)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return record_cuda_error(e);
+    if (dev < 0 || dev >= 64) return CIERA_ERR_UNSUPPORTED;
+    if (!cached[dev].load(std::memory_order_acquire)) {
+        for (const void* k : {(const void*)entropy_decode_kernel<false, kEntThreads, 5>, (const void*)entropy_decode_kernel<true, kEntThreads, 5>,
+                              (const void*)entropy_decode_kernel<false, kEntThreads, 8>, (const void*)entropy_decode_kernel<true, kEntThreads, 8>,
+                              (const void*)entropy_decode_kernel<false, kEntWide, 1>, (const void*)entropy_decode_kernel<true, kEntWide, 1>,
+                              (const void*)entropy_long_decode_kernel<false>, (const void*)entropy_long_decode_kernel<true>}) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecodeShared));
+            if (e != cudaSuccess) return record_cuda_error(e);
+        }
+        int sms = 0;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return record_cuda_error(e);
+        if (sms < 1) return CIERA_ERR_UNSUPPORTED;
+        cached[dev].store(sms, std::memory_order_release);
+    }
+    *sms_out = cached[dev].load(std::memory_order_acquire);
+    return CIERA_OK;
+}
+// wide blocks for the units as long as each has an SM to itself
+static bool wide_units(uint32_t units, int sms) { return units <= (uint32_t)sms; }
+// thread blocks to a chunk of kLongSegs segments: enough for five on every SM, at least a segment for each of their warps
+static uint32_t chunk_parts(uint32_t chunks, int sms) {
+    uint32_t parts = 1;
+    while (parts < kLongSegs / kEntWarps && chunks * parts < 5u * (uint32_t)sms) parts *= 2;
+    return parts;
+}
+
 extern "C" int ciera_entropy_encode(const ciera_plan* p, void* messages_dev, uint64_t* wire_bytes_dev, void* scratch_dev,
                                     void* stream) {
     int rc = check_entropy_args(p, messages_dev, wire_bytes_dev, scratch_dev);
@@ -1020,33 +1099,35 @@ extern "C" int ciera_entropy_encode(const ciera_plan* p, void* messages_dev, uin
     uint8_t* msgs = (uint8_t*)messages_dev;
     unsigned long long* wire = (unsigned long long*)wire_bytes_dev;
     const uint32_t n_long = (uint32_t)p->ent_long_units.size(), n_chunks = (uint32_t)p->ent_chunks.size();
+    int sms = 0;
+    if ((rc = entropy_device(&sms))) return rc;
+    cudaError_t e = cudaSuccess;
     if (n_long < p->n_units) {
-        auto* k = dt == CIERA_FP16 ? entropy_encode_kernel<true> : entropy_encode_kernel<false>;
-        k<<<p->n_units, kEntThreads, 0, s>>>(p->units_dev, p->seg_base_dev, dt, p->log2b, msgs, wire, slots, nw, sym);
+        const bool wide = wide_units(p->n_units - n_long, sms);
+        auto* k = dt == CIERA_FP16 ? (wide ? entropy_encode_kernel<true, kEntWide> : entropy_encode_kernel<true, kEntThreads>)
+                                   : (wide ? entropy_encode_kernel<false, kEntWide> : entropy_encode_kernel<false, kEntThreads>);
+        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev, dt, p->log2b,
+                         msgs, wire, slots, nw, sym);
+        if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
-        if ((rc = check_launch())) return rc;
     }
     if (n_long) {
-        cudaError_t e = cudaMemsetAsync(recs, 0, (size_t)n_long * kLongRec, s);  // the counts start at zero
+        const dim3 parts(n_chunks, chunk_parts(n_chunks, sms));
+        auto launch = [&](auto* k, dim3 grid, auto... args) {
+            if (e == cudaSuccess) e = launch_after(k, grid, kEntThreads, 0, s, args...);
+            if (e == cudaSuccess) count_launch();
+        };
+        e = cudaMemsetAsync(recs, 0, (size_t)n_long * kLongRec, s);  // the counts start at zero
+        if (dt == CIERA_FP16) launch(entropy_long_unpack_kernel, parts, p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire, sym);
+        launch(entropy_long_hist_kernel, parts, p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire, recs, sym);
+        launch(entropy_long_model_kernel, dim3(n_long), p->units_dev, p->ent_long_units_dev, dt, p->log2b, msgs, wire, recs);
+        launch(dt == CIERA_FP16 ? entropy_long_encode_kernel<true> : entropy_long_encode_kernel<false>, parts, p->units_dev,
+               p->seg_base_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire, recs, slots, nw, sym);
+        launch(entropy_long_layout_kernel, dim3(n_long), p->units_dev, p->seg_base_dev, p->ent_long_units_dev, dt, p->log2b, msgs,
+               wire, recs, nw, off);
+        launch(entropy_long_copy_kernel, parts, p->units_dev, p->seg_base_dev, p->ent_chunks_dev, dt, p->log2b, msgs, recs, slots,
+               nw, off);
         if (e != cudaSuccess) return record_cuda_error(e);
-        if (dt == CIERA_FP16) {
-            entropy_long_unpack_kernel<<<n_chunks, kEntThreads, 0, s>>>(p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs,
-                                                                        wire, sym);
-            count_launch();
-        }
-        entropy_long_hist_kernel<<<n_chunks, kEntThreads, 0, s>>>(p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire,
-                                                                  recs, sym);
-        entropy_long_model_kernel<<<n_long, kEntThreads, 0, s>>>(p->units_dev, p->ent_long_units_dev, dt, p->log2b, msgs,
-                                                                 wire, recs);
-        auto* k = dt == CIERA_FP16 ? entropy_long_encode_kernel<true> : entropy_long_encode_kernel<false>;
-        k<<<n_chunks, kEntThreads, 0, s>>>(p->units_dev, p->seg_base_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire, recs,
-                                           slots, nw, sym);
-        entropy_long_layout_kernel<<<n_long, kEntThreads, 0, s>>>(p->units_dev, p->seg_base_dev, p->ent_long_units_dev, dt,
-                                                                  p->log2b, msgs, wire, recs, nw, off);
-        entropy_long_copy_kernel<<<n_chunks, kEntThreads, 0, s>>>(p->units_dev, p->seg_base_dev, p->ent_chunks_dev, dt,
-                                                                  p->log2b, msgs, recs, slots, nw, off);
-        for (int i = 0; i < 5; ++i) count_launch();
-        if ((rc = check_launch())) return rc;
     }
     return CIERA_OK;
 }
@@ -1055,22 +1136,9 @@ extern "C" int ciera_entropy_decode(const ciera_plan* p, void* messages_dev, uin
                                     int32_t* status_dev, void* stream) {
     int rc = check_entropy_args(p, messages_dev, wire_bytes_dev, scratch_dev);
     if (rc || p->tiles.empty()) return rc;
-    static std::atomic<int> configured[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return record_cuda_error(e);
-    if (dev < 0 || dev >= 64) return CIERA_ERR_UNSUPPORTED;
-    if (!configured[dev].load(std::memory_order_acquire)) {
-        for (auto* k : {entropy_decode_kernel<false>, entropy_decode_kernel<true>}) {
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecodeShared));
-            if (e != cudaSuccess) return record_cuda_error(e);
-        }
-        for (auto* k : {entropy_long_decode_kernel<false>, entropy_long_decode_kernel<true>}) {
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecodeShared));
-            if (e != cudaSuccess) return record_cuda_error(e);
-        }
-        configured[dev].store(1, std::memory_order_release);
-    }
+    int sms = 0;
+    if ((rc = entropy_device(&sms))) return rc;
+    cudaError_t e = cudaSuccess;
     cudaStream_t s = (cudaStream_t)stream;
     const ScratchLayout L = scratch_layout(p);
     uint8_t* base = (uint8_t*)scratch_dev;
@@ -1083,21 +1151,31 @@ extern "C" int ciera_entropy_decode(const ciera_plan* p, void* messages_dev, uin
     unsigned long long* wire = (unsigned long long*)wire_bytes_dev;
     const uint32_t n_long = (uint32_t)p->ent_long_units.size(), n_chunks = (uint32_t)p->ent_chunks.size();
     if (n_long < p->n_units) {
-        auto* k = dt == CIERA_FP16 ? entropy_decode_kernel<true> : entropy_decode_kernel<false>;
-        k<<<p->n_units, kEntThreads, sizeof(DecodeShared), s>>>(p->units_dev, dt, p->log2b, msgs, wire, raw, status_dev);
+        const bool wide = wide_units(p->n_units - n_long, sms);
+        const bool few = p->n_units - n_long <= 5u * (uint32_t)sms;
+        auto* k = dt == CIERA_FP16 ? (wide  ? entropy_decode_kernel<true, kEntWide, 1>
+                                      : few ? entropy_decode_kernel<true, kEntThreads, 5>
+                                            : entropy_decode_kernel<true, kEntThreads, 8>)
+                                   : (wide  ? entropy_decode_kernel<false, kEntWide, 1>
+                                      : few ? entropy_decode_kernel<false, kEntThreads, 5>
+                                            : entropy_decode_kernel<false, kEntThreads, 8>);
+        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev, dt, p->log2b,
+                         msgs, wire, raw, status_dev);
+        if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
-        if ((rc = check_launch())) return rc;
     }
     if (n_long) {
-        entropy_long_parse_kernel<<<n_long, kEntThreads, 0, s>>>(p->units_dev, p->seg_base_dev, p->ent_long_units_dev, dt,
-                                                                 p->log2b, msgs, wire, recs, off, nw, status_dev);
-        auto* k = dt == CIERA_FP16 ? entropy_long_decode_kernel<true> : entropy_long_decode_kernel<false>;
-        k<<<n_chunks, kEntThreads, sizeof(DecodeShared), s>>>(p->units_dev, p->seg_base_dev, p->ent_chunks_dev, dt, p->log2b,
-                                                              msgs, recs, off, nw, raw, status_dev);
-        entropy_long_restore_kernel<<<n_chunks, kEntThreads, 0, s>>>(p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs,
-                                                                     wire, recs, raw);
-        for (int i = 0; i < 3; ++i) count_launch();
-        if ((rc = check_launch())) return rc;
+        const dim3 parts(n_chunks, chunk_parts(n_chunks, sms));
+        auto launch = [&](auto* k, dim3 grid, size_t smem, auto... args) {
+            if (e == cudaSuccess) e = launch_after(k, grid, kEntThreads, smem, s, args...);
+            if (e == cudaSuccess) count_launch();
+        };
+        launch(entropy_long_parse_kernel, dim3(n_long), 0, p->units_dev, p->seg_base_dev, p->ent_long_units_dev, dt, p->log2b, msgs,
+               wire, recs, off, nw, status_dev);
+        launch(dt == CIERA_FP16 ? entropy_long_decode_kernel<true> : entropy_long_decode_kernel<false>, parts, sizeof(DecodeShared),
+               p->units_dev, p->seg_base_dev, p->ent_chunks_dev, dt, p->log2b, msgs, recs, off, nw, raw, status_dev);
+        launch(entropy_long_restore_kernel, parts, 0, p->units_dev, p->ent_chunks_dev, dt, p->log2b, msgs, wire, recs, raw);
+        if (e != cudaSuccess) return record_cuda_error(e);
     }
     return CIERA_OK;
 }

@@ -72,3 +72,58 @@ def test_models_and_lengths():
     for u, part in zip(codec.units, parts):
         lo = int(u["weights_off"]) // 2
         assert np.array_equal(out[lo : lo + part.size], part)
+
+
+@pytest.mark.parametrize("dtype", [0, 2])
+@pytest.mark.parametrize("n_units", [148, 149, 741])
+def test_numbers_of_units(n_units, dtype):
+    """A wide thread block per unit up to one per SM, narrow ones beyond, and those in two builds by their number."""
+    from paper_2609_04609_b200 import runtime
+
+    name = {0: "bf16", 2: "fp16"}[dtype]
+    codec = guard(runtime.LayerCodec.from_tensors([4096 + 37 * (i % 5) for i in range(n_units)], 1, name, 64, DEV, slack=256))
+    gen = torch.Generator().manual_seed(n_units)
+    w = (torch.randn(codec.weights_bytes // 2, generator=gen) * 0.02).to({0: torch.bfloat16, 2: torch.float16}[dtype])
+    bits = w.view(torch.int16).numpy().view(np.uint16)
+    codec.init_caches(None)
+    codec.encode(to_dev_bytes(bits, DEV))
+    codec.entropy_encode()
+    torch.cuda.synchronize()
+    sent, wire = codec.msg_send.cpu().numpy(), codec.wire_bytes.cpu().numpy().copy()
+    codec.transport()
+    codec.entropy_decode()
+    torch.cuda.synchronize()
+    codec.check_status()
+    back, raw_wire = codec.msg_recv.cpu().numpy(), codec.wire_bytes.cpu().numpy()
+    for i, u in enumerate(codec.units):
+        n, lo, mo = int(u["n_values"]), int(u["weights_off"]) // 2, int(u["msg_off"])
+        raw = ora.encode(bits[lo : lo + n], np.zeros(n, np.uint8), dtype, 64)[0]
+        want = rans.entropy_encode_message(raw, n, dtype, 64)
+        assert want.size < raw.size and int(wire[i]) == want.size and int(raw_wire[i]) == raw.size
+        assert np.array_equal(sent[mo : mo + want.size], want) and np.array_equal(back[mo : mo + raw.size], raw)
+    codec.canaries.check("units")
+
+
+@pytest.mark.parametrize("chunks", [92, 100, 200, 400])
+def test_chunks_of_long_units_in_parts(chunks):
+    """One long unit of so many chunks that each is the work of 8, 8, 4 and 2 thread blocks: coded shorter, restored."""
+    from paper_2609_04609_b200 import runtime
+
+    codec = runtime.LayerCodec.from_tensors([262_144 * (chunks - 1) + 4097], 1, "bf16", 512, DEV)
+    gen = torch.Generator(DEV).manual_seed(chunks)
+    w = (torch.randn(codec.weights_bytes // 2, generator=gen, device=DEV) * 0.02).bfloat16().view(torch.uint8)
+    codec.init_caches(None)
+    codec.encode(w)
+    raw_wire = int(codec.wire_bytes[0])
+    raw = codec.msg_send[:raw_wire].clone()
+    codec.entropy_encode()
+    coded = int(codec.wire_bytes[0])
+    assert coded < 0.75 * raw_wire
+    codec.transport()
+    codec.entropy_decode()
+    codec.decode()
+    torch.cuda.synchronize()
+    codec.check_status()
+    assert int(codec.wire_bytes[0]) == raw_wire and torch.equal(codec.msg_recv[:raw_wire], raw)
+    n = 2 * int(codec.units[0]["n_values"])
+    assert torch.equal(codec.weights_out[:n], w[:n])
