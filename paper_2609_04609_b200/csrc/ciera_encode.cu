@@ -61,10 +61,27 @@
 namespace ciera {
 
 constexpr int kResolvers = 2;  // resolver warps (20 warps per block: two blocks per SM at 48 registers per thread)
-constexpr int kEncodeThreads = kThreads + 64 + 32 * kResolvers;  // consumers + producer + aggregator + resolvers
-constexpr int kProducerWarp = kWarps;                            // 16
-constexpr int kAggregatorWarp = kWarps + 1;                      // 17
-constexpr int kResolverWarp0 = kWarps + 2;                       // 18 ..
+// Consumer warps of a block, and how they share a tile.  With HashCache and 2-byte values, where the kernel is bound by
+// instruction issue, 8 warps take four pieces a thread: what a warp spends on a tile as such (waits, addresses, sending)
+// is spent half as often, and a warp's pieces are rows of 256 neighbouring values, so that rows of one block are added
+// up in registers before anything is exchanged between lanes: OLMoE-shaped layer 0.355 -> 0.302 ms with 512 values per
+// block, 0.400 -> 0.356 with 64, 0.393 -> 0.309 with 4096.  (Three blocks per SM instead of two: 0.297, 0.376, 0.306, and
+// small tables 8-15 % slower.  HASH == 3, whose consumers finish the hashes themselves, 0.494 -> 0.585: it keeps 16.)
+template <int DT, int HASH>
+constexpr int kConsumerWarps = (HASH == 1 || HASH == 2) && DT != CIERA_FP32 ? 8 : kWarps;
+template <int DT, int HASH>
+constexpr int kEncodeThreads = 32 * (kConsumerWarps<DT, HASH> + 2 + kResolvers);  // + producer, aggregator, resolvers
+template <int DT, int CW>
+struct Share {
+    using P = Piece<DT>;
+    static constexpr int kPerThread = kTileValues / (32 * CW * P::kValues);
+    // first value (inside the tile) of piece p of consumer thread tid
+    static __device__ __forceinline__ uint32_t start(uint32_t tid, int p) {
+        if (CW == kWarps) return P::start(tid, p);
+        return ((tid >> 5) * (uint32_t)kPerThread + (uint32_t)p) * (32u * P::kValues) + (tid & 31u) * P::kValues;
+    }
+};
+constexpr uint32_t kRowL2 = 8;  // log2(values of a row) in the second layout
 constexpr int kDescRing = 16;                                    // > exponent stages + 2
 constexpr int kVoteWords = 32;  // vote bits of a tile: up to 1024 pieces
 
@@ -416,7 +433,8 @@ template <int DT, bool BY_CONSUMERS>
 __device__ __forceinline__ uint32_t hash_block_bitmap(const ulonglong2* part, const ulonglong2* hold, ulonglong2* hash_dst,
                                                       uint32_t* bm, uint16_t* pre, uint32_t log2b, uint32_t nv,
                                                       uint32_t lane) {
-    constexpr uint32_t kGroupL2 = 5 + Piece<DT>::kLog2Values;  // log2(values of a warp's pieces)
+    // log2(values behind a partial sum): a warp's pieces, or in rows (8 consumer warps) all four of its rows
+    constexpr uint32_t kGroupL2 = kConsumerWarps<DT, 1> == kWarps ? 5 + Piece<DT>::kLog2Values : kRowL2 + 2;
     const uint32_t B = 1u << log2b;
     const uint32_t nbt = kTileValues >> log2b;
     const uint32_t nblk = (nv + B - 1u) >> log2b;
@@ -501,6 +519,36 @@ __device__ __forceinline__ void reduce_hash_terms(const uint64_t* a, const uint6
         const uint32_t r = lane & ((1u << l2) - 1u);
         if (r < 4) part[2 * ((r & 2u) ? e1 : e0) + (r & 1u)] = t;  // lanes 0..3: a of piece 0, b of piece 0, a, b of piece 1
     }
+}
+
+// The same for four rows of one warp (see Share): rows that lie in one block are added up first, entry of a group =
+// index of its values in units of the smaller of block and warp.  v0: the first value of this thread.  Blocks of 64 values and more (l2 >= 3); 9, 6 or 5 shuffles
+// of 64 bits for blocks of up to 256, 512, or 1024 values and more.
+__device__ __forceinline__ void reduce_hash_rows(uint64_t (&a)[4], uint64_t (&b)[4], uint32_t l2, uint32_t log2b, uint32_t v0,
+                                                 uint64_t* part, uint32_t lane) {
+    if (log2b > kRowL2 + 1) {
+        const uint64_t sa = (a[0] + a[1]) + (a[2] + a[3]), sb = (b[0] + b[1]) + (b[2] + b[3]);
+        reduce_hash_terms<1>(&sa, &sb, 5u, v0 >> (kRowL2 + 2), 0u, part, lane);
+        return;
+    }
+    if (log2b == kRowL2 + 1) {
+        const uint64_t sa[2] = {a[0] + a[1], a[2] + a[3]}, sb[2] = {b[0] + b[1], b[2] + b[3]};
+        reduce_hash_terms<2>(sa, sb, 5u, v0 >> log2b, (v0 >> log2b) + 1u, part, lane);
+        return;
+    }
+    const bool odd = (lane & 1u) != 0, second = (lane & 2u) != 0, third = (lane & 4u) != 0;
+    uint64_t k[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) k[p] = (odd ? b[p] : a[p]) + __shfl_xor_sync(0xffffffffu, odd ? a[p] : b[p], 1);
+    const uint64_t t0 = (second ? k[1] : k[0]) + __shfl_xor_sync(0xffffffffu, second ? k[0] : k[1], 2);
+    const uint64_t t1 = (second ? k[3] : k[2]) + __shfl_xor_sync(0xffffffffu, second ? k[2] : k[3], 2);
+    uint64_t u = (third ? t1 : t0) + __shfl_xor_sync(0xffffffffu, third ? t0 : t1, 4);
+#pragma unroll
+    for (uint32_t o = 3; o < 5; ++o)
+        if (o < l2) u += __shfl_xor_sync(0xffffffffu, u, 1u << o);
+    // lanes 0..7 of a group: bit 0 which sum, bits 1 and 2 the row
+    const uint32_t r = lane & ((1u << l2) - 1u);
+    if (r < 8u) part[2u * ((v0 + ((r >> 1) << kRowL2)) >> log2b) + (r & 1u)] = u;
 }
 
 // HashCache, consumers, kernel instance HASH == 3 (blocks that lie inside one warp's pieces and span at least two
@@ -638,14 +686,14 @@ __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t 
 // (CACHE = false, the sender with HashCache: payload only.)
 // (FULL: the tile is a full one, every piece complete.)
 // (STEP: the same bytes also go to the received message and to the receiver's cache.)
-template <int DT, bool CACHE, bool FULL, bool STEP>
+template <int DT, bool CACHE, bool FULL, bool STEP, class SHARE>
 __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm,
                                               const uint16_t* pre, uint64_t base, const uint8_t* s_exp, const StepTwins& tw,
                                               uint32_t tid) {
     using P = Piece<DT>;
 #pragma unroll
-    for (int p = 0; p < P::kPerThread; ++p) {
-        const uint32_t t0 = P::start(tid, p);
+    for (int p = 0; p < SHARE::kPerThread; ++p) {
+        const uint32_t t0 = SHARE::start(tid, p);
         const int nvalid = FULL ? (int)P::kValues : piece_valid<DT>(t0, ti.nv);
         if (nvalid == 0) continue;
         const uint32_t kb = t0 >> log2b;
@@ -917,9 +965,9 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
         // (as in the consumers' main loop: the two instances named there keep the one form that tests as it goes)
         constexpr bool kOneBody = (DT == CIERA_BF16 && HASH == 0 && !STEP) || (DT == CIERA_FP32 && HASH != 0);
         if (!kOneBody && ti.nv == (uint32_t)kTileValues)
-            write_changed<DT, HASH == 0, true, STEP>(ti, log2b, bm, pre, base, s_exp, tw, tid);
+            write_changed<DT, HASH == 0, true, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
         else
-            write_changed<DT, HASH == 0, false, STEP>(ti, log2b, bm, pre, base, s_exp, tw, tid);
+            write_changed<DT, HASH == 0, false, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
     } else if (DT != CIERA_FP16 && ti.nv == (uint32_t)kTileValues &&
                tile_payload_bytes >= (uint32_t)kTileValues / kGatherDensity) {
         // a full tile in which many exponents changed: gathered in shared memory, written out in whole pieces
@@ -942,7 +990,7 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
 // `cache` is the sender's exponent cache or, with HASH, its HashCache; `tile_hash` (HASH only) gives
 // the index of every tile's first block in it.
 template <int DT, bool FINE, int HASH, bool STEP>
-__global__ void __launch_bounds__(kEncodeThreads, kEncodeBlocksPerSM<DT, STEP>)
+__global__ void __launch_bounds__(kEncodeThreads<DT, HASH>, kEncodeBlocksPerSM<DT, STEP>)
 encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
               uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
@@ -951,6 +999,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     static_assert(!(HASH && FINE), "HashCache: blocks of 16 values and more");
     static_assert(!(HASH && STEP), "the whole step compares with the exponent cache");
     using P = Piece<DT>;
+    constexpr int CW = kConsumerWarps<DT, HASH>;
+    using S = Share<DT, CW>;
     constexpr int VB = Traits<DT>::kValueBytes;
     constexpr int SMB = Traits<DT>::kSmBytes;
     using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
@@ -982,19 +1032,19 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     const bool early_clear = spread_first < n_tiles && n_tiles - clear_first <= kEarlyClearTiles;
     volatile int* abort = &ctl->abort;
     // FINE: every consumer warp's gather space for its changed exponents (in place of the hash stages)
-    uint8_t* const s_gather = ring_h + (size_t)(warp < (uint32_t)kWarps ? warp : 0u) * kWarpGatherBytes;
+    uint8_t* const s_gather = ring_h + (size_t)(warp < (uint32_t)CW ? warp : 0u) * kWarpGatherBytes;
 
     if (tid == 0) {
         for (int s = 0; s < SW; ++s) {
             mbar_init(&ctl->full_w[s], 1);
-            mbar_init(&ctl->empty_w[s], kWarps);
+            mbar_init(&ctl->empty_w[s], CW);
         }
         for (int s = 0; s < SE; ++s) {
             mbar_init(&ctl->full_e[s], 1);
-            mbar_init(&ctl->voted[s], kWarps);
+            mbar_init(&ctl->voted[s], CW);
             mbar_init(&ctl->summed[s], 1);
             mbar_init(&ctl->resolved[s], 1);
-            mbar_init(&ctl->empty_e[s], kWarps);
+            mbar_init(&ctl->empty_e[s], CW);
         }
         ctl->abort = 0;
         ctl->issued = 0;
@@ -1007,7 +1057,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     // The block's tiles form a sequence k = 0, 1, 2, ... that only the producer knows in advance;
     // it closes the sequence with kResolvers end markers (one for each resolver warp), which the
     // other roles pass on to each other through the same barriers as real tiles.
-    if (warp == kProducerWarp) {
+    if (warp == (uint32_t)CW) {
         // ---------------------------------------------------------------- producer
         if (lane == 0) {
             TileWalk walk(seq_runs, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
@@ -1088,7 +1138,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 ctl->issued = k + 1;
             }
         }
-    } else if (warp == kAggregatorWarp) {
+    } else if (warp == (uint32_t)CW + 1u) {
         // ---------------------------------------------------------------- aggregator
         uint64_t run_incl = 0;  // payload bytes of the current alone-worked unit up to the last tile
         uint32_t byte_acc = 0;  // its bitmap byte in the making (tiles of fewer than 8 blocks)
@@ -1153,9 +1203,9 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if (seq) mbar_arrive(&ctl->resolved[se]);
             }
         }
-    } else if (warp >= kResolverWarp0) {
+    } else if (warp >= (uint32_t)CW + 2u) {
         // ---------------------------------------------------------------- resolvers (slots k = i, i + R, ...)
-        for (uint32_t k = warp - kResolverWarp0;; k += kResolvers) {
+        for (uint32_t k = warp - ((uint32_t)CW + 2u);; k += kResolvers) {
             const uint32_t se = k % SE;
             if (!mbar_wait(&ctl->summed[se], (k / SE) & 1u, abort, status)) break;
             const uint32_t tile = ctl->tile_idx[k % kDescRing];
@@ -1215,7 +1265,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 uint8_t* const s_w = ring_w + (size_t)sw * kWStage;
                 const uint8_t* const s_r = s_w + kWBytes;  // STEP: the receiver's cached exponents
                 uint8_t* const s_e = ring_e + (size_t)se * kEBytes;
-                uint64_t hash_a[P::kPerThread], hash_b[P::kPerThread];  // HASH: the pieces' sums of terms
+                uint64_t hash_a[S::kPerThread], hash_b[S::kPerThread];  // HASH: the pieces' sums of terms
                 // The pieces of this thread.  Most instances compile the loop twice: for full tiles (staged
                 // in shared memory, every piece complete, no tests on the way) and for a unit's last, short
                 // tile; that measured 2-12 % faster (fp16 most).  Two instances keep one loop that tests as it
@@ -1248,16 +1298,17 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     if constexpr (HASH == 3) {
                         // the tile's cached hashes have to be there now (they land on full_e)
                         if (!mbar_wait(&ctl->full_e[se], pe, abort, status)) break;
-                        finish_hash_groups<DT, P::kPerThread>(hash_a, hash_b, hash_lanes_l2, log2b, nv, tid,
+                        finish_hash_groups<DT, S::kPerThread>(hash_a, hash_b, hash_lanes_l2, log2b, nv, tid,
                                                               reinterpret_cast<const uint64_t*>(ring_h + (size_t)se * kHStage),
                                                               reinterpret_cast<uint64_t*>(ti.c_ptr),
                                                               reinterpret_cast<uint8_t*>(part), lane);
+                    } else if constexpr (S::kPerThread == 4) {
+                        reduce_hash_rows(hash_a, hash_b, hash_lanes_l2, log2b, S::start(tid, 0), part, lane);
                     } else {
-                        reduce_hash_terms<P::kPerThread>(hash_a, hash_b, hash_lanes_l2, (P::start(tid, 0) >> P::kLog2Values) >> hash_lanes_l2,
-                                                         (P::start(tid, P::kPerThread - 1) >> P::kLog2Values) >> hash_lanes_l2, part, lane);
+                        reduce_hash_terms<S::kPerThread>(hash_a, hash_b, hash_lanes_l2, (S::start(tid, 0) >> P::kLog2Values) >> hash_lanes_l2,
+                                                         (S::start(tid, S::kPerThread - 1) >> P::kLog2Values) >> hash_lanes_l2, part, lane);
                     }
                 }
-                if (kBulkOut && !kRebuild) fence_async_shared();
                 __syncwarp();  // the warp's shared-memory accesses above are ordered before lane 0's arrives
                 if (lane == 0) {
                     mbar_arrive(&ctl->voted[se]);
@@ -1367,7 +1418,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (uint32_t t = clear_first + tid; t < n_tiles; t += kEncodeThreads) st_status(tile_status + t, 0ull);
+        for (uint32_t t = clear_first + tid; t < n_tiles; t += kEncodeThreads<DT, HASH>) st_status(tile_status + t, 0ull);
         if (tid == 0) atomicExch(blocks_done, 0u);
     }
 }
@@ -1397,7 +1448,7 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
                                  (int)encode_smem_bytes<DT, FINE, HASH, STEP>(FINE ? 0u : HASH == 1 ? kHashShortRingsLog2 + 1u : kFineLog2));
         if (e != cudaSuccess) return record_cuda_error(e);
         int per_sm = 0, sms = 0, coop = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH, STEP>, kEncodeThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH, STEP>, kEncodeThreads<DT, HASH>, smem);
         if (e != cudaSuccess) return record_cuda_error(e);
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return record_cuda_error(e);
@@ -1457,10 +1508,10 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
         // GPU together, which is what the look-back between blocks relies on
         void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
                         &changed_blocks_dev, &ts, &ticket, &done, &status_dev, &tile_hash, &tw};
-        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads), args,
+        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
                                         smem, s);
     } else {
-        e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads, smem, s, tiles, nt, seq_runs, n_runs,
+        e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
                          spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
                          tile_hash, tw);
     }
