@@ -146,6 +146,10 @@ __device__ __forceinline__ void store_bytes_partial(uint8_t* dst, const uint32_t
 }
 
 
+// keeps the first n (0 .. 4) bytes of a word / the first n (0 .. 2) half-words
+__device__ __forceinline__ uint32_t keep_bytes(uint32_t w, int n) { return n >= 4 ? w : n <= 0 ? 0u : w & ((1u << (8 * n)) - 1u); }
+__device__ __forceinline__ uint32_t keep_halves(uint32_t w, int n) { return n >= 2 ? w : n <= 0 ? 0u : w & 0xFFFFu; }
+
 // ---- flags of fine blocks ------------------------------------------------------------------
 // bit 7 of every byte of the result tells whether that byte of d is non-zero
 __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t d) {
@@ -209,6 +213,12 @@ struct Piece<CIERA_BF16> {
         bf16_split4(x[0], x[1], e[0], s[0]);
         bf16_split4(x[2], x[3], e[1], s[1]);
     }
+    // the first nvalid values of a whole piece in shared memory; the others read as +0.0 (exponent 0)
+    __device__ __forceinline__ void split_first(const uint8_t* w, int nvalid) {
+        const uint4 a = Shared::ld16(w);
+        bf16_split4(keep_halves(a.x, nvalid), keep_halves(a.y, nvalid - 2), e[0], s[0]);
+        bf16_split4(keep_halves(a.z, nvalid - 4), keep_halves(a.w, nvalid - 6), e[1], s[1]);
+    }
     template <class M>
     __device__ __forceinline__ void load_exp_full(const uint8_t* src) {
         const uint2 v = M::ld8(src);
@@ -217,6 +227,11 @@ struct Piece<CIERA_BF16> {
     template <class M>
     __device__ __forceinline__ void store_exp_full(uint8_t* dst) const { M::st8(dst, make_uint2(e[0], e[1])); }
     __device__ __forceinline__ void load_exp_partial(const uint8_t* src, int nvalid) { load_bytes_partial<8>(e, src, nvalid); }
+    // the first nvalid exponents of a whole piece in shared memory; the others read as 0
+    __device__ __forceinline__ void load_exp_first(const uint8_t* src, int nvalid) {
+        const uint2 v = Shared::ld8(src);
+        e[0] = keep_bytes(v.x, nvalid); e[1] = keep_bytes(v.y, nvalid - 4);
+    }
     __device__ __forceinline__ void store_exp_partial(uint8_t* dst, int nvalid) const { store_bytes_partial<8>(dst, e, nvalid); }
     template <class M>
     __device__ __forceinline__ void load_sm_full(const uint8_t* src) {
@@ -291,6 +306,19 @@ struct Piece<CIERA_FP32> {
         for (int i = 0; i < 16; ++i) x[i] = i < nvalid ? p[i] : 0u;
         from_words(x);
     }
+    // the first nvalid values of a whole piece in shared memory; the others read as +0.0 (exponent 0)
+    __device__ __forceinline__ void split_first(const uint8_t* w, int nvalid) {
+        uint32_t x[16];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint4 v = Shared::ld16(w + 16 * i);
+            x[4 * i] = v.x; x[4 * i + 1] = v.y; x[4 * i + 2] = v.z; x[4 * i + 3] = v.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i >= nvalid) x[i] = 0u;
+        from_words(x);
+    }
     template <class M>
     __device__ __forceinline__ void load_exp_full(const uint8_t* src) {
         const uint4 v = M::ld16(src);
@@ -299,6 +327,12 @@ struct Piece<CIERA_FP32> {
     template <class M>
     __device__ __forceinline__ void store_exp_full(uint8_t* dst) const { M::st16(dst, make_uint4(e[0], e[1], e[2], e[3])); }
     __device__ __forceinline__ void load_exp_partial(const uint8_t* src, int nvalid) { load_bytes_partial<16>(e, src, nvalid); }
+    // the first nvalid exponents of a whole piece in shared memory; the others read as 0
+    __device__ __forceinline__ void load_exp_first(const uint8_t* src, int nvalid) {
+        const uint4 v = Shared::ld16(src);
+        e[0] = keep_bytes(v.x, nvalid); e[1] = keep_bytes(v.y, nvalid - 4);
+        e[2] = keep_bytes(v.z, nvalid - 8); e[3] = keep_bytes(v.w, nvalid - 12);
+    }
     __device__ __forceinline__ void store_exp_partial(uint8_t* dst, int nvalid) const { store_bytes_partial<16>(dst, e, nvalid); }
     template <class M>
     __device__ __forceinline__ void load_sm_full(const uint8_t* src) {
@@ -426,6 +460,13 @@ struct Piece<CIERA_FP16> {
             if (i < nvalid) w[i >> 1] |= (uint32_t)p[i] << (16 * (i & 1));
         split_words(w);
     }
+    // the first nvalid values of a whole piece in shared memory; the others read as +0.0
+    __device__ __forceinline__ void split_first(const uint8_t* src, int nvalid) {
+        const uint4 v = Shared::ld16(src);
+        const uint32_t w[4] = {keep_halves(v.x, nvalid), keep_halves(v.y, nvalid - 2), keep_halves(v.z, nvalid - 4),
+                               keep_halves(v.w, nvalid - 6)};
+        split_words(w);
+    }
     template <class M>
     __device__ __forceinline__ void merge_store_full(uint8_t* dst) const {
         uint32_t w[4];
@@ -448,6 +489,11 @@ struct Piece<CIERA_FP16> {
     template <class M>
     __device__ __forceinline__ void store_exp_full(uint8_t* dst) const { M::st8(dst, make_uint2(e[0], e[1])); }
     __device__ __forceinline__ void load_exp_partial(const uint8_t* src, int nvalid) { load_bytes_partial<8>(e, src, nvalid); }
+    // the first nvalid exponents of a whole piece in shared memory; the others read as 0
+    __device__ __forceinline__ void load_exp_first(const uint8_t* src, int nvalid) {
+        const uint2 v = Shared::ld8(src);
+        e[0] = keep_bytes(v.x, nvalid); e[1] = keep_bytes(v.y, nvalid - 4);
+    }
     __device__ __forceinline__ void store_exp_partial(uint8_t* dst, int nvalid) const { store_bytes_partial<8>(dst, e, nvalid); }
     __device__ __forceinline__ bool differs(const Piece& o) const { return ((e[0] ^ o.e[0]) | (e[1] ^ o.e[1])) != 0; }
     // one flag per block of 2^log2b values (log2b <= 3), lowest block first (the exponents lie one byte each, as for bf16)

@@ -767,33 +767,24 @@ __device__ __forceinline__ void reconstruct(const EncodeTileInfo& ti, uint32_t l
         if (nvalid == 0) continue;
         const uint32_t kb = t0 >> log2b;
         const bool changed = (bm[kb >> 5] >> (kb & 31u)) & 1u;
-        const uint8_t* const w = ti.w_src + (size_t)t0 * VB;
-        uint8_t* const out = const_cast<uint8_t*>(w) + tw.weights;
+        uint8_t* const out = const_cast<uint8_t*>(ti.w_src) + tw.weights + (size_t)t0 * VB;
+        const uint8_t* const r = ti.c_ptr + tw.cache + t0;
         P x;
-        if (FULL) {
-            x.template split_full<Shared>(s_w + (size_t)t0 * VB);
-            if (!changed) {
-                if (ti.r_staged)
-                    x.template load_exp_full<Shared>(s_r + t0);
-                else
-                    x.template load_exp_full<Global>(ti.c_ptr + tw.cache + t0);
-            }
-            if (BULK)
-                x.template merge_store_full<Shared>(s_w + (size_t)t0 * VB);
+        x.template split_full<Shared>(s_w + (size_t)t0 * VB);  // (values past the unit's end are not stored below)
+        if (!changed) {
+            if (ti.r_staged)
+                x.template load_exp_full<Shared>(s_r + t0);
+            else if (nvalid == P::kValues)
+                x.template load_exp_full<Global>(r);
             else
-                x.template merge_store_full<Global>(out);
-        } else {
-            const uint8_t* const r = ti.c_ptr + tw.cache + t0;
-            if (nvalid == P::kValues) {
-                x.template split_full<Global>(w);
-                if (!changed) x.template load_exp_full<Global>(r);
-                x.template merge_store_full<Global>(out);
-            } else {
-                x.split_partial(w, nvalid);
-                if (!changed) x.load_exp_partial(r, nvalid);
-                x.merge_store_partial(out, nvalid);
-            }
+                x.load_exp_partial(r, nvalid);
         }
+        if (BULK)
+            x.template merge_store_full<Shared>(s_w + (size_t)t0 * VB);
+        else if (nvalid == P::kValues)
+            x.template merge_store_full<Global>(out);
+        else
+            x.merge_store_partial(out, nvalid);
     }
 }
 
@@ -1112,28 +1103,25 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
                 }
+                // A unit's last, short tile is staged too, in whole 16-byte pieces: the up to 15 bytes behind its last value
+                // lie in the same piece of memory as that value, and the consumers drop them.
+                const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
+                const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
                 if constexpr (HASH) {
-                    // the cached hashes of the tile's blocks (16 bytes each) come in for every tile
-                    if (left >= (uint64_t)kTileValues) {
-                        mbar_arrive_expect_tx(&ctl->full_w[sw], kWBytes);
-                        bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
-                    } else {
-                        mbar_arrive(&ctl->full_w[sw]);
-                    }
-                    const uint32_t nblk = (uint32_t)((min((uint64_t)kTileValues, left) + (1u << log2b) - 1u) >> log2b);
+                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes);
+                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
+                    // the cached hashes of the tile's blocks (16 bytes each)
+                    const uint32_t nblk = (nvt + (1u << log2b) - 1u) >> log2b;
                     mbar_arrive_expect_tx(&ctl->full_e[se], nblk * 16u);
                     bulk_load(ring_h + (size_t)se * kHStage, cache + hb * 16ull, nblk * 16u, &ctl->full_e[se]);
-                } else if (left >= (uint64_t)kTileValues) {
-                    // all copies of the tile complete on the one barrier the consumers wait for
-                    mbar_arrive_expect_tx(&ctl->full_w[sw], kWBytes + kEBytes + (STEP && r_staged ? kEBytes : 0u));
-                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, kWBytes, &ctl->full_w[sw]);
-                    bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, kEBytes, &ctl->full_w[sw]);
-                    if (STEP && r_staged)
-                        bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, kEBytes,
-                                  &ctl->full_w[sw]);
                 } else {
-                    // short tile: consumers read global memory themselves
-                    mbar_arrive(&ctl->full_w[sw]);
+                    // all copies of the tile complete on the one barrier the consumers wait for
+                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes + e_bytes + (STEP && r_staged ? e_bytes : 0u));
+                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
+                    bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, e_bytes, &ctl->full_w[sw]);
+                    if (STEP && r_staged)
+                        bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, e_bytes,
+                                  &ctl->full_w[sw]);
                 }
                 ctl->issued = k + 1;
             }
@@ -1275,18 +1263,18 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if constexpr (kOneBody) {
                     // a plain loop that tests as it goes
 #define CIERA_PIECES_FULL false
-#define CIERA_PIECES_STAGED (nv == (uint32_t)kTileValues)
+#define CIERA_PIECES_WHOLE (nv == (uint32_t)kTileValues)
 #include "ciera_encode_pieces.inc"
 #undef CIERA_PIECES_FULL
-#undef CIERA_PIECES_STAGED
+#undef CIERA_PIECES_WHOLE
                 } else {
                     auto pieces = [&](auto full_tag) {
                         constexpr bool kFull = decltype(full_tag)::value;
 #define CIERA_PIECES_FULL kFull
-#define CIERA_PIECES_STAGED kFull
+#define CIERA_PIECES_WHOLE kFull
 #include "ciera_encode_pieces.inc"
 #undef CIERA_PIECES_FULL
-#undef CIERA_PIECES_STAGED
+#undef CIERA_PIECES_WHOLE
                     };
                     if (nv == (uint32_t)kTileValues)
                         pieces(std::true_type{});
