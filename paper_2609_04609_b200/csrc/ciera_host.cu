@@ -174,16 +174,27 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     // (While a run's number and table entry were still waited for at its start, whole units were the faster way
     // with 16 to 128 values per block, where the aggregator warp has the least time to spare; with the look-ahead
     // runs win there too: 0.2874 against 0.2917 ms with 64 values per block, 0.2898 against 0.3005 with 128.)
-    for (int pass = 0; pass < 2; ++pass) {
+    // Where the heads are long for the table -- fewer than kRunsPerBlock runs to a thread block -- they are cut into runs
+    // of `cap` tiles, every unit's first, then every unit's second, and so on, so that the blocks finish together: 374
+    // units of 28 tiles (bf16, 64 values per block, whole step) 160 -> 131 us, hashed sender 118 -> 92; 384 units of 16
+    // tiles 92 -> 82, 1024 of 32 215 -> 199.  With fewer units than blocks a unit's next run would be handed out while the
+    // one before it is still worked on: 256 units of 16 tiles 59.9 -> 62.6, so there the heads stay whole.
+    uint32_t cap = ~0u;
+    if (!p->spread_all && shorts.size() >= kEncodeBlocks)
+        cap = std::max(kSeqRunTiles, (uint32_t)(short_tiles / (kRunsPerBlock * kEncodeBlocks)) / kSeqRunTiles * kSeqRunTiles);
+    auto head_of = [](uint32_t n) { return n <= kSeqRunTiles ? n : (n - 1) / kSeqRunTiles * kSeqRunTiles; };
+    uint32_t longest_head = 0;
+    for (size_t i = 0; i + 1 < p->seq_first.size(); ++i)
+        longest_head = std::max(longest_head, head_of(p->seq_first[i + 1] - p->seq_first[i]));
+    for (uint32_t at = 0; at < longest_head; at += std::min(cap, longest_head)) {
         for (size_t i = 0; i + 1 < p->seq_first.size(); ++i) {
-            const uint32_t first = p->seq_first[i], end = p->seq_first[i + 1];
-            const uint32_t n = end - first;
-            const uint32_t head = n <= kSeqRunTiles ? n : (n - 1) / kSeqRunTiles * kSeqRunTiles;
-            if (pass == 0)
-                p->seq_runs.push_back({first, first + head});
-            else if (head < n)
-                p->seq_runs.push_back({first + head, end});
+            const uint32_t first = p->seq_first[i], head = head_of(p->seq_first[i + 1] - first);
+            if (at < head) p->seq_runs.push_back({first + at, first + at + std::min(cap, head - at)});
         }
+    }
+    for (size_t i = 0; i + 1 < p->seq_first.size(); ++i) {
+        const uint32_t first = p->seq_first[i], end = p->seq_first[i + 1], head = head_of(end - first);
+        if (first + head < end) p->seq_runs.push_back({first + head, end});
     }
     for (uint32_t u : longs) emit(u);
     // the same tiles by address, for steps on host weights

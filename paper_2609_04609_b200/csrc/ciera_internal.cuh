@@ -144,6 +144,8 @@ constexpr uint32_t kSeqMaxTiles = 32;
 // 768 tiles 26.2 / 12.9, 2048 tiles 40.0 / 34.6, 3072 tiles 47.1 / 50.0, 49152 tiles 570 / 625; units of 32 tiles:
 // 1536 tiles 50.4 / 23.5, 4096 tiles 76.5 / 63.0.
 constexpr uint32_t kSpreadShare = 197;
+constexpr uint32_t kEncodeBlocks = 296;  // the encode kernel's thread blocks on a B200, two on each of 148 SMs
+constexpr uint32_t kRunsPerBlock = 8;    // runs of short units to a block below which long runs are cut (ciera_plan_create)
 // A short unit is handed out in runs of this many tiles (all units' first runs, then all second runs, ...): the
 // smaller the piece of work a thread block draws, the less the blocks differ in when they finish.  A run's first
 // tile takes its payload offset from the status word that the run before it left.  A multiple of 4, so that tiles

@@ -153,3 +153,27 @@ def test_host_step_in_parts(dtype, block, pinned):
         for u in codec.units:
             lo, n = int(u["weights_off"]), int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]]
             assert np.array_equal(host[lo : lo + n], src.numpy()[lo : lo + n])
+
+
+@pytest.mark.parametrize("dtype,block", [(0, 512), (0, 4096), (1, 2), (2, 16)])
+def test_long_runs_cut(dtype, block):
+    """As many units of nine and ten tiles as the kernel has thread blocks: their runs of eight are handed out in pieces."""
+    from paper_2609_04609_b200 import runtime
+
+    sizes = [8192 * 10, 8192 * 9 + 1] * 148
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(block + dtype, DEV)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    w += [wl.step_clustered(w[0], gen, f=0.3)]
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    for t, step in ((1, _three_calls), (0, lambda c, x: c.step(x))):
+        exp = table.step(bits[t])
+        step(codec, to_dev_bytes(bits[t], DEV))
+        torch.cuda.synchronize()
+        codec.check_status()
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        compare_recon(codec, exp, bits[t], dtype, f"t={t}")
