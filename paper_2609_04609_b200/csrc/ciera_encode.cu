@@ -305,6 +305,7 @@ constexpr uint32_t kSeqTile = 1u, kSeqRunStart = 2u, kSeqRunEnd = 4u;
 // that at the start of a run neither the counter nor the table is waited for.
 struct TileWalk {
     const uint2* seq_runs;
+    const uint32_t* order;  // not null: the spread tiles are given by their places in this list
     unsigned int* run_ticket;
     uint32_t n_tiles, n_runs, G;
     uint32_t tile, end;      // current run: next tile, one past its last tile
@@ -314,9 +315,9 @@ struct TileWalk {
     uint32_t spread_tile;    // next spread tile of this block
     bool spread;
 
-    __device__ TileWalk(const uint2* runs, unsigned int* ticket, uint32_t nruns, uint32_t spread_first, uint32_t nt,
+    __device__ TileWalk(const uint2* runs, const uint32_t* places, unsigned int* ticket, uint32_t nruns, uint32_t spread_first, uint32_t nt,
                         uint32_t grid, uint32_t block)
-        : seq_runs(runs), run_ticket(ticket), n_tiles(nt), n_runs(nruns), G(grid), tile(0), end(0), spread(true) {
+        : seq_runs(runs), order(places), run_ticket(ticket), n_tiles(nt), n_runs(nruns), G(grid), tile(0), end(0), spread(true) {
         spread_tile = spread_first + block;  // tiles of longer units start after the short units' tiles
         next_run = block;
         after_run = block + grid;
@@ -333,7 +334,7 @@ struct TileWalk {
         if (spread) {
             if (spread_tile < n_tiles) {
                 seq = 0;
-                const uint32_t t = spread_tile;
+                const uint32_t t = order ? __ldg(order + spread_tile) : spread_tile;
                 spread_tile += G;
                 return t;
             }
@@ -982,7 +983,8 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
 // the index of every tile's first block in it.
 template <int DT, bool FINE, int HASH, bool STEP>
 __global__ void __launch_bounds__(kEncodeThreads<DT, HASH>, kEncodeBlocksPerSM<DT, STEP>)
-encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
+encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs,
+              const uint32_t* __restrict__ order, uint32_t n_runs,
               uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
               unsigned int* unit_ticket, unsigned int* blocks_done, int32_t* status,
@@ -1051,7 +1053,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     if (warp == (uint32_t)CW) {
         // ---------------------------------------------------------------- producer
         if (lane == 0) {
-            TileWalk walk(seq_runs, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
+            TileWalk walk(seq_runs, order, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
             uint32_t tile_nxt = walk.next(seq_nxt);
             TileDesc nxt;
@@ -1451,9 +1453,10 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
 
 // `scratch`: one status word per tile, then the run counter and the counter of finished blocks; all zero when
 // the kernel starts, and all zero again when it has finished without a device-side error.
-// part of a step: the tiles [lo, hi) of `tiles`, all of them spread; the last part empties the status words
+// part of a step: the tiles at places [lo, hi) of `order` (null: table order), all of them spread; the last part empties
+// the status words
 struct EncodePart {
-    const TileDesc* tiles;
+    const uint32_t* order;
     uint32_t lo, hi;
     bool last;
 };
@@ -1464,7 +1467,8 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     int limit = 0;
     const int rc = encode_grid_limit<DT, FINE, HASH, STEP>(p->log2b, &limit);
     if (rc) return rc;
-    const TileDesc* tiles = part ? part->tiles : p->tiles_dev;
+    const TileDesc* tiles = p->tiles_dev;
+    const uint32_t* order = part ? part->order : nullptr;
     const uint32_t all_tiles = (uint32_t)p->tiles.size();
     uint32_t nt = part ? part->hi : all_tiles;
     const uint32_t to_do = part ? part->hi - part->lo : all_tiles;
@@ -1494,12 +1498,12 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     if (has_spread && !one_each) {
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
-        void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
+        void* args[] = {&tiles, &nt, &seq_runs, &order, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
                         &changed_blocks_dev, &ts, &ticket, &done, &status_dev, &tile_hash, &tw};
         e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
                                         smem, s);
     } else {
-        e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
+        e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, order, n_runs,
                          spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
                          tile_hash, tw);
     }

@@ -83,7 +83,7 @@ ImageLayout image_layout(const ciera_plan* p) {
     L.elong_off = L.units_off + up16((size_t)p->n_units * sizeof(ciera_unit));
     L.echunk_off = L.elong_off + up16(p->ent_long_units.size() * sizeof(uint32_t));
     L.byaddr_off = L.echunk_off + up16(p->ent_chunks.size() * sizeof(ciera_plan::EntChunk));
-    L.thash_off = L.byaddr_off + p->tiles_by_address.size() * sizeof(TileDesc);
+    L.thash_off = L.byaddr_off + up16(p->tiles_by_address.size() * sizeof(uint32_t));
     L.runs_off = L.thash_off + up16(p->tiles.size() * sizeof(uint64_t));
     L.total = L.runs_off + p->seq_runs.size() * sizeof(ciera_plan::SeqRun) + 16;
     return L;
@@ -214,11 +214,11 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
             std::vector<uint32_t> first(n_units, 0);
             for (size_t t = 0; t < p->tiles.size(); ++t)
                 if (p->tiles[t].tile_in_unit == 0) first[p->tiles[t].unit] = (uint32_t)t;
-            p->tiles_by_address.reserve(p->tiles.size());
+            p->tiles_by_address.resize(p->tiles.size());
+            uint32_t at = 0;
             for (uint32_t u : order) {
-                const uint32_t at = (uint32_t)p->tiles_by_address.size(), nt = tiles_of(u);
-                p->tiles_by_address.insert(p->tiles_by_address.end(), p->tiles.begin() + first[u], p->tiles.begin() + first[u] + nt);
-                for (uint32_t j = 0; j < nt; ++j) p->tiles_by_address[at + j].first_tile = at;
+                const uint32_t nt = tiles_of(u);
+                for (uint32_t j = 0; j < nt; ++j) p->tiles_by_address[at++] = first[u] + j;
             }
         }
     }
@@ -252,7 +252,7 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     if (!p->long_units.empty()) memcpy(p->image.data() + L.long_off, p->long_units.data(), p->long_units.size() * 4);
     memcpy(p->image.data() + L.seq_off, p->seq_first.data(), p->seq_first.size() * 4);
     if (!p->tiles_by_address.empty())
-        memcpy(p->image.data() + L.byaddr_off, p->tiles_by_address.data(), p->tiles_by_address.size() * sizeof(TileDesc));
+        memcpy(p->image.data() + L.byaddr_off, p->tiles_by_address.data(), p->tiles_by_address.size() * sizeof(uint32_t));
     if (!p->tile_hash.empty()) memcpy(p->image.data() + L.thash_off, p->tile_hash.data(), p->tile_hash.size() * 8);
     if (!p->seq_runs.empty())
         memcpy(p->image.data() + L.runs_off, p->seq_runs.data(), p->seq_runs.size() * sizeof(ciera_plan::SeqRun));
@@ -322,7 +322,7 @@ extern "C" int ciera_plan_bind(ciera_plan* p, void* plan_dev, size_t plan_dev_by
     p->tiles_dev = (const TileDesc*)plan_dev;
     const ImageLayout L = image_layout(p);
     const uint8_t* base = (const uint8_t*)plan_dev;
-    p->tiles_by_address_dev = p->tiles_by_address.empty() ? p->tiles_dev : (const TileDesc*)(base + L.byaddr_off);
+    p->tiles_by_address_dev = p->tiles_by_address.empty() ? nullptr : (const uint32_t*)(base + L.byaddr_off);
     p->long_units_dev = (const uint32_t*)(base + L.long_off);
     p->seq_first_dev = (const uint32_t*)(base + L.seq_off);
     p->hash_base_dev = (const unsigned long long*)(base + L.hash_off);

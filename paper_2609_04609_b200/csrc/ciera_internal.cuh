@@ -183,9 +183,9 @@ struct ciera_plan {
     std::vector<uint32_t> unit_first;  // first tile of every unit (0xffffffff: a unit without values)
     std::vector<uint64_t> hash_base;   // index of every unit's first block in a per-block hash cache
     std::vector<uint64_t> tile_hash;   // the same for every tile's first block, in tile-table order
-    // the tiles of all units by ascending address of their weights, for steps on host weights; left empty where that
+    // the numbers of the tiles by ascending address of their weights, for steps on host weights; left empty where that
     // is the order of `tiles` already.  by_address_ok: the units' weights do not overlap.
-    std::vector<ciera::TileDesc> tiles_by_address;
+    std::vector<uint32_t> tiles_by_address;
     bool by_address_ok = false;
     uint64_t total_blocks = 0;
     std::vector<uint64_t> seg_base;    // index of every unit's first 4096-byte payload segment (entropy stage)
@@ -203,7 +203,7 @@ struct ciera_plan {
     std::vector<uint8_t> image;        // device image: tiles, long_units, seq_first, hash_base, unit_first, seg_base, units,
                                        // ent_long_units, ent_chunks, tiles_by_address, tile_hash, seq_runs
     const ciera::TileDesc* tiles_dev = nullptr;
-    const ciera::TileDesc* tiles_by_address_dev = nullptr;
+    const uint32_t* tiles_by_address_dev = nullptr;
     // Pairs of copy streams for steps on host weights: taken out for the length of a call, put back at its end and
     // reused by the next; as many as calls were ever made at the same time; destroyed with the plan.
     struct CopyLane {

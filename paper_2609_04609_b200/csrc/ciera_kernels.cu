@@ -436,15 +436,14 @@ static int host_step_in_parts(const ciera_plan* p, const void* weights_host, siz
     ciera_plan::CopyLane lane;
     rc = take_copy_lane(p, &lane);
     if (rc) return rc;
-    const std::vector<TileDesc>& tiles = p->tiles_by_address.empty() ? p->tiles : p->tiles_by_address;
-    const uint32_t nt = (uint32_t)tiles.size();
+    const uint32_t nt = (uint32_t)p->tiles.size();
     cudaError_t e = join(lane.in, s, lane.event);
     uint32_t lo = 0;
     uint64_t from = 0;  // weights up to this byte are on their way
     for (uint32_t k = 1; k <= parts && e == cudaSuccess && rc == CIERA_OK; ++k) {
         const uint32_t hi = k == parts ? nt : (uint32_t)((uint64_t)nt * (2u * k - 1u) / (2u * parts - 2u));
         if (hi == lo) continue;
-        uint64_t to = hi < nt ? tiles[hi].w_off : (uint64_t)weights_bytes;
+        uint64_t to = hi < nt ? p->tiles[p->tiles_by_address.empty() ? hi : p->tiles_by_address[hi]].w_off : (uint64_t)weights_bytes;
         if (to > weights_bytes) to = weights_bytes;
         if (to < from) to = from;
         const uint64_t n = to - from;
