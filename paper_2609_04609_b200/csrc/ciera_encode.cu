@@ -619,17 +619,13 @@ struct HashTile {
     ulonglong2* dst;
 };
 
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH>
 __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, bool publish,
-                                                   const uint32_t* ballot, uint32_t* bm, uint16_t* pre, uint8_t* msgs,
-                                                   const StepTwins& tw, unsigned long long* tile_status, const HashTile& ht,
+                                                   const uint32_t* ballot, uint32_t* bm, uint16_t* pre,
+                                                   unsigned long long* tile_status, const HashTile& ht, uint32_t nv,
                                                    uint32_t lane) {
-    const uint64_t N = td.n_unit;
     const uint32_t B = 1u << log2b;
     const uint32_t nbt = kTileValues >> log2b;
-    const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
-    const uint32_t nv = (uint32_t)min((uint64_t)kTileValues, N - v0);
-    uint8_t* msg = msgs + td.msg_off;
 
     uint32_t run;
     if constexpr (HASH)
@@ -651,34 +647,41 @@ __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t 
         const unsigned long long flag = td.tile_in_unit == 0 ? kFlagPrefix : kFlagAggregate;
         if (lane == 0) st_status(tile_status + tile, flag | ((unsigned long long)mybits << kBitsShift) | agg);
     }
-    // bitmap bytes of this tile (tiles of >= 8 blocks own whole bytes)
-    if (FINE) {
-        // at least 128 bytes per full tile, starting on a 128-byte boundary of the (16-byte aligned) slot
-        const uint64_t byte0 = (uint64_t)td.tile_in_unit * (nbt >> 3);
-        const uint32_t nbytes = (((nv + B - 1u) >> log2b) + 7u) >> 3;
-        uint32_t* dst32 = reinterpret_cast<uint32_t*>(msg + byte0);
-        // 16 bytes at a time, then the last words, then the last bytes
-        const uint32_t quads = nbytes >> 4;
-        auto twin32 = reinterpret_cast<uint32_t*>(msg + byte0 + tw.msg);
-        for (uint32_t c = lane; c < quads; c += 32) {
-            const uint4 v = reinterpret_cast<const uint4*>(bm)[c];
-            reinterpret_cast<uint4*>(dst32)[c] = v;
-            if (STEP) reinterpret_cast<uint4*>(twin32)[c] = v;
-        }
-        for (uint32_t w = 4u * quads + lane; w < (nbytes >> 2); w += 32) {
-            dst32[w] = bm[w];
-            if (STEP) twin32[w] = bm[w];
-        }
-        const uint32_t done = nbytes & ~3u;
-        if (lane < nbytes - done)
-            put_byte<STEP>(msg + byte0 + done + lane, (uint8_t)(bm[done >> 2] >> (lane * 8u)), tw.msg);
-    } else if (nbt >= 8) {
-        const uint64_t byte0 = (uint64_t)td.tile_in_unit * (nbt >> 3);
-        const uint32_t nbytes = (((nv + B - 1u) >> log2b) + 7u) >> 3;
-        for (uint32_t b = lane; b < nbytes; b += 32)
-            put_byte<STEP>(msg + byte0 + b, (uint8_t)(bm[b >> 2] >> ((b & 3u) * 8u)), tw.msg);
-    }
     return agg;
+}
+
+// The tile's bytes of the bitmap (tiles of >= 8 blocks own whole bytes).  `dst`: where they go; `nblk`: blocks of the tile.
+// Fine blocks: at least 128 bytes per full tile, starting on a 128-byte boundary of the (16-byte aligned) slot.
+template <bool STEP>
+__device__ __forceinline__ void store_bitmap_fine(uint8_t* dst, const uint32_t* bm, uint32_t nblk, const StepTwins& tw,
+                                                  uint32_t lane) {
+    const uint32_t nbytes = (nblk + 7u) >> 3;
+    uint32_t* const dst32 = reinterpret_cast<uint32_t*>(dst);
+    uint32_t* const twin32 = reinterpret_cast<uint32_t*>(dst + tw.msg);
+    // 16 bytes at a time, then the last words, then the last bytes
+    const uint32_t quads = nbytes >> 4;
+    for (uint32_t c = lane; c < quads; c += 32) {
+        const uint4 v = reinterpret_cast<const uint4*>(bm)[c];
+        reinterpret_cast<uint4*>(dst32)[c] = v;
+        if (STEP) reinterpret_cast<uint4*>(twin32)[c] = v;
+    }
+    for (uint32_t w = 4u * quads + lane; w < (nbytes >> 2); w += 32) {
+        dst32[w] = bm[w];
+        if (STEP) twin32[w] = bm[w];
+    }
+    const uint32_t done = nbytes & ~3u;
+    if (lane < nbytes - done) put_byte<STEP>(dst + done + lane, (uint8_t)(bm[done >> 2] >> (lane * 8u)), tw.msg);
+}
+// Coarse blocks: lane l holds word l of the flags; a tile of 32 blocks and more starts on a word boundary.
+template <bool STEP>
+__device__ __forceinline__ void store_bitmap(uint8_t* dst, uint32_t word, uint32_t nblk, const StepTwins& tw, uint32_t lane) {
+    const uint32_t nbytes = (nblk + 7u) >> 3;
+    if (4u * lane + 4u <= nbytes) {
+        *reinterpret_cast<uint32_t*>(dst + 4u * lane) = word;
+        if (STEP) *reinterpret_cast<uint32_t*>(dst + tw.msg + 4u * lane) = word;
+    } else {
+        for (uint32_t b = 4u * lane; b < nbytes; ++b) put_byte<STEP>(dst + b, (uint8_t)(word >> ((b & 3u) * 8u)), tw.msg);
+    }
 }
 
 // payload <- exponents of changed blocks in block order; cache refreshed for the same blocks.
@@ -1153,14 +1156,21 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 ht.part = reinterpret_cast<const ulonglong2*>(ring_h + (size_t)se * kHStage + kHoldBytes);
                 ht.dst = reinterpret_cast<ulonglong2*>(ctl->info[k % kDescRing].c_ptr);
             }
-            const uint64_t agg = aggregate_tile<DT, FINE, HASH, STEP>(td, tile, log2b, !seq, ctl->ballot[se], ctl->bm[se],
-                                                                      ctl->pre[se], msgs, tw, tile_status, ht, lane);
+            const uint32_t nbt = kTileValues >> log2b;
+            const uint32_t nv = (uint32_t)min((uint64_t)kTileValues, td.n_unit - (uint64_t)td.tile_in_unit * kTileValues);
+            const uint32_t nblk = (nv + (1u << log2b) - 1u) >> log2b;
+            const bool last = td.tile_in_unit == td.n_tiles_unit - 1u;
+            uint8_t* const msg = msgs + td.msg_off;
+            uint8_t* const bitmap_dst = msg + (uint64_t)td.tile_in_unit * (nbt >> 3);
+            const uint64_t agg = aggregate_tile<DT, FINE, HASH>(td, tile, log2b, !seq, ctl->ballot[se], ctl->bm[se], ctl->pre[se],
+                                                                tile_status, ht, nv, lane);
+            uint64_t excl = 0;
             if (seq) {
                 // the run is this block's: the tile's offset is the running sum; a run that does not start its
                 // unit carries on from the inclusive offset that the run before it left in its last tile's
                 // status word (that run went out many draws earlier; the wait is bounded all the same; reading
                 // the word in the producer thread instead, tiles ahead, was slower)
-                uint64_t excl = run_incl;
+                excl = run_incl;
                 if (td.tile_in_unit == 0)
                     excl = 0;
                 else if (seq_bits & kSeqRunStart) {
@@ -1169,22 +1179,31 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     if (lane == 0) st_status(tile_status + tile - 1, 0ull);  // its one reader leaves the word empty again
                 }
                 run_incl = excl + agg;
-                if ((seq_bits & kSeqRunEnd) && td.tile_in_unit != td.n_tiles_unit - 1u && lane == 0)
-                    st_status(tile_status + tile, kFlagPrefix | run_incl);
-                const uint32_t nbt = kTileValues >> log2b;
-                const bool last = td.tile_in_unit == td.n_tiles_unit - 1u;
+                if ((seq_bits & kSeqRunEnd) && !last && lane == 0) st_status(tile_status + tile, kFlagPrefix | run_incl);
+            }
+            // What the others wait for goes out before the tile's bitmap and the unit's totals: the chain votes - sums -
+            // offset - sending is what small tables wait for.  The flags that are still needed are in registers by then, since
+            // the stage may be refilled.  (Whole step of 4736 units of 67 values 45 -> 41 us, sender with 64 values per block
+            // 0.281 -> 0.274 ms per OLMoE-shaped layer; with HashCache the other order is the faster one for small tables.)
+            uint32_t word = 0;
+            if (FINE)
+                store_bitmap_fine<STEP>(bitmap_dst, ctl->bm[se], nblk, tw, lane);
+            else if (32u * lane < nbt)
+                word = ctl->bm[se][lane];
+            auto report = [&]() {
+                if (!FINE && nbt >= 8) store_bitmap<STEP>(bitmap_dst, word, nblk, tw, lane);
+                if (!seq) return;
                 if (nbt < 8) {
                     const uint32_t tpb = 8u / nbt, p = td.tile_in_unit & (tpb - 1u);
-                    byte_acc = (p == 0 ? 0u : byte_acc) | (ctl->bm[se][0] << (p * nbt));
+                    byte_acc = (p == 0 ? 0u : byte_acc) | (word << (p * nbt));  // (lane 0)
                     if ((p == tpb - 1u || last) && lane == 0)
-                        put_byte<STEP>(msgs + td.msg_off + td.tile_in_unit / tpb, (uint8_t)byte_acc, tw.msg);
+                        put_byte<STEP>(msg + td.tile_in_unit / tpb, (uint8_t)byte_acc, tw.msg);
                 }
                 if (last) finish_unit<DT, STEP>(td, log2b, run_incl, msgs, tw.msg, wire_bytes, changed_blocks, lane);
-                if (lane == 0) {
-                    ctl->base[se] = excl;
-                    ctl->agg[se] = agg;
-                }
-            } else if (lane == 0) {
+            };
+            if constexpr (HASH != 0) report();
+            if (lane == 0) {
+                if (seq) ctl->base[se] = excl;
                 ctl->agg[se] = agg;
             }
             __syncwarp();
@@ -1192,6 +1211,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 mbar_arrive(&ctl->summed[se]);
                 if (seq) mbar_arrive(&ctl->resolved[se]);
             }
+            if constexpr (HASH == 0) report();
         }
     } else if (warp >= (uint32_t)CW + 2u) {
         // ---------------------------------------------------------------- resolvers (slots k = i, i + R, ...)
@@ -1217,12 +1237,13 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             }
             if (ctl->seq[k % kDescRing] != 0) continue;  // the aggregator has done it all
             const TileDesc td = ctl->desc[k % kDescRing];
-            const uint64_t excl = resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, tw.msg, wire_bytes,
-                                                         changed_blocks, tile_status, status, lane);
-            if (lane == 0) {
-                ctl->base[se] = excl;
-                mbar_arrive(&ctl->resolved[se]);
-            }
+            resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, tw.msg, wire_bytes, changed_blocks,
+                                   tile_status, status, lane, [&](uint64_t excl) {
+                                       if (lane == 0) {
+                                           ctl->base[se] = excl;
+                                           mbar_arrive(&ctl->resolved[se]);
+                                       }
+                                   });
         }
     } else {
         // ---------------------------------------------------------------- consumers

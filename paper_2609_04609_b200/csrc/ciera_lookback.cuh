@@ -76,12 +76,13 @@ __device__ __forceinline__ void finish_unit(const TileDesc& td, uint32_t log2b, 
 
 // Resolver warp, one spread tile: exclusive prefix of the payload bytes over the earlier tiles of
 // the same unit by a single-pass look-back over the status words, then the duties that need it.
-// Returns the tile's exclusive payload offset inside its unit.
-template <int DT, bool TWICE>
-__device__ __forceinline__ uint64_t resolve_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, uint64_t agg,
+// `known` is called with the tile's exclusive payload offset inside its unit as soon as there is one (the tile's flags
+// in `bm` are not read after that).
+template <int DT, bool TWICE, class KNOWN>
+__device__ __forceinline__ void resolve_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, uint64_t agg,
                                                  const uint32_t* bm, uint8_t* msgs, int64_t twin,
                                                  unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
-                                                 int32_t* status, uint32_t lane) {
+                                                 int32_t* status, uint32_t lane, KNOWN known) {
     const uint32_t nbt = kTileValues >> log2b;
     uint8_t* msg = msgs + td.msg_off;
     const uint32_t mybits = nbt < 8 ? bm[0] : 0u;
@@ -103,6 +104,8 @@ __device__ __forceinline__ uint64_t resolve_tile(const TileDesc& td, uint32_t ti
         if (lane == 0)
             st_status(tile_status + tile, kFlagPrefix | ((unsigned long long)mybits << kBitsShift) | (excl + agg));
     }
+    __syncwarp();  // every lane has read its flags
+    known(excl);
 
     // tiles of fewer than 8 blocks share a bitmap byte: the last tile of each byte collects the
     // bits its predecessors published in their status words
@@ -122,7 +125,6 @@ __device__ __forceinline__ uint64_t resolve_tile(const TileDesc& td, uint32_t ti
     }
     if (td.tile_in_unit == td.n_tiles_unit - 1u)
         finish_unit<DT, TWICE>(td, log2b, excl + agg, msgs, twin, wire_bytes, changed_blocks, lane);
-    return excl;
 }
 
 }  // namespace ciera
