@@ -473,12 +473,12 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* scan, uint3
 }
 
 // ------------------------------------------------------------------------------------------ sender
-// units of up to kLongSegs segment slots: one thread block per unit, start to end
+// units of up to long_slots (at most kLongSegs) segment slots: one thread block per unit, start to end
 
 template <bool HALF, int T>  // HALF: fp16, five-bit symbols (see the head of this file); T: threads of the block
 __global__ void __launch_bounds__(T, T == kEntWide ? 1 : 5)
 entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long long* __restrict__ seg_base,
-                      int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
+                      uint32_t long_slots, int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
                       uint8_t* scratch_slots, uint32_t* scratch_nw, uint8_t* scratch_sym) {
     __shared__ uint32_t s_hist[T / 32][256];  // the warps' private histograms, then the two small lists of step 4
     __shared__ uint16_t s_f[256];
@@ -488,7 +488,7 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     pdl_wait();
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
-    if (un.n_values == 0 || segments_of(un.n_values) > kLongSegs) return;
+    if (un.n_values == 0 || segments_of(un.n_values) > long_slots) return;
     const uint64_t payoff = payload_offset_of(un.n_values, dt, log2b);
     const uint64_t Q = wire_bytes[unit] - payoff;
     // nothing to code; or a length that no sender step reports (shorter than the fixed sections, more
@@ -794,7 +794,7 @@ __device__ __forceinline__ void raise_corrupt(int32_t* status) {
 // more than 5, the 48 registers shorten the chain: 512 units 55 us against 70, 192 units 48 against 57)
 template <bool HALF, int T, int BLOCKS>
 __global__ void __launch_bounds__(T, BLOCKS)
-entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log2b, uint8_t* msgs,
+entropy_decode_kernel(const ciera_unit* __restrict__ units, uint32_t long_slots, int dt, uint32_t log2b, uint8_t* msgs,
                       unsigned long long* wire_bytes, uint8_t* scratch_raw, int32_t* status) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     DecodeShared& sh = *reinterpret_cast<DecodeShared*>(smem_raw);
@@ -802,7 +802,7 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
     const uint64_t N = un.n_values;
-    if (N == 0 || segments_of(N) > kLongSegs) return;
+    if (N == 0 || segments_of(N) > long_slots) return;
     uint8_t* const msg = msgs + un.msg_off;
     const uint64_t payoff = payload_offset_of(N, dt, log2b);
     if (tid == 0) {
@@ -1075,7 +1075,7 @@ static int entropy_device(int* sms_out) {
     return CIERA_OK;
 }
 // wide blocks for the units as long as each has an SM to itself
-static bool wide_units(uint32_t units, int sms) { return units <= (uint32_t)sms; }
+static bool wide_units(uint32_t units) { return units <= kEntWideUnits; }
 // thread blocks to a chunk of kLongSegs segments: enough for five on every SM, at least a segment for each of their warps
 static uint32_t chunk_parts(uint32_t chunks, int sms) {
     uint32_t parts = 1;
@@ -1103,11 +1103,11 @@ extern "C" int ciera_entropy_encode(const ciera_plan* p, void* messages_dev, uin
     if ((rc = entropy_device(&sms))) return rc;
     cudaError_t e = cudaSuccess;
     if (n_long < p->n_units) {
-        const bool wide = wide_units(p->n_units - n_long, sms);
+        const bool wide = wide_units(p->n_units - n_long);
         auto* k = dt == CIERA_FP16 ? (wide ? entropy_encode_kernel<true, kEntWide> : entropy_encode_kernel<true, kEntThreads>)
                                    : (wide ? entropy_encode_kernel<false, kEntWide> : entropy_encode_kernel<false, kEntThreads>);
-        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev, dt, p->log2b,
-                         msgs, wire, slots, nw, sym);
+        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev,
+                         p->ent_long_slots, dt, p->log2b, msgs, wire, slots, nw, sym);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }
@@ -1151,16 +1151,16 @@ extern "C" int ciera_entropy_decode(const ciera_plan* p, void* messages_dev, uin
     unsigned long long* wire = (unsigned long long*)wire_bytes_dev;
     const uint32_t n_long = (uint32_t)p->ent_long_units.size(), n_chunks = (uint32_t)p->ent_chunks.size();
     if (n_long < p->n_units) {
-        const bool wide = wide_units(p->n_units - n_long, sms);
-        const bool few = p->n_units - n_long <= 5u * (uint32_t)sms;
+        const bool wide = wide_units(p->n_units - n_long);
+        const bool few = p->n_units - n_long <= kEntFewUnits;
         auto* k = dt == CIERA_FP16 ? (wide  ? entropy_decode_kernel<true, kEntWide, 1>
                                       : few ? entropy_decode_kernel<true, kEntThreads, 5>
                                             : entropy_decode_kernel<true, kEntThreads, 8>)
                                    : (wide  ? entropy_decode_kernel<false, kEntWide, 1>
                                       : few ? entropy_decode_kernel<false, kEntThreads, 5>
                                             : entropy_decode_kernel<false, kEntThreads, 8>);
-        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev, dt, p->log2b,
-                         msgs, wire, raw, status_dev);
+        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev,
+                         p->ent_long_slots, dt, p->log2b, msgs, wire, raw, status_dev);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }

@@ -132,6 +132,13 @@ __host__ __device__ inline size_t workspace_total_bytes(size_t nt) {
     return (workspace_prefix_offset(nt) + nt * sizeof(uint32_t) + 15) / 16 * 16;
 }
 
+// Entropy stage: a unit of at most 64 segment slots is coded by one thread block, of 32 warps as long as there are no more
+// such units than SMs (kEntWideUnits), else of 8; longer ones by several blocks.  Up to kEntSplitUnits units, blocks of 8
+// warps leave most of the GPU idle, so there units of more than kEntSplitSlots are coded by several blocks as well: step with
+// the stage, 208 units of 62 slots 433 -> 277 us, 192 of 32 (every block changed) 355 -> 222; 384 units of 32 slots 206 -> 214.
+// kEntFewUnits: up to here the receiver's build for 5 blocks per SM is the faster one.
+constexpr uint32_t kEntWideUnits = 148, kEntSplitUnits = 296, kEntSplitSlots = 16, kEntFewUnits = 740;
+
 // The tile table lists the tiles of "short" units (up to this many tiles) first, longest units
 // first, then the tiles of the longer units.  The encode kernel lets one thread block work through
 // a short unit tile after tile (the tile's place in the payload is then a running sum inside the
@@ -191,7 +198,8 @@ struct ciera_plan {
     std::vector<uint64_t> seg_base;    // index of every unit's first 4096-byte payload segment (entropy stage)
     uint64_t total_segments = 0;
     uint64_t cache_extent = 0;         // max over units of cache_off + n_values
-    // entropy stage: units of more than 64 segment slots, and their chunks of 64 slots
+    // entropy stage: units of more than ent_long_slots segment slots, and their chunks of 64 slots
+    uint32_t ent_long_slots = 64;
     // {unit, first segment of the chunk inside the unit, index among the long units, 0}
     struct EntChunk {
         uint32_t unit, first_seg, long_index, zero;

@@ -75,13 +75,14 @@ def test_models_and_lengths():
 
 
 @pytest.mark.parametrize("dtype", [0, 2])
-@pytest.mark.parametrize("n_units", [148, 149, 741])
-def test_numbers_of_units(n_units, dtype):
-    """A wide thread block per unit up to one per SM, narrow ones beyond, and those in two builds by their number."""
+@pytest.mark.parametrize("n_units,size", [(148, 4096), (149, 4096), (741, 4096), (149, 65_500), (297, 65_500)])
+def test_numbers_of_units(n_units, size, dtype):
+    """A wide thread block per unit up to one per SM, narrow ones beyond, and those in two builds by their number; among
+    few units those of more than 16 segment slots take several blocks."""
     from paper_2609_04609_b200 import runtime
 
     name = {0: "bf16", 2: "fp16"}[dtype]
-    codec = guard(runtime.LayerCodec.from_tensors([4096 + 37 * (i % 5) for i in range(n_units)], 1, name, 64, DEV, slack=256))
+    codec = guard(runtime.LayerCodec.from_tensors([size + 37 * (i % 5) for i in range(n_units)], 1, name, 64, DEV, slack=256))
     gen = torch.Generator().manual_seed(n_units)
     w = (torch.randn(codec.weights_bytes // 2, generator=gen) * 0.02).to({0: torch.bfloat16, 2: torch.float16}[dtype])
     bits = w.view(torch.int16).numpy().view(np.uint16)
