@@ -144,7 +144,17 @@ __device__ __forceinline__ void store_bytes_partial(uint8_t* dst, const uint32_t
     for (int i = 0; i < NB; ++i)
         if (i < nbytes) dst[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
 }
-
+template <int NH>
+__device__ __forceinline__ void store_halves_partial(uint8_t* dst, const uint32_t* w, int nhalves) {
+    uint16_t* const p = reinterpret_cast<uint16_t*>(dst);
+#pragma unroll
+    for (int i = 0; i < NH; ++i)
+        if (i < nhalves) p[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+}
+__device__ __forceinline__ void load_16_bytes(const uint8_t* src, uint32_t* w) {  // from shared memory
+    const uint4 v = Shared::ld16(src);
+    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+}
 
 // keeps the first n (0 .. 4) bytes of a word / the first n (0 .. 2) half-words
 __device__ __forceinline__ uint32_t keep_bytes(uint32_t w, int n) { return n >= 4 ? w : n <= 0 ? 0u : w & ((1u << (8 * n)) - 1u); }
@@ -189,6 +199,7 @@ struct Piece<CIERA_BF16> {
     static constexpr int kPerThread = 2;  // pieces per thread
     static constexpr int kExpWords = 2;
     static constexpr int kSmWords = 2;
+    static constexpr int kWeightWords = 4;
     // first value (inside the tile) of piece p of consumer thread tid
     static __device__ __forceinline__ uint32_t start(uint32_t tid, int p) {
         return (uint32_t)p * (kTileValues / 2) + tid * 8u;
@@ -253,10 +264,22 @@ struct Piece<CIERA_BF16> {
         uint32_t x[4];
         bf16_merge4(e[0], s[0], x[0], x[1]);
         bf16_merge4(e[1], s[1], x[2], x[3]);
-        uint16_t* p = reinterpret_cast<uint16_t*>(w);
+        store_halves_partial<8>(w, x, nvalid);
+    }
+    // the weights at `src` (shared memory) with this piece's exponents in place of their own
+    __device__ __forceinline__ void exchange(const uint8_t* src, uint32_t (&w)[kWeightWords]) const {
+        load_weights(src, w);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < nvalid) p[i] = (uint16_t)(x[i >> 1] >> (16 * (i & 1)));
+        for (int i = 0; i < 4; ++i)
+            w[i] = bitselect(0x7F807F80u, __byte_perm(e[i >> 1], 0u, (i & 1) ? 0x4342u : 0x4140u) << 7, w[i]);
+    }
+    static __device__ __forceinline__ void load_weights(const uint8_t* src, uint32_t (&w)[kWeightWords]) { load_16_bytes(src, w); }
+    template <class M>
+    static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
+        M::st16(dst, make_uint4(w[0], w[1], w[2], w[3]));
+    }
+    static __device__ __forceinline__ void store_weights_first(uint8_t* dst, const uint32_t (&w)[kWeightWords], int nvalid) {
+        store_halves_partial<8>(dst, w, nvalid);
     }
     __device__ __forceinline__ bool differs(const Piece& o) const { return ((e[0] ^ o.e[0]) | (e[1] ^ o.e[1])) != 0; }
     // one flag per block of 2^log2b values (log2b <= 3), lowest block first
@@ -276,6 +299,7 @@ struct Piece<CIERA_FP32> {
     static constexpr int kPerThread = 1;
     static constexpr int kExpWords = 4;
     static constexpr int kSmWords = 12;
+    static constexpr int kWeightWords = 16;
     static __device__ __forceinline__ uint32_t start(uint32_t tid, int) { return tid * 16u; }
 
     uint32_t e[kExpWords];
@@ -375,6 +399,32 @@ struct Piece<CIERA_FP32> {
         for (int i = 0; i < 16; ++i)
             if (i < nvalid) p[i] = x[i];
     }
+    // the weights at `src` (shared memory) with this piece's exponents in place of their own
+    __device__ __forceinline__ void exchange(const uint8_t* src, uint32_t (&w)[kWeightWords]) const {
+        load_weights(src, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            w[4 * i] = bitselect(0x7F800000u, e[i] << 23, w[4 * i]);
+            w[4 * i + 1] = bitselect(0x7F800000u, e[i] << 15, w[4 * i + 1]);
+            w[4 * i + 2] = bitselect(0x7F800000u, e[i] << 7, w[4 * i + 2]);
+            w[4 * i + 3] = bitselect(0x7F800000u, e[i] >> 1, w[4 * i + 3]);
+        }
+    }
+    static __device__ __forceinline__ void load_weights(const uint8_t* src, uint32_t (&w)[kWeightWords]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) load_16_bytes(src + 16 * i, w + 4 * i);
+    }
+    template <class M>
+    static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) M::st16(dst + 16 * i, make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]));
+    }
+    static __device__ __forceinline__ void store_weights_first(uint8_t* dst, const uint32_t (&w)[kWeightWords], int nvalid) {
+        uint32_t* const p = reinterpret_cast<uint32_t*>(dst);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i < nvalid) p[i] = w[i];
+    }
     __device__ __forceinline__ bool differs(const Piece& o) const {
         return ((e[0] ^ o.e[0]) | (e[1] ^ o.e[1]) | (e[2] ^ o.e[2]) | (e[3] ^ o.e[3])) != 0;
     }
@@ -401,9 +451,12 @@ struct Piece<CIERA_FP16> {
     static constexpr int kLog2Values = 3;
     static constexpr int kPerThread = 2;
     static constexpr int kExpWords = 2;
+    static constexpr int kWeightWords = 4;
     static __device__ __forceinline__ uint32_t start(uint32_t tid, int p) {
         return (uint32_t)p * (kTileValues / 2) + tid * 8u;
     }
+
+    static constexpr uint32_t kWarpSmBytes = 32u * 11u;  // packed sign-plus-mantissa of a warp's 32 pieces
 
     uint32_t e[2];  // 8 exponents, one byte each (0..31)
     uint32_t s[3];  // 88 bits of sign-plus-mantissa
@@ -425,25 +478,30 @@ struct Piece<CIERA_FP16> {
         s[1] = (p[1] >> 10) | (p[2] << 12);
         s[2] = (p[2] >> 20) | (p[3] << 2);
     }
+    // two values at a time: their exponents to bits 14:10 and 30:26, their fields (bits 21:0) as split_words left them
     __device__ __forceinline__ void merge_words(uint32_t w[4]) const {
-        uint32_t f[8];
-        f[0] = s[0] & 0x7FFu;
-        f[1] = (s[0] >> 11) & 0x7FFu;
-        f[2] = ((s[0] >> 22) | (s[1] << 10)) & 0x7FFu;
-        f[3] = (s[1] >> 1) & 0x7FFu;
-        f[4] = (s[1] >> 12) & 0x7FFu;
-        f[5] = ((s[1] >> 23) | (s[2] << 9)) & 0x7FFu;
-        f[6] = (s[2] >> 2) & 0x7FFu;
-        f[7] = (s[2] >> 13) & 0x7FFu;
+        const uint32_t p[4] = {s[0], __funnelshift_r(s[0], s[1], 22), __funnelshift_r(s[1], s[2], 12), s[2] >> 2};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t ex = (e[i >> 2] >> (8 * (i & 3))) & 0x1Fu;
-            const uint32_t v = (f[i] & 0x3FFu) | ((f[i] & 0x400u) << 5) | (ex << 10);
-            if (i & 1)
-                w[i >> 1] |= v << 16;
-            else
-                w[i >> 1] = v;
-        }
+        for (int i = 0; i < 4; ++i)
+            w[i] = (p[i] & 0x3FFu) | ((p[i] << 5) & 0x03FF8000u) | ((p[i] << 10) & 0x80000000u) | exponent_bits(i);
+    }
+    // the exponents of values 2 i and 2 i + 1 where they lie in their two values
+    __device__ __forceinline__ uint32_t exponent_bits(int i) const {
+        return (__byte_perm(e[i >> 1], 0u, (i & 1) ? 0x4342u : 0x4140u) << 10) & 0x7C007C00u;
+    }
+    // the weights at `src` (shared memory) with this piece's exponents in place of their own
+    __device__ __forceinline__ void exchange(const uint8_t* src, uint32_t (&w)[kWeightWords]) const {
+        load_weights(src, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = (w[i] & 0x83FF83FFu) | exponent_bits(i);
+    }
+    static __device__ __forceinline__ void load_weights(const uint8_t* src, uint32_t (&w)[kWeightWords]) { load_16_bytes(src, w); }
+    template <class M>
+    static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
+        M::st16(dst, make_uint4(w[0], w[1], w[2], w[3]));
+    }
+    static __device__ __forceinline__ void store_weights_first(uint8_t* dst, const uint32_t (&w)[kWeightWords], int nvalid) {
+        store_halves_partial<8>(dst, w, nvalid);
     }
     template <class M>
     __device__ __forceinline__ void split_full(const uint8_t* src) {
@@ -476,10 +534,7 @@ struct Piece<CIERA_FP16> {
     __device__ __forceinline__ void merge_store_partial(uint8_t* dst, int nvalid) const {
         uint32_t w[4];
         merge_words(w);
-        uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (i < nvalid) d16[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+        store_halves_partial<8>(dst, w, nvalid);
     }
     template <class M>
     __device__ __forceinline__ void load_exp_full(const uint8_t* src) {
@@ -504,22 +559,30 @@ struct Piece<CIERA_FP16> {
         return word_block_flags(e[0] ^ o.e[0], log2b) | (word_block_flags(e[1] ^ o.e[1], log2b) << per_word);
     }
 
-    // the 8 exponents as 40 bits: low word and high byte
+    // the 8 exponents as 40 bits: low word and high byte (four bytes of 5 bits -> two fields of 10 -> one of 20)
     __device__ __forceinline__ void pack_exponents(uint32_t& lo, uint32_t& hi) const {
-        uint32_t x[8];
+        uint32_t z[2];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = (e[i >> 2] >> (8 * (i & 3))) & 0x1Fu;
-        lo = x[0] | (x[1] << 5) | (x[2] << 10) | (x[3] << 15) | (x[4] << 20) | (x[5] << 25) | (x[6] << 30);
-        hi = (x[6] >> 2) | (x[7] << 3);
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t v = (e[i] & 0x001F001Fu) | ((e[i] >> 3) & 0x03E003E0u);
+            z[i] = (v & 0x3FFu) | ((v >> 6) & 0xFFC00u);
+        }
+        lo = z[0] | (z[1] << 20);
+        hi = z[1] >> 12;
     }
     __device__ __forceinline__ void unpack_exponents(uint32_t lo, uint32_t hi) {
-        uint32_t x[8];
+        const uint32_t z[2] = {lo, (lo >> 20) | (hi << 12)};
 #pragma unroll
-        for (int i = 0; i < 6; ++i) x[i] = (lo >> (5 * i)) & 0x1Fu;
-        x[6] = ((lo >> 30) | (hi << 2)) & 0x1Fu;
-        x[7] = (hi >> 3) & 0x1Fu;
-        e[0] = x[0] | (x[1] << 8) | (x[2] << 16) | (x[3] << 24);
-        e[1] = x[4] | (x[5] << 8) | (x[6] << 16) | (x[7] << 24);
+        for (int i = 0; i < 2; ++i) {
+            const uint32_t v = (z[i] & 0x3FFu) | ((z[i] << 6) & 0x03FF0000u);
+            e[i] = (v & 0x001F001Fu) | ((v << 3) & 0x1F001F00u);
+        }
+    }
+    // the packed exponents of a whole piece from shared memory (any alignment): the two words that hold the 5 bytes
+    __device__ __forceinline__ void load_packed_exponents(const uint8_t* src) {
+        const uint32_t skew = (uint32_t)reinterpret_cast<uintptr_t>(src) & 3u;
+        const uint32_t w0 = Shared::ld4(src - skew), w1 = Shared::ld4(src - skew + 4);
+        unpack_exponents(__funnelshift_r(w0, w1, 8u * skew), w1 >> (8u * skew));
     }
     // the packed exponents of the piece from `src` (5 bytes, any alignment; nvalid < 8: fewer)
     template <class M>
@@ -560,9 +623,22 @@ struct Piece<CIERA_FP16> {
         const uint32_t a = lane & 3u, sh = 8u * a;
         const uint32_t next0 = __shfl_down_sync(0xffffffffu, s[0], 1);
         uint32_t* dst = reinterpret_cast<uint32_t*>(section + (size_t)11 * (piece - a)) + 3u * a;
-        dst[0] = sh ? (s[0] >> sh) | (s[1] << (32u - sh)) : s[0];
-        dst[1] = sh ? (s[1] >> sh) | (s[2] << (32u - sh)) : s[1];
+        dst[0] = __funnelshift_r(s[0], s[1], sh);
+        dst[1] = __funnelshift_r(s[1], s[2], sh);
         if (a != 3u) dst[2] = (s[2] >> sh) | (next0 << (24u - sh));
+    }
+    // The same for the warp's 32 pieces by way of 352 bytes of shared memory (`gather`, 16-byte aligned), from which
+    // 22 lanes write 16 bytes each, and again `twin` bytes further on.
+    __device__ __forceinline__ void store_sm_warp(uint8_t* section, uint32_t piece, uint8_t* gather, int64_t twin, uint32_t lane) const {
+        store_sm_group(gather, lane, lane);
+        __syncwarp();
+        if (lane < kWarpSmBytes / 16u) {
+            const uint4 v = ld_shared16(gather + 16u * lane);
+            uint8_t* const dst = section + (size_t)11 * (piece - lane) + 16u * lane;
+            st_stream16(dst, v);
+            st_stream16(dst + twin, v);
+        }
+        __syncwarp();  // the gather space is free again
     }
     // byte by byte (pieces of a tile with a ragged end)
     __device__ __forceinline__ void load_sm_bytes(const uint8_t* src, int nvalid) {

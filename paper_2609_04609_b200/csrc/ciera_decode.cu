@@ -689,10 +689,9 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
                         x.template load_sm_group<Shared>(st, t0 >> 3, lane);
                         chg = (word >> (kb & 31u)) & 1u;
                         if (chg)
-                            x.template load_packed_exponents<Shared>(
-                                st + kSmTile + kTileValues + r->pay_skew + (size_t)payload_bytes_of_blocks<DT>(rank, log2b) +
-                                    5u * ((t0 & bmask) >> 3),
-                                P::kValues);
+                            // (its second word ends at most 3 bytes after the slice, inside the stage's slack)
+                            x.load_packed_exponents(st + kSmTile + kTileValues + r->pay_skew +
+                                                    (size_t)payload_bytes_of_blocks<DT>(rank, log2b) + 5u * ((t0 & bmask) >> 3));
                         else
                             x.template load_exp_full<Shared>(st + kSmTile + t0);
                     } else if (!FINE) {

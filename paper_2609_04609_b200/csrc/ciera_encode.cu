@@ -702,13 +702,45 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
         if (nvalid == 0) continue;
         const uint32_t kb = t0 >> log2b;
         const uint32_t word = bm[kb >> 5];
-        if (!((word >> (kb & 31u)) & 1u)) continue;
+        const bool changed = (word >> (kb & 31u)) & 1u;
+        if constexpr (DT == CIERA_FP16 && FULL && STEP) {
+            // Blocks of 32 values and more: four neighbouring lanes' pieces make 20 bytes = 5 aligned words.  Lane a
+            // of the four writes word a -- the top of its neighbour's 40 bits, then its own -- and lane 3 the last one.
+            // Ten byte stores per piece and message pair bound the step by issue and LSU: with the words, the gathered
+            // sign-plus-mantissa and the exchange of exponents in place an OLMoE-shaped fp16 layer takes 0.600 ms
+            // instead of 0.677 at 32 values per block, 0.611 instead of 0.652 at 512 (its bytes: 0.57 ms at the copy
+            // peak).  The sender alone is bound by HBM with byte stores as well (0.300 ms) and keeps them.
+            if (log2b >= 5u) {
+                if (!__any_sync(0xffffffffu, changed)) continue;
+                P x;
+                x.template load_exp_full<Shared>(s_exp + t0);
+                uint32_t lo, hi;
+                x.pack_exponents(lo, hi);
+                const uint32_t top = __funnelshift_r(lo, hi, 8);  // bits 39:8
+                const uint32_t before = __shfl_up_sync(0xffffffffu, top, 1);
+                if (!changed) continue;
+                const uint32_t rank = pre[kb >> 5] + __popc(word & ((1u << (kb & 31u)) - 1u));
+                const uint32_t in_block = (t0 & ((1u << log2b) - 1u)) >> 3, a = in_block & 3u;
+                uint32_t* const dst = reinterpret_cast<uint32_t*>(ti.pay_dst + base + payload_bytes_of_blocks<DT>(rank, log2b) +
+                                                                  5u * (in_block - a)) + a;
+                const uint32_t own = __funnelshift_l(before, lo, 8u * a);
+                __stcs(dst, own);
+                if (a == 3u) __stcs(dst + 1, top);
+                uint32_t* const twin = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dst) + tw.msg);
+                __stcs(twin, own);
+                if (a == 3u) __stcs(twin + 1, top);
+                x.template store_exp_full<Global>(ti.c_ptr + t0);
+                x.template store_exp_full<Global>(ti.c_ptr + t0 + tw.cache);
+                continue;
+            }
+        }
+        if (!changed) continue;
         const uint32_t rank = pre[kb >> 5] + __popc(word & ((1u << (kb & 31u)) - 1u));
         uint8_t* cdst = ti.c_ptr + t0;
         P x;
         x.template load_exp_full<Shared>(s_exp + t0);
         if constexpr (DT == CIERA_FP16) {
-            // five packed bytes per piece (fewer for the unit's last, short piece), byte by byte
+            // blocks of 16 values, short tiles: five packed bytes per piece (fewer for the last one), byte by byte
             uint8_t* pdst = ti.pay_dst + base + payload_bytes_of_blocks<DT>(rank, log2b) +
                             5u * ((t0 & ((1u << log2b) - 1u)) >> 3);
             uint32_t lo, hi;
@@ -754,9 +786,9 @@ __device__ __forceinline__ void bulk_store_tile_part(const EncodeTileInfo& ti, c
     bulk_commit();
 }
 
-// STEP, coarse blocks: the receiver's part of one tile.  Every consumer thread splits its pieces of the tile once
-// more (the stage still holds the weights), takes the exponents of an unchanged block from the receiver's cache and
-// those of a changed one as they travel in the payload, merges them with the sign-plus-mantissa as it travels and
+// STEP, coarse blocks: the receiver's part of one tile.  Every consumer thread takes its pieces of the tile once
+// more (the stage still holds the weights: sign and mantissa as they travel, and the exponents of changed blocks as
+// they travel in the payload), puts the receiver's cached exponents of the unchanged blocks into their places and
 // stores the reconstructed weights.  (The receiver's cache of changed blocks is refreshed by write_changed.)
 // BULK: the thread's weights are left in their place of the stage instead.
 template <int DT, bool FULL, bool BULK>
@@ -773,22 +805,25 @@ __device__ __forceinline__ void reconstruct(const EncodeTileInfo& ti, uint32_t l
         const bool changed = (bm[kb >> 5] >> (kb & 31u)) & 1u;
         uint8_t* const out = const_cast<uint8_t*>(ti.w_src) + tw.weights + (size_t)t0 * VB;
         const uint8_t* const r = ti.c_ptr + tw.cache + t0;
-        P x;
-        x.template split_full<Shared>(s_w + (size_t)t0 * VB);  // (values past the unit's end are not stored below)
+        uint32_t w[P::kWeightWords];
         if (!changed) {
+            P x;
             if (ti.r_staged)
                 x.template load_exp_full<Shared>(s_r + t0);
             else if (nvalid == P::kValues)
                 x.template load_exp_full<Global>(r);
             else
                 x.load_exp_partial(r, nvalid);
+            x.exchange(s_w + (size_t)t0 * VB, w);
+            if (BULK) P::template store_weights<Shared>(s_w + (size_t)t0 * VB, w);
+        } else if (!BULK) {
+            P::load_weights(s_w + (size_t)t0 * VB, w);
         }
-        if (BULK)
-            x.template merge_store_full<Shared>(s_w + (size_t)t0 * VB);
-        else if (nvalid == P::kValues)
-            x.template merge_store_full<Global>(out);
+        if (BULK) continue;
+        if (nvalid == P::kValues)
+            P::template store_weights<Global>(out, w);
         else
-            x.merge_store_partial(out, nvalid);
+            P::store_weights_first(out, w, nvalid);
     }
 }
 
@@ -888,8 +923,12 @@ __device__ __forceinline__ void write_changed_fine(const EncodeTileInfo& ti, con
 // up to 15 bytes of skew in front (the gathered run starts at the same address modulo 16 as its place in the
 // payload), up to 512 bytes, rounded up to whole 16-byte pieces.
 constexpr uint32_t kWarpGatherBytes = 16u + 512u + 16u;
+// FINE: for the changed exponents; fp16 with STEP: for the packed sign-plus-mantissa.
+template <int DT, bool FINE, bool STEP>
+constexpr uint32_t kGatherBytes = FINE ? kWarpGatherBytes : DT == CIERA_FP16 && STEP ? Piece<CIERA_FP16>::kWarpSmBytes : 0u;
 // The gathering pays from about one changed exponent byte in four (measured with one value per block: 3.4 % changed
-// 0.322 ms per layer gathered against 0.316 ms stored one by one, 50 % changed 0.429 against 0.548 ms).
+// 0.322 ms per layer gathered against 0.316 ms stored one by one, 50 % changed 0.429 against 0.548 ms; fp16, whole step,
+// 40 % changed 0.795 against 1.18 ms; fp16's sender alone would gain 11 % there and lose 1-2 % with few changes).
 constexpr uint32_t kGatherDensity = 4;
 
 // Fine blocks, full tile.  A warp's 32 threads hold the flags of 512 consecutive values, so the changed blocks of
@@ -899,11 +938,12 @@ constexpr uint32_t kGatherDensity = 4;
 // shared memory -- every thread walks its set flags as before, but stores into the warp's gather space -- and
 // then writes it out in whole 16-byte pieces, one per lane, with single bytes only at the two ragged ends.
 // The cache is refreshed by whole sectors as in write_changed_fine.
-template <int LB, bool STEP>
+template <int DT, int LB, bool STEP>
 __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti, const uint32_t* bm, const uint16_t* pre,
                                                         uint64_t base, const uint8_t* s_exp, uint8_t* s_gather,
                                                         const StepTwins& tw, uint32_t tid) {
     constexpr uint32_t kFlags = 16u >> LB;  // flags per thread
+    constexpr uint32_t kBlockBytes = (uint32_t)payload_bytes_of_blocks<DT>(1, LB);
     const uint32_t lane = tid & 31u;
     const uint32_t bit0 = tid * kFlags;
     const uint32_t word = bm[bit0 >> 5], sh = bit0 & 31u;
@@ -916,15 +956,21 @@ __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti
     const uint32_t rank0 = __shfl_sync(0xffffffffu, rank, 0);
     const uint32_t total = __shfl_sync(0xffffffffu, rank + (uint32_t)__popc(bits), 31) - rank0;
     if (total == 0) return;
-    uint8_t* const gdst = ti.pay_dst + base + ((uint64_t)rank0 << LB);  // where the warp's run goes
-    const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(gdst) & 15u);  // a multiple of the block size
-    uint8_t* out = s_gather + skew + ((rank - rank0) << LB);
+    uint8_t* const gdst = ti.pay_dst + base + (uint64_t)rank0 * kBlockBytes;  // where the warp's run goes
+    const uint32_t skew = (uint32_t)(reinterpret_cast<uintptr_t>(gdst) & 15u);  // (not fp16: a multiple of the block size)
+    uint8_t* out = s_gather + skew + (rank - rank0) * kBlockBytes;
     while (bits) {
         const uint32_t j = (uint32_t)__ffs(bits) - 1u;
         bits &= bits - 1u;
         const uint8_t* src = s_exp + ((bit0 + j) << LB);
         if (LB == 0) {
             *out = *src;
+        } else if constexpr (DT == CIERA_FP16) {  // five bits each, the block rounded up to whole bytes
+            unsigned long long packed = 0;
+#pragma unroll
+            for (uint32_t i = 0; i < (1u << LB); ++i) packed |= (unsigned long long)(src[i] & 31u) << (5u * i);
+#pragma unroll
+            for (uint32_t k = 0; k < kBlockBytes; ++k) out[k] = (uint8_t)(packed >> (8u * k));
         } else if (LB == 1) {
             *reinterpret_cast<uint16_t*>(out) = *reinterpret_cast<const uint16_t*>(src);
         } else if (LB == 2) {
@@ -932,12 +978,12 @@ __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti
         } else {
             st_shared8(out, ld_shared8(src));
         }
-        out += 1u << LB;
+        out += kBlockBytes;
     }
     __syncwarp();
     // write-out: piece c covers bytes [16 c, 16 c + 16) of the gather space; the run occupies [skew, skew + len)
     // (the ragged ends byte by byte, one byte per lane; whole pieces in between, one per lane)
-    const uint32_t end = skew + (total << LB);
+    const uint32_t end = skew + total * kBlockBytes;
     uint8_t* const g16 = gdst - skew;
     const uint32_t head_end = min((skew + 15u) & ~15u, end);  // first 16-byte boundary at or after the run's start
     const uint32_t tail_start = max(head_end, end & ~15u);     // last 16-byte boundary at or before its end
@@ -963,16 +1009,15 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
             write_changed<DT, HASH == 0, true, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
         else
             write_changed<DT, HASH == 0, false, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
-    } else if (DT != CIERA_FP16 && ti.nv == (uint32_t)kTileValues &&
-               tile_payload_bytes >= (uint32_t)kTileValues / kGatherDensity) {
+    } else if ((STEP || DT != CIERA_FP16) && ti.nv == (uint32_t)kTileValues && tile_payload_bytes >= (uint32_t)kTileValues / kGatherDensity) {
         // a full tile in which many exponents changed: gathered in shared memory, written out in whole pieces
         switch (log2b) {
-            case 0: write_changed_fine_full<0, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
-            case 1: write_changed_fine_full<1, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
-            case 2: write_changed_fine_full<2, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
-            default: write_changed_fine_full<3, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            case 0: write_changed_fine_full<DT, 0, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            case 1: write_changed_fine_full<DT, 1, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            case 2: write_changed_fine_full<DT, 2, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
+            default: write_changed_fine_full<DT, 3, STEP>(ti, bm, pre, base, s_exp, s_gather, tw, tid); break;
         }
-    } else {  // few changes (a store per changed block is cheaper than the gathering), a unit's last, short tile, or fp16
+    } else {  // few changes (a store per changed block is cheaper than the gathering), a unit's last, short tile, or fp16's sender alone
         switch (log2b) {
             case 0: write_changed_fine<DT, 0, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
             case 1: write_changed_fine<DT, 1, STEP>(ti, bm, pre, base, s_exp, tw, tid); break;
@@ -1027,8 +1072,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const bool early_clear = spread_first < n_tiles && n_tiles - clear_first <= kEarlyClearTiles;
     volatile int* abort = &ctl->abort;
-    // FINE: every consumer warp's gather space for its changed exponents (in place of the hash stages)
-    uint8_t* const s_gather = ring_h + (size_t)(warp < (uint32_t)CW ? warp : 0u) * kWarpGatherBytes;
+    // every consumer warp's gather space (in place of the hash stages)
+    uint8_t* const s_gather = ring_h + (size_t)(warp < (uint32_t)CW ? warp : 0u) * kGatherBytes<DT, FINE, STEP>;
 
     if (tid == 0) {
         for (int s = 0; s < SW; ++s) {
@@ -1440,8 +1485,14 @@ static size_t encode_smem_bytes(uint32_t log2b) {
     using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
     constexpr int SW = Cfg::kWStages, SE = Cfg::kEStages;
     const size_t hash_stage = HASH ? (size_t)hash_hold_bytes<DT>(log2b) + hash_part_bytes<DT>(log2b) : 0;
+    // the SM's 228 KB hold that many blocks, with the 1 KB each that the system takes
+    static_assert(HASH || kEncodeBlocksPerSM<DT, STEP> *
+                                  ((size_t)SW * kTileValues * (Traits<DT>::kValueBytes + (STEP ? 1 : 0)) + (size_t)SE * kTileValues +
+                                   sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)kWarps * kGatherBytes<DT, FINE, STEP> + 1024) <=
+                              233472,
+                  "thread blocks per SM");
     return (size_t)SW * kTileValues * (Traits<DT>::kValueBytes + (STEP ? 1 : 0)) + (size_t)SE * kTileValues +
-           sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)SE * hash_stage + (FINE ? (size_t)kWarps * kWarpGatherBytes : 0);
+           sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)SE * hash_stage + (size_t)kWarps * kGatherBytes<DT, FINE, STEP>;
 }
 
 // Largest grid whose blocks are all resident at once, per device and block size (0 = not yet known).
