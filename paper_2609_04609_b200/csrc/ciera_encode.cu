@@ -1365,6 +1365,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                                                          (S::start(tid, S::kPerThread - 1) >> P::kLog2Values) >> hash_lanes_l2, part, lane);
                     }
                 }
+                if (kBulkOut && !kRebuild) fence_async_shared();  // the reconstructed weights, before lane 0's bulk store reads them
                 __syncwarp();  // the warp's shared-memory accesses above are ordered before lane 0's arrives
                 if (lane == 0) {
                     mbar_arrive(&ctl->voted[se]);
