@@ -353,7 +353,8 @@ CIERA_API int ciera_roundtrip_host(const ciera_plan* plan, const void* weights_h
  *                   need not be initialised
  *   status_dev      device int32 or NULL: CIERA_ERR_CORRUPT if a coded section is inconsistent
  *                   (that unit's payload is then left as received)
- * One launch each, one thread block per unit; nothing waits inside the kernels. */
+ * One launch each for short units, a thread block per unit; longer units are cut into chunks of 64 segments, which
+ * takes up to six launches more (decode: three).  Nothing waits inside the kernels. */
 CIERA_API size_t ciera_plan_entropy_scratch_bytes(const ciera_plan* plan);
 CIERA_API int ciera_entropy_encode(const ciera_plan* plan, void* messages_dev, uint64_t* wire_bytes_dev, void* scratch_dev,
                                    void* stream);
