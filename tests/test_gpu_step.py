@@ -177,3 +177,29 @@ def test_long_runs_cut(dtype, block):
         compare_step(codec, exp, bits[t], f"t={t}")
         compare_caches(codec, table, f"t={t}")
         compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+
+
+@pytest.mark.parametrize("block", [1, 2, 8, 512])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_receiver_with_other_exponents_many_times(dtype, block):
+    """The receiver's cache holds other exponents than the sender's, so that every reconstructed word differs from the
+    weights it was staged with: a store that picks up the stage too early shows (fp32 leaves it by the copy engine)."""
+    from paper_2609_04609_b200 import ciera, runtime
+
+    one, three = (runtime.LayerCodec.from_tensors(SIZES, 1, NAME[dtype], block, DEV) for _ in range(2))
+    gen = wl.make_generator(11 * block + dtype, DEV)
+    n = one.weights_bytes // wl.VALUE_BYTES[NAME[dtype]]
+    for rep in range(40):
+        a = wl.init_weights(n, NAME[dtype], gen)
+        b, other = wl.inject_exponent_changes(a, gen, 0.05), wl.init_weights(n, NAME[dtype], gen)
+        for codec in (one, three):
+            codec.init_caches(a.view(torch.uint8))
+            ciera.cache_init(codec.plan, codec.receiver_cache, other.view(torch.uint8))
+        one.step(b.view(torch.uint8))
+        _three_calls(three, b.view(torch.uint8))
+        torch.cuda.synchronize()
+        one.check_status()
+        for u in one.units:
+            lo = int(u["weights_off"])
+            hi = lo + int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]]
+            assert torch.equal(one.weights_out[lo:hi], three.weights_out[lo:hi]), f"pass {rep}, values from {lo}"
