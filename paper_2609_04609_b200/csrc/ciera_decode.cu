@@ -101,7 +101,6 @@ struct __align__(16) DecodeRing {
     uint32_t nv;                             // values in the tile
     uint32_t tile;                           // the tile's number, or kNoTile: this producer has no more work
     uint32_t pay_skew;                       // fine: bytes in front of the slice in its stage (0 .. 15)
-    uint32_t ws;                             // count from the scratch (units that went through the prefix kernel)
     uint32_t direct;                         // coarse: 1 = the few unchanged pieces read their cached exponents from global memory
     uint16_t pre[kBm];                       // set flags before each word
     // raw material of coarse blocks, fetched asynchronously one tile ahead:
@@ -111,6 +110,15 @@ struct __align__(16) DecodeRing {
 
 static_assert(offsetof(DecodeRing<true>, bm) % 16 == 0 && offsetof(DecodeRing<true>, pre) % 4 == 0,
               "with blocks of one value the flags are digested 16 bytes at a time");
+
+// Units that went through the prefix kernel: the scratch holds, for every tile, the changed blocks of its segment up
+// to and with the tile.  Before tile j there are those of tile j - 1 (unless j starts its segment) and the last count
+// of every earlier segment: one word per lane, fetched into `words` and added up later.
+__device__ __forceinline__ bool prefix_lane(const TileDesc& td, bool fine, uint32_t lane, uint32_t& at) {
+    const uint32_t seg = prefix_segment(td.n_tiles_unit, fine), j = td.tile_in_unit;
+    at = min((lane + 1u) * seg, j) - 1u;
+    return lane * seg < j;
+}
 
 template <int S, int R, bool FINE>
 struct DecodeCtl {
@@ -126,7 +134,7 @@ struct DecodeCtl {
 // slot `r`: the unit's words before the tile (direct units) or the tile's count from the scratch
 // (long units), and the tile's own words.  Nothing is held in registers meanwhile.
 template <bool FINE>
-__device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t tile, uint32_t log2b, const uint8_t* msgs,
+__device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t log2b, const uint8_t* msgs,
                                              const uint32_t* ws_prefix, DecodeRing<FINE>* r, uint32_t lane) {
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td.msg_off);
     const uint64_t kb0 = ((uint64_t)td.tile_in_unit * kTileValues) >> log2b;  // first block of the tile
@@ -136,7 +144,9 @@ __device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t tile, 
         // every unit of more than one tile has its counts in the scratch; the tile's own flags are
         // 128 to 1024 bytes that start on a 128-byte boundary of the slot: 16 bytes per copy,
         // never past the bitmap's padded end
-        if (td.tile_in_unit != 0 && lane == 0) cp_async4(&r->ws, ws_prefix + tile);
+        // (the counts go to where the counts before each word will be)
+        uint32_t at;
+        if (prefix_lane(td, true, lane, at)) cp_async4(reinterpret_cast<uint32_t*>(r->pre) + lane, ws_prefix + td.first_tile + at);
         const uint32_t chunks = nbt >> 7;  // 8 .. 64 copies of four words
         for (uint32_t c = lane; c < chunks; c += 32) {
             const uint64_t w = (kb0 >> 5) + 4ull * c;
@@ -151,8 +161,9 @@ __device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t tile, 
             const uint32_t w = lane + 32u * i;
             if (w < nwords) cp_async4(&r->raw_pre[w], bm32 + w);
         }
-    } else if (lane == 0) {
-        cp_async4(&r->ws, ws_prefix + tile);
+    } else {
+        uint32_t at;
+        if (prefix_lane(td, false, lane, at)) cp_async4(&r->raw_pre[lane], ws_prefix + td.first_tile + at);
     }
     // the tile's own bits: nbt >= 32 -> words (kb0 >> 5) + lane; nbt < 32 -> part of one word
     const uint32_t own_words = nbt >= 32 ? (nbt >> 5) : 1u;
@@ -174,6 +185,11 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
     const uint32_t nv = (uint32_t)min((uint64_t)kTileValues, td.n_unit - v0);
     const uint32_t nblk = (nv + (1u << log2b) - 1u) >> log2b;  // valid blocks of this tile
     uint32_t cnt = 0;
+    if (FINE || nb > kDirectBlocks) {
+        uint32_t at;
+        if (prefix_lane(td, FINE, lane, at)) cnt = FINE ? reinterpret_cast<const uint32_t*>(r->pre)[lane] : r->raw_pre[lane];
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+    }
     if (FINE && log2b == 0) {
         // blocks of one value: 256 words; lane l takes words 8 l .. 8 l + 7, one scan does for the tile
         uint32_t w[8], before8[8], sum = 0;
@@ -206,7 +222,7 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
         for (int i = 0; i < 4; ++i) pre32[i] = (base + before8[2 * i]) | ((base + before8[2 * i + 1]) << 16);
         own_total = __shfl_sync(0xffffffffu, incl, 31);
         __syncwarp();
-        return td.tile_in_unit != 0 ? r->ws : 0u;
+        return cnt;
     }
     if (FINE) {
         // flags past the tile's last block are dropped (words past the bitmap's end were not fetched)
@@ -232,7 +248,7 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
         }
         own_total = run;
         __syncwarp();
-        return td.tile_in_unit != 0 ? r->ws : 0u;
+        return cnt;
     }
     if (nb <= kDirectBlocks) {
         const uint32_t nfull = (uint32_t)(kb0 >> 5);
@@ -245,8 +261,6 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
                 cnt += __popc(r->raw_pre[w] & ((1u << (kb0 & 31u)) - 1u));
         }
         cnt = __reduce_add_sync(0xffffffffu, cnt);
-    } else {
-        cnt = r->ws;
     }
     uint32_t word = 0;
     if (nbt >= 32) {
@@ -485,7 +499,7 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
         cp_async_wait<1>();  // D_0
         __syncwarp();
         if (t_cur != kNoTile)
-            fetch_bitmap(ctl->ring[seq(0) % kDecRing].desc, t_cur, log2b, msgs, ws_prefix, &ctl->ring[seq(0) % kDecRing], lane);
+            fetch_bitmap(ctl->ring[seq(0) % kDecRing].desc, log2b, msgs, ws_prefix, &ctl->ring[seq(0) % kDecRing], lane);
         cp_async_commit();
         for (uint32_t jj = 0;; ++jj) {
             const uint32_t k = seq(jj);
@@ -505,7 +519,7 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
             __syncwarp();
             if (t_nxt != kNoTile) {
                 Ring* rn = &ctl->ring[seq(jj + 1u) % kDecRing];
-                fetch_bitmap(rn->desc, t_nxt, log2b, msgs, ws_prefix, rn, lane);
+                fetch_bitmap(rn->desc, log2b, msgs, ws_prefix, rn, lane);
             }
             cp_async_commit();
 
@@ -805,26 +819,31 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
     }
 }
 
-// Changed blocks before every tile of the long units (more than kDirectBlocks blocks): one thread
-// block per long unit, a running count over the unit's tiles in chunks of 256.
+// Changed blocks of the tiles of the long units (more than kDirectBlocks blocks): one thread block per segment of
+// such a unit, a running count over the segment's tiles in chunks of 256.  One thread block per unit left the GPU idle
+// in tables of few units; receiver of 3 x 12 489 655 fp16 values on 4 shards, 2 per block: 122 -> 53 us; 3 x 14 885 525
+// bf16 on 2, 16 per block: 46 -> 39; one unit of 10^8, 32 per block: 143 -> 75; of 2 x 10^8, 512 per block: 207 -> 136.
+// (Tables of many short units pay for the fetch by all lanes: OLMoE-shaped layer, 1 value per block, bf16 322 -> 329 us,
+// fp16 462 -> 490.)
 __global__ void __launch_bounds__(256)
-decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ long_first_tiles, uint32_t log2b,
+decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ segments, uint32_t log2b,
                      const uint8_t* __restrict__ msgs, uint32_t* __restrict__ ws_prefix) {
     __shared__ uint32_t s_warp[8];
     __shared__ uint32_t s_carry;
     pdl_wait();
-    const uint32_t first = long_first_tiles[blockIdx.x];
-    const TileDesc td0 = load_tile_desc(tiles + first);
+    const TileDesc td0 = load_tile_desc(tiles + segments[blockIdx.x]);
+    const uint32_t first = td0.first_tile, j_begin = td0.tile_in_unit;
+    const uint32_t j_end = min(j_begin + prefix_segment(td0.n_tiles_unit, false), td0.n_tiles_unit);
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td0.msg_off);
     const uint64_t nb = num_blocks(td0.n_unit, log2b);
     const uint32_t nbt = kTileValues >> log2b;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     if (tid == 0) s_carry = 0;
     __syncthreads();
-    for (uint32_t j0 = 0; j0 < td0.n_tiles_unit; j0 += 256u) {
+    for (uint32_t j0 = j_begin; j0 < j_end; j0 += 256u) {
         const uint32_t j = j0 + tid;
         uint32_t cnt = 0;
-        if (j < td0.n_tiles_unit) {
+        if (j < j_end) {
             const uint64_t kb0 = (uint64_t)j * nbt;
             if (nbt >= 32) {
                 for (uint32_t w = 0; w < (nbt >> 5); ++w) {
@@ -851,7 +870,7 @@ decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restr
         uint32_t wbase = 0;
         for (uint32_t w = 0; w < warp; ++w) wbase += s_warp[w];
         const uint32_t carry = s_carry;
-        if (j < td0.n_tiles_unit) ws_prefix[first + j] = carry + wbase + incl - cnt;
+        if (j < j_end) ws_prefix[first + j] = carry + wbase + incl;
         __syncthreads();
         if (tid == 255) s_carry = carry + wbase + incl;
         __syncthreads();
@@ -862,22 +881,23 @@ decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restr
 // 256 words of flags: the warps take the unit's tiles in turn and each counts a tile's flags with
 // all its lanes (consecutive words, coalesced), then the counts are scanned as above.
 __global__ void __launch_bounds__(256)
-decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ long_first_tiles,
+decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ segments,
                           uint32_t log2b, const uint8_t* __restrict__ msgs, uint32_t* __restrict__ ws_prefix) {
     __shared__ uint32_t s_cnt[256];
     __shared__ uint32_t s_warp[8];
     __shared__ uint32_t s_carry;
     pdl_wait();
-    const uint32_t first = long_first_tiles[blockIdx.x];
-    const TileDesc td0 = load_tile_desc(tiles + first);
+    const TileDesc td0 = load_tile_desc(tiles + segments[blockIdx.x]);
+    const uint32_t first = td0.first_tile, j_begin = td0.tile_in_unit;
+    const uint32_t j_end = min(j_begin + prefix_segment(td0.n_tiles_unit, true), td0.n_tiles_unit);
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td0.msg_off);
     const uint64_t nb = num_blocks(td0.n_unit, log2b);
     const uint32_t words = kTileValues >> (log2b + 5);  // words of flags per tile
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     if (tid == 0) s_carry = 0;
     __syncthreads();
-    for (uint32_t j0 = 0; j0 < td0.n_tiles_unit; j0 += 256u) {
-        for (uint32_t t = warp; t < 256u && j0 + t < td0.n_tiles_unit; t += 8u) {
+    for (uint32_t j0 = j_begin; j0 < j_end; j0 += 256u) {
+        for (uint32_t t = warp; t < 256u && j0 + t < j_end; t += 8u) {
             const uint64_t w0 = (uint64_t)(j0 + t) * words;
             uint32_t c = 0;
             for (uint32_t m = lane; m < words; m += 32u) {
@@ -893,7 +913,7 @@ decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __
         }
         __syncthreads();
         const uint32_t j = j0 + tid;
-        const uint32_t cnt = j < td0.n_tiles_unit ? s_cnt[tid] : 0u;
+        const uint32_t cnt = j < j_end ? s_cnt[tid] : 0u;
         uint32_t incl = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -905,7 +925,7 @@ decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __
         uint32_t wbase = 0;
         for (uint32_t w = 0; w < warp; ++w) wbase += s_warp[w];
         const uint32_t carry = s_carry;
-        if (j < td0.n_tiles_unit) ws_prefix[first + j] = carry + wbase + incl - cnt;
+        if (j < j_end) ws_prefix[first + j] = carry + wbase + incl;
         __syncthreads();
         if (tid == 255) s_carry = carry + wbase + incl;
         __syncthreads();
@@ -983,11 +1003,11 @@ extern "C" int ciera_decode(const ciera_plan* p, const void* messages_dev, void*
     // alone), and behind it the per-tile counts of the units that go through the prefix kernel
     unsigned int* ticket = (unsigned int*)((uint8_t*)workspace_dev + workspace_ticket_offset(nt));
     uint32_t* ws_prefix = (uint32_t*)((uint8_t*)workspace_dev + workspace_prefix_offset(nt));
-    const uint32_t n_long = (uint32_t)p->long_units.size();
-    if (n_long) {
+    const uint32_t n_segments = (uint32_t)p->prefix_segments.size();
+    if (n_segments) {
         const cudaError_t e =
-            launch_after(is_fine(p->log2b) ? decode_prefix_fine_kernel : decode_prefix_kernel, dim3(n_long), 256, 0, s, p->tiles_dev,
-                         p->long_units_dev, p->log2b, (const uint8_t*)messages_dev, ws_prefix);
+            launch_after(is_fine(p->log2b) ? decode_prefix_fine_kernel : decode_prefix_kernel, dim3(n_segments), 256, 0, s, p->tiles_dev,
+                         p->prefix_segments_dev, p->log2b, (const uint8_t*)messages_dev, ws_prefix);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }

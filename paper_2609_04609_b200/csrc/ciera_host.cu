@@ -75,7 +75,7 @@ ImageLayout image_layout(const ciera_plan* p) {
     ImageLayout L;
     L.tiles = p->tiles.size() * sizeof(TileDesc);
     L.long_off = L.tiles;
-    L.seq_off = L.long_off + up16(p->long_units.size() * sizeof(uint32_t));
+    L.seq_off = L.long_off + up16(p->prefix_segments.size() * sizeof(uint32_t));
     L.hash_off = L.seq_off + up16(p->seq_first.size() * sizeof(uint32_t));
     L.first_off = L.hash_off + up16((size_t)p->n_units * sizeof(uint64_t));
     L.seg_off = L.first_off + up16((size_t)p->n_units * sizeof(uint32_t));
@@ -155,7 +155,8 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
             p->tiles.push_back(t);
         }
         const bool needs_prefix = is_fine(p->log2b) ? nt > 1 : (un.n_values + block - 1) / block > kDecodeDirectBlocks;
-        if (needs_prefix) p->long_units.push_back(first);
+        if (needs_prefix)
+            for (uint32_t j = 0; j < nt; j += prefix_segment(nt, is_fine(p->log2b))) p->prefix_segments.push_back(first + j);
     };
     for (uint32_t u : shorts) {
         p->seq_first.push_back((uint32_t)p->tiles.size());
@@ -257,7 +258,7 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     const ImageLayout L = image_layout(p);
     p->image.assign(L.total, 0);
     if (L.tiles) memcpy(p->image.data(), p->tiles.data(), L.tiles);
-    if (!p->long_units.empty()) memcpy(p->image.data() + L.long_off, p->long_units.data(), p->long_units.size() * 4);
+    if (!p->prefix_segments.empty()) memcpy(p->image.data() + L.long_off, p->prefix_segments.data(), p->prefix_segments.size() * 4);
     memcpy(p->image.data() + L.seq_off, p->seq_first.data(), p->seq_first.size() * 4);
     if (!p->tiles_by_address.empty())
         memcpy(p->image.data() + L.byaddr_off, p->tiles_by_address.data(), p->tiles_by_address.size() * sizeof(uint32_t));
@@ -331,7 +332,7 @@ extern "C" int ciera_plan_bind(ciera_plan* p, void* plan_dev, size_t plan_dev_by
     const ImageLayout L = image_layout(p);
     const uint8_t* base = (const uint8_t*)plan_dev;
     p->tiles_by_address_dev = p->tiles_by_address.empty() ? nullptr : (const uint32_t*)(base + L.byaddr_off);
-    p->long_units_dev = (const uint32_t*)(base + L.long_off);
+    p->prefix_segments_dev = (const uint32_t*)(base + L.long_off);
     p->seq_first_dev = (const uint32_t*)(base + L.seq_off);
     p->hash_base_dev = (const unsigned long long*)(base + L.hash_off);
     p->unit_first_dev = (const uint32_t*)(base + L.first_off);

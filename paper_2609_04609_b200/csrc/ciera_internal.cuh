@@ -88,6 +88,14 @@ __host__ __device__ inline uint64_t pad16(uint64_t x) { return (x + 15ull) & ~15
 __host__ __device__ inline uint64_t num_blocks(uint64_t n, uint32_t log2b) {
     return (n + (1ull << log2b) - 1) >> log2b;
 }
+// Tiles per segment of a unit of n_tiles tiles whose changed blocks before each tile are counted ahead of decode
+// (a power of two; at most 32 segments, so that one lane each can fetch their totals; a segment has work enough
+// for one thread block of the prefix kernel: with fine blocks 128 bytes to 1 KB of flags per tile, else a few words)
+__host__ __device__ inline uint32_t prefix_segment(uint32_t n_tiles, bool fine) {
+    uint32_t s = fine ? 16u : 256u;
+    while (32u * s < n_tiles) s *= 2u;
+    return s;
+}
 __host__ __device__ inline uint64_t bitmap_bytes(uint64_t n, uint32_t log2b) { return (num_blocks(n, log2b) + 7) >> 3; }
 __host__ __device__ inline uint64_t sm_offset(uint64_t n, uint32_t log2b) { return pad16(bitmap_bytes(n, log2b)); }
 __host__ __device__ inline uint64_t payload_offset(uint64_t n, uint32_t sm_bytes_per_value, uint32_t log2b) {
@@ -180,7 +188,7 @@ struct ciera_plan {
     bool has_empty_units = false;
     std::vector<ciera_unit> units;
     std::vector<ciera::TileDesc> tiles;
-    std::vector<uint32_t> long_units;  // first tile of every unit whose decode needs the prefix kernel
+    std::vector<uint32_t> prefix_segments;  // first tiles of the segments of every unit whose decode needs the prefix kernel
     std::vector<uint32_t> seq_first;   // first tile of every short unit, in table order, + end marker
     struct SeqRun {
         uint32_t lo, hi;               // tiles [lo, hi) of the table
@@ -208,7 +216,7 @@ struct ciera_plan {
     std::vector<EntChunk> ent_chunks;
     const uint32_t* ent_long_units_dev = nullptr;
     const uint4* ent_chunks_dev = nullptr;
-    std::vector<uint8_t> image;        // device image: tiles, long_units, seq_first, hash_base, unit_first, seg_base, units,
+    std::vector<uint8_t> image;        // device image: tiles, prefix_segments, seq_first, hash_base, unit_first, seg_base, units,
                                        // ent_long_units, ent_chunks, tiles_by_address, tile_hash, seq_runs
     const ciera::TileDesc* tiles_dev = nullptr;
     const uint32_t* tiles_by_address_dev = nullptr;
@@ -221,7 +229,7 @@ struct ciera_plan {
     };
     mutable std::mutex lanes_mutex;
     mutable std::vector<CopyLane> lanes;
-    const uint32_t* long_units_dev = nullptr;
+    const uint32_t* prefix_segments_dev = nullptr;
     const uint32_t* seq_first_dev = nullptr;
     const uint2* seq_runs_dev = nullptr;
     const unsigned long long* hash_base_dev = nullptr;
