@@ -13,6 +13,7 @@ static std::atomic<uint64_t> g_launches{0};
 
 int record_cuda_error(cudaError_t e) {
     g_last_cuda_error = (int)e;
+    cudaGetLastError();  // reported here: the launch check of the next call must not find it again
     return CIERA_ERR_CUDA;
 }
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -281,11 +282,7 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
 
 extern "C" void ciera_plan_destroy(ciera_plan* plan) {
     if (plan)
-        for (const ciera_plan::CopyLane& lane : plan->lanes) {  // (work still queued there runs to its end)
-            cudaStreamDestroy(lane.in);
-            cudaStreamDestroy(lane.out);
-            cudaEventDestroy(lane.event);
-        }
+        for (const ciera_plan::CopyLane& lane : plan->lanes) destroy_copy_lane(lane);  // (work still queued there runs to its end)
     delete plan;
 }
 

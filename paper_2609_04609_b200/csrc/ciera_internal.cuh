@@ -176,6 +176,9 @@ __host__ __device__ inline uint64_t transport_chunk_bytes(uint32_t sm_bytes_per_
     return (uint64_t)kTileValues * (sm_bytes_per_value + 1) + bitmap_share;
 }
 
+// the largest number of parts that a step on host weights is cut into
+constexpr uint32_t kHostPartsMax = 64;
+
 }  // namespace ciera
 
 // The plan object behind the opaque handle.
@@ -226,6 +229,7 @@ struct ciera_plan {
         int device;
         cudaStream_t in, out;
         cudaEvent_t event;
+        cudaEvent_t arrived[ciera::kHostPartsMax];  // behind each part's weights
     };
     mutable std::mutex lanes_mutex;
     mutable std::vector<CopyLane> lanes;
@@ -266,6 +270,7 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 int check_launch();                            // cudaGetLastError -> status
+void destroy_copy_lane(const ciera_plan::CopyLane& lane);
 // the persistent sender kernel with HashCache in place of the exponent cache (ciera_encode.cu)
 int launch_encode_hashed(const ciera_plan* p, const void* weights_dev, void* hash_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,

@@ -1,6 +1,9 @@
 // Auxiliary sm_100a kernels of libciera: cache initialisation, the transport stand-in, and the
 // host-buffer round trip.  (Encode and decode live in ciera_encode.cu / ciera_decode.cu.)
+#include <algorithm>
+
 #include "ciera_bits.cuh"
+#include "ciera_host_step.hpp"
 #include "ciera_lookback.cuh"
 #include "ciera_pipe.cuh"
 
@@ -375,8 +378,6 @@ extern "C" int ciera_transport(const ciera_plan* p, const void* src_messages_dev
 // 8 pieces, 2.73 in 32, about 20 us a piece).  Both together are least near sqrt(link time / 20 us) = sqrt(MB) parts.
 // 100 MB of bf16 weights: as a whole 3.72 ms, 8 parts 2.45, 16 equal parts 2.52, 32 equal parts 2.86; 25 MB: as a whole
 // 0.935 ms, 6 parts 0.727, 12 parts 0.811.
-constexpr uint32_t kHostPartsMax = 64;
-
 // parts to cut the step into; 1: as a whole
 static uint32_t host_step_parts(const ciera_plan* p, const void* in, const void* out, size_t bytes, cudaStream_t s) {
     uint32_t parts = 1;
@@ -388,44 +389,96 @@ static uint32_t host_step_parts(const ciera_plan* p, const void* in, const void*
         cudaGetLastError();
         return 1;
     }
-    for (const void* q : {in, out}) {
-        cudaPointerAttributes a;
-        if (cudaPointerGetAttributes(&a, q) != cudaSuccess || a.type != cudaMemoryTypeHost) {
-            cudaGetLastError();
-            return 1;
+    for (const void* q : {in, out})
+        for (const void* end : {q, (const void*)((const uint8_t*)q + bytes - 1)}) {
+            cudaPointerAttributes a;
+            if (cudaPointerGetAttributes(&a, end) != cudaSuccess || a.type != cudaMemoryTypeHost) {
+                cudaGetLastError();
+                return 1;
+            }
         }
-    }
     return parts;
 }
 
-static int take_copy_lane(const ciera_plan* p, ciera_plan::CopyLane* lane) {
+void ciera::destroy_copy_lane(const ciera_plan::CopyLane& lane) {
+    if (lane.in) cudaStreamDestroy(lane.in);
+    if (lane.out) cudaStreamDestroy(lane.out);
+    if (lane.event) cudaEventDestroy(lane.event);
+    for (cudaEvent_t a : lane.arrived)
+        if (a) cudaEventDestroy(a);
+}
+
+// (with events for that many parts)
+static int take_copy_lane(const ciera_plan* p, uint32_t parts, ciera_plan::CopyLane* lane) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return record_cuda_error(e);
+    *lane = {};
+    lane->device = dev;
     {
         std::lock_guard<std::mutex> hold(p->lanes_mutex);
         for (size_t i = 0; i < p->lanes.size(); ++i)
             if (p->lanes[i].device == dev) {
                 *lane = p->lanes[i];
                 p->lanes.erase(p->lanes.begin() + i);
-                return CIERA_OK;
+                break;
             }
     }
-    *lane = {dev, nullptr, nullptr, nullptr};
-    e = cudaStreamCreateWithFlags(&lane->in, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&lane->out, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&lane->event, cudaEventDisableTiming);
+    if (!lane->in) e = cudaStreamCreateWithFlags(&lane->in, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !lane->out) e = cudaStreamCreateWithFlags(&lane->out, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !lane->event) e = cudaEventCreateWithFlags(&lane->event, cudaEventDisableTiming);
+    for (uint32_t k = 0; k < parts; ++k)
+        if (e == cudaSuccess && !lane->arrived[k]) e = cudaEventCreateWithFlags(&lane->arrived[k], cudaEventDisableTiming);
     if (e == cudaSuccess) return CIERA_OK;
-    if (lane->in) cudaStreamDestroy(lane->in);
-    if (lane->out) cudaStreamDestroy(lane->out);
+    destroy_copy_lane(*lane);
     return record_cuda_error(e);
 }
 
-// `to` waits for what `from` holds so far (one event serves them all: a wait refers to the record before it)
-static cudaError_t join(cudaStream_t to, cudaStream_t from, cudaEvent_t event) {
+// `to` waits for what `from` holds so far
+static cudaError_t wait_for(cudaStream_t to, cudaStream_t from, cudaEvent_t event) {
     const cudaError_t e = cudaEventRecord(event, from);
     return e != cudaSuccess ? e : cudaStreamWaitEvent(to, event, 0);
 }
+
+// queues the parts of one step (see ciera_host_step.hpp)
+struct HostStepOps {
+    struct Part {
+        uint32_t lo, hi;    // tiles by address
+        uint64_t from, to;  // bytes of the weights
+    };
+    const ciera_plan* p;
+    const ciera_device_buffers* b;
+    const uint8_t* in;
+    uint8_t* out;
+    const ciera_plan::CopyLane& lane;
+    cudaStream_t s;
+    Part part[kHostPartsMax];
+
+    static int status_of(cudaError_t e) { return e != cudaSuccess ? record_cuda_error(e) : CIERA_OK; }
+    int copy_in(uint32_t k) {
+        const Part& t = part[k];
+        cudaError_t e = cudaSuccess;
+        if (t.to > t.from) e = cudaMemcpyAsync((uint8_t*)b->weights_dev + t.from, in + t.from, t.to - t.from, cudaMemcpyHostToDevice, lane.in);
+        if (e == cudaSuccess) e = cudaEventRecord(lane.arrived[k], lane.in);
+        return status_of(e);
+    }
+    int step(uint32_t k) {
+        const cudaError_t e = cudaStreamWaitEvent(s, lane.arrived[k], 0);
+        return e != cudaSuccess ? record_cuda_error(e) : launch_step_part(p, b, part[k].lo, part[k].hi, s);
+    }
+    int copy_out(uint32_t k) {
+        const Part& t = part[k];
+        cudaError_t e = wait_for(lane.out, s, lane.event);
+        if (e == cudaSuccess && t.to > t.from)
+            e = cudaMemcpyAsync(out + t.from, (const uint8_t*)b->weights_out_dev + t.from, t.to - t.from, cudaMemcpyDeviceToHost, lane.out);
+        return status_of(e);
+    }
+    void clear() { cudaMemsetAsync(b->workspace_dev, 0, workspace_total_bytes(p->tiles.size()), s); }
+    int join() {
+        const cudaError_t e1 = wait_for(s, lane.in, lane.event), e2 = wait_for(s, lane.out, lane.event);
+        return status_of(e1 != cudaSuccess ? e1 : e2);
+    }
+};
 
 static int host_step_in_parts(const ciera_plan* p, const void* weights_host, size_t weights_bytes, void* weights_out_host,
                               const ciera_device_buffers* b, uint32_t parts, cudaStream_t s) {
@@ -434,37 +487,28 @@ static int host_step_in_parts(const ciera_plan* p, const void* weights_host, siz
                               b->weights_out_dev, b->wire_bytes_dev, b->changed_blocks_dev, b->workspace_dev, s);
     if (rc) return rc;
     ciera_plan::CopyLane lane;
-    rc = take_copy_lane(p, &lane);
+    rc = take_copy_lane(p, parts, &lane);
     if (rc) return rc;
+    HostStepOps op{p, b, (const uint8_t*)weights_host, (uint8_t*)weights_out_host, lane, s, {}};
     const uint32_t nt = (uint32_t)p->tiles.size();
-    cudaError_t e = join(lane.in, s, lane.event);
-    uint32_t lo = 0;
-    uint64_t from = 0;  // weights up to this byte are on their way
-    for (uint32_t k = 1; k <= parts && e == cudaSuccess && rc == CIERA_OK; ++k) {
+    uint32_t n = 0, lo = 0;
+    uint64_t from = 0;
+    for (uint32_t k = 1; k <= parts; ++k) {
         const uint32_t hi = k == parts ? nt : (uint32_t)((uint64_t)nt * (2u * k - 1u) / (2u * parts - 2u));
         if (hi == lo) continue;
         uint64_t to = hi < nt ? p->tiles[p->tiles_by_address.empty() ? hi : p->tiles_by_address[hi]].w_off : (uint64_t)weights_bytes;
-        if (to > weights_bytes) to = weights_bytes;
-        if (to < from) to = from;
-        const uint64_t n = to - from;
-        if (n) e = cudaMemcpyAsync((uint8_t*)b->weights_dev + from, (const uint8_t*)weights_host + from, n, cudaMemcpyHostToDevice, lane.in);
-        if (e == cudaSuccess) e = join(s, lane.in, lane.event);
-        if (e == cudaSuccess) rc = launch_step_part(p, b, lo, hi, s);
-        if (e == cudaSuccess && rc == CIERA_OK) e = join(lane.out, s, lane.event);
-        if (e == cudaSuccess && rc == CIERA_OK && n)
-            e = cudaMemcpyAsync((uint8_t*)weights_out_host + from, (const uint8_t*)b->weights_out_dev + from, n, cudaMemcpyDeviceToHost, lane.out);
+        to = std::max(from, std::min(to, (uint64_t)weights_bytes));
+        op.part[n++] = {lo, hi, from, to};
         from = to;
         lo = hi;
     }
-    // whatever happened, the caller's stream waits for what has been queued
-    const cudaError_t e2 = join(s, lane.in, lane.event), e3 = join(s, lane.out, lane.event);
+    const cudaError_t e = wait_for(lane.in, s, lane.event);
+    rc = e != cudaSuccess ? record_cuda_error(e) : run_host_parts(op, n);
     {
         std::lock_guard<std::mutex> hold(p->lanes_mutex);
         p->lanes.push_back(lane);
     }
-    if (rc) return rc;
-    if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
-    return e != cudaSuccess ? record_cuda_error(e) : CIERA_OK;
+    return rc;
 }
 
 extern "C" int ciera_roundtrip_host(const ciera_plan* p, const void* weights_host, size_t weights_bytes,

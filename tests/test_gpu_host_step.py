@@ -1,0 +1,91 @@
+"""Steps on host weights (``ciera_roundtrip_host``): what a copy that the runtime refuses leaves behind, buffers that
+overlap, several threads and streams; against the oracle, tolerance 0.
+
+A copy is made to fail on the host: the runtime refuses a range that is page-locked at both ends and not in the middle."""
+import ctypes
+import mmap
+
+import numpy as np
+import pytest
+import torch
+
+from harness import OracleTable, compare_caches, compare_recon, compare_step, sender_scratch_is_clean, to_dev_bytes
+from paper_2609_04609_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+SIZES = [8192 * 40 + 3, 100, 8192 * 900 + 4097, 8192 * 12 + 5, 1_000_000]  # about 18 MB in bf16: four parts
+
+
+class HalfPinned:
+    """Host memory of ``size`` bytes of which only the first and the last quarter are page-locked."""
+
+    def __init__(self, size):
+        page = mmap.PAGESIZE
+        self.map = mmap.mmap(-1, (size + page - 1) // page * page)
+        self.tensor = torch.frombuffer(self.map, dtype=torch.uint8)[:size]
+        base, quarter = self.tensor.data_ptr(), len(self.map) // 4 // page * page
+        self.locked = [(base, quarter), (base + len(self.map) - quarter, quarter)]
+        for at, n in self.locked:
+            assert int(torch.cuda.cudart().cudaHostRegister(at, n, 0)) == 0
+
+    def release(self):
+        for at, _ in self.locked:
+            assert int(torch.cuda.cudart().cudaHostUnregister(at)) == 0
+
+
+def _make(sizes=SIZES, block=512, seed=3, steps=3):
+    from paper_2609_04609_b200 import runtime
+
+    codec = runtime.LayerCodec.from_tensors(sizes, 1, "bf16", block, DEV)
+    table = OracleTable(codec.units, 0, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(seed)
+    w = [wl.init_weights(codec.weights_bytes // 2, "bf16", gen)]
+    for _ in range(steps):
+        w.append(wl.step_clustered(w[-1], gen, f=0.3))
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    staging = torch.empty(codec.weights_bytes, dtype=torch.uint8, device=DEV)
+    return codec, table, bits, staging
+
+
+def _pinned(bits):
+    return torch.from_numpy(bits.view(np.uint8).copy()).pin_memory()
+
+
+def _compare(codec, table, exp, bits, label):
+    torch.cuda.synchronize()
+    codec.check_status()
+    compare_step(codec, exp, bits, label)
+    compare_caches(codec, table, label)
+    compare_recon(codec, exp, bits, 0, label)
+
+
+@pytest.mark.parametrize("side", ["in", "out"])
+def test_a_copy_that_fails_half_way(side):
+    from paper_2609_04609_b200 import ciera
+
+    codec, table, bits, staging = _make()
+    good_out = torch.zeros(codec.weights_bytes, dtype=torch.uint8).pin_memory()
+    holed = HalfPinned(codec.weights_bytes)
+    holed.tensor.copy_(torch.from_numpy(bits[1].view(np.uint8)))
+    before = codec.sender_cache.clone(), codec.receiver_cache.clone()
+    with pytest.raises(ciera.CieraError) as e:
+        if side == "in":
+            codec.step_host(holed.tensor, good_out, staging)
+        else:
+            codec.step_host(_pinned(bits[1]), holed.tensor, staging)
+    assert e.value.status == ciera.ERR_CUDA
+    torch.cuda.synchronize()
+    holed.release()
+    assert sender_scratch_is_clean(codec)
+    if side == "in":  # nothing was stepped
+        assert torch.equal(codec.sender_cache, before[0]) and torch.equal(codec.receiver_cache, before[1])
+    else:  # the step on the device is complete
+        _compare(codec, table, table.step(bits[1]), bits[1], "step whose way out failed")
+    for t in (2, 3):
+        codec.step_host(_pinned(bits[t]), good_out, staging)
+        _compare(codec, table, table.step(bits[t]), bits[t], f"t={t}")
+    ciera.cache_init(codec.plan, codec.sender_cache, staging)  # (the earlier error is not reported twice)
