@@ -298,8 +298,9 @@ CIERA_API int ciera_decode(const ciera_plan* plan, const void* messages_dev, voi
  * one GPU: every byte of a message is stored to both buffers as it is made, and the receiver's part works on it
  * before it leaves the chip, so nothing that the step itself has written is fetched again.  The receiver's weights
  * come from its own cache and the message's contents, as in ciera_decode.
- * Arguments as for the three calls; msg_send_dev and msg_recv_dev are different buffers, weights_out_dev may be
- * weights_dev.
+ * Arguments as for the three calls.  One launch needs the buffers apart, but for weights_out_dev, which may be
+ * weights_dev; where they overlap in any other way (say, reconstructed weights over the message that was sent), or where
+ * units share weights that are reconstructed in place, the call runs the three kernels one after the other.
  */
 CIERA_API int ciera_step(const ciera_plan* plan, const void* weights_dev, void* sender_cache_dev, void* msg_send_dev,
                          void* msg_recv_dev, void* receiver_cache_dev, void* weights_out_dev, uint64_t* wire_bytes_dev,

@@ -1679,6 +1679,26 @@ static StepTwins step_twins(const void* weights, const void* sender_cache, const
                      (int64_t)((intptr_t)weights_out - (intptr_t)weights)};
 }
 
+// One launch reads and writes all buffers of a step side by side.  Three calls in a row only need what is live between
+// them: the reconstructed weights may go to where the weights lay a little further on, or to where the message was sent
+// from.  Here, each buffer has to have its place to itself, but for weights that are reconstructed in place (the same
+// bytes, tile by tile, unless units share theirs).
+bool ciera::step_buffers_apart(const ciera_plan* p, const void* weights, const void* sender_cache, const void* msg_send,
+                               const void* msg_recv, const void* receiver_cache, const void* weights_out) {
+    struct {
+        uintptr_t at;
+        uint64_t bytes;
+    } const r[6] = {{(uintptr_t)weights, p->weights_extent},  {(uintptr_t)weights_out, p->weights_extent},
+                    {(uintptr_t)sender_cache, p->cache_extent}, {(uintptr_t)receiver_cache, p->cache_extent},
+                    {(uintptr_t)msg_send, p->msg_extent},       {(uintptr_t)msg_recv, p->msg_extent}};
+    for (int i = 0; i < 6; ++i)
+        for (int j = i + 1; j < 6; ++j) {
+            if (i == 0 && j == 1 && weights == weights_out && p->by_address_ok) continue;
+            if (r[i].at < r[j].at + r[j].bytes && r[j].at < r[i].at + r[i].bytes) return false;
+        }
+    return true;
+}
+
 // The checks of a step, and the outputs of units without tiles.
 int ciera::step_begin(const ciera_plan* p, const void* weights_dev, const void* sender_cache_dev, const void* msg_send_dev,
                             const void* msg_recv_dev, const void* receiver_cache_dev, const void* weights_out_dev,
@@ -1711,6 +1731,14 @@ extern "C" int ciera_step(const ciera_plan* p, const void* weights_dev, void* se
     const int rc = step_begin(p, weights_dev, sender_cache_dev, msg_send_dev, msg_recv_dev, receiver_cache_dev,
                                     weights_out_dev, wire_bytes_dev, changed_blocks_dev, workspace_dev, s);
     if (rc || p->tiles.empty()) return rc;
+    if (!step_buffers_apart(p, weights_dev, sender_cache_dev, msg_send_dev, msg_recv_dev, receiver_cache_dev, weights_out_dev)) {
+        int r = ciera_encode(p, weights_dev, sender_cache_dev, msg_send_dev, wire_bytes_dev, changed_blocks_dev, workspace_dev,
+                             status_dev, stream);
+        if (r == CIERA_OK) r = ciera_transport(p, msg_send_dev, msg_recv_dev, wire_bytes_dev, workspace_dev, status_dev, stream);
+        if (r == CIERA_OK)
+            r = ciera_decode(p, msg_recv_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev, workspace_dev, status_dev, stream);
+        return r;
+    }
     const StepTwins tw = step_twins(weights_dev, sender_cache_dev, msg_send_dev, msg_recv_dev, receiver_cache_dev, weights_out_dev);
     return launch_encode_any(p, weights_dev, sender_cache_dev, msg_send_dev, wire_bytes_dev, changed_blocks_dev,
                              workspace_dev, status_dev, s, &tw);

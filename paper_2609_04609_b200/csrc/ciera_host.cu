@@ -244,7 +244,11 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         // the payload of a unit has at most n_values bytes: that many 4096-byte segments
         p->seg_base[u] = p->total_segments;
         p->total_segments += (units_host[u].n_values + 4095) / 4096;
-        p->cache_extent = std::max<uint64_t>(p->cache_extent, units_host[u].cache_off + units_host[u].n_values);
+        if (units_host[u].n_values) {
+            p->cache_extent = std::max<uint64_t>(p->cache_extent, units_host[u].cache_off + units_host[u].n_values);
+            p->weights_extent = std::max<uint64_t>(p->weights_extent, units_host[u].weights_off + units_host[u].n_values * vb);
+            p->msg_extent = std::max<uint64_t>(p->msg_extent, units_host[u].msg_off + units_host[u].msg_capacity);
+        }
         const uint64_t slots = (units_host[u].n_values + 4095) / 4096;
         if (slots > p->ent_long_slots) {  // the entropy stage spreads such a unit over several thread blocks
             const uint32_t li = (uint32_t)p->ent_long_units.size();

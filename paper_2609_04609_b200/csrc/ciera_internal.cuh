@@ -208,7 +208,8 @@ struct ciera_plan {
     uint64_t total_blocks = 0;
     std::vector<uint64_t> seg_base;    // index of every unit's first 4096-byte payload segment (entropy stage)
     uint64_t total_segments = 0;
-    uint64_t cache_extent = 0;         // max over units of cache_off + n_values
+    // the ends of the units' furthest values and slots in the three kinds of buffers, in bytes
+    uint64_t cache_extent = 0, weights_extent = 0, msg_extent = 0;
     // entropy stage: units of more than ent_long_slots segment slots, and their chunks of 64 slots
     uint32_t ent_long_slots = 64;
     // {unit, first segment of the chunk inside the unit, index among the long units, 0}
@@ -279,6 +280,9 @@ int launch_encode_hashed(const ciera_plan* p, const void* weights_dev, void* has
 int step_begin(const ciera_plan* p, const void* weights_dev, const void* sender_cache_dev, const void* msg_send_dev,
                const void* msg_recv_dev, const void* receiver_cache_dev, const void* weights_out_dev, uint64_t* wire_bytes_dev,
                uint32_t* changed_blocks_dev, const void* workspace_dev, cudaStream_t s);
+// whether the buffers of a step lie apart, so that one launch may work on all of them
+bool step_buffers_apart(const ciera_plan* p, const void* weights, const void* sender_cache, const void* msg_send,
+                        const void* msg_recv, const void* receiver_cache, const void* weights_out);
 // ciera_step on the tiles [lo, hi) of the plan's tiles by address; parts of one step go to one stream in order
 int launch_step_part(const ciera_plan* p, const ciera_device_buffers* b, uint32_t lo, uint32_t hi, cudaStream_t s);
 }  // namespace ciera

@@ -379,10 +379,16 @@ extern "C" int ciera_transport(const ciera_plan* p, const void* src_messages_dev
 // 100 MB of bf16 weights: as a whole 3.72 ms, 8 parts 2.45, 16 equal parts 2.52, 32 equal parts 2.86; 25 MB: as a whole
 // 0.935 ms, 6 parts 0.727, 12 parts 0.811.
 // parts to cut the step into; 1: as a whole
-static uint32_t host_step_parts(const ciera_plan* p, const void* in, const void* out, size_t bytes, cudaStream_t s) {
+static uint32_t host_step_parts(const ciera_plan* p, const ciera_device_buffers* b, const void* in, const void* out, size_t bytes,
+                                cudaStream_t s) {
     uint32_t parts = 1;
     while (parts < kHostPartsMax && ((uint64_t)(parts + 1) * (parts + 1) << 20) <= bytes) ++parts;
     if (parts < 2 || !p->by_address_ok) return 1;
+    if (!step_buffers_apart(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->msg_recv_dev, b->receiver_cache_dev, b->weights_out_dev))
+        return 1;
+    // (a part goes out while others still come in: in place, or with both ranges apart)
+    const uintptr_t a0 = (uintptr_t)in, a1 = (uintptr_t)out;
+    if (a0 != a1 && a0 < a1 + bytes && a1 < a0 + bytes) return 1;
     // (inside a capture no streams are made; pageable memory is copied synchronously, which parts would only slow down)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
@@ -519,7 +525,7 @@ extern "C" int ciera_roundtrip_host(const ciera_plan* p, const void* weights_hos
     if (!b || !weights_host || !weights_out_host) return CIERA_ERR_INVALID_ARG;
     if (p->tiles.empty()) return CIERA_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    const uint32_t parts = host_step_parts(p, weights_host, weights_out_host, weights_bytes, s);
+    const uint32_t parts = host_step_parts(p, b, weights_host, weights_out_host, weights_bytes, s);
     if (parts > 1) {
         rc = host_step_in_parts(p, weights_host, weights_bytes, weights_out_host, b, parts, s);
         if (rc) return rc;

@@ -105,7 +105,8 @@ class LayerCodec:
                      self.wire_bytes if check_length else None, self.workspace, self.status, stream)
 
     def step(self, weights: torch.Tensor, weights_out: Optional[torch.Tensor] = None, stream=None) -> None:
-        """encode, transport and decode in one launch."""
+        """encode, transport and decode in one launch (in three where ``weights_out`` overlaps another buffer without
+        being ``weights`` itself)."""
         out = self.weights_out if weights_out is None else weights_out
         ciera.step(self.plan, weights, self.sender_cache, self.msg_send, self.msg_recv, self.receiver_cache, out,
                    self.wire_bytes, self.changed_blocks, self.workspace, self.status, stream)

@@ -89,3 +89,18 @@ def test_a_copy_that_fails_half_way(side):
         codec.step_host(_pinned(bits[t]), good_out, staging)
         _compare(codec, table, table.step(bits[t]), bits[t], f"t={t}")
     ciera.cache_init(codec.plan, codec.sender_cache, staging)  # (the earlier error is not reported twice)
+
+
+@pytest.mark.parametrize("shift", [-(1 << 20), 0, 16, 1 << 20, 8 << 20])
+def test_host_ranges_that_overlap(shift):
+    """The step reads all of its weights before it writes any: the output may lie over the input, shifted or not."""
+    codec, table, bits, staging = _make(steps=1)
+    n = codec.weights_bytes
+    room = torch.zeros(n + (9 << 20), dtype=torch.uint8).pin_memory()
+    src, out = room[1 << 20 :][:n], room[(1 << 20) + shift :][:n]
+    src.copy_(torch.from_numpy(bits[1].view(np.uint8)))
+    codec.step_host(src, out, staging)
+    _compare(codec, table, table.step(bits[1]), bits[1], f"shift {shift}")
+    for u in codec.units:
+        lo, hi = int(u["weights_off"]), int(u["weights_off"]) + 2 * int(u["n_values"])
+        assert np.array_equal(out.numpy()[lo:hi], bits[1].view(np.uint8)[lo:hi])

@@ -203,3 +203,38 @@ def test_receiver_with_other_exponents_many_times(dtype, block):
             lo = int(u["weights_off"])
             hi = lo + int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]]
             assert torch.equal(one.weights_out[lo:hi], three.weights_out[lo:hi]), f"pass {rep}, values from {lo}"
+
+
+@pytest.mark.parametrize("block", [1, 512])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+@pytest.mark.parametrize("where", ["weights - 64 KB", "weights + 16", "weights + 24 MB", "sent message"])
+def test_output_over_buffers_that_the_three_calls_are_done_with(dtype, block, where):
+    """Where the reconstructed weights go over bytes that the sender has read or sent by then, a step does what the three
+    calls do: the message holds the weights as they were."""
+    from paper_2609_04609_b200 import runtime
+
+    codec = runtime.LayerCodec.from_tensors(SIZES + [8192 * 4000], 1, NAME[dtype], block, DEV)
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(17 * block + dtype)
+    w0 = wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)
+    bits = [wl.as_bits(x) for x in (w0, wl.step_clustered(w0, gen, f=0.3))]
+    n = codec.weights_bytes
+    room = torch.zeros(n + (25 << 20), dtype=torch.uint8, device=DEV)
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    w = room[1 << 17 :][:n]
+    w.copy_(torch.from_numpy(bits[1].view(np.uint8)))
+    if where == "sent message":
+        codec.weights_out = codec.msg_send[:n]
+    else:
+        at = {"weights - 64 KB": -(1 << 16), "weights + 16": 16, "weights + 24 MB": 24 << 20}[where]
+        codec.weights_out = room[(1 << 17) + at :][:n]
+    exp = table.step(bits[1])
+    codec.step(w)
+    torch.cuda.synchronize()
+    codec.check_status()
+    if where == "sent message":
+        codec.msg_send = codec.msg_recv  # (what was sent is gone; what arrived is compared twice)
+    compare_step(codec, exp, bits[1], where)
+    compare_caches(codec, table, where)
+    compare_recon(codec, exp, bits[1], dtype, where)
