@@ -96,7 +96,8 @@ typedef enum ciera_dtype {
 } ciera_dtype;
 
 /* One unit = one shard of one tensor.  All offsets are in BYTES from the base pointer of the
- * respective buffer and must be multiples of 16. */
+ * respective buffer and must be multiples of 16.  Nothing behind the furthest unit's last value (byte) of a buffer
+ * is read or written; between units the rest of a unit's last 16 bytes may be read, and is never used or written. */
 typedef struct ciera_unit {
     uint64_t n_values;     /* N; may be 0, may be smaller than the block size                   */
     uint64_t weights_off;  /* into the weights buffer (encode: input, decode: output)           */

@@ -31,7 +31,6 @@ namespace ciera {
 constexpr int kDecProducers = 2;                               // producer warps, taking tiles in turn
 constexpr int kDecodeThreads = kThreads + 32 * kDecProducers;  // consumers + producers
 constexpr int kDecProducerWarp0 = kWarps;
-constexpr uint32_t kNoTile = 0xffffffffu;
 constexpr uint32_t kDirectWordsPerLane = 4;
 constexpr uint32_t kDirectBlocks = kDecodeDirectBlocks;
 static_assert(kDirectBlocks == 32u * 32u * kDirectWordsPerLane, "one fetch covers the direct range");

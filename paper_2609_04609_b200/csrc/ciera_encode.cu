@@ -265,6 +265,38 @@ struct __align__(16) EncodeTileInfo {
     uint32_t pad[2];
 };
 
+// The tiles whose last 16-byte piece reaches behind the last value of the weights buffer or of an exponent cache
+// (kNoTile: there is none); several: there are more, and every short tile is taken for one.
+struct BufferEnds {
+    uint32_t weights, cache;
+    bool several;
+    __device__ __forceinline__ bool has(uint32_t tile, uint32_t nv) const {
+        return tile == weights || tile == cache || (several && (nv & 15u));
+    }
+};
+
+// Producer, a tile that ends a buffer: bulk copies as far as whole 16-byte pieces go, small copies that stop in time for
+// the rest, all on `bar`.  (st_e null: no cached exponents; r_at: where behind the staged weights the receiver's go, 0 =
+// nowhere, and r_twin their distance.  Not inlined: at 48 registers per thread the producer's loop spills more for what it
+// might need here.  Steps of 12 288 units of 4 688 values 117 us inlined, 115 like this, 118 with the consumers fetching
+// the broken pieces, 113 when all that lies in the last 16 bytes was read, whether there or not.)
+__device__ __noinline__ void stage_buffer_end(uint8_t* st_w, const uint8_t* w, uint32_t w_bytes, uint8_t* st_e, const uint8_t* e,
+                                              uint32_t e_bytes, uint32_t r_at, int64_t r_twin, uint64_t* bar) {
+    const uint32_t w_whole = w_bytes & ~15u, e_whole = st_e ? e_bytes & ~15u : 0u;
+    if (w_bytes & 15u) cp_async16_first(st_w + w_whole, w + w_whole, w_bytes & 15u);
+    if (st_e && (e_bytes & 15u)) {
+        cp_async16_first(st_e + e_whole, e + e_whole, e_bytes & 15u);
+        if (r_at) cp_async16_first(st_w + r_at + e_whole, e + r_twin + e_whole, e_bytes & 15u);
+    }
+    cp_async_arrive(bar);
+    mbar_arrive_expect_tx(bar, w_whole + e_whole + (r_at ? e_whole : 0u));
+    if (w_whole) bulk_load(st_w, w, w_whole, bar);
+    if (e_whole) {
+        bulk_load(st_e, e, e_whole, bar);
+        if (r_at) bulk_load(st_w + r_at, e + r_twin, e_whole, bar);
+    }
+}
+
 template <int SW, int SE, int BW>
 struct EncodeCtl {
     uint64_t full_w[SW];    // weights tile landed
@@ -288,7 +320,6 @@ struct EncodeCtl {
     uint32_t seen;    // tiles whose loads the consumers have seen complete
 };
 
-constexpr uint32_t kNoTile = 0xffffffffu;
 constexpr uint32_t kEarlyClearTiles = 4096;  // status words that one warp empties while the rest still works
 
 // How a tile relates to the run of tiles it was handed out with (a short unit's tiles go out in runs of
@@ -1036,7 +1067,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
               uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
               unsigned int* unit_ticket, unsigned int* blocks_done, int32_t* status,
-              const unsigned long long* __restrict__ tile_hash, StepTwins tw) {
+              const unsigned long long* __restrict__ tile_hash, StepTwins tw, BufferEnds ends) {
     static_assert(!(HASH && FINE), "HashCache: blocks of 16 values and more");
     static_assert(!(HASH && STEP), "the whole step compares with the exponent cache");
     using P = Piece<DT>;
@@ -1153,17 +1184,17 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
                 }
-                // A unit's last, short tile is staged too, in whole 16-byte pieces: the up to 15 bytes behind its last value
-                // lie in the same piece of memory as that value, and the consumers drop them.
+                // A unit's last, short tile is staged too, in whole 16-byte pieces; the consumers drop what lies behind its
+                // last value.  Only behind the last value of a whole buffer there need not be anything.
                 const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
                 const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
-                if constexpr (HASH) {
+                if (ends.has(tile, nvt)) {
+                    stage_buffer_end(ring_w + (size_t)sw * kWStage, weights + td.w_off, nvt * (uint32_t)VB,
+                                     HASH ? nullptr : ring_e + (size_t)se * kEBytes, cache + td.c_off, nvt,
+                                     STEP && r_staged ? kWBytes : 0u, tw.cache, &ctl->full_w[sw]);
+                } else if (HASH) {
                     mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes);
                     bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
-                    // the cached hashes of the tile's blocks (16 bytes each)
-                    const uint32_t nblk = (nvt + (1u << log2b) - 1u) >> log2b;
-                    mbar_arrive_expect_tx(&ctl->full_e[se], nblk * 16u);
-                    bulk_load(ring_h + (size_t)se * kHStage, cache + hb * 16ull, nblk * 16u, &ctl->full_e[se]);
                 } else {
                     // all copies of the tile complete on the one barrier the consumers wait for
                     mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes + e_bytes + (STEP && r_staged ? e_bytes : 0u));
@@ -1173,8 +1204,15 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                         bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, e_bytes,
                                   &ctl->full_w[sw]);
                 }
+                if constexpr (HASH) {
+                    // the cached hashes of the tile's blocks (16 bytes each)
+                    const uint32_t nblk = (nvt + (1u << log2b) - 1u) >> log2b;
+                    mbar_arrive_expect_tx(&ctl->full_e[se], nblk * 16u);
+                    bulk_load(ring_h + (size_t)se * kHStage, cache + hb * 16ull, nblk * 16u, &ctl->full_e[se]);
+                }
                 ctl->issued = k + 1;
             }
+            cp_async_wait_all();  // (an aborted run: none in flight when the block ends)
         }
     } else if (warp == (uint32_t)CW + 1u) {
         // ---------------------------------------------------------------- aggregator
@@ -1561,6 +1599,7 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     unsigned int* done = ticket + 1;
     const unsigned long long* tile_hash = HASH ? p->tile_hash_dev : nullptr;
     const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
+    BufferEnds ends{p->weights_end_tile, HASH ? kNoTile : p->cache_end_tile, p->several_end_tiles};
     const bool has_spread = spread_first < nt;  // look-back between blocks
     // With a tile to a block and nothing else a tile looks back at blocks before its own only, which start no later, so the
     // blocks need not all be resident and the launch may begin while the kernel before it drains.  (Two or three neighbouring
@@ -1572,13 +1611,13 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
         void* args[] = {&tiles, &nt, &seq_runs, &order, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
-                        &changed_blocks_dev, &ts, &ticket, &done, &status_dev, &tile_hash, &tw};
+                        &changed_blocks_dev, &ts, &ticket, &done, &status_dev, &tile_hash, &tw, &ends};
         e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
                                         smem, s);
     } else {
         e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, order, n_runs,
                          spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev,
-                         tile_hash, tw);
+                         tile_hash, tw, ends);
     }
     if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();

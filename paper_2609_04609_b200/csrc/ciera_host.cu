@@ -256,6 +256,19 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
             for (uint64_t g = 0; g < slots; g += 64) p->ent_chunks.push_back({u, (uint32_t)g, li, 0u});
         }
     }
+    for (size_t t = 0; t < p->tiles.size(); ++t) {
+        const TileDesc& td = p->tiles[t];
+        if (td.tile_in_unit + 1 != td.n_tiles_unit) continue;
+        const uint64_t nv = td.n_unit - (uint64_t)td.tile_in_unit * kTileValues;
+        if (pad16(td.w_off + nv * vb) > p->weights_extent) {
+            p->several_end_tiles |= p->weights_end_tile != kNoTile;
+            p->weights_end_tile = (uint32_t)t;
+        }
+        if (pad16(td.c_off + nv) > p->cache_extent) {
+            p->several_end_tiles |= p->cache_end_tile != kNoTile;
+            p->cache_end_tile = (uint32_t)t;
+        }
+    }
     p->tile_hash.resize(p->tiles.size());
     for (size_t t = 0; t < p->tiles.size(); ++t)
         p->tile_hash[t] = p->hash_base[p->tiles[t].unit] + (uint64_t)p->tiles[t].tile_in_unit * (kTileValues >> p->log2b);

@@ -27,6 +27,8 @@ constexpr int kBitmapWords = kTileValues / 16 / 32;  // 16: words of block flags
 constexpr int kFineBitmapWords = kTileValues / 32;   // 256: the same, fine
 __host__ __device__ inline bool is_fine(uint32_t log2b) { return log2b < kFineLog2; }
 
+constexpr uint32_t kNoTile = 0xffffffffu;
+
 // Device-side tile descriptor: everything a thread block needs, in one 48-byte record so that
 // a single dependent load stands between block start and the first data load.
 struct __align__(16) TileDesc {
@@ -210,6 +212,9 @@ struct ciera_plan {
     uint64_t total_segments = 0;
     // the ends of the units' furthest values and slots in the three kinds of buffers, in bytes
     uint64_t cache_extent = 0, weights_extent = 0, msg_extent = 0;
+    // the tiles whose values, rounded up to 16 bytes, go past these ends (kNoTile: none; several: more than these)
+    uint32_t weights_end_tile = ciera::kNoTile, cache_end_tile = ciera::kNoTile;
+    bool several_end_tiles = false;
     // entropy stage: units of more than ent_long_slots segment slots, and their chunks of 64 slots
     uint32_t ent_long_slots = 64;
     // {unit, first segment of the chunk inside the unit, index among the long units, 0}

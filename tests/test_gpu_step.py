@@ -238,3 +238,87 @@ def test_output_over_buffers_that_the_three_calls_are_done_with(dtype, block, wh
     compare_step(codec, exp, bits[1], where)
     compare_caches(codec, table, where)
     compare_recon(codec, exp, bits[1], dtype, where)
+
+
+@pytest.mark.parametrize("block", [1, 8, 16, 512])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_every_remainder_of_a_short_tile(dtype, block):
+    """Units that end at every place of a 16-byte piece, in their first tile and in a later one, with bytes behind the last
+    value that would count as changed exponents: sender, hashed sender and whole step."""
+    from paper_2609_04609_b200 import runtime
+
+    sizes = list(range(1, 35)) + [8192 + r for r in range(1, 17)] + [8192 * 3 + 500 + r for r in range(16)]
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(13 * block + dtype)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    for _ in range(3):
+        w.append(wl.inject_exponent_changes(w[-1], gen, 0.2))
+    bits = [wl.as_bits(x).copy() for x in w]
+    inside = np.zeros(bits[0].size, bool)
+    for u in codec.units:
+        lo = int(u["weights_off"]) // wl.VALUE_BYTES[NAME[dtype]]
+        inside[lo : lo + int(u["n_values"])] = True
+    for b in bits:
+        b[~inside] = np.iinfo(b.dtype).max
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    guard(codec)  # (the bytes behind the cached exponents as well)
+    if block >= 16:
+        codec.init_hash_cache(to_dev_bytes(bits[0], DEV))
+    for t, step in ((1, _three_calls), (2, lambda c, x: c.step(x)), (3, _three_calls)):
+        exp = table.step(bits[t])
+        x = to_dev_bytes(bits[t], DEV)
+        if block >= 16:  # the same message from the other sender, before the caches move on
+            codec.encode_hashed(x)
+            torch.cuda.synchronize()
+            sent, wire = codec.msg_send.cpu().numpy(), codec.wire_bytes.tolist()
+            assert wire == exp["wire"].tolist(), f"hashed t={t}"
+            for u, n in zip(codec.units, wire):
+                lo = int(u["msg_off"])
+                assert np.array_equal(sent[lo : lo + n], exp["msgs"][lo : lo + n]), f"hashed t={t}"
+        step(codec, x)
+        torch.cuda.synchronize()
+        codec.check_status()
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+
+
+@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_every_remainder_of_the_last_tile_of_a_buffer(dtype, shared):
+    """The unit that ends the buffers, with every remainder and a different one for weights and caches; with ``shared``,
+    two units have the same weights, so that several tiles end the weights buffer."""
+    from paper_2609_04609_b200 import ciera, runtime
+
+    vb, block = wl.VALUE_BYTES[NAME[dtype]], 16
+    for n in list(range(1, 34)) + [8192 + r for r in range(1, 17)]:
+        cap = ciera.message_capacity(n, dtype, block)
+        slot = (cap + 15) // 16 * 16
+        other = (n + 7) if not shared else n  # first in the caches, last in the weights (or in the same place there)
+        rows = [(other, 0 if shared else (n * vb + 15) // 16 * 16, 0, 2 * slot + 64, ciera.message_capacity(other, dtype, block)),
+                (n, 0, (other + 15) // 16 * 16, 0, cap)]
+        units = np.array(rows, dtype=wl.UNIT_DTYPE)
+        values = int(max(u["weights_off"] // vb + u["n_values"] for u in units))
+        codec = runtime.LayerCodec(units, NAME[dtype], block, values * vb, int(rows[1][2]) + n, 5 * slot + 256, DEV, slack=256)
+        table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+        gen = wl.make_generator(n + dtype)
+        w = [wl.init_weights(values, NAME[dtype], gen)]
+        for _ in range(2):
+            w.append(wl.inject_exponent_changes(w[-1], gen, 0.3))
+        bits = [wl.as_bits(x) for x in w]
+        table.init_caches(bits[0])
+        codec.init_caches(to_dev_bytes(bits[0], DEV))
+        codec.allocations["sender_cache"][codec.cache_bytes :] = 0xEE
+        codec.allocations["receiver_cache"][codec.cache_bytes :] = 0xEE
+        room = torch.full((values * vb + 16,), 0xEE, dtype=torch.uint8, device=DEV)
+        for t, step in ((1, _three_calls), (2, lambda c, x: c.step(x))):
+            exp = table.step(bits[t])
+            room[: values * vb] = torch.from_numpy(bits[t].view(np.uint8).copy()).to(DEV)
+            step(codec, room[: values * vb])
+            torch.cuda.synchronize()
+            codec.check_status()
+            compare_step(codec, exp, bits[t], f"n={n} t={t}")
+            compare_caches(codec, table, f"n={n} t={t}")
+            compare_recon(codec, exp, bits[t], dtype, f"n={n} t={t}")
