@@ -334,6 +334,7 @@ constexpr uint32_t kSeqTile = 1u, kSeqRunStart = 2u, kSeqRunEnd = 4u;
 // back to zero for the next launch.  The walk keeps two runs in hand besides the current one: the number of
 // the run after next (its draw is on its way) and the table entry of the next run (its load is on its way), so
 // that at the start of a run neither the counter nor the table is waited for.
+template <bool ORDERED>  // the spread tiles may be given by their places in a list (steps in parts)
 struct TileWalk {
     const uint2* seq_runs;
     const uint32_t* order;  // not null: the spread tiles are given by their places in this list
@@ -365,7 +366,7 @@ struct TileWalk {
         if (spread) {
             if (spread_tile < n_tiles) {
                 seq = 0;
-                const uint32_t t = order ? __ldg(order + spread_tile) : spread_tile;
+                const uint32_t t = ORDERED && order ? __ldg(order + spread_tile) : spread_tile;
                 spread_tile += G;
                 return t;
             }
@@ -1132,7 +1133,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     if (warp == (uint32_t)CW) {
         // ---------------------------------------------------------------- producer
         if (lane == 0) {
-            TileWalk walk(seq_runs, order, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
+            TileWalk<STEP> walk(seq_runs, order, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
             uint32_t tile_nxt = walk.next(seq_nxt);
             TileDesc nxt;
