@@ -100,6 +100,7 @@ struct __align__(16) DecodeRing {
     uint32_t nv;                             // values in the tile
     uint32_t tile;                           // the tile's number, or kNoTile: this producer has no more work
     uint32_t pay_skew;                       // fine: bytes in front of the slice in its stage (0 .. 15)
+    uint32_t ws;                             // count from the scratch (units of one segment)
     uint32_t direct;                         // coarse: 1 = the few unchanged pieces read their cached exponents from global memory
     uint16_t pre[kBm];                       // set flags before each word
     // raw material of coarse blocks, fetched asynchronously one tile ahead:
@@ -110,9 +111,13 @@ struct __align__(16) DecodeRing {
 static_assert(offsetof(DecodeRing<true>, bm) % 16 == 0 && offsetof(DecodeRing<true>, pre) % 4 == 0,
               "with blocks of one value the flags are digested 16 bytes at a time");
 
-// Units that went through the prefix kernel: the scratch holds, for every tile, the changed blocks of its segment up
+// Units that went through the prefix kernel.  SEGMENTED: the scratch holds, for every tile, the changed blocks of its segment up
 // to and with the tile.  Before tile j there are those of tile j - 1 (unless j starts its segment) and the last count
-// of every earlier segment: one word per lane, fetched into `words` and added up later.
+// of every earlier segment: one word per lane, fetched into `words` and added up later.  Otherwise every such unit of
+// the table is one segment (fine blocks: up to 16 tiles, as in layers cut into many shards), and the scratch holds the
+// count before each tile: one word.  With fine blocks the producers set the kernel's pace, so that case has an instance
+// of its own: receiver of an OLMoE-shaped fp32 layer in blocks of one value 613 us, 633 with SEGMENTED, 627 with both
+// ways in one instance.
 __device__ __forceinline__ bool prefix_lane(const TileDesc& td, bool fine, uint32_t lane, uint32_t& at) {
     const uint32_t seg = prefix_segment(td.n_tiles_unit, fine), j = td.tile_in_unit;
     at = min((lane + 1u) * seg, j) - 1u;
@@ -132,8 +137,8 @@ struct DecodeCtl {
 // Starts the asynchronous fetch of the bitmap words a producer needs for one tile into the ring
 // slot `r`: the unit's words before the tile (direct units) or the tile's count from the scratch
 // (long units), and the tile's own words.  Nothing is held in registers meanwhile.
-template <bool FINE>
-__device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t log2b, const uint8_t* msgs,
+template <bool FINE, bool SEGMENTED>
+__device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t tile, uint32_t log2b, const uint8_t* msgs,
                                              const uint32_t* ws_prefix, DecodeRing<FINE>* r, uint32_t lane) {
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td.msg_off);
     const uint64_t kb0 = ((uint64_t)td.tile_in_unit * kTileValues) >> log2b;  // first block of the tile
@@ -144,8 +149,12 @@ __device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t log2b,
         // 128 to 1024 bytes that start on a 128-byte boundary of the slot: 16 bytes per copy,
         // never past the bitmap's padded end
         // (the counts go to where the counts before each word will be)
-        uint32_t at;
-        if (prefix_lane(td, true, lane, at)) cp_async4(reinterpret_cast<uint32_t*>(r->pre) + lane, ws_prefix + td.first_tile + at);
+        if constexpr (SEGMENTED) {
+            uint32_t at;
+            if (prefix_lane(td, true, lane, at)) cp_async4(reinterpret_cast<uint32_t*>(r->pre) + lane, ws_prefix + td.first_tile + at);
+        } else {
+            if (td.tile_in_unit != 0 && lane == 0) cp_async4(&r->ws, ws_prefix + tile);
+        }
         const uint32_t chunks = nbt >> 7;  // 8 .. 64 copies of four words
         for (uint32_t c = lane; c < chunks; c += 32) {
             const uint64_t w = (kb0 >> 5) + 4ull * c;
@@ -174,7 +183,7 @@ __device__ __forceinline__ void fetch_bitmap(const TileDesc& td, uint32_t log2b,
 
 // Turns a completed fetch into the tile's block flags (r->bm, r->pre).  Returns the number of
 // changed blocks before the tile; `own_total` gets the number of changed blocks of the tile.
-template <bool FINE>
+template <bool FINE, bool SEGMENTED>
 __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const TileDesc& td, uint32_t log2b, uint32_t lane,
                                                   uint32_t& own_total) {
     const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
@@ -184,7 +193,7 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
     const uint32_t nv = (uint32_t)min((uint64_t)kTileValues, td.n_unit - v0);
     const uint32_t nblk = (nv + (1u << log2b) - 1u) >> log2b;  // valid blocks of this tile
     uint32_t cnt = 0;
-    if (FINE || nb > kDirectBlocks) {
+    if (SEGMENTED && (FINE || nb > kDirectBlocks)) {
         uint32_t at;
         if (prefix_lane(td, FINE, lane, at)) cnt = FINE ? reinterpret_cast<const uint32_t*>(r->pre)[lane] : r->raw_pre[lane];
         cnt = __reduce_add_sync(0xffffffffu, cnt);
@@ -221,7 +230,7 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
         for (int i = 0; i < 4; ++i) pre32[i] = (base + before8[2 * i]) | ((base + before8[2 * i + 1]) << 16);
         own_total = __shfl_sync(0xffffffffu, incl, 31);
         __syncwarp();
-        return cnt;
+        return SEGMENTED ? cnt : td.tile_in_unit != 0 ? r->ws : 0u;
     }
     if (FINE) {
         // flags past the tile's last block are dropped (words past the bitmap's end were not fetched)
@@ -247,7 +256,7 @@ __device__ __forceinline__ uint64_t digest_bitmap(DecodeRing<FINE>* r, const Til
         }
         own_total = run;
         __syncwarp();
-        return cnt;
+        return SEGMENTED ? cnt : td.tile_in_unit != 0 ? r->ws : 0u;
     }
     if (nb <= kDirectBlocks) {
         const uint32_t nfull = (uint32_t)(kb0 >> 5);
@@ -427,7 +436,7 @@ __host__ __device__ constexpr uint32_t decode_stage_bytes() {
            ((FINE || DT == CIERA_FP16) ? 16u : 0u);
 }
 
-template <int DT, bool FINE>
+template <int DT, bool FINE, bool SEGMENTED>
 __global__ void __launch_bounds__(kDecodeThreads, DecodeCfg<DT, FINE>::kBlocksPerSM)
 decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log2b, const uint8_t* msgs, uint8_t* cache,
               uint8_t* __restrict__ weights, const unsigned long long* __restrict__ wire_bytes,
@@ -498,7 +507,7 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
         cp_async_wait<1>();  // D_0
         __syncwarp();
         if (t_cur != kNoTile)
-            fetch_bitmap(ctl->ring[seq(0) % kDecRing].desc, log2b, msgs, ws_prefix, &ctl->ring[seq(0) % kDecRing], lane);
+            fetch_bitmap<FINE, SEGMENTED>(ctl->ring[seq(0) % kDecRing].desc, t_cur, log2b, msgs, ws_prefix, &ctl->ring[seq(0) % kDecRing], lane);
         cp_async_commit();
         for (uint32_t jj = 0;; ++jj) {
             const uint32_t k = seq(jj);
@@ -518,14 +527,14 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
             __syncwarp();
             if (t_nxt != kNoTile) {
                 Ring* rn = &ctl->ring[seq(jj + 1u) % kDecRing];
-                fetch_bitmap(rn->desc, log2b, msgs, ws_prefix, rn, lane);
+                fetch_bitmap<FINE, SEGMENTED>(rn->desc, t_nxt, log2b, msgs, ws_prefix, rn, lane);
             }
             cp_async_commit();
 
             Ring* r = &ctl->ring[k % kDecRing];
             const TileDesc td = r->desc;
             uint32_t own = 0;
-            const uint64_t before = digest_bitmap(r, td, log2b, lane, own);
+            const uint64_t before = digest_bitmap<FINE, SEGMENTED>(r, td, log2b, lane, own);
             const uint64_t N = td.n_unit;
             const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
             const uint64_t smoff = sm_offset(N, log2b);
@@ -822,8 +831,6 @@ decode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, uint32_t log
 // such a unit, a running count over the segment's tiles in chunks of 256.  One thread block per unit left the GPU idle
 // in tables of few units; receiver of 3 x 12 489 655 fp16 values on 4 shards, 2 per block: 122 -> 53 us; 3 x 14 885 525
 // bf16 on 2, 16 per block: 46 -> 39; one unit of 10^8, 32 per block: 143 -> 75; of 2 x 10^8, 512 per block: 207 -> 136.
-// (Tables of many short units pay for the fetch by all lanes: OLMoE-shaped layer, 1 value per block, bf16 322 -> 329 us,
-// fp16 462 -> 490.)
 __global__ void __launch_bounds__(256)
 decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ segments, uint32_t log2b,
                      const uint8_t* __restrict__ msgs, uint32_t* __restrict__ ws_prefix) {
@@ -879,6 +886,7 @@ decode_prefix_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restr
 // The same for fine blocks, where every unit of more than one tile comes here and a tile has 32 to
 // 256 words of flags: the warps take the unit's tiles in turn and each counts a tile's flags with
 // all its lanes (consecutive words, coalesced), then the counts are scanned as above.
+template <bool SEGMENTED>  // (see prefix_lane)
 __global__ void __launch_bounds__(256)
 decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __restrict__ segments,
                           uint32_t log2b, const uint8_t* __restrict__ msgs, uint32_t* __restrict__ ws_prefix) {
@@ -887,8 +895,8 @@ decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __
     __shared__ uint32_t s_carry;
     pdl_wait();
     const TileDesc td0 = load_tile_desc(tiles + segments[blockIdx.x]);
-    const uint32_t first = td0.first_tile, j_begin = td0.tile_in_unit;
-    const uint32_t j_end = min(j_begin + prefix_segment(td0.n_tiles_unit, true), td0.n_tiles_unit);
+    const uint32_t first = td0.first_tile, j_begin = SEGMENTED ? td0.tile_in_unit : 0u;
+    const uint32_t j_end = SEGMENTED ? min(j_begin + prefix_segment(td0.n_tiles_unit, true), td0.n_tiles_unit) : td0.n_tiles_unit;
     const uint32_t* bm32 = reinterpret_cast<const uint32_t*>(msgs + td0.msg_off);
     const uint64_t nb = num_blocks(td0.n_unit, log2b);
     const uint32_t words = kTileValues >> (log2b + 5);  // words of flags per tile
@@ -924,7 +932,7 @@ decode_prefix_fine_kernel(const TileDesc* __restrict__ tiles, const uint32_t* __
         uint32_t wbase = 0;
         for (uint32_t w = 0; w < warp; ++w) wbase += s_warp[w];
         const uint32_t carry = s_carry;
-        if (j < j_end) ws_prefix[first + j] = carry + wbase + incl;
+        if (j < j_end) ws_prefix[first + j] = carry + wbase + incl - (SEGMENTED ? 0u : cnt);
         __syncthreads();
         if (tid == 255) s_carry = carry + wbase + incl;
         __syncthreads();
@@ -940,7 +948,7 @@ static size_t decode_smem_bytes() {
     return (size_t)S * stage + out + sizeof(DecodeCtl<S, Cfg::kRing, FINE>);
 }
 
-template <int DT, bool FINE>
+template <int DT, bool FINE, bool SEGMENTED>
 static int decode_grid_limit(int* out) {
     static std::atomic<int> cached[64];  // (zero-initialised; any host thread may be the first to fill an entry)
     int dev = 0;
@@ -949,10 +957,10 @@ static int decode_grid_limit(int* out) {
     if (dev < 0 || dev >= 64) return CIERA_ERR_UNSUPPORTED;
     if (cached[dev].load(std::memory_order_acquire) == 0) {
         const size_t smem = decode_smem_bytes<DT, FINE>();
-        e = cudaFuncSetAttribute(decode_kernel<DT, FINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(decode_kernel<DT, FINE, SEGMENTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return record_cuda_error(e);
         int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_kernel<DT, FINE>, kDecodeThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, decode_kernel<DT, FINE, SEGMENTED>, kDecodeThreads, smem);
         if (e != cudaSuccess) return record_cuda_error(e);
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return record_cuda_error(e);
@@ -963,21 +971,30 @@ static int decode_grid_limit(int* out) {
     return CIERA_OK;
 }
 
-template <int DT, bool FINE>
+template <int DT, bool FINE, bool SEGMENTED>
 static int launch_decode(const ciera_plan* p, const void* messages_dev, void* receiver_cache_dev, void* weights_out_dev,
                          const uint64_t* wire_bytes_dev, const uint32_t* ws_prefix, unsigned int* ticket, int32_t* status_dev,
                          cudaStream_t s) {
     int limit = 0;
-    const int rc = decode_grid_limit<DT, FINE>(&limit);
+    const int rc = decode_grid_limit<DT, FINE, SEGMENTED>(&limit);
     if (rc) return rc;
     const uint32_t nt = (uint32_t)p->tiles.size();
     const uint32_t grid = nt < (uint32_t)limit ? nt : (uint32_t)limit;
     const cudaError_t e = launch_after(
-        decode_kernel<DT, FINE>, dim3(grid), kDecodeThreads, decode_smem_bytes<DT, FINE>(), s, p->tiles_dev, nt, p->log2b, (const uint8_t*)messages_dev, (uint8_t*)receiver_cache_dev, (uint8_t*)weights_out_dev,
+        decode_kernel<DT, FINE, SEGMENTED>, dim3(grid), kDecodeThreads, decode_smem_bytes<DT, FINE>(), s, p->tiles_dev, nt, p->log2b, (const uint8_t*)messages_dev, (uint8_t*)receiver_cache_dev, (uint8_t*)weights_out_dev,
         (const unsigned long long*)wire_bytes_dev, ws_prefix, ticket, status_dev);
     if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
     return CIERA_OK;
+}
+
+// picks the kernel for the plan's block class
+template <int DT>
+static int launch_decode_of(const ciera_plan* p, const void* messages_dev, void* receiver_cache_dev, void* weights_out_dev,
+                            const uint64_t* wire_bytes_dev, const uint32_t* ws_prefix, unsigned int* ticket, int32_t* status_dev,
+                            cudaStream_t s) {
+    auto* launch = !is_fine(p->log2b) ? launch_decode<DT, false, true> : p->prefix_segmented ? launch_decode<DT, true, true> : launch_decode<DT, true, false>;
+    return launch(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev, ws_prefix, ticket, status_dev, s);
 }
 
 }  // namespace ciera
@@ -1005,24 +1022,11 @@ extern "C" int ciera_decode(const ciera_plan* p, const void* messages_dev, void*
     const uint32_t n_segments = (uint32_t)p->prefix_segments.size();
     if (n_segments) {
         const cudaError_t e =
-            launch_after(is_fine(p->log2b) ? decode_prefix_fine_kernel : decode_prefix_kernel, dim3(n_segments), 256, 0, s, p->tiles_dev,
+            launch_after(!is_fine(p->log2b) ? decode_prefix_kernel : p->prefix_segmented ? decode_prefix_fine_kernel<true> : decode_prefix_fine_kernel<false>, dim3(n_segments), 256, 0, s, p->tiles_dev,
                          p->prefix_segments_dev, p->log2b, (const uint8_t*)messages_dev, ws_prefix);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }
-    const bool fine = is_fine(p->log2b);
-    if (p->dtype == CIERA_FP16)
-        return fine ? launch_decode<CIERA_FP16, true>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                      ws_prefix, ticket, status_dev, s)
-                    : launch_decode<CIERA_FP16, false>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                       ws_prefix, ticket, status_dev, s);
-    if (p->dtype == CIERA_BF16)
-        return fine ? launch_decode<CIERA_BF16, true>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                      ws_prefix, ticket, status_dev, s)
-                    : launch_decode<CIERA_BF16, false>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                       ws_prefix, ticket, status_dev, s);
-    return fine ? launch_decode<CIERA_FP32, true>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                  ws_prefix, ticket, status_dev, s)
-                : launch_decode<CIERA_FP32, false>(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev,
-                                                   ws_prefix, ticket, status_dev, s);
+    auto* launch = p->dtype == CIERA_FP16 ? launch_decode_of<CIERA_FP16> : p->dtype == CIERA_BF16 ? launch_decode_of<CIERA_BF16> : launch_decode_of<CIERA_FP32>;
+    return launch(p, messages_dev, receiver_cache_dev, weights_out_dev, wire_bytes_dev, ws_prefix, ticket, status_dev, s);
 }

@@ -157,7 +157,10 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         }
         const bool needs_prefix = is_fine(p->log2b) ? nt > 1 : (un.n_values + block - 1) / block > kDecodeDirectBlocks;
         if (needs_prefix)
-            for (uint32_t j = 0; j < nt; j += prefix_segment(nt, is_fine(p->log2b))) p->prefix_segments.push_back(first + j);
+            for (uint32_t j = 0; j < nt; j += prefix_segment(nt, is_fine(p->log2b))) {
+                p->prefix_segments.push_back(first + j);
+                p->prefix_segmented |= j != 0;
+            }
     };
     for (uint32_t u : shorts) {
         p->seq_first.push_back((uint32_t)p->tiles.size());

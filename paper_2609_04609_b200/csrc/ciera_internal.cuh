@@ -194,6 +194,7 @@ struct ciera_plan {
     std::vector<ciera_unit> units;
     std::vector<ciera::TileDesc> tiles;
     std::vector<uint32_t> prefix_segments;  // first tiles of the segments of every unit whose decode needs the prefix kernel
+    bool prefix_segmented = false;          // one of these units has several segments
     std::vector<uint32_t> seq_first;   // first tile of every short unit, in table order, + end marker
     struct SeqRun {
         uint32_t lo, hi;               // tiles [lo, hi) of the table
