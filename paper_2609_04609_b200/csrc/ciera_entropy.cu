@@ -1106,7 +1106,7 @@ extern "C" int ciera_entropy_encode(const ciera_plan* p, void* messages_dev, uin
         const bool wide = wide_units(p->n_units - n_long);
         auto* k = dt == CIERA_FP16 ? (wide ? entropy_encode_kernel<true, kEntWide> : entropy_encode_kernel<true, kEntThreads>)
                                    : (wide ? entropy_encode_kernel<false, kEntWide> : entropy_encode_kernel<false, kEntThreads>);
-        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev,
+        e = launch_when(wide, k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev,
                          p->ent_long_slots, dt, p->log2b, msgs, wire, slots, nw, sym);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
@@ -1159,7 +1159,7 @@ extern "C" int ciera_entropy_decode(const ciera_plan* p, void* messages_dev, uin
                                    : (wide  ? entropy_decode_kernel<false, kEntWide, 1>
                                       : few ? entropy_decode_kernel<false, kEntThreads, 5>
                                             : entropy_decode_kernel<false, kEntThreads, 8>);
-        e = launch_after(k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev,
+        e = launch_when(wide, k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev,
                          p->ent_long_slots, dt, p->log2b, msgs, wire, raw, status_dev);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();

@@ -257,8 +257,10 @@ void count_launch();                           // launch accounting
 // become resident as soon as there is room, set themselves up and wait in pdl_wait() -- which every thread of such a
 // kernel calls before it touches global memory -- until the kernel before has finished and its writes are visible.
 // Sender step of 64 tiles, back to back: 8.2 -> 6.3 us; no difference where the kernels are long.
+// (early false: an ordinary launch.  For grids of a few blocks per SM that do not balance themselves: begun while a
+// persistent kernel drains, they are packed onto the SMs that it leaves first.)
 template <class... P, class... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_when(bool early, void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, A&&... args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -268,8 +270,12 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, uint32_t threads, size
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, uint32_t threads, size_t smem, cudaStream_t s, A&&... args) {
+    return launch_when(true, kernel, grid, threads, smem, s, args...);
 }
 // (and lets the kernel behind it begin in turn)
 __device__ __forceinline__ void pdl_wait() {
