@@ -28,6 +28,8 @@
 // units go through a chain of launches whose grids run over chunks of 64 segments, so that their
 // work spreads over the GPU: sender = histogram, model, segments, layout, copy; receiver = layout,
 // segments, restore.  Nothing waits for another thread block anywhere.
+#include <type_traits>
+
 #include "ciera_bits.cuh"
 
 namespace ciera {
@@ -38,12 +40,14 @@ constexpr uint32_t kSegment = 4096;                              // bytes of raw
 constexpr uint32_t kSegWordsMax = kSegment * kProbBits / 16;     // 3072: a symbol adds at most 12 bits
 constexpr uint32_t kSegSlot = 4 * 32 + 2 * kSegWordsMax;         // 6272 bytes: states + words
 constexpr int kEntThreads = 256, kEntWarps = kEntThreads / 32;
-// A unit's thread block has kEntThreads threads where there are units enough to fill the GPU, else kEntWide: a segment
-// is a serial chain of 128 steps (about 8 us), and a block codes as many segments at a time as it has warps.  Four units of
-// 32 segments, sender's / receiver's stage: 66 / 92 us with 8 warps, 32 / 31 with 32; 192 units of 8 segments are better off
-// with 8 (both stages and the step: 79 us against 107).
-constexpr int kEntWide = 1024;
-constexpr uint32_t kLongSegs = 64;  // units with more segment slots than this take the chunked path
+// A unit's thread block has kEntThreads threads where there are units enough to fill the GPU, else kEntMiddle (two blocks
+// to an SM) or kEntWide (one), as long as all of them are resident at once: a segment is a serial chain of 128 steps
+// (about 8 us), and a block codes as many segments at a time as it has warps.  Sender's / receiver's stage, us: four units
+// of 32 segments 66 / 92 with 8 warps, 32 / 31 with 32; 160 units of 32 slots, 7 of them in use, 41 / 62 with 8 warps, 27 / 33
+// with 16 (cut into several blocks each: 42 / 54), all in use 100 / 127 and 64 / 65 (cut: 55 / 60); 288 units of 32 slots, 7
+// in use, 47 / 66 and 30 / 33.  Whole step with the stage, 192 units of 8 segments: 79 with 8 warps, 107 with 32.
+constexpr int kEntWide = 1024, kEntMiddle = 512;
+constexpr uint32_t kLongSegs = kEntLongSlots;  // units with more segment slots than this take the chunked path
 
 __host__ __device__ inline uint64_t segments_of(uint64_t bytes) { return (bytes + kSegment - 1) / kSegment; }
 __host__ __device__ inline uint32_t segment_bytes(uint32_t nw) { return 4u * 32u + 2u * nw + ((nw & 1u) ? 2u : 0u); }
@@ -473,12 +477,12 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* scan, uint3
 }
 
 // ------------------------------------------------------------------------------------------ sender
-// units of up to long_slots (at most kLongSegs) segment slots: one thread block per unit, start to end
+// units of up to kLongSegs segment slots: one thread block per unit, start to end
 
 template <bool HALF, int T>  // HALF: fp16, five-bit symbols (see the head of this file); T: threads of the block
-__global__ void __launch_bounds__(T, T == kEntWide ? 1 : 5)
+__global__ void __launch_bounds__(T, T == kEntWide ? 1 : T == kEntMiddle ? 2 : 5)
 entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long long* __restrict__ seg_base,
-                      uint32_t long_slots, int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
+                      int dt, uint32_t log2b, uint8_t* msgs, unsigned long long* wire_bytes,
                       uint8_t* scratch_slots, uint32_t* scratch_nw, uint8_t* scratch_sym) {
     __shared__ uint32_t s_hist[T / 32][256];  // the warps' private histograms, then the two small lists of step 4
     __shared__ uint16_t s_f[256];
@@ -488,7 +492,7 @@ entropy_encode_kernel(const ciera_unit* __restrict__ units, const unsigned long 
     pdl_wait();
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
-    if (un.n_values == 0 || segments_of(un.n_values) > long_slots) return;
+    if (un.n_values == 0 || segments_of(un.n_values) > kLongSegs) return;
     const uint64_t payoff = payload_offset_of(un.n_values, dt, log2b);
     const uint64_t Q = wire_bytes[unit] - payoff;
     // nothing to code; or a length that no sender step reports (shorter than the fixed sections, more
@@ -794,7 +798,7 @@ __device__ __forceinline__ void raise_corrupt(int32_t* status) {
 // more than 5, the 48 registers shorten the chain: 512 units 55 us against 70, 192 units 48 against 57)
 template <bool HALF, int T, int BLOCKS>
 __global__ void __launch_bounds__(T, BLOCKS)
-entropy_decode_kernel(const ciera_unit* __restrict__ units, uint32_t long_slots, int dt, uint32_t log2b, uint8_t* msgs,
+entropy_decode_kernel(const ciera_unit* __restrict__ units, int dt, uint32_t log2b, uint8_t* msgs,
                       unsigned long long* wire_bytes, uint8_t* scratch_raw, int32_t* status) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     DecodeShared& sh = *reinterpret_cast<DecodeShared*>(smem_raw);
@@ -802,7 +806,7 @@ entropy_decode_kernel(const ciera_unit* __restrict__ units, uint32_t long_slots,
     const uint32_t unit = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const ciera_unit un = units[unit];
     const uint64_t N = un.n_values;
-    if (N == 0 || segments_of(N) > long_slots) return;
+    if (N == 0 || segments_of(N) > kLongSegs) return;
     uint8_t* const msg = msgs + un.msg_off;
     const uint64_t payoff = payload_offset_of(N, dt, log2b);
     if (tid == 0) {
@@ -1060,7 +1064,7 @@ static int entropy_device(int* sms_out) {
     if (!cached[dev].load(std::memory_order_acquire)) {
         for (const void* k : {(const void*)entropy_decode_kernel<false, kEntThreads, 5>, (const void*)entropy_decode_kernel<true, kEntThreads, 5>,
                               (const void*)entropy_decode_kernel<false, kEntThreads, 8>, (const void*)entropy_decode_kernel<true, kEntThreads, 8>,
-                              (const void*)entropy_decode_kernel<false, kEntWide, 1>, (const void*)entropy_decode_kernel<true, kEntWide, 1>,
+                              (const void*)entropy_decode_kernel<false, kEntMiddle, 2>, (const void*)entropy_decode_kernel<true, kEntMiddle, 2>, (const void*)entropy_decode_kernel<false, kEntWide, 1>, (const void*)entropy_decode_kernel<true, kEntWide, 1>,
                               (const void*)entropy_long_decode_kernel<false>, (const void*)entropy_long_decode_kernel<true>}) {
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DecodeShared));
             if (e != cudaSuccess) return record_cuda_error(e);
@@ -1074,8 +1078,10 @@ static int entropy_device(int* sms_out) {
     *sms_out = cached[dev].load(std::memory_order_acquire);
     return CIERA_OK;
 }
-// wide blocks for the units as long as each has an SM to itself
-static bool wide_units(uint32_t units) { return units <= kEntWideUnits; }
+// threads of the blocks that code a unit each
+static int unit_threads(uint32_t units, int sms) {
+    return units <= (uint32_t)sms ? kEntWide : units <= 2u * (uint32_t)sms ? kEntMiddle : kEntThreads;
+}
 // thread blocks to a chunk of kLongSegs segments: enough for five on every SM, at least a segment for each of their warps
 static uint32_t chunk_parts(uint32_t chunks, int sms) {
     uint32_t parts = 1;
@@ -1103,11 +1109,15 @@ extern "C" int ciera_entropy_encode(const ciera_plan* p, void* messages_dev, uin
     if ((rc = entropy_device(&sms))) return rc;
     cudaError_t e = cudaSuccess;
     if (n_long < p->n_units) {
-        const bool wide = wide_units(p->n_units - n_long);
-        auto* k = dt == CIERA_FP16 ? (wide ? entropy_encode_kernel<true, kEntWide> : entropy_encode_kernel<true, kEntThreads>)
-                                   : (wide ? entropy_encode_kernel<false, kEntWide> : entropy_encode_kernel<false, kEntThreads>);
-        e = launch_when(wide, k, dim3(p->n_units), wide ? kEntWide : kEntThreads, 0, s, p->units_dev, p->seg_base_dev,
-                         p->ent_long_slots, dt, p->log2b, msgs, wire, slots, nw, sym);
+        const int threads = unit_threads(p->n_units - n_long, sms);
+        auto pick = [&](auto half) {
+            constexpr bool kHalf = decltype(half)::value;
+            return threads == kEntWide     ? entropy_encode_kernel<kHalf, kEntWide>
+                   : threads == kEntMiddle ? entropy_encode_kernel<kHalf, kEntMiddle>
+                                           : entropy_encode_kernel<kHalf, kEntThreads>;
+        };
+        e = launch_when(threads == kEntWide, dt == CIERA_FP16 ? pick(std::true_type{}) : pick(std::false_type{}), dim3(p->n_units),
+                        threads, 0, s, p->units_dev, p->seg_base_dev, dt, p->log2b, msgs, wire, slots, nw, sym);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }
@@ -1151,16 +1161,17 @@ extern "C" int ciera_entropy_decode(const ciera_plan* p, void* messages_dev, uin
     unsigned long long* wire = (unsigned long long*)wire_bytes_dev;
     const uint32_t n_long = (uint32_t)p->ent_long_units.size(), n_chunks = (uint32_t)p->ent_chunks.size();
     if (n_long < p->n_units) {
-        const bool wide = wide_units(p->n_units - n_long);
-        const bool few = p->n_units - n_long <= kEntFewUnits;
-        auto* k = dt == CIERA_FP16 ? (wide  ? entropy_decode_kernel<true, kEntWide, 1>
-                                      : few ? entropy_decode_kernel<true, kEntThreads, 5>
-                                            : entropy_decode_kernel<true, kEntThreads, 8>)
-                                   : (wide  ? entropy_decode_kernel<false, kEntWide, 1>
-                                      : few ? entropy_decode_kernel<false, kEntThreads, 5>
-                                            : entropy_decode_kernel<false, kEntThreads, 8>);
-        e = launch_when(wide, k, dim3(p->n_units), wide ? kEntWide : kEntThreads, sizeof(DecodeShared), s, p->units_dev,
-                         p->ent_long_slots, dt, p->log2b, msgs, wire, raw, status_dev);
+        const int threads = unit_threads(p->n_units - n_long, sms);
+        const bool few = p->n_units - n_long <= 5u * (uint32_t)sms;  // (see entropy_decode_kernel)
+        auto pick = [&](auto half) {
+            constexpr bool kHalf = decltype(half)::value;
+            return threads == kEntWide     ? entropy_decode_kernel<kHalf, kEntWide, 1>
+                   : threads == kEntMiddle ? entropy_decode_kernel<kHalf, kEntMiddle, 2>
+                   : few                   ? entropy_decode_kernel<kHalf, kEntThreads, 5>
+                                           : entropy_decode_kernel<kHalf, kEntThreads, 8>;
+        };
+        e = launch_when(threads == kEntWide, dt == CIERA_FP16 ? pick(std::true_type{}) : pick(std::false_type{}), dim3(p->n_units),
+                        threads, sizeof(DecodeShared), s, p->units_dev, dt, p->log2b, msgs, wire, raw, status_dev);
         if (e != cudaSuccess) return record_cuda_error(e);
         count_launch();
     }

@@ -231,14 +231,6 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     p->unit_first.assign(n_units, 0xffffffffu);
     for (size_t t = 0; t < p->tiles.size(); ++t)
         if (p->tiles[t].tile_in_unit == 0) p->unit_first[p->tiles[t].unit] = (uint32_t)t;
-    {
-        uint32_t units = 0;
-        for (uint32_t u = 0; u < n_units; ++u) {
-            const uint64_t slots = (units_host[u].n_values + 4095) / 4096;
-            units += slots != 0 && slots <= 64;
-        }
-        if (units > kEntWideUnits && units <= kEntSplitUnits) p->ent_long_slots = kEntSplitSlots;
-    }
     p->hash_base.resize(n_units);
     p->seg_base.resize(n_units);
     for (uint32_t u = 0; u < n_units; ++u) {
@@ -253,10 +245,10 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
             p->msg_extent = std::max<uint64_t>(p->msg_extent, units_host[u].msg_off + units_host[u].msg_capacity);
         }
         const uint64_t slots = (units_host[u].n_values + 4095) / 4096;
-        if (slots > p->ent_long_slots) {  // the entropy stage spreads such a unit over several thread blocks
+        if (slots > kEntLongSlots) {  // the entropy stage spreads such a unit over several thread blocks
             const uint32_t li = (uint32_t)p->ent_long_units.size();
             p->ent_long_units.push_back(u);
-            for (uint64_t g = 0; g < slots; g += 64) p->ent_chunks.push_back({u, (uint32_t)g, li, 0u});
+            for (uint64_t g = 0; g < slots; g += kEntLongSlots) p->ent_chunks.push_back({u, (uint32_t)g, li, 0u});
         }
     }
     for (size_t t = 0; t < p->tiles.size(); ++t) {

@@ -142,12 +142,8 @@ __host__ __device__ inline size_t workspace_total_bytes(size_t nt) {
     return (workspace_prefix_offset(nt) + nt * sizeof(uint32_t) + 15) / 16 * 16;
 }
 
-// Entropy stage: a unit of at most 64 segment slots is coded by one thread block, of 32 warps as long as there are no more
-// such units than SMs (kEntWideUnits), else of 8; longer ones by several blocks.  Up to kEntSplitUnits units, blocks of 8
-// warps leave most of the GPU idle, so there units of more than kEntSplitSlots are coded by several blocks as well: step with
-// the stage, 208 units of 62 slots 433 -> 277 us, 192 of 32 (every block changed) 355 -> 222; 384 units of 32 slots 206 -> 214.
-// kEntFewUnits: up to here the receiver's build for 5 blocks per SM is the faster one.
-constexpr uint32_t kEntWideUnits = 148, kEntSplitUnits = 296, kEntSplitSlots = 16, kEntFewUnits = 740;
+// Entropy stage: a unit of up to this many segment slots is coded by one thread block, a longer one by several.
+constexpr uint32_t kEntLongSlots = 64;
 
 // The tile table lists the tiles of "short" units (up to this many tiles) first, longest units
 // first, then the tiles of the longer units.  The encode kernel lets one thread block work through
@@ -216,8 +212,7 @@ struct ciera_plan {
     // the tiles whose values, rounded up to 16 bytes, go past these ends (kNoTile: none; several: more than these)
     uint32_t weights_end_tile = ciera::kNoTile, cache_end_tile = ciera::kNoTile;
     bool several_end_tiles = false;
-    // entropy stage: units of more than ent_long_slots segment slots, and their chunks of 64 slots
-    uint32_t ent_long_slots = 64;
+    // entropy stage: units of more than kEntLongSlots segment slots, and their chunks of as many
     // {unit, first segment of the chunk inside the unit, index among the long units, 0}
     struct EntChunk {
         uint32_t unit, first_seg, long_index, zero;

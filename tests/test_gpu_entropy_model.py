@@ -75,10 +75,11 @@ def test_models_and_lengths():
 
 
 @pytest.mark.parametrize("dtype", [0, 2])
-@pytest.mark.parametrize("n_units,size", [(148, 4096), (149, 4096), (741, 4096), (149, 65_500), (297, 65_500)])
+@pytest.mark.parametrize("n_units,size", [(148, 4096), (149, 4096), (741, 4096), (149, 65_500), (297, 65_500), (296, 4096), (296, 65_500),
+                                          (740, 4096), (160, 131_072)])
 def test_numbers_of_units(n_units, size, dtype):
-    """A wide thread block per unit up to one per SM, narrow ones beyond, and those in two builds by their number; among
-    few units those of more than 16 segment slots take several blocks."""
+    """A thread block of 32 warps per unit up to one per SM, of 16 up to two, narrow ones beyond, and those in two builds
+    by their number."""
     from paper_2609_04609_b200 import runtime
 
     name = {0: "bf16", 2: "fp16"}[dtype]
