@@ -15,10 +15,13 @@
  *   - Every function returns a ciera_status (0 = CIERA_OK, negative = error).  Nothing throws,
  *     nothing is printed, and no codec state lives in the library: caches, messages and scratch
  *     are the caller's buffers.  What the library does keep per process: the launch counter, the
- *     thread's last CUDA error, and per device the grid sizes it has worked out for its kernels.
+ *     thread's last CUDA error, per device the grid sizes it has worked out for its kernels, and up to
+ *     eight pairs of copy streams with their events, made by ciera_roundtrip_host when it first needs
+ *     them (all but one pair are given up when the last plan is destroyed).
  *   - "dev" pointers are CUDA device pointers, "host" pointers are ordinary host pointers.
  *     The library never allocates device memory: the caller owns every device buffer and
- *     passes scratch space explicitly.  The only host allocation is the plan object.  (One
+ *     passes scratch space explicitly.  The only host allocations are the plan object and the
+ *     records of those copy streams.  (One
  *     exception, stated where it is declared: ciera_encode_noalloc works in a fixed device array
  *     that is part of the library image, for callers that cannot supply scratch.)
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Device work is
@@ -326,10 +329,18 @@ typedef struct ciera_device_buffers {
 } ciera_device_buffers;
 
 /* One sender + receiver step of Algorithm 1 on weights that live in HOST memory:
- * copy `weights_host` (weights_bytes, ideally pinned) to the device, ciera_encode,
- * ciera_transport, ciera_decode, copy the reconstructed weights to `weights_out_host` and the
- * per-unit wire lengths to `wire_bytes_host` ([n_units], may be NULL).  Everything is enqueued on
- * `stream`; the host buffers must stay valid until the stream has drained. */
+ * copy `weights_host` (weights_bytes, ideally pinned) to the device, step as ciera_step does, copy the
+ * reconstructed weights to `weights_out_host` (which may be or overlap `weights_host`) and the per-unit wire
+ * lengths to `wire_bytes_host` ([n_units], may be NULL).
+ *   - Pinned weights of 4 MB and more are stepped in parts, so that the host link carries both directions at
+ *     once: the copies run on streams of the library, between what `stream` held before and what it is given
+ *     next, and a part is one kernel launch on `stream`.  Pageable memory, and a stream that is being captured:
+ *     as a whole, all on `stream`.
+ *   - The host buffers must stay valid until `stream` has drained.
+ *   - Any number of threads and streams may step at the same time, each with buffers of its own.
+ *   - If a copy to the device cannot be queued, nothing is stepped; if one back cannot, the step on the device
+ *     is complete.  After any other CUDA error the caches may hold the exponents of some tiles already; the
+ *     workspace can be used again in every case. */
 CIERA_API int ciera_roundtrip_host(const ciera_plan* plan, const void* weights_host, size_t weights_bytes,
                          void* weights_out_host, uint64_t* wire_bytes_host, const ciera_device_buffers* bufs,
                          void* stream);

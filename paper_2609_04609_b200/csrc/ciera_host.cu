@@ -289,13 +289,14 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         }
     }
     *plan_out = p;
+    count_plan(1);
     return CIERA_OK;
 }
 
 extern "C" void ciera_plan_destroy(ciera_plan* plan) {
-    if (plan)
-        for (const ciera_plan::CopyLane& lane : plan->lanes) destroy_copy_lane(lane);  // (work still queued there runs to its end)
+    if (!plan) return;
     delete plan;
+    count_plan(-1);
 }
 
 extern "C" uint32_t ciera_plan_n_units(const ciera_plan* p) { return p ? p->n_units : 0; }

@@ -5,7 +5,6 @@
 #include <stdint.h>
 
 #include <atomic>
-#include <mutex>
 #include <vector>
 
 #include "ciera.h"
@@ -225,16 +224,6 @@ struct ciera_plan {
                                        // ent_long_units, ent_chunks, tiles_by_address, tile_hash, seq_runs
     const ciera::TileDesc* tiles_dev = nullptr;
     const uint32_t* tiles_by_address_dev = nullptr;
-    // Pairs of copy streams for steps on host weights: taken out for the length of a call, put back at its end and
-    // reused by the next; as many as calls were ever made at the same time; destroyed with the plan.
-    struct CopyLane {
-        int device;
-        cudaStream_t in, out;
-        cudaEvent_t event;
-        cudaEvent_t arrived[ciera::kHostPartsMax];  // behind each part's weights
-    };
-    mutable std::mutex lanes_mutex;
-    mutable std::vector<CopyLane> lanes;
     const uint32_t* prefix_segments_dev = nullptr;
     const uint32_t* seq_first_dev = nullptr;
     const uint2* seq_runs_dev = nullptr;
@@ -278,7 +267,7 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 int check_launch();                            // cudaGetLastError -> status
-void destroy_copy_lane(const ciera_plan::CopyLane& lane);
+void count_plan(int change);                   // plans that exist
 // the persistent sender kernel with HashCache in place of the exponent cache (ciera_encode.cu)
 int launch_encode_hashed(const ciera_plan* p, const void* weights_dev, void* hash_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,

@@ -1,6 +1,8 @@
 // Auxiliary sm_100a kernels of libciera: cache initialisation, the transport stand-in, and the
 // host-buffer round trip.  (Encode and decode live in ciera_encode.cu / ciera_decode.cu.)
 #include <algorithm>
+#include <mutex>
+#include <new>
 
 #include "ciera_bits.cuh"
 #include "ciera_host_step.hpp"
@@ -406,38 +408,88 @@ static uint32_t host_step_parts(const ciera_plan* p, const ciera_device_buffers*
     return parts;
 }
 
-void ciera::destroy_copy_lane(const ciera_plan::CopyLane& lane) {
-    if (lane.in) cudaStreamDestroy(lane.in);
-    if (lane.out) cudaStreamDestroy(lane.out);
-    if (lane.event) cudaEventDestroy(lane.event);
-    for (cudaEvent_t a : lane.arrived)
+// A lane: two streams that carry a step's copies and the events that tie them to the caller's stream.  Making one takes
+// 0.13 ms (a process's first streams: a millisecond and more), as long as copying 4 MB both ways, so lanes are kept: taken
+// out for the length of a call, put back at its end, shared by all plans.  A caller's stream gets the lane that served it
+// last, so that steps on different streams do not wait for one another's copies as long as there are no more streams than
+// lanes kept.  When the last plan goes, all but one of the kept lanes go.  First step of a fresh plan, 4 / 8 MB: as a whole
+// 220 / 390 us, in parts with streams of the plan's own 320 / 440, like this 177 / 301.
+struct CopyLane {
+    int device;
+    cudaStream_t user;  // the caller's stream that it served last
+    cudaStream_t in, out;
+    cudaEvent_t event;
+    cudaEvent_t arrived[kHostPartsMax];  // behind each part's weights
+};
+constexpr int kKeptLanes = 8;
+static std::mutex g_lanes_mutex;
+static CopyLane* g_lanes[kKeptLanes];  // the one put back longest ago first
+static int g_n_lanes = 0, g_n_plans = 0;
+
+static void destroy_copy_lane(CopyLane* lane) {  // (work still queued there runs to its end)
+    if (lane->in) cudaStreamDestroy(lane->in);
+    if (lane->out) cudaStreamDestroy(lane->out);
+    if (lane->event) cudaEventDestroy(lane->event);
+    for (cudaEvent_t a : lane->arrived)
         if (a) cudaEventDestroy(a);
+    delete lane;
+}
+static CopyLane* drop_kept_lane(int i) {  // (holding the mutex)
+    CopyLane* const lane = g_lanes[i];
+    --g_n_lanes;
+    for (; i < g_n_lanes; ++i) g_lanes[i] = g_lanes[i + 1];
+    return lane;
 }
 
-// (with events for that many parts)
-static int take_copy_lane(const ciera_plan* p, uint32_t parts, ciera_plan::CopyLane* lane) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return record_cuda_error(e);
-    *lane = {};
-    lane->device = dev;
+void ciera::count_plan(int change) {
+    CopyLane* gone[kKeptLanes];
+    int n = 0;
     {
-        std::lock_guard<std::mutex> hold(p->lanes_mutex);
-        for (size_t i = 0; i < p->lanes.size(); ++i)
-            if (p->lanes[i].device == dev) {
-                *lane = p->lanes[i];
-                p->lanes.erase(p->lanes.begin() + i);
-                break;
-            }
+        std::lock_guard<std::mutex> hold(g_lanes_mutex);
+        g_n_plans += change;
+        while (g_n_plans == 0 && g_n_lanes > 1) gone[n++] = drop_kept_lane(0);
     }
+    while (n) destroy_copy_lane(gone[--n]);
+}
+
+// a lane for steps on `s`, with events for that many parts; null: there is none to be had
+static CopyLane* take_copy_lane(cudaStream_t s, uint32_t parts) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    CopyLane* lane = nullptr;
+    {
+        std::lock_guard<std::mutex> hold(g_lanes_mutex);
+        int found = -1;
+        for (int i = g_n_lanes; i-- > 0 && found < 0;)
+            if (g_lanes[i]->device == dev && g_lanes[i]->user == s) found = i;
+        for (int i = 0; g_n_lanes == kKeptLanes && i < g_n_lanes && found < 0; ++i)
+            if (g_lanes[i]->device == dev) found = i;
+        if (found >= 0) lane = drop_kept_lane(found);
+    }
+    if (!lane) lane = new (std::nothrow) CopyLane{};
+    if (!lane) return nullptr;
+    lane->device = dev;
+    lane->user = s;
+    cudaError_t e = cudaSuccess;
     if (!lane->in) e = cudaStreamCreateWithFlags(&lane->in, cudaStreamNonBlocking);
     if (e == cudaSuccess && !lane->out) e = cudaStreamCreateWithFlags(&lane->out, cudaStreamNonBlocking);
     if (e == cudaSuccess && !lane->event) e = cudaEventCreateWithFlags(&lane->event, cudaEventDisableTiming);
     for (uint32_t k = 0; k < parts; ++k)
         if (e == cudaSuccess && !lane->arrived[k]) e = cudaEventCreateWithFlags(&lane->arrived[k], cudaEventDisableTiming);
-    if (e == cudaSuccess) return CIERA_OK;
-    destroy_copy_lane(*lane);
-    return record_cuda_error(e);
+    if (e == cudaSuccess) return lane;
+    cudaGetLastError();
+    destroy_copy_lane(lane);
+    return nullptr;
+}
+
+static void put_copy_lane(CopyLane* lane) {
+    CopyLane* gone = nullptr;
+    {
+        std::lock_guard<std::mutex> hold(g_lanes_mutex);
+        if (g_n_lanes == kKeptLanes) gone = drop_kept_lane(0);
+        g_lanes[g_n_lanes++] = lane;
+    }
+    if (gone) destroy_copy_lane(gone);
 }
 
 // `to` waits for what `from` holds so far
@@ -456,7 +508,7 @@ struct HostStepOps {
     const ciera_device_buffers* b;
     const uint8_t* in;
     uint8_t* out;
-    const ciera_plan::CopyLane& lane;
+    const CopyLane& lane;
     cudaStream_t s;
     Part part[kHostPartsMax];
 
@@ -487,13 +539,10 @@ struct HostStepOps {
 };
 
 static int host_step_in_parts(const ciera_plan* p, const void* weights_host, size_t weights_bytes, void* weights_out_host,
-                              const ciera_device_buffers* b, uint32_t parts, cudaStream_t s) {
+                              const ciera_device_buffers* b, uint32_t parts, const CopyLane& lane, cudaStream_t s) {
     // the checks of ciera_step, and the outputs of units without values
     int rc = step_begin(p, b->weights_dev, b->sender_cache_dev, b->msg_send_dev, b->msg_recv_dev, b->receiver_cache_dev,
                               b->weights_out_dev, b->wire_bytes_dev, b->changed_blocks_dev, b->workspace_dev, s);
-    if (rc) return rc;
-    ciera_plan::CopyLane lane;
-    rc = take_copy_lane(p, parts, &lane);
     if (rc) return rc;
     HostStepOps op{p, b, (const uint8_t*)weights_host, (uint8_t*)weights_out_host, lane, s, {}};
     const uint32_t nt = (uint32_t)p->tiles.size();
@@ -510,10 +559,6 @@ static int host_step_in_parts(const ciera_plan* p, const void* weights_host, siz
     }
     const cudaError_t e = wait_for(lane.in, s, lane.event);
     rc = e != cudaSuccess ? record_cuda_error(e) : run_host_parts(op, n);
-    {
-        std::lock_guard<std::mutex> hold(p->lanes_mutex);
-        p->lanes.push_back(lane);
-    }
     return rc;
 }
 
@@ -526,8 +571,10 @@ extern "C" int ciera_roundtrip_host(const ciera_plan* p, const void* weights_hos
     if (p->tiles.empty()) return CIERA_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t parts = host_step_parts(p, b, weights_host, weights_out_host, weights_bytes, s);
-    if (parts > 1) {
-        rc = host_step_in_parts(p, weights_host, weights_bytes, weights_out_host, b, parts, s);
+    CopyLane* const lane = parts > 1 ? take_copy_lane(s, parts) : nullptr;
+    if (lane) {
+        rc = host_step_in_parts(p, weights_host, weights_bytes, weights_out_host, b, parts, *lane, s);
+        put_copy_lane(lane);
         if (rc) return rc;
     } else {
         cudaError_t e = cudaMemcpyAsync(b->weights_dev, weights_host, weights_bytes, cudaMemcpyHostToDevice, s);

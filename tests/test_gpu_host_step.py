@@ -104,3 +104,71 @@ def test_host_ranges_that_overlap(shift):
     for u in codec.units:
         lo, hi = int(u["weights_off"]), int(u["weights_off"]) + 2 * int(u["n_values"])
         assert np.array_equal(out.numpy()[lo:hi], bits[1].view(np.uint8)[lo:hi])
+
+
+def test_two_threads_on_one_plan():
+    """Steps in parts from two threads on one plan, each with a stream and buffers of its own, at the same time."""
+    import threading
+
+    from paper_2609_04609_b200 import ciera, runtime
+
+    first, table0, bits0, staging0 = _make(seed=5, steps=4)
+    second, table1, bits1, staging1 = _make(seed=6, steps=4)
+    second.plan = first.plan  # (the same table of units)
+    jobs = [(first, table0, bits0, staging0), (second, table1, bits1, staging1)]
+    errors = []
+
+    def work(codec, table, bits, staging):
+        try:
+            stream = torch.cuda.Stream()
+            out = torch.zeros(codec.weights_bytes, dtype=torch.uint8).pin_memory()
+            for t in range(1, len(bits)):
+                src = _pinned(bits[t])
+                exp = table.step(bits[t])
+                codec.step_host(src, out, staging, stream=stream)
+                stream.synchronize()
+                codec.check_status()
+                compare_step(codec, exp, bits[t], f"t={t}")
+                compare_recon(codec, exp, bits[t], 0, f"t={t}")
+                for u in codec.units:
+                    lo, hi = int(u["weights_off"]), int(u["weights_off"]) + 2 * int(u["n_values"])
+                    assert np.array_equal(out.numpy()[lo:hi], bits[t].view(np.uint8)[lo:hi]), f"t={t}"
+        except Exception as e:  # (reported by the main thread)
+            errors.append(e)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for x in threads:
+        x.start()
+    for x in threads:
+        x.join()
+    assert not errors, errors
+    for codec, table, bits, _ in jobs:
+        compare_caches(codec, table, "threads")
+
+
+def test_more_streams_than_the_library_keeps_copy_streams_for():
+    """Twelve codecs, a stream each, stepped round and round without waiting in between; plans come and go meanwhile."""
+    from paper_2609_04609_b200 import runtime
+
+    made = [_make([8192 * 300 + i, 4099], seed=20 + i, steps=2) for i in range(12)]
+    streams = [torch.cuda.Stream() for _ in made]
+    outs = [torch.zeros(m[0].weights_bytes, dtype=torch.uint8).pin_memory() for m in made]
+    srcs = [[_pinned(b) for b in m[2]] for m in made]
+    torch.cuda.synchronize()
+    for t in (1, 2, 1, 2):
+        for i, (codec, _, _, staging) in enumerate(made):
+            codec.step_host(srcs[i][t], outs[i], staging, stream=streams[i])
+    torch.cuda.synchronize()
+    for i, (codec, table, bits, _) in enumerate(made):
+        codec.check_status()
+        for t in (1, 2, 1, 2):
+            exp = table.step(bits[t])
+        compare_step(codec, exp, bits[2], f"codec {i}")
+        compare_caches(codec, table, f"codec {i}")
+        compare_recon(codec, exp, bits[2], 0, f"codec {i}")
+    del made, codec, table
+    codec, table, bits, staging = _make(steps=1)  # after the last plan went, and its streams with it
+    out = torch.zeros(codec.weights_bytes, dtype=torch.uint8).pin_memory()
+    codec.step_host(_pinned(bits[1]), out, staging)
+    _compare(codec, table, table.step(bits[1]), bits[1], "fresh")
