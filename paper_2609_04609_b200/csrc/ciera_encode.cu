@@ -1609,8 +1609,12 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
     BufferEnds ends{p->weights_end_tile, HASH ? kNoTile : p->cache_end_tile, p->several_end_tiles};
     const bool has_spread = spread_first < nt;  // look-back between blocks
-    // With a tile to a block and nothing else a tile looks back at blocks before its own only, which start no later, so the
-    // blocks need not all be resident and the launch may begin while the kernel before it drains.  (Two or three neighbouring
+    // With a tile to a block and nothing else a tile looks back at blocks before its own only, so the blocks need not all be
+    // resident and the launch may begin while the kernel before it drains -- provided that blocks start in the order of their
+    // numbers, which the hardware does and the programming model does not promise (the runs of short units rest on it too: a
+    // block's first two are given by its number).  Were a block to start after one that waits for it, with all SMs taken by
+    // other kernels for longer than the bound on the wait, the step would end with CIERA_ERR_TIMEOUT, not hang.  Drawing the
+    // tile from a counter instead costs a round trip before the first load: 64 tiles 6.6 -> 7.0 us.  (Two or three neighbouring
     // tiles to a block would keep that for more tables; measured on whole steps back to back: 384 tiles 15.3 us against
     // 14.1 with a cooperative launch and every grid-th tile, 768 tiles 18.3 against 20.1, 1024 tiles in fours 30.1 against 25.0.)
     const bool one_each = n_runs == 0 && to_do <= grid;

@@ -322,3 +322,34 @@ def test_every_remainder_of_the_last_tile_of_a_buffer(dtype, shared):
             compare_step(codec, exp, bits[t], f"n={n} t={t}")
             compare_caches(codec, table, f"n={n} t={t}")
             compare_recon(codec, exp, bits[t], dtype, f"n={n} t={t}")
+
+
+def test_small_tables_on_several_streams_beside_a_large_one():
+    """Tables of a tile to a thread block (look-back between blocks that need not all be resident), of a few tiles to a
+    block and of runs, stepped over and over on streams of their own while a large table keeps the SMs busy."""
+    from paper_2609_04609_b200 import runtime
+
+    gen = wl.make_generator(77, DEV)
+    tables = [[524_288], [8192 * 250], [3_000_005, 131_072], [8192] * 40, [2_097_152] * 3, [8192 * 5 + 3] * 300, [8192 * 290 + 1], [4099]]
+    jobs = []
+    for i, sizes in enumerate(tables + [[2_097_152] * 48]):
+        dtype = (0, 1, 2)[i % 3]
+        codec = runtime.LayerCodec.from_tensors(sizes, 4, NAME[dtype], (512, 16, 1, 64)[i % 4], DEV)
+        a = wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)
+        w = [wl.step_clustered(a, gen, f=0.3).view(torch.uint8), a.view(torch.uint8)]
+        codec.init_caches(w[1])
+        jobs.append((codec, w, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for it in range(60):
+        for i, (codec, w, stream) in enumerate(jobs):
+            for rep in range(1 if i == len(jobs) - 1 else 3):
+                codec.step(w[(3 * it + rep) & 1 if i < len(jobs) - 1 else it & 1], None, stream)
+    torch.cuda.synchronize()
+    for i, (codec, w, _) in enumerate(jobs):
+        codec.check_status()
+        last = w[(3 * 59 + 2) & 1 if i < len(jobs) - 1 else 59 & 1]
+        vb = wl.VALUE_BYTES[codec.dtype_name]
+        for u in codec.units:
+            lo, hi = int(u["weights_off"]), int(u["weights_off"]) + vb * int(u["n_values"])
+            assert torch.equal(codec.weights_out[lo:hi], last[lo:hi]), f"table {i}"
+        assert torch.equal(codec.sender_cache, codec.receiver_cache), f"table {i}"
