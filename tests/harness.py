@@ -3,9 +3,24 @@
 Lives in tests/ and is used by tests only.  The oracle runner keeps its own flat caches in the
 same layout as the device buffers so that results can be compared byte for byte."""
 import numpy as np
+import pytest
 import torch
 
 from oracle import ciera_oracle as ora
+
+def one_launch(codec, w):
+    """The whole step by ``ciera_step``."""
+    codec.step(w)
+
+
+def three_calls(codec, w):
+    """The same step by the three calls it stands for."""
+    codec.encode(w)
+    codec.transport()
+    codec.decode()
+
+
+both_ways = pytest.mark.parametrize("step", [one_launch, three_calls], ids=["one-launch", "three-calls"])
 
 VB = {0: 2, 1: 4, 2: 2}
 WDT = {0: np.uint16, 1: np.uint32, 2: np.uint16}

@@ -172,3 +172,51 @@ def test_entropy_decode_flags_a_damaged_section(rt, n_values, dtype):
     torch.cuda.synchronize()
     assert int(codec.status.item()) == ciera.ERR_CORRUPT
     assert torch.equal(codec.msg_recv, damaged) and not torch.equal(damaged, before)  # left as received
+
+
+@pytest.mark.parametrize("dtype,block,sizes", [(0, 512, [131_072, 70_001, 5]), (2, 64, [600_001, 131_072]), (0, 64, [4096] * 200),
+                                               (1, 512, [4096 * 3] * 320)])
+def test_steps_with_the_stage_replayed_from_a_cuda_graph(rt, dtype, block, sizes):
+    """Sender, stage, transport, stage, receiver captured once and replayed on new weights in the same buffer: few units
+    (wide thread blocks), a unit that is cut into chunks, some more units, many."""
+    ciera, runtime = rt
+    name = {0: "bf16", 1: "fp32", 2: "fp16"}[dtype]
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, name, block, DEV, slack=256))
+    n = codec.weights_bytes // wl.VALUE_BYTES[name]
+    traj = [wl.as_bits(w) for w in wl.trajectory(n, name, 55 + block, 4, "clustered", f=0.3)]
+    wdt = traj[0].dtype
+    codec.init_caches(to_dev_bytes(traj[0], DEV))
+    caches = [ora.cache_init(traj[0][int(u["weights_off"]) // wdt.itemsize :][: int(u["n_values"])], int(u["n_values"]), dtype)
+              for u in codec.units]
+    w_in = to_dev_bytes(traj[1], DEV).clone()
+
+    def step():
+        codec.encode(w_in)
+        codec.entropy_encode()
+        codec.transport()
+        codec.entropy_decode()
+        codec.decode()
+
+    def check(w, label):
+        torch.cuda.synchronize()
+        codec.check_status()
+        codec.canaries.check(label)
+        sent, back, wire = codec.msg_send.cpu().numpy(), codec.msg_recv.cpu().numpy(), codec.wire_bytes.tolist()
+        out = codec.weights_out.cpu().numpy().view(wdt)
+        for i, u in enumerate(codec.units):
+            lo, nn, mo = int(u["weights_off"]) // wdt.itemsize, int(u["n_values"]), int(u["msg_off"])
+            raw = ora.encode(w[lo : lo + nn], caches[i], dtype, block)[0]
+            want = rans.entropy_encode_message(raw, nn, dtype, block)
+            assert np.array_equal(sent[mo : mo + want.size], want), f"{label}: coded message {i}"
+            assert wire[i] == raw.size and np.array_equal(back[mo : mo + raw.size], raw), f"{label}: restored message {i}"
+            assert np.array_equal(out[lo : lo + nn], w[lo : lo + nn]), f"{label}: weights {i}"
+
+    step()  # outside the capture first
+    check(traj[1], "eager")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        step()
+    for t in (2, 3, 4):
+        w_in.copy_(to_dev_bytes(traj[t], DEV))
+        graph.replay()
+        check(traj[t], f"replay t={t}")

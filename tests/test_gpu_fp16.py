@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes
+from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes, one_launch, three_calls
 from paper_2609_04609_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -30,20 +30,21 @@ def _run(rt, sizes, shards, block, traj_fn, zero_cache=False, label=""):
     n = codec.weights_bytes // 2
     traj = traj_fn(n)
     first = None if zero_cache else traj[0]
-    codec.init_caches(None if first is None else to_dev_bytes(first, DEV))
-    table.init_caches(first)
-    compare_caches(codec, table, label + " init")
     stats = []
-    for t, w in enumerate(traj[1:], 1):
-        codec.step(to_dev_bytes(w, DEV))
-        torch.cuda.synchronize()
-        codec.check_status()
-        exp = table.step(w)
-        wire, chg = compare_step(codec, exp, w, f"{label} t={t}")
-        compare_caches(codec, table, f"{label} t={t}")
-        compare_recon(codec, exp, w, FP16, f"{label} t={t}")
-        stats.append((int(chg.sum()), codec.n_blocks()))
-    return stats
+    for step in (one_launch, three_calls):  # the trajectory from the start by either
+        codec.init_caches(None if first is None else to_dev_bytes(first, DEV))
+        table.init_caches(first)
+        compare_caches(codec, table, label + " init")
+        for t, w in enumerate(traj[1:], 1):
+            step(codec, to_dev_bytes(w, DEV))
+            torch.cuda.synchronize()
+            codec.check_status()
+            exp = table.step(w)
+            wire, chg = compare_step(codec, exp, w, f"{label} t={t} {step.__name__}")
+            compare_caches(codec, table, f"{label} t={t} {step.__name__}")
+            compare_recon(codec, exp, w, FP16, f"{label} t={t} {step.__name__}")
+            stats.append((int(chg.sum()), codec.n_blocks()))
+    return stats[: len(traj) - 1]
 
 
 @pytest.mark.parametrize("block", [1, 2, 4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, 4096])

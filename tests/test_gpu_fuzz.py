@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes
+from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes, one_launch, three_calls
 from oracle import ciera_oracle as ora
 from oracle import rans_oracle as rans
 from paper_2609_04609_b200 import workloads as wl
@@ -67,22 +67,25 @@ def _trajectory(rng, n, dtype):
 def test_random_tables_full_step(rt, seed):
     ciera, runtime = rt
     rng, sizes, shards, dtype, block = _random_case(1000 + seed)
-    codec = guard(runtime.LayerCodec.from_tensors(sizes, shards, NAME[dtype], block, DEV, slack=256))
-    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
-    n = codec.weights_bytes // VB[dtype]
+    ways = (one_launch, three_calls)
+    codecs = [guard(runtime.LayerCodec.from_tensors(sizes, shards, NAME[dtype], block, DEV, slack=256)) for _ in ways]
+    table = OracleTable(codecs[0].units, dtype, block, codecs[0].cache_bytes, codecs[0].msg_bytes)
+    n = codecs[0].weights_bytes // VB[dtype]
     traj = _trajectory(rng, max(n, 1), dtype)
     from_zero = bool(rng.integers(0, 2))
-    codec.init_caches(None if from_zero else to_dev_bytes(traj[0], DEV))
+    for codec in codecs:
+        codec.init_caches(None if from_zero else to_dev_bytes(traj[0], DEV))
     table.init_caches(None if from_zero else traj[0])
-    label = f"seed {seed} sizes {sizes} shards {shards} {NAME[dtype]} B={block}"
     for t, w in enumerate(traj[1:], 1):
-        codec.step(to_dev_bytes(w, DEV))
-        torch.cuda.synchronize()
-        codec.check_status()
         exp = table.step(w)
-        compare_step(codec, exp, w, f"{label} t={t}")
-        compare_caches(codec, table, f"{label} t={t}")
-        compare_recon(codec, exp, w, dtype, f"{label} t={t}")
+        for codec, step in zip(codecs, ways):
+            label = f"seed {seed} sizes {sizes} shards {shards} {NAME[dtype]} B={block} t={t} {step.__name__}"
+            step(codec, to_dev_bytes(w, DEV))
+            torch.cuda.synchronize()
+            codec.check_status()
+            compare_step(codec, exp, w, label)
+            compare_caches(codec, table, label)
+            compare_recon(codec, exp, w, dtype, label)
 
 
 @pytest.mark.parametrize("seed", range(N_HASHED))

@@ -7,7 +7,8 @@ import numpy as np
 import pytest
 import torch
 
-from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes
+from harness import (OracleTable, both_ways, compare_caches, compare_recon, compare_step, guard, one_launch, three_calls,
+                     to_dev_bytes)
 from paper_2609_04609_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -34,6 +35,13 @@ def _make(rt, sizes, n_shards, dtype, block):
 
 
 def _run_trajectory(rt, codec, table, traj, dtype, zero_cache=False, label=""):
+    """The trajectory from the start by whole steps in one launch, and once more by the three calls."""
+    stats = _run_once(codec, table, traj, dtype, zero_cache, label, one_launch)
+    assert _run_once(codec, table, traj, dtype, zero_cache, label + " three calls", three_calls) == stats
+    return stats
+
+
+def _run_once(codec, table, traj, dtype, zero_cache, label, step):
     w0 = traj[0]
     if zero_cache:
         codec.init_caches(None)
@@ -45,7 +53,7 @@ def _run_trajectory(rt, codec, table, traj, dtype, zero_cache=False, label=""):
     stats = []
     for t, w in enumerate(traj[1:], 1):
         wd = to_dev_bytes(w, DEV)
-        codec.step(wd)
+        step(codec, wd)
         torch.cuda.synchronize()
         codec.check_status()
         exp = table.step(w)
@@ -262,13 +270,16 @@ def test_pipelined_stack_equals_serial(rt):
             assert torch.equal(x, y)
 
 
+@both_ways
 @pytest.mark.parametrize("sizes,dtype,block", [([3_000_005, 131_072, 70_001], 0, 512), ([200_000, 5, 8192 * 3], 0, 4),
-                                               ([131_072, 70_001], 1, 64), ([131_072, 70_001], 2, 512)])
-def test_steps_replayed_from_a_cuda_graph(rt, sizes, dtype, block):
+                                               ([131_072, 70_001], 1, 64), ([131_072, 70_001], 2, 512),
+                                               ([8192 * 80 + 5, 8192 * 3], 0, 1), ([3_000_005, 70_001], 0, 64)])
+def test_steps_replayed_from_a_cuda_graph(rt, sizes, dtype, block, step):
     """A whole step (sender, transport, receiver) is a handful of kernel launches that read their sizes on the
     device and leave the scratch as they found it, so it can be captured once in a CUDA graph and replayed on new
-    weights in the same buffer.  Every replay must equal the oracle's step bit for bit, with a long unit
-    (cooperative launch, prefix kernel) in the table as well."""
+    weights in the same buffer.  Every replay must equal the oracle's step bit for bit, with long units in the table
+    as well (cooperative launch; by the three calls also the prefix kernel: blocks of 64, and of 1 over several
+    segments)."""
     ciera, runtime = rt
     name = {0: "bf16", 1: "fp32", 2: "fp16"}[dtype]
     codec = guard(runtime.LayerCodec.from_tensors(sizes, 2, name, block, DEV, slack=256))
@@ -278,13 +289,13 @@ def test_steps_replayed_from_a_cuda_graph(rt, sizes, dtype, block):
     codec.init_caches(to_dev_bytes(traj[0], DEV))
     table.init_caches(traj[0])
     w_in = to_dev_bytes(traj[1], DEV).clone()
-    codec.step(w_in)  # outside the capture first: the first calls query occupancy and set kernel attributes
+    step(codec, w_in)  # outside the capture first: the first calls query occupancy and set kernel attributes
     torch.cuda.synchronize()
     codec.check_status()
     compare_step(codec, table.step(traj[1]), traj[1], "eager")
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
-        codec.step(w_in)
+        step(codec, w_in)
     for t in (2, 3, 4):
         w_in.copy_(to_dev_bytes(traj[t], DEV))
         graph.replay()
@@ -296,8 +307,9 @@ def test_steps_replayed_from_a_cuda_graph(rt, sizes, dtype, block):
         compare_recon(codec, exp, traj[t], dtype, f"replay t={t}")
 
 
+@both_ways
 @pytest.mark.parametrize("dtype,block", [(0, 1), (0, 8), (0, 512), (2, 1), (2, 4), (2, 64), (1, 2), (1, 512)])
-def test_every_pattern_against_every_cached_exponent(rt, dtype, block):
+def test_every_pattern_against_every_cached_exponent(rt, dtype, block, step):
     """The complete per-value map on the GPU: every 16-bit pattern of bf16 and fp16 (zeros, subnormals, infinities,
     NaNs with every payload) against every value the cached exponent can have (256 / 32) -- 16.7 M / 2.1 M values in
     one unit, cache rows shuffled so that changed and unchanged blocks mix; for fp32 every exponent field x both
@@ -332,7 +344,7 @@ def test_every_pattern_against_every_cached_exponent(rt, dtype, block):
     w_dev[lo : lo + w.nbytes] = torch.from_numpy(w.view(np.uint8)).to(DEV)
     for cache in (codec.sender_cache, codec.receiver_cache):
         cache[co : co + n] = torch.from_numpy(cache0).to(DEV)
-    codec.step(w_dev)
+    step(codec, w_dev)
     torch.cuda.synchronize()
     codec.check_status()
     codec.canaries.check("every pattern")
@@ -400,11 +412,14 @@ def test_resume_from_saved_caches_or_from_the_weights(rt, dtype, block):
         compare_step(hashed, want, traj[3], "HashCache rebuilt from the weights")
 
 
+@pytest.mark.parametrize("mode", ["plain", "timers", "entropy", "hashed", "alternating"])
 @pytest.mark.parametrize("n_layers", [1, 3])
-def test_pipeline_of_many_iterations_reuses_layer_buffers_safely(rt, n_layers):
-    """Many iterations back to back on two streams, alternating between two iterates: with a single
-    layer the next iteration's sender side would overwrite the message that is still being decoded
-    unless it waits for that decode.  Every iteration must come out exact and with a clean status."""
+def test_pipeline_of_many_iterations_reuses_layer_buffers_safely(rt, n_layers, mode):
+    """Many iterations back to back, alternating between two iterates.  With timers, the entropy stage or the hashed
+    sender the layers run on two streams: with a single layer the next iteration's sender side would overwrite
+    the message that is still being decoded unless it waits for that decode.  Without them a layer is one launch;
+    ``alternating`` goes from one way to the other and back with nothing in between.  Every iteration must come out
+    exact and with a clean status."""
     ciera, runtime = rt
     shapes = [r * c for r, c in wl.olmoe_layer_shapes(8)]
     layers, wa, wb = [], [], []
@@ -418,23 +433,33 @@ def test_pipeline_of_many_iterations_reuses_layer_buffers_safely(rt, n_layers):
         wa.append(to_dev_bytes(wl.as_bits(w0), DEV))
         wb.append(to_dev_bytes(wl.as_bits(w1), DEV))
         codec.init_caches(wa[-1])
-    outs = [[torch.empty_like(c.weights_out) for c in layers] for _ in range(8)]
-    pipe = runtime.LayerPipeline(layers)
+        if mode == "hashed":
+            codec.init_hash_cache(wa[-1])
+    iterations = 12 if mode == "alternating" else 8
+    outs = [[torch.empty_like(c.weights_out) for c in layers] for _ in range(iterations)]
+    pipe = runtime.LayerPipeline(layers, entropy=mode == "entropy")
+    timers = []
     torch.cuda.synchronize()
-    for i in range(8):
-        pipe.step(wb if i % 2 == 0 else wa, outs[i])
+    for i in range(iterations):
+        two_streams = mode == "timers" or (mode == "alternating" and i % 5 in (1, 2))
+        launches0 = ciera.kernel_launch_count()
+        pipe.step(wb if i % 2 == 0 else wa, outs[i], timers if two_streams else None)
+        per_layer = (ciera.kernel_launch_count() - launches0) / n_layers
+        assert per_layer == (1 if mode in ("plain", "alternating") and not two_streams else 5 if mode == "entropy" else 3)
     pipe.wait()
     torch.cuda.synchronize()
     for c in layers:
         c.check_status()
-    for i in range(8):
+    for i in range(iterations):
         want = wb if i % 2 == 0 else wa
         for l in range(n_layers):
             assert torch.equal(outs[i][l][: want[l].numel()], want[l]), f"iteration {i}, layer {l}"
+    assert len(timers) == n_layers * {"timers": iterations, "alternating": 5}.get(mode, 0)
 
 
+@both_ways
 @pytest.mark.parametrize("dtype,block", [(0, 512), (1, 512), (0, 64)])
-def test_full_size_layer_sampled_units(rt, dtype, block):
+def test_full_size_layer_sampled_units(rt, dtype, block, step):
     """One full OLMoE-shaped layer (64 experts x 3 matrices, 16 shards: 3072 units, 402 653 184 values) in the
     launch configuration the benchmark times, generated on the device.  The round trip is checked everywhere
     (device-side comparison); messages, lengths, counts and caches of sampled units are checked against the
@@ -459,7 +484,7 @@ def test_full_size_layer_sampled_units(rt, dtype, block):
     wdt = WDT[dtype]
     prev = b0
     for cur in (b1, b2):
-        codec.step(cur)
+        step(codec, cur)
         torch.cuda.synchronize()
         codec.check_status()
         assert torch.equal(codec.weights_out[: cur.numel()], cur), "round trip is not bit-exact"
@@ -480,8 +505,9 @@ def test_full_size_layer_sampled_units(rt, dtype, block):
     assert q > (0.99 if block >= 256 else 0.8)  # the i.i.d. step changes (nearly) every block
 
 
+@both_ways
 @pytest.mark.parametrize("n_shards", [8, 64])
-def test_config5_full_size_mixed_shapes(rt, n_shards):
+def test_config5_full_size_mixed_shapes(rt, n_shards, step):
     """The mixed-shape sweep at full size in ONE plan: 256 fine-grained experts x (2048x512, 2048x512, 512x2048)
     plus dense tensors of 4 KB ... 256 MB (bf16) and one ragged 1000-value tensor, cut into 8 or 64 shards.  At 8
     shards the 256 MB tensor gives units of 16.8 M values = 2048 tiles (tiles spread over the thread blocks,
@@ -530,7 +556,7 @@ def test_config5_full_size_mixed_shapes(rt, n_shards):
     for c, seg in [(0.001, 0), (0.01, 0), (0.1, 0), (0.5, 0), (0.001, 512), (0.01, 512), (0.1, 512), (0.5, 512)]:
         w = wl.inject_exponent_changes(w, gen, c, seg)
         cur = as_bytes(w)
-        codec.step(cur)
+        step(codec, cur)
         torch.cuda.synchronize()
         codec.check_status()
         label = f"config5 shards={n_shards} c={c} seg={seg}"
@@ -554,9 +580,11 @@ def test_config5_full_size_mixed_shapes(rt, n_shards):
         prev = cur
 
 
-@pytest.mark.parametrize("block", [512, 1])
-def test_buffers_beyond_four_gib(rt, block):
-    """(With blocks of 512 values, and of one value: the fine-block kernels and their prefix kernel.)
+@pytest.mark.parametrize("block,steps_by", [(512, (one_launch, three_calls)), (1, (three_calls, one_launch))],
+                         ids=["512", "1"])
+def test_buffers_beyond_four_gib(rt, block, steps_by):
+    """(With blocks of 512 values, and of one value: the fine-block kernels and their prefix kernel.  One step in one
+    launch, one by the three calls.)
     One plan whose buffers are larger than 4 GiB each: 4.56 G bf16 values (9.1 GB of weights, 4.6 GB per cache,
     9.1 GB per message buffer), so that byte offsets pass 2^32 in every buffer and 2^33 in weights and messages --
     no 32-bit offset arithmetic survives this.  34 tensors of 128 Mi values in 4 shards (units of 4096 tiles: spread
@@ -621,7 +649,7 @@ def test_buffers_beyond_four_gib(rt, block):
     for t, make in enumerate(steps):
         w_next = chunked(make, like=w)
         cur = as_bytes(w_next)
-        codec.step(cur)
+        steps_by[t](codec, cur)
         torch.cuda.synchronize()
         codec.check_status()
         label = f"beyond 4 GiB, step {t}"
@@ -760,6 +788,19 @@ def test_one_unit_of_more_than_two_to_the_32_values(rt):
     assert sent > 2 ** 30 // 2 and int(codec.changed_blocks[0].item()) == changed
     assert int(codec.wire_bytes[0].item()) == pay_off + sent
     assert pay_off > 2 ** 32 and torch.equal(codec.msg_recv[: pay_off + sent], msg[: pay_off + sent])
+
+    # transport and receiver on their own: the same message arrives and gives the same weights
+    codec.msg_recv.zero_()
+    codec.weights_out.zero_()
+    guard(codec)
+    ciera.cache_init(codec.plan, codec.receiver_cache, b0)
+    codec.transport()
+    codec.decode()
+    torch.cuda.synchronize()
+    codec.check_status()
+    codec.canaries.check("one unit of more than 2^32 values, three calls")
+    assert torch.equal(codec.msg_recv[: pay_off + sent], msg[: pay_off + sent])
+    assert torch.equal(codec.weights_out[: 2 * n], b1) and torch.equal(codec.receiver_cache[:n], codec.sender_cache[:n])
 
     # the same step by the hashed sender gives the same message; then once through the entropy stage and back
     # (its chain of launches for long units, a quarter of a million segments)

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, to_dev_bytes
+from harness import OracleTable, compare_caches, compare_recon, compare_step, guard, one_launch, three_calls, to_dev_bytes
 from paper_2609_04609_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -18,15 +18,9 @@ SIZES = [1, 7, 8, 9, 255, 256, 257, 0, 511, 513, 4096, 8191, 8192, 8193, 8192 * 
 STATE = ("sender_cache", "receiver_cache", "weights_out", "wire_bytes", "changed_blocks")
 
 
-def _three_calls(codec, w):
-    codec.encode(w)
-    codec.transport()
-    codec.decode()
-
-
 @pytest.mark.parametrize("block", [1, 2, 4, 8, 16, 32, 256, 512, 1024, 2048, 4096])
 @pytest.mark.parametrize("dtype", [0, 1, 2])
-def test_one_launch_equals_three_calls_equals_the_oracle(dtype, block):
+def test_one_launch_equalsthree_calls_equals_the_oracle(dtype, block):
     from paper_2609_04609_b200 import ciera, runtime
 
     one, three = (guard(runtime.LayerCodec.from_tensors(SIZES, 1, NAME[dtype], block, DEV, slack=256)) for _ in range(2))
@@ -46,7 +40,7 @@ def test_one_launch_equals_three_calls_equals_the_oracle(dtype, block):
         launches0 = ciera.kernel_launch_count()
         one.step(dev[t])
         assert ciera.kernel_launch_count() - launches0 == 1
-        _three_calls(three, dev[t])
+        three_calls(three, dev[t])
         torch.cuda.synchronize()
         for codec in (one, three):
             codec.check_status()
@@ -58,7 +52,7 @@ def test_one_launch_equals_three_calls_equals_the_oracle(dtype, block):
     for codec in (one, three):
         ciera.cache_init(codec.plan, codec.receiver_cache, other)
     one.step(dev[1])
-    _three_calls(three, dev[1])
+    three_calls(three, dev[1])
     torch.cuda.synchronize()
     for codec in (one, three):
         codec.check_status()
@@ -105,7 +99,7 @@ def test_runs_of_short_units(dtype, block):
     bits = [wl.as_bits(x) for x in w]
     table.init_caches(bits[0])
     codec.init_caches(to_dev_bytes(bits[0], DEV))
-    for t, step in ((1, _three_calls), (0, lambda c, x: c.step(x))):
+    for t, step in ((1, three_calls), (0, one_launch)):
         exp = table.step(bits[t])
         step(codec, to_dev_bytes(bits[t], DEV))
         torch.cuda.synchronize()
@@ -169,7 +163,7 @@ def test_long_runs_cut(dtype, block):
     bits = [wl.as_bits(x) for x in w]
     table.init_caches(bits[0])
     codec.init_caches(to_dev_bytes(bits[0], DEV))
-    for t, step in ((1, _three_calls), (0, lambda c, x: c.step(x))):
+    for t, step in ((1, three_calls), (0, one_launch)):
         exp = table.step(bits[t])
         step(codec, to_dev_bytes(bits[t], DEV))
         torch.cuda.synchronize()
@@ -196,7 +190,7 @@ def test_receiver_with_other_exponents_many_times(dtype, block):
             codec.init_caches(a.view(torch.uint8))
             ciera.cache_init(codec.plan, codec.receiver_cache, other.view(torch.uint8))
         one.step(b.view(torch.uint8))
-        _three_calls(three, b.view(torch.uint8))
+        three_calls(three, b.view(torch.uint8))
         torch.cuda.synchronize()
         one.check_status()
         for u in one.units:
@@ -208,7 +202,7 @@ def test_receiver_with_other_exponents_many_times(dtype, block):
 @pytest.mark.parametrize("block", [1, 512])
 @pytest.mark.parametrize("dtype", [0, 1, 2])
 @pytest.mark.parametrize("where", ["weights - 64 KB", "weights + 16", "weights + 24 MB", "sent message"])
-def test_output_over_buffers_that_the_three_calls_are_done_with(dtype, block, where):
+def test_output_over_buffers_that_thethree_calls_are_done_with(dtype, block, where):
     """Where the reconstructed weights go over bytes that the sender has read or sent by then, a step does what the three
     calls do: the message holds the weights as they were."""
     from paper_2609_04609_b200 import runtime
@@ -266,7 +260,7 @@ def test_every_remainder_of_a_short_tile(dtype, block):
     guard(codec)  # (the bytes behind the cached exponents as well)
     if block >= 16:
         codec.init_hash_cache(to_dev_bytes(bits[0], DEV))
-    for t, step in ((1, _three_calls), (2, lambda c, x: c.step(x)), (3, _three_calls)):
+    for t, step in ((1, three_calls), (2, one_launch), (3, three_calls)):
         exp = table.step(bits[t])
         x = to_dev_bytes(bits[t], DEV)
         if block >= 16:  # the same message from the other sender, before the caches move on
@@ -313,7 +307,7 @@ def test_every_remainder_of_the_last_tile_of_a_buffer(dtype, shared):
         codec.allocations["sender_cache"][codec.cache_bytes :] = 0xEE
         codec.allocations["receiver_cache"][codec.cache_bytes :] = 0xEE
         room = torch.full((values * vb + 16,), 0xEE, dtype=torch.uint8, device=DEV)
-        for t, step in ((1, _three_calls), (2, lambda c, x: c.step(x))):
+        for t, step in ((1, three_calls), (2, one_launch)):
             exp = table.step(bits[t])
             room[: values * vb] = torch.from_numpy(bits[t].view(np.uint8).copy()).to(DEV)
             step(codec, room[: values * vb])
