@@ -15,7 +15,8 @@ the steps alternate between them (the set of changed exponents between A and B i
 both directions), so every step is a real encode against a cache left by the previous one and
 the K timed steps run back to back.
 
-Prints ONE JSON line (rank 0).  ``--impl reference`` times the CPU oracle instead.
+Prints ONE JSON line on stdout (rank 0); the side tables go to stderr, as a line of their own.  ``--impl reference`` times
+the CPU oracle instead.
 """
 from __future__ import annotations
 
@@ -385,7 +386,7 @@ def run_reference(args):
     gbps = nvals * vb / (ms * 1e-3) / 1e9
     total_units = len(shapes) * args.shards * args.layers
     sample = f"{n_units} of {total_units} units ({nvals} values) per step"
-    config = workload_config(args)
+    config = workload_config(args, oracle=True)
     config["workload"] += (f" -- each step of this arm is a sample of {n_units} of the {total_units} units; ms_per_step is "
                            f"the time of that sample, value (GB/s of weights) is what compares with the other arm")
     print(json.dumps({
@@ -398,7 +399,12 @@ def run_reference(args):
     }))
 
 
-def workload_config(args):
+def steps_in_one_launch(args):
+    """A layer's step is one launch (ciera_step) where nothing stands between sender and receiver."""
+    return not args.entropy and args.detect == "compare"
+
+
+def workload_config(args, oracle=False):
     full = args.layers == 16 and args.experts == 64 and args.shapes == "olmoe"
     upd = f"update model {args.update}" + (f" f={args.f}" if args.update == "clustered" else "") + (
         f" c={args.inject}" + (f" in segments of {args.inject_seg}" if args.inject_seg else "") if args.update == "inject" else "")
@@ -412,8 +418,12 @@ def workload_config(args):
     return {
         "workload": f"{what}, {args.shards} simulated shards per matrix, block {args.block}, {upd}",
         "l2": "inputs larger than L2 (no flush needed)",
-        "schedule": args.schedule,
-        "round_trip": "encode + device-to-device transport + decode",
+        "schedule": "host threads" if oracle else "one launch per layer, one after the other" if steps_in_one_launch(args)
+                    else args.schedule,
+        "round_trip": "encode + decode on the CPU" if oracle else
+                      "sender and receiver of a layer in one launch (ciera_step): the message is stored to both buffers as it is "
+                      "made and not read back; three_calls: encode + device-to-device transport + decode as launches of their own"
+                      if steps_in_one_launch(args) else "encode + device-to-device transport + decode",
         "change_detection": "exact comparison with a sender-side exponent cache" if args.detect == "compare"
                             else "128-bit hash per block (HashCache), the persistent kernel in its HashCache form",
     }
@@ -550,12 +560,21 @@ def main():
     for c in layers:
         c.check_status()
 
-    # ---- two steps with events around every kernel on the two streams (overlapped figures; with events between
-    #      them, sender, transport and receiver are launches of their own)
-    for _ in range(2):
+    # ---- the same K steps with events around every kernel on the two streams: sender, transport and receiver are
+    #      launches of their own then, as they are where the message goes to another rank
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    barrier()
+    t0.record(cur)
+    s_enc.wait_event(t0)
+    s_dec.wait_event(t0)
+    for _ in range(args.steps):
         pipe.step(weights_of(step_i), None, timers)
         step_i += 1
+    cur.wait_stream(s_enc)
+    cur.wait_stream(s_dec)
+    t1.record(cur)
     barrier()
+    three_ms = max_over_ranks(t0.elapsed_time(t1), world, device) / args.steps
 
     # ---- the same K steps once more on ONE stream: kernels do not overlap, so the CUDA events
     #      around each launch time that kernel alone (used for the roofline entries)
@@ -600,8 +619,7 @@ def main():
     dec_gbs = a_dec / (dec_ms * 1e-3) / 1e9
     tra_gbs = a_tra / (tra_ms * 1e-3) / 1e9
     # a layer of the timed step: where it is one launch, the message is written to both buffers and not read again
-    one_launch = not args.entropy and args.detect == "compare"
-    a_step = a_enc + a_dec + (0 if one_launch else a_tra)  # (the copy's write stands for the receiver's read)
+    a_step = a_enc + a_dec + (0 if steps_in_one_launch(args) else a_tra)  # (the copy's write stands for the receiver's read)
     path_gbs = len(layers) * a_step / (ms_per_step * 1e-3) / 1e9
 
     # ---- correctness at full size: exact round trip everywhere, oracle on sampled units
@@ -630,7 +648,7 @@ def main():
         coded = {"bytes_ratio_coded": coded_bytes / weight_bytes,
                  "entropy_encode_ms": ent_ms[0], "entropy_decode_ms": ent_ms[1],
                  "per": "layer launch, serial re-run",
-                 "note": "rANS of the changed exponents, static 12-bit model per unit; one block per unit"}
+                 "note": "rANS of the changed exponents, static 12-bit model per unit"}
 
     traffic, traffic_note = None, "no ncu capture on record for this workload"
     if args.dtype == "bf16" and args.block == 512 and args.update == "clustered" and args.f == 0.22 and args.shapes == "olmoe":
@@ -651,6 +669,8 @@ def main():
         "dtype": "u32",
         "data": "synthetic",
         "config": workload_config(args),
+        "three_calls": {"value": whole_job_gbps(world, weight_bytes, three_ms), "ms_per_step": three_ms,
+                        "per": "the same steps by encode, transport and decode on two streams"},
         "gpu_launches": int(launches),
         "clocks": clocks,
         "verified_bit_exact": verified,
@@ -664,7 +684,7 @@ def main():
         "kernel_ms": {"encode": enc_ms, "transport": tra_ms, "decode": dec_ms,
                       "per": "layer launch; serial re-run of the timed steps on one stream"},
         "kernel_ms_overlapped": {"encode": ovl_ms[0], "transport": ovl_ms[1], "decode": ovl_ms[2],
-                                 "per": "layer launch of two more steps on two streams (kernels overlap)"},
+                                 "per": "layer launch of the three_calls steps (kernels overlap)"},
         "serial_ms_per_step": serial_ms_per_step,
         "serial_step_ms_spread": step_spread,
         "kernel_ms_x_sm_mhz": ({"encode": enc_ms * clocks["sm_mhz"], "transport": tra_ms * clocks["sm_mhz"],
@@ -734,9 +754,16 @@ def main():
                                          f"encode+decode round trip, {dt:.2f} s wall on {threads} threads",
                                "single_thread_value": n1 * vb / d1 / 1e9}
     if rank == 0:
-        print(json.dumps(out))
+        # the line itself is short enough for whoever reads the end of a log; everything else goes to stderr
+        print(json.dumps({"bench_details": {k: v for k, v in out.items() if k not in HEADLINE_KEYS}}), file=sys.stderr, flush=True)
+        print(json.dumps({k: out[k] for k in HEADLINE_KEYS if k in out}), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+HEADLINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                 "dtype", "data", "config", "three_calls", "gpu_launches", "clocks", "verified_bit_exact", "oracle_sampled_units",
+                 "block_change_rate_q", "bytes_ratio", "kernel_ms", "roofline", "e2e", "cpu_baseline")
 
 
 # The other workloads of the build's configuration list, one layer each, kernels timed one after the other on one
@@ -784,16 +811,17 @@ def entropy_roofline(symbols, enc_ms, dec_ms, sm_mhz, sms=148):
         rec = json.load(open(TRAFFIC_FILE))["entropy_stage_bf16_B512_clustered_f0.22"]
     except Exception:
         return None
+    current = rec.get("csrc_sha256") == csrc_digest()
     peak = sms * 4 * (sm_mhz or 1965.0) * 1e6  # warp instructions per second
     out = {"bound": "issue", "unit": "G warp-instructions/s", "peak": peak / 1e9, "symbols_per_launch": symbols,
            "derivation": "148 SMs x 4 schedulers x 1 warp instruction per clock x sampled SM MHz"}
     for name, ms, key in (("encode", enc_ms, "warp_instructions_per_symbol_encode"),
                           ("decode", dec_ms, "warp_instructions_per_symbol_decode")):
-        ach = rec[key] * symbols / (ms * 1e-3)
-        out[name] = {"warp_instructions_per_symbol": rec[key], "achieved": ach / 1e9, "frac": ach / peak,
-                     "payload_GBps": symbols / (ms * 1e-3) / 1e9}
-    if rec.get("csrc_sha256") != csrc_digest():
-        out["note"] = "instruction counts per symbol are from an ncu capture of earlier kernel sources"
+        ach = rec[key] * symbols / (ms * 1e-3) if current else None
+        out[name] = {"warp_instructions_per_symbol": rec[key] if current else None, "achieved": ach / 1e9 if current else None,
+                     "frac": ach / peak if current else None, "payload_GBps": symbols / (ms * 1e-3) / 1e9}
+    if not current:
+        out["note"] = "kernel sources changed since the ncu capture on record; re-capture to fill this in"
     return out
 
 

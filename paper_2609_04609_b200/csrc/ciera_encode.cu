@@ -4,14 +4,16 @@
 // first.  A block first takes its share of the tiles of the longer units, spread tile by tile over
 // the blocks (block c takes tiles T0 + c, T0 + c + G, ...; neighbouring tiles of a unit are then
 // worked on by neighbouring blocks at about the same time, and their payload offsets come from a
-// single-pass look-back over per-tile status words; this part needs all blocks resident, so a
-// plan with longer units is launched cooperatively).  Then it works through the short units in runs
-// of four tiles, drawing the next run's number from a counter in the scratch (every unit's first run
-// goes out before any unit's second run, and so on): a tile's place in its unit's payload is then a
-// running sum inside the block, which a run that does not start its unit takes over from the status
-// word of the tile before it -- written many draws earlier -- and all SMs stay busy to the end
-// whatever their individual pace (with whole units of 16 tiles as the piece of work drawn, the blocks
-// finished up to a unit apart: 0.921 of the copy peak against 0.935).
+// single-pass look-back over per-tile status words; with more than one tile to a block this part
+// needs all blocks resident, so such a plan is launched cooperatively).  Then it works through the
+// short units in runs of their tiles -- a long first run, a last run of at most four (see
+// ciera_plan_create) --, drawing the next run's number from a counter in the scratch (every unit's
+// first run goes out before any unit's second run, and so on): a tile's place in its unit's payload
+// is then a running sum inside the block, which a run that does not start its unit takes over from
+// the status word of the tile before it -- written many draws earlier -- and all SMs stay busy to the
+// end whatever their individual pace (with whole units of 16 tiles as the piece of work drawn, the
+// blocks finished up to a unit apart: 0.921 of the copy peak against 0.935).  Tables with few tiles in
+// short units have all of their tiles spread (kSpreadShare).
 // A thread block has four roles:
 //
 //   producer warp   runs ahead of the others: for each of its tiles it fetches the tile
@@ -48,8 +50,8 @@
 // 11.1 bytes per bf16 value move.  Here every byte of a message is stored to both buffers as it is made, and the
 // consumers reconstruct a tile's weights from what travels (sign-plus-mantissa, exponents of changed blocks) and
 // the receiver's cached exponents while the tile is still in shared memory: 8.9 bytes.  Measured per OLMoE-shaped
-// layer, B = 512, q = 0.22: bf16 0.711 -> 0.579 ms (0.95 of the copy peak), fp32 1.500 -> 1.108 (0.94); every block
-// changed, bf16: 0.941 -> 0.719.
+// layer, B = 512, q = 0.22: bf16 0.694 -> 0.572 ms (0.93 of the copy peak), fp32 1.436 -> 1.084 (0.94); every block
+// changed, bf16: 0.933 -> 0.724.
 #include <cstddef>
 #include <type_traits>
 
@@ -64,9 +66,10 @@ constexpr int kResolvers = 2;  // resolver warps (20 warps per block: two blocks
 // Consumer warps of a block, and how they share a tile.  With HashCache and 2-byte values, where the kernel is bound by
 // instruction issue, 8 warps take four pieces a thread: what a warp spends on a tile as such (waits, addresses, sending)
 // is spent half as often, and a warp's pieces are rows of 256 neighbouring values, so that rows of one block are added
-// up in registers before anything is exchanged between lanes: OLMoE-shaped layer 0.355 -> 0.302 ms with 512 values per
-// block, 0.400 -> 0.356 with 64, 0.393 -> 0.309 with 4096.  (Three blocks per SM instead of two: 0.297, 0.376, 0.306, and
-// small tables 8-15 % slower.  HASH == 3, whose consumers finish the hashes themselves, 0.494 -> 0.585: it keeps 16.)
+// up in registers before anything is exchanged between lanes: OLMoE-shaped layer 0.357 -> 0.305 ms with 512 values per
+// block (0.311 with inputs changing from pass to pass), 0.399 -> 0.361 with 64, 0.397 -> 0.319 with 4096.  (Three blocks per
+// SM instead of two: 2 % faster with 512 values per block, 5 % slower with 64, small tables 8-15 % slower.  HASH == 3, whose
+// consumers finish the hashes themselves, 0.494 -> 0.585: it keeps 16.)
 template <int DT, int HASH>
 constexpr int kConsumerWarps = (HASH == 1 || HASH == 2) && DT != CIERA_FP32 ? 8 : kWarps;
 template <int DT, int HASH>

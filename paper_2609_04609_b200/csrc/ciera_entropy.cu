@@ -149,9 +149,11 @@ __device__ __forceinline__ void normalise_model(const uint32_t* h, uint64_t P, u
 // m = floor(P / f) and e = (m + 1) * f - P:
 //   f = 1                     m = 2^32 - 1 gives x - 1 (x > 0), the missing 1 * (4096 - f) goes into c
 //   f a power of two          m = 2^31, shift s - 1
-//   f * 2^20 * e <= P         q = ((m + 1) * x) / P, the round-up reciprocal (all f < 2^11, most others)
-//   else                      q = (m * (x + 1)) / P, the round-down one: exact if f * 2^20 * (f - e) <= P, which
-//                             follows from e > P / (f * 2^20) >= 2^23 / f for 2^11 < f < 2^12
+//   f * 2^20 * e <= P         q = ((m + 1) * x) / P, the round-up reciprocal (all f < 2^11, most others; Granlund and
+//                             Montgomery, Division by Invariant Integers using Multiplication, 1994)
+//   else                      q = (m * (x + 1)) / P, the round-down one (Robison, N-Bit Unsigned Division via N-Bit
+//                             Multiply-Add, 2005): exact if f * 2^20 * (f - e) <= P, which follows from
+//                             e > P / (f * 2^20) >= 2^23 / f for 2^11 < f < 2^12
 // At most one symbol is of the last kind; whether there is one comes back (the same in all threads).  An entry of 16
 // bytes holds what a coder step needs:
 //   {multiplier, largest x below f * 2^20, c, (4096 - f) << 5 | shift, bit 31: x + 1}

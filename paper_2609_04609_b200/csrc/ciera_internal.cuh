@@ -154,7 +154,9 @@ constexpr uint32_t kSeqMaxTiles = 32;
 // encode kernel spreads all tiles of such a table.  197 = 2/3 of the 296 thread blocks that a B200
 // holds, where the two ways cross.  Whole step, bf16, units of 16 tiles, in runs / spread: 64 tiles 26.4 / 7.7 us,
 // 768 tiles 26.2 / 12.9, 2048 tiles 40.0 / 34.6, 3072 tiles 47.1 / 50.0, 49152 tiles 570 / 625; units of 32 tiles:
-// 1536 tiles 50.4 / 23.5, 4096 tiles 76.5 / 63.0.
+// 1536 tiles 50.4 / 23.5, 4096 tiles 76.5 / 63.0.  (Measured on the bf16 step, which has 296 blocks; the plan does not know
+// which kernel will run.  The fp32 step has 148, so its ways cross at half as many tiles, which has not been measured; of 78
+// tables in all precisions none is slower than with runs only, the hashed sender's included.)
 constexpr uint32_t kSpreadShare = 197;
 constexpr uint32_t kEncodeBlocks = 296;  // the encode kernel's thread blocks on a B200, two on each of 148 SMs
 constexpr uint32_t kRunsPerBlock = 8;    // runs of short units to a block below which long runs are cut (ciera_plan_create)
