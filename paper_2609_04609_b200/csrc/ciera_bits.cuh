@@ -274,6 +274,11 @@ struct Piece<CIERA_BF16> {
             w[i] = bitselect(0x7F807F80u, __byte_perm(e[i >> 1], 0u, (i & 1) ? 0x4342u : 0x4140u) << 7, w[i]);
     }
     static __device__ __forceinline__ void load_weights(const uint8_t* src, uint32_t (&w)[kWeightWords]) { load_16_bytes(src, w); }
+    // the exponents of a piece's weights
+    __device__ __forceinline__ void exponents_of(const uint32_t (&w)[kWeightWords]) {
+        bf16_split4(w[0], w[1], e[0], s[0]);
+        bf16_split4(w[2], w[3], e[1], s[1]);
+    }
     template <class M>
     static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
         M::st16(dst, make_uint4(w[0], w[1], w[2], w[3]));
@@ -414,6 +419,11 @@ struct Piece<CIERA_FP32> {
 #pragma unroll
         for (int i = 0; i < 4; ++i) load_16_bytes(src + 16 * i, w + 4 * i);
     }
+    // the exponents of a piece's weights
+    __device__ __forceinline__ void exponents_of(const uint32_t (&w)[kWeightWords]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e[i] = fp32_exp4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+    }
     template <class M>
     static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
 #pragma unroll
@@ -496,6 +506,8 @@ struct Piece<CIERA_FP16> {
         for (int i = 0; i < 4; ++i) w[i] = (w[i] & 0x83FF83FFu) | exponent_bits(i);
     }
     static __device__ __forceinline__ void load_weights(const uint8_t* src, uint32_t (&w)[kWeightWords]) { load_16_bytes(src, w); }
+    // the exponents of a piece's weights
+    __device__ __forceinline__ void exponents_of(const uint32_t (&w)[kWeightWords]) { split_words(w); }
     template <class M>
     static __device__ __forceinline__ void store_weights(uint8_t* dst, const uint32_t (&w)[kWeightWords]) {
         M::st16(dst, make_uint4(w[0], w[1], w[2], w[3]));

@@ -218,13 +218,27 @@ struct EncodeStepCfg<CIERA_FP32, true> {
     static constexpr int kDefer = 2;
     static constexpr int kBmWords = kFineBitmapWords;
 };
+// LONG, the whole step on tables of long units (coarse blocks).  What bounds these tables is not memory but that every tile waits
+// for the votes of all tiles before it in its unit: loads take 3 to 12 us when hundreds of tiles are in flight, and blocks
+// that were two tiles from their oldest unsent payload stood still for the slowest (one tensor of 2^28 bf16 values on 4 shards:
+// 477 us, with made-up offsets 414, and 370 if in addition blocks may take tiles at their own pace).  So the exponents' ring only
+// holds the cached ones until they are compared, both caches are refreshed as soon as a tile's flags are there, its payload goes
+// out kDefer tiles later from the cache (see FromCache), tiles are drawn (see TileWalk), and the look-back reads groups: 394 us,
+// 0.90 of the copy peak.  Where offsets need no look-back, in runs of short units, the other instance stays 1 % ahead.
+template <int DT>
+struct EncodeLongCfg {
+    static constexpr int kWStages = DT == CIERA_FP32 ? 4 : 3;
+    static constexpr int kEStages = DT == CIERA_FP32 ? 4 : 3;
+    static constexpr int kDefer = 6;
+    static constexpr int kBmWords = kBitmapWords;
+};
 template <int DT, bool STEP>
 constexpr int kEncodeBlocksPerSM = STEP && DT == CIERA_FP32 ? 1 : 2;
 // Values of changed blocks from which a tile counts as dense, rounded down to whole blocks: three of four with 2048 values per
 // block and one of two with 4096, where pieces that are missing lie in long stretches.  (Half an OLMoE-shaped layer, 0.57 of
 // the blocks of 4096 changed: bf16 331 us, 338 with two of two; fp32 581 and 590; 2048, 0.59 changed, 338 and 342.)
 constexpr uint32_t kDenseValues = (uint32_t)kTileValues / 8u * 7u;
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH, bool STEP, bool LONG = false>
 struct EncodeCfgOf {
     using type = EncodeHashCfg<DT, HASH>;
 };
@@ -236,6 +250,14 @@ template <int DT, bool FINE>
 struct EncodeCfgOf<DT, FINE, 0, true> {
     using type = EncodeStepCfg<DT, FINE>;
 };
+template <int DT>
+struct EncodeCfgOf<DT, false, 0, true, true> {
+    using type = EncodeLongCfg<DT>;
+};
+// A tile's votes, flags and offset live in a ring of their own; it is as long as the ring of exponents, which waits for the
+// sending too, but for LONG.
+template <class Cfg, bool LONG>
+constexpr int kResultStages = LONG ? Cfg::kDefer + 1 : Cfg::kEStages;
 
 // Distances, in bytes, from the sender's buffers to their counterparts on the receiver's side (STEP; else unused):
 // unit layouts are the same on both sides, so one distance serves a whole buffer.
@@ -304,24 +326,24 @@ __device__ __noinline__ void stage_buffer_end(uint8_t* st_w, const uint8_t* w, u
     mbar_arrive(bar);
 }
 
-template <int SW, int SE, int BW>
+template <int SW, int SE, int SR, int BW>
 struct EncodeCtl {
     uint64_t full_w[SW];    // weights tile landed
     uint64_t empty_w[SW];   // all 16 consumer warps have read it
     uint64_t full_e[SE];    // cached-exponent tile landed
-    uint64_t voted[SE];     // all 16 consumer warps have left their exponents there and voted
-    uint64_t summed[SE];    // aggregator has published the tile's status and block flags
-    uint64_t resolved[SE];  // a resolver knows the tile's offset in the unit's payload
+    uint64_t voted[SR];     // all 16 consumer warps have left their exponents there and voted
+    uint64_t summed[SR];    // aggregator has published the tile's status and block flags
+    uint64_t resolved[SR];  // a resolver knows the tile's offset in the unit's payload
     uint64_t empty_e[SE];   // all 16 consumer warps have sent the tile's changed exponents
     TileDesc desc[kDescRing];
     EncodeTileInfo info[kDescRing];
     uint32_t tile_idx[kDescRing];  // table index of the tile in desc[]; kNoTile = end marker
     uint32_t seq[kDescRing];       // kSeq* bits: tile of a run that this block works through alone, first / last of the run
-    uint32_t ballot[SE][kVoteWords];  // coarse blocks: "my piece differs" votes
-    uint32_t bm[SE][BW];              // block flags of the tile (16-byte aligned: checked where the kernel starts)
-    uint16_t pre[SE][BW];             // set flags before each word of bm
-    unsigned long long agg[SE];
-    unsigned long long base[SE];
+    uint32_t ballot[SR][kVoteWords];  // coarse blocks: "my piece differs" votes
+    uint32_t bm[SR][BW];              // block flags of the tile (16-byte aligned: checked where the kernel starts)
+    uint16_t pre[SR][BW];             // set flags before each word of bm
+    unsigned long long agg[SR];
+    unsigned long long base[SR];
     int abort;
     uint32_t issued;  // tiles whose loads have been started (producer)
     uint32_t seen;    // tiles whose loads the consumers have seen complete
@@ -341,7 +363,10 @@ constexpr uint32_t kSeqTile = 1u, kSeqRunStart = 2u, kSeqRunEnd = 4u;
 // back to zero for the next launch.  The walk keeps two runs in hand besides the current one: the number of
 // the run after next (its draw is on its way) and the table entry of the next run (its load is on its way), so
 // that at the start of a run neither the counter nor the table is waited for.
-template <bool ORDERED>  // the spread tiles may be given by their places in a list (steps in parts)
+// DRAWN (LONG): a block's spread tiles after the second are drawn from a counter of their own, from exactly n_spread - G times,
+// so that blocks may work at their own pace; a tile is drawn when the loads of the one before it have been started, not
+// earlier, since all later tiles of its unit wait for its votes.
+template <bool ORDERED, bool DRAWN>  // ORDERED: the spread tiles may be given by their places in a list (steps in parts)
 struct TileWalk {
     const uint2* seq_runs;
     const uint32_t* order;  // not null: the spread tiles are given by their places in this list
@@ -351,12 +376,14 @@ struct TileWalk {
     uint2 next_range;        // the next run's tiles (valid if next_run < n_runs)
     uint32_t next_run;       // number of the next run
     uint32_t after_run;      // number of the run after that
-    uint32_t spread_tile;    // next spread tile of this block
+    uint32_t spread_tile;    // next spread tile of this block, or its number as drawn
+    uint32_t first_drawn;    // DRAWN: the tile with drawn number 0
+    uint32_t taken;          // DRAWN: spread tiles so far
     bool spread;
 
     __device__ TileWalk(const uint2* runs, const uint32_t* places, unsigned int* ticket, uint32_t nruns, uint32_t spread_first, uint32_t nt,
                         uint32_t grid, uint32_t block)
-        : seq_runs(runs), order(places), run_ticket(ticket), n_tiles(nt), n_runs(nruns), G(grid), tile(0), end(0), spread(true) {
+        : seq_runs(runs), order(places), run_ticket(ticket), n_tiles(nt), n_runs(nruns), G(grid), tile(0), end(0), first_drawn(spread_first + 2u * grid), taken(0), spread(true) {
         spread_tile = spread_first + block;  // tiles of longer units start after the short units' tiles
         next_run = block;
         after_run = block + grid;
@@ -371,10 +398,16 @@ struct TileWalk {
     // next tile, or kNoTile; `seq` gets the kSeq* bits of the tile
     __device__ uint32_t next(uint32_t& seq) {
         if (spread) {
-            if (spread_tile < n_tiles) {
+            uint32_t at = spread_tile;
+            if (DRAWN && taken >= 2u) {
+                at += first_drawn;
+                if (at + 1u == n_tiles + G) atomicExch(run_ticket + 2, 0u);  // that was the launch's last draw
+            }
+            if (at < n_tiles) {
                 seq = 0;
-                const uint32_t t = ORDERED && order ? __ldg(order + spread_tile) : spread_tile;
-                spread_tile += G;
+                const uint32_t t = ORDERED && order ? __ldg(order + at) : at;
+                spread_tile = !DRAWN || taken == 0u ? at + G : atomicAdd(run_ticket + 2, 1u);
+                if (DRAWN) ++taken;
                 return t;
             }
             spread = false;
@@ -392,6 +425,8 @@ struct TileWalk {
         if (tile + 1u == end) seq |= kSeqRunEnd;
         return tile++;
     }
+    // the tile that next() returned is a spread one, and the next one has been drawn: it is fetched late
+    __device__ bool late() const { return DRAWN && spread && taken >= 2u; }
 };
 
 // Fine blocks: the consumers have written the block flags themselves; fills pre (set bits before
@@ -658,10 +693,10 @@ struct HashTile {
     ulonglong2* dst;
 };
 
-template <int DT, bool FINE, int HASH>
+template <int DT, bool FINE, int HASH, class WORD>
 __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, bool publish,
                                                    const uint32_t* ballot, uint32_t* bm, uint16_t* pre,
-                                                   unsigned long long* tile_status, const HashTile& ht, uint32_t nv,
+                                                   WORD* tile_status, unsigned long long* groups, const HashTile& ht, uint32_t nv,
                                                    uint32_t lane) {
     const uint32_t B = 1u << log2b;
     const uint32_t nbt = kTileValues >> log2b;
@@ -681,10 +716,14 @@ __device__ __forceinline__ uint64_t aggregate_tile(const TileDesc& td, uint32_t 
         if ((bm[kb >> 5] >> (kb & 31u)) & 1u) agg -= block_payload_bytes(B, DT) - block_payload_bytes(rem, DT);
     }
     if (publish) {
-        // a unit's first tile knows its prefix (0) already
         const uint32_t mybits = nbt < 8 ? bm[0] : 0u;
-        const unsigned long long flag = td.tile_in_unit == 0 ? kFlagPrefix : kFlagAggregate;
-        if (lane == 0) st_status(tile_status + tile, flag | ((unsigned long long)mybits << kBitsShift) | agg);
+        if constexpr (sizeof(WORD) == 4) {
+            if (lane == 0) report_tile(tile_status, groups, td, tile, mybits, (uint32_t)agg);
+        } else {
+            // a unit's first tile knows its prefix (0) already
+            const unsigned long long flag = td.tile_in_unit == 0 ? kFlagPrefix : kFlagAggregate;
+            if (lane == 0) st_status(tile_status + tile, flag | ((unsigned long long)mybits << kBitsShift) | agg);
+        }
     }
     return agg;
 }
@@ -724,15 +763,14 @@ __device__ __forceinline__ void store_bitmap(uint8_t* dst, uint32_t word, uint32
 }
 
 // payload <- exponents of changed blocks in block order; cache refreshed for the same blocks.
-// Every consumer thread sends the exponents of its own pieces (left in the stage's shared-memory
-// tile) if their block changed; `base` is the tile's exclusive offset in the unit's payload.
-// (CACHE = false, the sender with HashCache: payload only.)
+// Every consumer thread sends the exponents of its own pieces if their block changed; `source(x, p, t0, nvalid)` puts those of
+// piece p into x, and `base` is the tile's exclusive offset in the unit's payload.
+// (CACHE = false, the sender with HashCache, and LONG: payload only.)
 // (FULL: the tile is a full one, every piece complete.)
 // (STEP: the same bytes also go to the received message and to the receiver's cache.)
-template <int DT, bool CACHE, bool FULL, bool STEP, class SHARE>
+template <int DT, bool CACHE, bool FULL, bool STEP, class SHARE, class SOURCE>
 __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm,
-                                              const uint16_t* pre, uint64_t base, const uint8_t* s_exp, const StepTwins& tw,
-                                              uint32_t tid) {
+                                              const uint16_t* pre, uint64_t base, const StepTwins& tw, uint32_t tid, SOURCE source) {
     using P = Piece<DT>;
 #pragma unroll
     for (int p = 0; p < SHARE::kPerThread; ++p) {
@@ -752,7 +790,7 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
             if (log2b >= 5u) {
                 if (!__any_sync(0xffffffffu, changed)) continue;
                 P x;
-                x.template load_exp_full<Shared>(s_exp + t0);
+                source(x, p, t0, nvalid);
                 uint32_t lo, hi;
                 x.pack_exponents(lo, hi);
                 const uint32_t top = __funnelshift_r(lo, hi, 8);  // bits 39:8
@@ -768,6 +806,7 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
                 uint32_t* const twin = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dst) + tw.msg);
                 __stcs(twin, own);
                 if (a == 3u) __stcs(twin + 1, top);
+                if (!CACHE) continue;
                 x.template store_exp_full<Global>(ti.c_ptr + t0);
                 x.template store_exp_full<Global>(ti.c_ptr + t0 + tw.cache);
                 continue;
@@ -777,7 +816,7 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
         const uint32_t rank = pre[kb >> 5] + __popc(word & ((1u << (kb & 31u)) - 1u));
         uint8_t* cdst = ti.c_ptr + t0;
         P x;
-        x.template load_exp_full<Shared>(s_exp + t0);
+        source(x, p, t0, nvalid);
         if constexpr (DT == CIERA_FP16) {
             // blocks of 16 values, short tiles: five packed bytes per piece (fewer for the last one), byte by byte
             uint8_t* pdst = ti.pay_dst + base + payload_bytes_of_blocks<DT>(rank, log2b) +
@@ -804,18 +843,57 @@ __device__ __forceinline__ void write_changed(const EncodeTileInfo& ti, uint32_t
             if (CACHE) x.template store_exp_full<Global>(cdst);
             if (STEP) {
                 x.template store_exp_full<Global>(pdst + tw.msg);
-                x.template store_exp_full<Global>(cdst + tw.cache);
+                if (CACHE) x.template store_exp_full<Global>(cdst + tw.cache);
             }
         } else {
             x.store_exp_partial(pdst, nvalid);
             if (CACHE) x.store_exp_partial(cdst, nvalid);
             if (STEP) {
                 x.store_exp_partial(pdst + tw.msg, nvalid);
-                x.store_exp_partial(cdst + tw.cache, nvalid);
+                if (CACHE) x.store_exp_partial(cdst + tw.cache, nvalid);
             }
         }
     }
 }
+
+// Sources of write_changed.  Of a stage in shared memory: new exponents or, LONG, the weights.
+template <int DT, bool LONG>
+__device__ __forceinline__ auto from_stage(const uint8_t* stage) {
+    return [stage](Piece<DT>& x, int, uint32_t t0, int nvalid) {
+        using P = Piece<DT>;
+        if (LONG && nvalid != P::kValues) {
+            x.split_first(stage + (size_t)t0 * Traits<DT>::kValueBytes, nvalid);
+        } else if constexpr (LONG) {
+            uint32_t w[P::kWeightWords];
+            P::load_weights(stage + (size_t)t0 * Traits<DT>::kValueBytes, w);
+            x.exponents_of(w);
+        } else {
+            x.template load_exp_full<Shared>(stage + t0);
+        }
+    };
+}
+// LONG: of the refreshed cache, where the same thread has put them (they are in L2 still), fetched ahead of the sending.
+template <int DT>
+struct FromCache {
+    Piece<DT> x[Piece<DT>::kPerThread];
+    __device__ __forceinline__ void fetch(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm, uint32_t tid) {
+        using P = Piece<DT>;
+#pragma unroll
+        for (int p = 0; p < P::kPerThread; ++p) {
+            const uint32_t t0 = P::start(tid, p), kb = t0 >> log2b;
+            const int nvalid = piece_valid<DT>(t0, ti.nv);
+            if (nvalid == 0 || !((bm[kb >> 5] >> (kb & 31u)) & 1u)) continue;
+            if (nvalid == P::kValues)
+                x[p].template load_exp_full<Global>(ti.c_ptr + t0);
+            else
+                x[p].load_exp_partial(ti.c_ptr + t0, nvalid);
+        }
+    }
+    __device__ __forceinline__ void operator()(Piece<DT>& to, int p, uint32_t, int) const {
+#pragma unroll
+        for (int i = 0; i < Piece<DT>::kExpWords; ++i) to.e[i] = x[p].e[i];
+    }
+};
 
 // STEP, fp32: one warp's 2 KB of reconstructed weights from the stage to global memory (one thread).
 __device__ __forceinline__ void bulk_store_tile_part(const EncodeTileInfo& ti, const StepTwins& tw, const uint8_t* s_w,
@@ -828,9 +906,10 @@ __device__ __forceinline__ void bulk_store_tile_part(const EncodeTileInfo& ti, c
 // STEP, coarse blocks: the receiver's part of one tile.  Every consumer thread takes its pieces of the tile once
 // more (the stage still holds the weights: sign and mantissa as they travel, and the exponents of changed blocks as
 // they travel in the payload), puts the receiver's cached exponents of the unchanged blocks into their places and
-// stores the reconstructed weights.  (The receiver's cache of changed blocks is refreshed by write_changed.)
+// stores the reconstructed weights.  (Changed blocks: both caches are refreshed here, LONG, or by
+// write_changed.)
 // BULK: the thread's weights are left in their place of the stage instead.
-template <int DT, bool FULL, bool BULK>
+template <int DT, bool FULL, bool BULK, bool LONG>
 __device__ __forceinline__ void reconstruct(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm, uint8_t* s_w,
                                             const uint8_t* s_r, const StepTwins& tw, uint32_t tid) {
     using P = Piece<DT>;
@@ -855,8 +934,20 @@ __device__ __forceinline__ void reconstruct(const EncodeTileInfo& ti, uint32_t l
                 x.load_exp_partial(r, nvalid);
             x.exchange(s_w + (size_t)t0 * VB, w);
             if (BULK) P::template store_weights<Shared>(s_w + (size_t)t0 * VB, w);
-        } else if (!BULK) {
+        } else if (LONG || !BULK) {
             P::load_weights(s_w + (size_t)t0 * VB, w);
+            if (LONG) {
+                P x;
+                x.exponents_of(w);
+                uint8_t* const c = ti.c_ptr + t0;
+                if (nvalid == P::kValues) {
+                    x.template store_exp_full<Global>(c);
+                    x.template store_exp_full<Global>(c + tw.cache);
+                } else {
+                    x.store_exp_partial(c, nvalid);
+                    x.store_exp_partial(c + tw.cache, nvalid);
+                }
+            }
         }
         if (BULK) continue;
         if (nvalid == P::kValues)
@@ -1036,7 +1127,7 @@ __device__ __forceinline__ void write_changed_fine_full(const EncodeTileInfo& ti
     __syncwarp();  // the gather space is free again
 }
 
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH, bool STEP, bool LONG>
 __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t log2b, const uint32_t* bm,
                                              const uint16_t* pre, uint64_t base, uint32_t tile_payload_bytes,
                                              const uint8_t* s_exp, uint8_t* s_gather, const StepTwins& tw,
@@ -1045,9 +1136,11 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
         // (as in the consumers' main loop: the two instances named there keep the one form that tests as it goes)
         constexpr bool kOneBody = (DT == CIERA_BF16 && HASH == 0 && !STEP) || (DT == CIERA_FP32 && HASH != 0);
         if (!kOneBody && ti.nv == (uint32_t)kTileValues)
-            write_changed<DT, HASH == 0, true, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
+            write_changed<DT, HASH == 0 && !LONG, true, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, tw, tid,
+                                                                                                from_stage<DT, LONG>(s_exp));
         else
-            write_changed<DT, HASH == 0, false, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, s_exp, tw, tid);
+            write_changed<DT, HASH == 0 && !LONG, false, STEP, Share<DT, kConsumerWarps<DT, HASH>>>(ti, log2b, bm, pre, base, tw, tid,
+                                                                                                 from_stage<DT, LONG>(s_exp));
     } else if ((STEP || DT != CIERA_FP16) && ti.nv == (uint32_t)kTileValues && tile_payload_bytes >= (uint32_t)kTileValues / kGatherDensity) {
         // a full tile in which many exponents changed: gathered in shared memory, written out in whole pieces
         switch (log2b) {
@@ -1070,39 +1163,44 @@ __device__ __forceinline__ void send_changed(const EncodeTileInfo& ti, uint32_t 
 // tables in a LayerPipeline 28.0 -> 29.3 us.)  per_tile: with STEP the list of tiles by address or null, with HASH `tile_hash`.
 // `cache` is the sender's exponent cache or, with HASH, its HashCache; `tile_hash` (HASH only) gives
 // the index of every tile's first block in it.
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH, bool STEP, bool LONG>
 __global__ void __launch_bounds__(kEncodeThreads<DT, HASH>, kEncodeBlocksPerSM<DT, STEP>)
 encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
               uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
-              unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
-              unsigned int* unit_ticket, unsigned int* blocks_done, int32_t* status,
+              unsigned long long* wire_bytes, uint32_t* changed_blocks, void* status_words,
+              unsigned long long* groups, unsigned int* counters, int32_t* status,
               const void* __restrict__ per_tile, StepTwins tw, BufferEnds ends) {
     const uint32_t* const order = STEP ? static_cast<const uint32_t*>(per_tile) : nullptr;
     const unsigned long long* const tile_hash = HASH ? static_cast<const unsigned long long*>(per_tile) : nullptr;
+    using Word = std::conditional_t<LONG, uint32_t, unsigned long long>;
+    Word* const tile_status = static_cast<Word*>(status_words);
+    unsigned int* const blocks_done = counters + 1;
     static_assert(!(HASH && FINE), "HashCache: blocks of 16 values and more");
+    static_assert(!LONG || (STEP && !FINE), "long units: the whole step with coarse blocks");
     static_assert(!(HASH && STEP), "the whole step compares with the exponent cache");
     using P = Piece<DT>;
     constexpr int CW = kConsumerWarps<DT, HASH>;
     using S = Share<DT, CW>;
     constexpr int VB = Traits<DT>::kValueBytes;
     constexpr int SMB = Traits<DT>::kSmBytes;
-    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
+    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP, LONG>::type;
     constexpr int SW = Cfg::kWStages;
     constexpr int SE = Cfg::kEStages;
+    constexpr int SR = kResultStages<Cfg, LONG>;
     constexpr int kDefer = Cfg::kDefer;
     // coarse blocks: a tile's weights are reconstructed one slot after its votes, when its block flags are there
     constexpr bool kRebuild = STEP && !FINE;
     // fp32: the reconstructed weights of a full tile leave the stage by one bulk store per warp (64 bytes per lane
     // scatter over the stores of a warp)
     constexpr bool kBulkOut = STEP && DT == CIERA_FP32;
-    static_assert(kDescRing > SE + 2 && SE > kDefer, "ring depths");
+    static_assert(kDescRing > (LONG ? SW + SR : SE) + 2 && SR > kDefer && SR >= SW && (LONG || SE == SR), "ring depths");
     constexpr uint32_t kWBytes = kTileValues * VB;
     constexpr uint32_t kEBytes = kTileValues;
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t* const ring_w = smem;
     constexpr uint32_t kWStage = kWBytes + (STEP ? kEBytes : 0u);  // STEP: then the receiver's cached exponents
     uint8_t* const ring_e = smem + (size_t)SW * kWStage;
-    using Ctl = EncodeCtl<SW, SE, Cfg::kBmWords>;
+    using Ctl = EncodeCtl<SW, SE, SR, Cfg::kBmWords>;
     Ctl* ctl = reinterpret_cast<Ctl*>(ring_e + (size_t)SE * kEBytes);
     // HASH: per stage of the exponent ring, the tile's cached hashes and then the partial sums
     static_assert(sizeof(Ctl) % 16 == 0, "the hash stages follow the control block");
@@ -1124,10 +1222,12 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         }
         for (int s = 0; s < SE; ++s) {
             mbar_init(&ctl->full_e[s], 1);
+            mbar_init(&ctl->empty_e[s], CW);
+        }
+        for (int s = 0; s < SR; ++s) {
             mbar_init(&ctl->voted[s], CW);
             mbar_init(&ctl->summed[s], 1);
             mbar_init(&ctl->resolved[s], 1);
-            mbar_init(&ctl->empty_e[s], CW);
         }
         ctl->abort = 0;
         ctl->issued = 0;
@@ -1143,7 +1243,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     if (warp == (uint32_t)CW) {
         // ---------------------------------------------------------------- producer
         if (lane == 0) {
-            TileWalk<STEP> walk(seq_runs, order, unit_ticket, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
+            TileWalk<STEP, LONG> walk(seq_runs, order, counters, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
             uint32_t tile_nxt = walk.next(seq_nxt);
             TileDesc nxt;
@@ -1158,13 +1258,15 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 const uint32_t tile = tile_nxt;
                 const uint32_t seq = seq_nxt;
                 const unsigned long long hb = hb_nxt;
-                if (tile != kNoTile) {
+                auto fetch = [&]() {
                     tile_nxt = walk.next(seq_nxt);
                     if (tile_nxt != kNoTile) {
                         nxt = load_tile_desc(tiles + tile_nxt);
                         if (HASH) hb_nxt = __ldg(tile_hash + tile_nxt);
                     }
-                }
+                };
+                const bool late = walk.late();
+                if (tile != kNoTile && !late) fetch();
                 const uint32_t sw = k % SW, se = k % SE;
                 if (k >= (uint32_t)SW && !mbar_wait(&ctl->empty_w[sw], ((k / SW) & 1u) ^ 1u, abort, status)) break;
                 if (k >= (uint32_t)SE && !mbar_wait(&ctl->empty_e[se], ((k / SE) & 1u) ^ 1u, abort, status)) break;
@@ -1188,10 +1290,10 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     ti.c_ptr = HASH ? cache + hb * 16ull : cache + td.c_off;
                     ti.w_src = weights + td.w_off;
                     ti.nv = (uint32_t)min((uint64_t)kTileValues, left);
-                    // Only unchanged blocks need the receiver's cached exponents.  Where the tile that this stage held
+                    // Only unchanged blocks need the receiver's cached exponents.  Where the tile one ring of stages
                     // before was dense (see kDenseValues) they are not staged: with every block changed that is 1 byte
                     // of 12 per value that need not be read.
-                    r_staged = FINE || k < (uint32_t)SE || ctl->agg[se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
+                    r_staged = FINE || k < (uint32_t)(LONG ? SW : SE) || ctl->agg[LONG ? (k - SW) % SR : se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
                     ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
                 }
@@ -1222,6 +1324,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     bulk_load(ring_h + (size_t)se * kHStage, cache + hb * 16ull, nblk * 16u, &ctl->full_e[se]);
                 }
                 ctl->issued = k + 1;
+                if (late) fetch();
             }
             cp_async_wait_all();  // (an aborted run: none in flight when the block ends)
         }
@@ -1231,11 +1334,11 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         uint32_t byte_acc = 0;  // its bitmap byte in the making (tiles of fewer than 8 blocks)
         uint32_t markers = 0;
         for (uint32_t k = 0;; ++k) {
-            const uint32_t se = k % SE;
-            if (!mbar_wait(&ctl->voted[se], (k / SE) & 1u, abort, status)) break;
+            const uint32_t se = k % SE, sr = k % SR;
+            if (!mbar_wait(&ctl->voted[sr], (k / SR) & 1u, abort, status)) break;
             const uint32_t tile = ctl->tile_idx[k % kDescRing];
             if (tile == kNoTile) {  // pass the end marker on to the resolver in charge of slot k
-                if (lane == 0) mbar_arrive(&ctl->summed[se]);
+                if (lane == 0) mbar_arrive(&ctl->summed[sr]);
                 if (++markers == (uint32_t)kResolvers) break;
                 continue;
             }
@@ -1256,8 +1359,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             const bool last = td.tile_in_unit == td.n_tiles_unit - 1u;
             uint8_t* const msg = msgs + td.msg_off;
             uint8_t* const bitmap_dst = msg + (uint64_t)td.tile_in_unit * (nbt >> 3);
-            const uint64_t agg = aggregate_tile<DT, FINE, HASH>(td, tile, log2b, !seq, ctl->ballot[se], ctl->bm[se], ctl->pre[se],
-                                                                tile_status, ht, nv, lane);
+            const uint64_t agg = aggregate_tile<DT, FINE, HASH>(td, tile, log2b, !seq, ctl->ballot[sr], ctl->bm[sr], ctl->pre[sr],
+                                                                tile_status, groups, ht, nv, lane);
             uint64_t excl = 0;
             if (seq) {
                 // the run is this block's: the tile's offset is the running sum; a run that does not start its
@@ -1268,12 +1371,12 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if (td.tile_in_unit == 0)
                     excl = 0;
                 else if (seq_bits & kSeqRunStart) {
-                    excl = wait_status(tile_status + tile - 1, status) & kValueMask;
+                    excl = wait_status(tile_status + tile - 1, status) & (LONG ? (Word)kShortValueMask : (Word)kValueMask);
                     __syncwarp();
-                    if (lane == 0) st_status(tile_status + tile - 1, 0ull);  // its one reader leaves the word empty again
+                    if (lane == 0) st_status(tile_status + tile - 1, (Word)0);  // its one reader leaves the word empty again
                 }
                 run_incl = excl + agg;
-                if ((seq_bits & kSeqRunEnd) && !last && lane == 0) st_status(tile_status + tile, kFlagPrefix | run_incl);
+                if ((seq_bits & kSeqRunEnd) && !last && lane == 0) st_status(tile_status + tile, (LONG ? (Word)kShortPrefix : (Word)kFlagPrefix) | (Word)run_incl);
             }
             // What the others wait for goes out before the tile's bitmap and the unit's totals: the chain votes - sums -
             // offset - sending is what small tables wait for.  The flags that are still needed are in registers by then, since
@@ -1284,9 +1387,9 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             // fp32, two of 30 000 001, 108 -> 111.)
             uint32_t word = 0;
             if (FINE)
-                store_bitmap_fine<STEP>(bitmap_dst, ctl->bm[se], nblk, tw, lane);
+                store_bitmap_fine<STEP>(bitmap_dst, ctl->bm[sr], nblk, tw, lane);
             else if (32u * lane < nbt)
-                word = ctl->bm[se][lane];
+                word = ctl->bm[sr][lane];
             auto report = [&]() {
                 if (!FINE && nbt >= 8) store_bitmap<STEP>(bitmap_dst, word, nblk, tw, lane);
                 if (!seq) return;
@@ -1301,21 +1404,21 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             const bool report_first = HASH != 0 || (!STEP && DT != CIERA_FP32 && !seq && n_tiles - spread_first >= 4u * gridDim.x);
             if (report_first) report();
             if (lane == 0) {
-                if (seq) ctl->base[se] = excl;
-                ctl->agg[se] = agg;
+                if (seq) ctl->base[sr] = excl;
+                ctl->agg[sr] = agg;
             }
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(&ctl->summed[se]);
-                if (seq) mbar_arrive(&ctl->resolved[se]);
+                mbar_arrive(&ctl->summed[sr]);
+                if (seq) mbar_arrive(&ctl->resolved[sr]);
             }
             if (!report_first) report();
         }
     } else if (warp >= (uint32_t)CW + 2u) {
         // ---------------------------------------------------------------- resolvers (slots k = i, i + R, ...)
         for (uint32_t k = warp - ((uint32_t)CW + 2u);; k += kResolvers) {
-            const uint32_t se = k % SE;
-            if (!mbar_wait(&ctl->summed[se], (k / SE) & 1u, abort, status)) break;
+            const uint32_t sr = k % SR;
+            if (!mbar_wait(&ctl->summed[sr], (k / SR) & 1u, abort, status)) break;
             const uint32_t tile = ctl->tile_idx[k % kDescRing];
             if (tile == kNoTile) {
                 if (early_clear) {
@@ -1327,7 +1430,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     }
                     if (__shfl_sync(0xffffffffu, last, 0)) {
                         __threadfence();
-                        for (uint32_t t = clear_first + lane; t < n_tiles; t += 32u) st_status(tile_status + t, 0ull);
+                        clear_status(tile_status, groups, clear_first, n_tiles, lane, 32u);
                         if (lane == 0) atomicExch(blocks_done, 0u);
                     }
                 }
@@ -1335,11 +1438,11 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             }
             if (ctl->seq[k % kDescRing] != 0) continue;  // the aggregator has done it all
             const TileDesc td = ctl->desc[k % kDescRing];
-            resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[se], ctl->bm[se], msgs, tw.msg, wire_bytes, changed_blocks,
-                                   tile_status, status, lane, [&](uint64_t excl) {
+            resolve_tile<DT, STEP>(td, tile, log2b, ctl->agg[sr], ctl->bm[sr], msgs, tw.msg, wire_bytes, changed_blocks,
+                                   tile_status, groups, status, lane, [&](uint64_t excl) {
                                        if (lane == 0) {
-                                           ctl->base[se] = excl;
-                                           mbar_arrive(&ctl->resolved[se]);
+                                           ctl->base[sr] = excl;
+                                           mbar_arrive(&ctl->resolved[sr]);
                                        }
                                    });
         }
@@ -1347,13 +1450,20 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         // ---------------------------------------------------------------- consumers
         uint32_t k_end = kNoTile;  // slot of the first end marker, once seen
         uint32_t k = 0;
-        // stage and phase of slot k in the two rings, and of slot k - kDefer in the exponent ring, kept
+        // stage and phase of slot k in the rings, and of slot k - kDefer in the ring of results, kept
         // as running counters (the ring depths are no powers of two)
-        uint32_t sw = 0, pw = 0, se = 0, pe = 0, je = 0, pj = 0;
-        uint32_t rw = 0, re = 0, pr = 0;  // kRebuild: stages of slot k - 1 in the two rings, phase in the exponent ring
+        uint32_t sw = 0, pw = 0, se = 0, pe = 0, sr = 0, je = 0, pj = 0;
+        uint32_t rw = 0, rr = 0, pr = 0;  // kRebuild: stages of slot k - 1 in the rings of weights and results, phase in the latter
         // HASH: the lanes of a warp that share a block (a power of two, at most the warp) add up their terms
         const uint32_t hash_lanes_l2 = min(5u, log2b - (uint32_t)P::kLog2Values);
         for (;; ++k) {
+            // LONG: a spread tile is sent kDefer slots later, from the cache: its exponents are fetched here
+            std::conditional_t<LONG, FromCache<DT>, int> ahead;
+            bool deferred = false;
+            if constexpr (LONG) {
+                deferred = k >= (uint32_t)kDefer && k - kDefer < k_end && ctl->seq[(k - kDefer) % kDescRing] == 0;
+                if (deferred) ahead.fetch(ctl->info[(k - kDefer) % kDescRing], log2b, ctl->bm[je], tid);
+            }
             // (the producer starts the loads of slot k only once both of its stages are free, and the cached
             // exponents land on the same barrier as the weights; with HashCache the cached hashes, which only
             // the aggregator reads, land on full_e)
@@ -1364,7 +1474,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if (k_end == kNoTile) k_end = k;
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(&ctl->voted[se]);  // pass the end marker on to the aggregator
+                    mbar_arrive(&ctl->voted[sr]);  // pass the end marker on to the aggregator
                     mbar_arrive(&ctl->empty_w[sw]);  // and hand the marker's (unused) stages back
                     mbar_arrive(&ctl->empty_e[se]);
                 }
@@ -1421,7 +1531,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 if (kBulkOut && !kRebuild) fence_async_shared();  // the reconstructed weights, before lane 0's bulk store reads them
                 __syncwarp();  // the warp's shared-memory accesses above are ordered before lane 0's arrives
                 if (lane == 0) {
-                    mbar_arrive(&ctl->voted[se]);
+                    mbar_arrive(&ctl->voted[sr]);
+                    if (LONG) mbar_arrive(&ctl->empty_e[se]);
                     if (!kRebuild) {
                         if (kBulkOut && nv == (uint32_t)kTileValues) {
                             bulk_store_tile_part(ti, tw, s_w, warp);
@@ -1434,28 +1545,31 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             if constexpr (kRebuild) {
                 // the receiver's part of the tile before this one: its block flags are there by now
                 if (k != 0 && k - 1u < k_end) {
-                    if (!mbar_wait(&ctl->summed[re], pr, abort, status)) break;
+                    if (!mbar_wait(&ctl->summed[rr], pr, abort, status)) break;
                     const EncodeTileInfo ti = ctl->info[(k - 1u) % kDescRing];
                     uint8_t* const s_w = ring_w + (size_t)rw * kWStage;
                     const bool full = ti.nv == (uint32_t)kTileValues;
                     if (full)
-                        reconstruct<DT, true, kBulkOut>(ti, log2b, ctl->bm[re], s_w, s_w + kWBytes, tw, tid);
+                        reconstruct<DT, true, kBulkOut, LONG>(ti, log2b, ctl->bm[rr], s_w, s_w + kWBytes, tw, tid);
                     else
-                        reconstruct<DT, false, false>(ti, log2b, ctl->bm[re], s_w, s_w + kWBytes, tw, tid);
+                        reconstruct<DT, false, false, LONG>(ti, log2b, ctl->bm[rr], s_w, s_w + kWBytes, tw, tid);
                     if (kBulkOut) fence_async_shared();
                     __syncwarp();
+                    if (kBulkOut && full && lane == 0) bulk_store_tile_part(ti, tw, s_w, warp);
+                    if (LONG && ctl->seq[(k - 1u) % kDescRing] != 0) {  // a tile of a run: its offset came with its flags
+                        send_changed<DT, FINE, HASH, STEP, LONG>(ti, log2b, ctl->bm[rr], ctl->pre[rr], ctl->base[rr],
+                                                                 (uint32_t)ctl->agg[rr], s_w, s_gather, tw, tid);
+                        __syncwarp();
+                    }
                     if (lane == 0) {
-                        if (kBulkOut && full) {
-                            bulk_store_tile_part(ti, tw, s_w, warp);
-                            bulk_wait_read<0>();
-                        }
+                        if (kBulkOut && full) bulk_wait_read<0>();
                         mbar_arrive(&ctl->empty_w[rw]);
                     }
                 }
                 if (k != 0) {
                     if (++rw == (uint32_t)SW) rw = 0;
-                    if (++re == (uint32_t)SE) {
-                        re = 0;
+                    if (++rr == (uint32_t)SR) {
+                        rr = 0;
                         pr ^= 1u;
                     }
                 }
@@ -1463,15 +1577,24 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
 
             // the changed exponents of the tile handled kDefer slots ago: its offset is known by now
             if (k >= (uint32_t)kDefer) {
-                if (k - kDefer < k_end) {
+                if constexpr (LONG) {
+                    if (deferred) {
+                        if (!mbar_wait(&ctl->resolved[je], pj, abort, status)) break;
+                        const EncodeTileInfo ti = ctl->info[(k - kDefer) % kDescRing];
+                        if (ti.nv == (uint32_t)kTileValues)
+                            write_changed<DT, false, true, STEP, S>(ti, log2b, ctl->bm[je], ctl->pre[je], ctl->base[je], tw, tid, ahead);
+                        else
+                            write_changed<DT, false, false, STEP, S>(ti, log2b, ctl->bm[je], ctl->pre[je], ctl->base[je], tw, tid, ahead);
+                    }
+                } else if (k - kDefer < k_end) {
                     if (!mbar_wait(&ctl->resolved[je], pj, abort, status)) break;
-                    send_changed<DT, FINE, HASH, STEP>(ctl->info[(k - kDefer) % kDescRing], log2b, ctl->bm[je], ctl->pre[je],
-                                                 ctl->base[je], (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes,
-                                                 s_gather, tw, tid);
+                    send_changed<DT, FINE, HASH, STEP, false>(ctl->info[(k - kDefer) % kDescRing], log2b, ctl->bm[je], ctl->pre[je],
+                                                        ctl->base[je], (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes,
+                                                        s_gather, tw, tid);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->empty_e[je]);
                 }
-                if (++je == (uint32_t)SE) {
+                if (++je == (uint32_t)SR) {
                     je = 0;
                     pj ^= 1u;
                 }
@@ -1485,16 +1608,29 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 se = 0;
                 pe ^= 1u;
             }
+            if (++sr == (uint32_t)SR) sr = 0;
         }
         // tiles whose changed exponents are still to be sent (when kDefer > kResolvers)
         if (!*abort && k_end != kNoTile) {
             for (uint32_t j = k + 1u >= (uint32_t)kDefer ? k + 1u - kDefer : 0u; j < k_end; ++j) {
-                const uint32_t je = j % SE;
-                if (!mbar_wait(&ctl->resolved[je], (j / SE) & 1u, abort, status)) break;
-                send_changed<DT, FINE, HASH, STEP>(ctl->info[j % kDescRing], log2b, ctl->bm[je], ctl->pre[je], ctl->base[je],
-                                             (uint32_t)ctl->agg[je], ring_e + (size_t)je * kEBytes, s_gather, tw, tid);
+                const uint32_t je = j % SR;
+                if (LONG && ctl->seq[j % kDescRing] != 0) continue;  // sent already
+                if (!mbar_wait(&ctl->resolved[je], (j / SR) & 1u, abort, status)) break;
+                const EncodeTileInfo ti = ctl->info[j % kDescRing];
+                if constexpr (LONG) {
+                    if (j + (uint32_t)SW < k_end) {
+                        FromCache<DT> ahead;
+                        ahead.fetch(ti, log2b, ctl->bm[je], tid);
+                        write_changed<DT, false, false, STEP, S>(ti, log2b, ctl->bm[je], ctl->pre[je], ctl->base[je], tw, tid, ahead);
+                        continue;
+                    }
+                }
+                // (LONG: the weights stage has not been filled again)
+                send_changed<DT, FINE, HASH, STEP, LONG>(ti, log2b, ctl->bm[je], ctl->pre[je], ctl->base[je], (uint32_t)ctl->agg[je],
+                                                         LONG ? ring_w + (size_t)(j % SW) * kWStage : ring_e + (size_t)je * kEBytes,
+                                                         s_gather, tw, tid);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&ctl->empty_e[je]);
+                if (!LONG && lane == 0) mbar_arrive(&ctl->empty_e[je]);
             }
         }
     }
@@ -1528,29 +1664,29 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     __syncthreads();
     if (s_last) {
         __threadfence();
-        for (uint32_t t = clear_first + tid; t < n_tiles; t += kEncodeThreads<DT, HASH>) st_status(tile_status + t, 0ull);
+        clear_status(tile_status, groups, clear_first, n_tiles, tid, (uint32_t)kEncodeThreads<DT, HASH>);
         if (tid == 0) atomicExch(blocks_done, 0u);
     }
 }
 
 // (with HashCache the size depends on the block size: see hash_hold_bytes, hash_part_bytes)
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH, bool STEP, bool LONG>
 static size_t encode_smem_bytes(uint32_t log2b) {
-    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP>::type;
+    using Cfg = typename EncodeCfgOf<DT, FINE, HASH, STEP, LONG>::type;
     constexpr int SW = Cfg::kWStages, SE = Cfg::kEStages;
     const size_t hash_stage = HASH ? (size_t)hash_hold_bytes<DT>(log2b) + hash_part_bytes<DT>(log2b) : 0;
     // the SM's 228 KB hold that many blocks, with the 1 KB each that the system takes
     static_assert(HASH || kEncodeBlocksPerSM<DT, STEP> *
                                   ((size_t)SW * kTileValues * (Traits<DT>::kValueBytes + (STEP ? 1 : 0)) + (size_t)SE * kTileValues +
-                                   sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)kWarps * kGatherBytes<DT, FINE, STEP> + 1024) <=
+                                   sizeof(EncodeCtl<SW, SE, kResultStages<Cfg, LONG>, Cfg::kBmWords>) + (size_t)kWarps * kGatherBytes<DT, FINE, STEP> + 1024) <=
                               233472,
                   "thread blocks per SM");
     return (size_t)SW * kTileValues * (Traits<DT>::kValueBytes + (STEP ? 1 : 0)) + (size_t)SE * kTileValues +
-           sizeof(EncodeCtl<SW, SE, Cfg::kBmWords>) + (size_t)SE * hash_stage + (size_t)kWarps * kGatherBytes<DT, FINE, STEP>;
+           sizeof(EncodeCtl<SW, SE, kResultStages<Cfg, LONG>, Cfg::kBmWords>) + (size_t)SE * hash_stage + (size_t)kWarps * kGatherBytes<DT, FINE, STEP>;
 }
 
 // Largest grid whose blocks are all resident at once, per device and block size (0 = not yet known).
-template <int DT, bool FINE, int HASH, bool STEP>
+template <int DT, bool FINE, int HASH, bool STEP, bool LONG>
 static int encode_grid_limit(uint32_t log2b, int* out) {
     static std::atomic<int> cached[64][16];  // (zero-initialised; any host thread may be the first to fill an entry)
     int dev = 0;
@@ -1558,13 +1694,13 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
     if (e != cudaSuccess) return record_cuda_error(e);
     if (dev < 0 || dev >= 64 || log2b >= 16) return CIERA_ERR_UNSUPPORTED;
     if (cached[dev][log2b].load(std::memory_order_acquire) == 0) {
-        const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
+        const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP, LONG>(log2b);
         // (the limit set here is the largest any block size asks for: the smallest block of the class)
-        e = cudaFuncSetAttribute(encode_kernel<DT, FINE, HASH, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)encode_smem_bytes<DT, FINE, HASH, STEP>(FINE ? 0u : HASH == 1 ? kHashShortRingsLog2 + 1u : kFineLog2));
+        e = cudaFuncSetAttribute(encode_kernel<DT, FINE, HASH, STEP, LONG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)encode_smem_bytes<DT, FINE, HASH, STEP, LONG>(FINE ? 0u : HASH == 1 ? kHashShortRingsLog2 + 1u : kFineLog2));
         if (e != cudaSuccess) return record_cuda_error(e);
         int per_sm = 0, sms = 0, coop = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH, STEP>, kEncodeThreads<DT, HASH>, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, encode_kernel<DT, FINE, HASH, STEP, LONG>, kEncodeThreads<DT, HASH>, smem);
         if (e != cudaSuccess) return record_cuda_error(e);
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return record_cuda_error(e);
@@ -1586,12 +1722,12 @@ struct EncodePart {
     uint32_t lo, hi;
     bool last;
 };
-template <int DT, bool FINE, int HASH = 0, bool STEP = false>
+template <int DT, bool FINE, int HASH = 0, bool STEP = false, bool LONG = false>
 static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                          uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
                          cudaStream_t s, StepTwins tw = StepTwins{0, 0, 0}, const EncodePart* part = nullptr) {
     int limit = 0;
-    const int rc = encode_grid_limit<DT, FINE, HASH, STEP>(p->log2b, &limit);
+    const int rc = encode_grid_limit<DT, FINE, HASH, STEP, LONG>(p->log2b, &limit);
     if (rc) return rc;
     const TileDesc* tiles = p->tiles_dev;
     const uint32_t all_tiles = (uint32_t)p->tiles.size();
@@ -1608,11 +1744,10 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     uint8_t* c = (uint8_t*)sender_cache_dev;
     uint8_t* m = (uint8_t*)messages_dev;
     unsigned long long* wb = (unsigned long long*)wire_bytes_dev;
-    unsigned long long* ts = (unsigned long long*)scratch;
-    unsigned int* ticket = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(all_tiles));
-    unsigned int* done = ticket + 1;
+    unsigned long long* groups = (unsigned long long*)((uint8_t*)scratch + workspace_groups_offset(all_tiles));
+    unsigned int* counters = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(all_tiles));
     const void* per_tile = HASH ? static_cast<const void*>(p->tile_hash_dev) : part ? part->order : nullptr;
-    const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP>(log2b);
+    const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP, LONG>(log2b);
     BufferEnds ends{p->weights_end_tile, HASH ? kNoTile : p->cache_end_tile, p->several_end_tiles};
     const bool has_spread = spread_first < nt;  // look-back between blocks
     // With a tile to a block and nothing else a tile looks back at blocks before its own only, so the blocks need not all be
@@ -1629,12 +1764,12 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
         void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
-                        &changed_blocks_dev, &ts, &ticket, &done, &status_dev, &per_tile, &tw, &ends};
-        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
+                        &changed_blocks_dev, &scratch, &groups, &counters, &status_dev, &per_tile, &tw, &ends};
+        e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP, LONG>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
                                         smem, s);
     } else {
-        e = launch_after(encode_kernel<DT, FINE, HASH, STEP>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
-                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, ts, ticket, done, status_dev, per_tile, tw, ends);
+        e = launch_after(encode_kernel<DT, FINE, HASH, STEP, LONG>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
+                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, scratch, groups, counters, status_dev, per_tile, tw, ends);
     }
     if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
@@ -1646,6 +1781,9 @@ template <int DT>
 static int launch_encode_of(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                             uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
                             cudaStream_t s, const StepTwins* tw, const EncodePart* part) {
+    if (tw && !is_fine(p->log2b) && p->long_tiles >= kLongTilesMin)
+        return launch_encode<DT, false, 0, true, true>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev,
+                                                       scratch, status_dev, s, *tw, part);
     auto launch = [&](auto fine, auto step) {
         return launch_encode<DT, decltype(fine)::value, 0, decltype(step)::value>(
             p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev, scratch, status_dev, s,

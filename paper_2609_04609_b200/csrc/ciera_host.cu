@@ -201,7 +201,10 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         const uint32_t first = p->seq_first[i], end = p->seq_first[i + 1], head = head_of(end - first);
         if (first + head < end) p->seq_runs.push_back({first + head, end});
     }
-    for (uint32_t u : longs) emit(u);
+    for (uint32_t u : longs) {
+        emit(u);
+        p->long_tiles += tiles_of(u);
+    }
     // the same tiles by address, for steps on host weights
     {
         std::vector<uint32_t> order;

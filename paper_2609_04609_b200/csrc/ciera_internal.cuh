@@ -51,6 +51,19 @@ constexpr unsigned long long kFlagPrefix = 2ull << 62;
 constexpr unsigned long long kValueMask = (1ull << 56) - 1;
 constexpr int kBitsShift = 56;
 
+// The whole step on tables of long units (LONG in ciera_encode.cu) keeps shorter words per tile, and words per group of 32
+// tiles that start at a multiple of 32 and belong to one unit.
+//   tile   bits 31:30 as above, bits 29:24 the tile's own bitmap bits, bits 23:0 payload bytes of the tile (at most
+//          kTileValues) or, handed on by a run, of its unit so far (at most kSeqMaxTiles times that)
+//   group  bits 63:62 2 = the value goes back to the unit's first tile, bits 61:56 tiles that have reported, bits 55:0 payload
+//          bytes; everything in it is added, in any order
+constexpr uint32_t kShortAggregate = 1u << 30;
+constexpr uint32_t kShortPrefix = 2u << 30;
+constexpr uint32_t kShortValueMask = (1u << 24) - 1;
+constexpr int kShortBitsShift = 24;
+constexpr uint32_t kGroupTilesLog2 = 5, kGroupTiles = 1u << kGroupTilesLog2;
+constexpr int kGroupCountShift = 56;
+
 // Upper bound on polls of one status word before a tile gives up and raises CIERA_ERR_TIMEOUT.
 constexpr uint32_t kMaxPolls = 1u << 21;
 
@@ -127,13 +140,15 @@ constexpr uint32_t kDecodeDirectBlocks = 4096;
 
 // Layout of the scratch ("workspace") of a plan with nt tiles, shared by the sender, transport and receiver calls:
 //   [0, 8 nt)             one 64-bit look-back status word per tile                     (sender)
-//   [8 nt, + 16)          the sender's run counter and its counter of finished blocks   (sender)
+//                         or, the whole step on long units: a 32-bit word per tile, then a 64-bit word per whole group
+//   [8 nt, + 16)          the sender's counters of runs, of finished blocks and of spread tiles (sender)
 //   [8 nt + 16, + 16)     the counter that transport and receiver hand their tiles out from, and their count of
 //                         thread blocks (producer warps) that have drawn their last number
 //   [8 nt + 32, + 4 nt)   changed blocks before each tile of the units that go through the receiver's prefix kernel
 // Sender, transport and receiver each need their counters all zero when they start and leave them so (the last
 // thread block to finish clears them), so that no call needs a clearing launch in front of its kernel; transport
 // and receiver touch nothing of the sender's, and the per-tile counts need no initial value.
+__host__ __device__ inline size_t workspace_groups_offset(size_t nt) { return (nt * sizeof(uint32_t) + 7) / 8 * 8; }
 __host__ __device__ inline size_t workspace_sender_counters_offset(size_t nt) { return nt * sizeof(unsigned long long); }
 __host__ __device__ inline size_t workspace_ticket_offset(size_t nt) { return workspace_sender_counters_offset(nt) + 16; }
 __host__ __device__ inline size_t workspace_prefix_offset(size_t nt) { return workspace_ticket_offset(nt) + 16; }
@@ -149,6 +164,11 @@ constexpr uint32_t kEntLongSlots = 64;
 // a short unit tile after tile (the tile's place in the payload is then a running sum inside the
 // block) and spreads everything else tile by tile over all blocks.
 constexpr uint32_t kSeqMaxTiles = 32;
+// Tiles of longer units from which a whole step with coarse blocks is run by the instance for long units: 8 to each of the 296
+// thread blocks of a B200.  With few tiles to a block the sending that is put off has nothing to hide behind.  bf16, four long
+// units, by the other instance / by this one: 1024 tiles 28.4 / 28.6 us, 2048 tiles 42.0 / 41.8, 4096 tiles 72.3 / 64.4,
+// 8192 tiles 129.4 / 112.1, 32768 tiles 476.9 / 394.5; fp32 4096 tiles 127.1 / 111.3, 16384 tiles 468.5 / 388.4.
+constexpr uint32_t kLongTilesMin = 8 * 296;
 // That needs many more units than thread blocks: a table whose short units' tiles are fewer than kSpreadShare times
 // the longest of these units would leave most of the GPU idle while a few blocks work through their units, so the
 // encode kernel spreads all tiles of such a table.  197 = 2/3 of the 296 thread blocks that a B200
@@ -196,6 +216,7 @@ struct ciera_plan {
     struct SeqRun {
         uint32_t lo, hi;               // tiles [lo, hi) of the table
     };
+    uint32_t long_tiles = 0;           // tiles of the units that are spread tile by tile for their length
     bool spread_all = false;           // the short units' tiles are spread too (kSpreadShare)
     std::vector<SeqRun> seq_runs;      // the short units' runs of tiles in the order they are handed out
     std::vector<uint32_t> unit_first;  // first tile of every unit (0xffffffff: a unit without values)

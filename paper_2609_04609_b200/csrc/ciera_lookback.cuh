@@ -43,6 +43,114 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
     return v;
 }
 
+// The short words and the groups of the whole step on long units (see ciera_internal.cuh).
+__device__ __forceinline__ uint32_t ld_status(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_status(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void add_status(unsigned long long* p, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// As wait_status (`st`: what was read last).
+__device__ __forceinline__ uint32_t wait_status(const uint32_t* p, uint32_t st, int32_t* status) {
+    uint32_t polls = 0;
+    while ((st >> 30) == 0) {
+        if (++polls > kMaxPolls) {
+            if (status) atomicCAS(status, 0, (int32_t)CIERA_ERR_TIMEOUT);
+            return kShortPrefix;
+        }
+        if (polls > 16) __nanosleep(polls > 1024 ? 400 : 40);
+        st = ld_status(p);
+    }
+    return st;
+}
+__device__ __forceinline__ uint32_t wait_status(const uint32_t* p, int32_t* status) { return wait_status(p, ld_status(p), status); }
+
+// A spread tile's payload bytes for the tiles behind it: its own status word and, where its group of 32 lies inside its
+// unit, its group's (one thread).
+__device__ __forceinline__ void report_tile(uint32_t* tile_status, unsigned long long* groups, const TileDesc& td, uint32_t tile,
+                                            uint32_t bits, uint32_t bytes) {
+    st_status(tile_status + tile, kShortAggregate | (bits << kShortBitsShift) | bytes);
+    const uint32_t head = tile & ~(kGroupTiles - 1u);
+    if (head >= td.first_tile && head + kGroupTiles - td.first_tile <= td.n_tiles_unit)
+        add_status(groups + (tile >> kGroupTilesLog2), (1ull << kGroupCountShift) | bytes);
+}
+
+// Empties the status words of the tiles [lo, hi) and of their groups (thread `me` of n).
+template <class WORD>
+__device__ __forceinline__ void clear_status(WORD* tile_status, unsigned long long* groups, uint32_t lo, uint32_t hi, uint32_t me,
+                                             uint32_t n) {
+    for (uint32_t t = lo + me; t < hi; t += n) st_status(tile_status + t, (WORD)0);
+    if (sizeof(WORD) == 8) return;  // no groups
+    for (uint32_t g = (lo >> kGroupTilesLog2) + me; g < hi >> kGroupTilesLog2; g += n) st_status(groups + g, 0ull);
+}
+
+// Payload bytes of the unit's tiles before `tile` (one warp; first < tile): the words of the group that the tile is in, the
+// words of the groups before it back to one that knows its prefix, and, where it comes to that, the words between
+// the unit's first tile and its first whole group.  Tile words and the nearest 32 groups are fetched at once, so that the
+// hundreds of tiles in work cost one round trip, where a word per tile, 32 to a round trip, took up to nine.  The last tile
+// of a group adds the prefix to the group's word.
+__device__ __forceinline__ uint64_t look_back(const uint32_t* tile_status, unsigned long long* groups, uint32_t first, uint32_t tile,
+                                              int32_t* status, uint32_t lane) {
+    const uint32_t head = tile & ~(kGroupTiles - 1u);
+    const uint32_t whole = (first + kGroupTiles - 1u) & ~(kGroupTiles - 1u);  // the unit's first whole group starts here
+    const bool near = tile - first <= kGroupTiles;  // the words before the tile reach back to the unit's start
+    const uint32_t lo = near ? first : head;        // words [lo, tile), at most 32
+    const uint32_t far_end = near ? first : whole;  // words [first, far_end), fewer than 32
+    const bool has_near = lo + lane < tile, has_far = first + lane < far_end;
+    uint32_t a = 0, c = 0;
+    if (has_near) a = ld_status(tile_status + lo + lane);
+    if (has_far) c = ld_status(tile_status + first + lane);
+    // (32 bits hold it: a prefix lies at most as many groups back as can be in work, some 150 of 2^18 bytes)
+    uint32_t sum = 0;
+    uint64_t prefix = 0;
+    bool from_start = true;  // no prefix was found: the words between first and far_end count
+    if (!near) {
+        const uint32_t g_first = whole >> kGroupTilesLog2;
+        for (uint32_t g = head >> kGroupTilesLog2; g > g_first; g -= min(32u, g - g_first)) {
+            const bool has = g_first + lane < g;  // lane l: the l-th group before group g
+            const unsigned long long* const p = groups + (g - 1u - (has ? lane : 0u));
+            unsigned long long st = has ? ld_status(p) : 0ull;
+            uint32_t polls = 0, known;
+            for (;;) {
+                const bool ready = !has || ((st >> kGroupCountShift) & 63ull) == (unsigned long long)kGroupTiles;
+                known = __ballot_sync(0xffffffffu, ready && (st >> 62) == 2ull);
+                const uint32_t needed = known ? (known & (0u - known)) - 1u : 0xffffffffu;  // lanes below the nearest prefix
+                if ((__ballot_sync(0xffffffffu, !ready) & needed) == 0u) break;
+                if (++polls > kMaxPolls) {
+                    if (status && lane == 0) atomicCAS(status, 0, (int32_t)CIERA_ERR_TIMEOUT);
+                    known = 1u;
+                    st = kFlagPrefix;
+                    break;
+                }
+                if (polls > 16) __nanosleep(polls > 1024 ? 400 : 40);
+                if (!ready) st = ld_status(p);
+            }
+            const uint32_t at = known ? (uint32_t)__ffs(known) - 1u : 32u;
+            if (lane < at) sum += (uint32_t)(st & kValueMask);
+            if (known) {
+                prefix = __shfl_sync(0xffffffffu, st & kValueMask, (int)at);
+                from_start = false;
+                break;
+            }
+        }
+    }
+    uint32_t near_sum = 0;
+    if (has_near) near_sum = wait_status(tile_status + lo + lane, a, status) & kShortValueMask;
+    if (has_far && from_start) sum += wait_status(tile_status + first + lane, c, status) & kShortValueMask;
+    __syncwarp();
+    const uint64_t excl = prefix + __reduce_add_sync(0xffffffffu, sum) + __reduce_add_sync(0xffffffffu, near_sum);
+    if (head >= first && tile - head == kGroupTiles - 1u) {
+        const uint64_t before_group = excl - __reduce_add_sync(0xffffffffu, lo + lane >= head ? near_sum : 0u);
+        if (lane == 0) add_status(groups + (head >> kGroupTilesLog2), kFlagPrefix + before_group);
+    }
+    return excl;
+}
+
 // One byte of a message; with TWICE also `twin` bytes further on (the whole-step kernel writes a message into the
 // sender's and the receiver's buffer alike).
 template <bool TWICE>
@@ -76,19 +184,23 @@ __device__ __forceinline__ void finish_unit(const TileDesc& td, uint32_t log2b, 
 
 // Resolver warp, one spread tile: exclusive prefix of the payload bytes over the earlier tiles of
 // the same unit by a single-pass look-back over the status words, then the duties that need it.
+// (WORD: short words and groups, or one 64-bit word per tile.)
 // `known` is called with the tile's exclusive payload offset inside its unit as soon as there is one (the tile's flags
 // in `bm` are not read after that).
-template <int DT, bool TWICE, class KNOWN>
+template <int DT, bool TWICE, class WORD, class KNOWN>
 __device__ __forceinline__ void resolve_tile(const TileDesc& td, uint32_t tile, uint32_t log2b, uint64_t agg,
                                                  const uint32_t* bm, uint8_t* msgs, int64_t twin,
-                                                 unsigned long long* wire_bytes, uint32_t* changed_blocks, unsigned long long* tile_status,
-                                                 int32_t* status, uint32_t lane, KNOWN known) {
+                                                 unsigned long long* wire_bytes, uint32_t* changed_blocks, WORD* tile_status,
+                                                 unsigned long long* groups, int32_t* status, uint32_t lane, KNOWN known) {
+    constexpr bool kShort = sizeof(WORD) == 4;
     const uint32_t nbt = kTileValues >> log2b;
     uint8_t* msg = msgs + td.msg_off;
     const uint32_t mybits = nbt < 8 ? bm[0] : 0u;
 
     uint64_t excl = 0;
-    if (td.tile_in_unit != 0) {
+    if constexpr (kShort) {
+        if (td.tile_in_unit != 0) excl = look_back(tile_status, groups, td.first_tile, tile, status, lane);
+    } else if (td.tile_in_unit != 0) {
         int64_t hi = (int64_t)tile - 1;
         while (true) {
             const int64_t idx = hi - (int64_t)lane;
@@ -115,8 +227,8 @@ __device__ __forceinline__ void resolve_tile(const TileDesc& td, uint32_t tile, 
         if (p == tpb - 1u || td.tile_in_unit == td.n_tiles_unit - 1u) {
             uint32_t part = 0;
             if (lane < p) {
-                unsigned long long st = wait_status(tile_status + (tile - p + lane), status);
-                part = (uint32_t)((st >> kBitsShift) & 0x3Full) << (lane * nbt);
+                const auto st = wait_status(tile_status + (tile - p + lane), status);
+                part = (uint32_t)((st >> (kShort ? kShortBitsShift : kBitsShift)) & 0x3Fu) << (lane * nbt);
             }
             __syncwarp();
             part = __reduce_or_sync(0xffffffffu, part);

@@ -347,3 +347,43 @@ def test_small_tables_on_several_streams_beside_a_large_one():
             lo, hi = int(u["weights_off"]), int(u["weights_off"]) + vb * int(u["n_values"])
             assert torch.equal(codec.weights_out[lo:hi], last[lo:hi]), f"table {i}"
         assert torch.equal(codec.sender_cache, codec.receiver_cache), f"table {i}"
+
+
+@pytest.mark.parametrize("block", [16, 512, 4096])
+@pytest.mark.parametrize("dtype", [0, 1, 2])
+def test_tables_of_long_units(dtype, block):
+    """Thousands of tiles in units of more than 32: units that start inside, and on the edge of, the groups of 32 tiles
+    whose words the look-back reads, ragged ends, and runs of short units beside them; hardly any, some and nearly all
+    blocks changed; once more in parts from host memory."""
+    from paper_2609_04609_b200 import runtime
+
+    tile = 8192
+    sizes = [tile * 33, tile * 1024, tile * 40 + 3, tile * 35 - 4097, tile * 1300 + 77, 100] + [tile * 5] * 240
+    codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(17 * block + dtype, DEV)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    for model, kw in (("clustered", {"f": 0.3}), ("inject", {"c": 0.9}), ("inject", {"c": 1e-5}), ("clustered", {"f": 0.2})):
+        step = wl.step_clustered if model == "clustered" else wl.inject_exponent_changes
+        w.append(step(w[-1], gen, **kw))
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    for t in (1, 2, 3, 4):
+        exp = table.step(bits[t])
+        if t < 4:
+            codec.step(to_dev_bytes(bits[t], DEV))
+        else:
+            host = torch.from_numpy(bits[t].view(np.uint8).copy()).pin_memory()
+            out = torch.zeros_like(host).pin_memory()
+            codec.step_host(host, out, torch.empty(host.numel(), dtype=torch.uint8, device=DEV))
+        torch.cuda.synchronize()
+        codec.check_status()
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        if t < 4:
+            compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+        else:
+            for u in codec.units:
+                lo, hi = (int(u["weights_off"]) + k * int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]] for k in (0, 1))
+                assert torch.equal(out[lo:hi], host[lo:hi])
