@@ -429,6 +429,15 @@ struct TileWalk {
     __device__ bool late() const { return DRAWN && spread && taken >= 2u; }
 };
 
+// The first tile that the walk of `block` will hand out, from the tables alone.
+template <bool ORDERED>
+__device__ __forceinline__ uint32_t first_tile(const uint2* runs, const uint32_t* places, uint32_t n_runs, uint32_t spread_first,
+                                               uint32_t n_tiles, uint32_t block) {
+    const uint32_t at = spread_first + block;
+    if (at < n_tiles) return ORDERED && places ? __ldg(places + at) : at;
+    return block < n_runs ? __ldg(runs + block).x : kNoTile;
+}
+
 // Fine blocks: the consumers have written the block flags themselves; fills pre (set bits before
 // each word) and returns the number of changed blocks of the tile (one warp).
 // Lane l takes the W = nwords / 32 consecutive words l W .. l W + W - 1 (1, 2, 4 or 8), so that one scan over
@@ -1234,6 +1243,13 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         ctl->seen = 0;
         mbar_fence_init();
     }
+    // The producer fetches what the kernel before this one cannot be writing, the tables, before it waits for that kernel.
+    // (One matrix of 524 288 values on 4 shards, whole step: EARLY_NUMBERS)
+    TileDesc nxt;
+    if (tid == 32u * (uint32_t)CW) {
+        const uint32_t first = first_tile<STEP>(seq_runs, order, n_runs, spread_first, n_tiles, blockIdx.x);
+        if (first != kNoTile) nxt = load_tile_desc(tiles + first);
+    }
     pdl_wait();
     __syncthreads();
 
@@ -1245,13 +1261,9 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         if (lane == 0) {
             TileWalk<STEP, LONG> walk(seq_runs, order, counters, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
-            uint32_t tile_nxt = walk.next(seq_nxt);
-            TileDesc nxt;
-            unsigned long long hb_nxt = 0;  // HASH: index of the tile's first block in HashCache
-            if (tile_nxt != kNoTile) {      // descriptors are fetched one tile ahead
-                nxt = load_tile_desc(tiles + tile_nxt);
-                if (HASH) hb_nxt = __ldg(tile_hash + tile_nxt);
-            }
+            uint32_t tile_nxt = walk.next(seq_nxt);  // (descriptors are fetched one tile ahead, the first one above)
+            unsigned long long hb_nxt = 0;           // HASH: index of the tile's first block in HashCache
+            if (HASH && tile_nxt != kNoTile) hb_nxt = __ldg(tile_hash + tile_nxt);
             uint32_t markers = 0;
             for (uint32_t k = 0;; ++k) {
                 const TileDesc td = nxt;
@@ -1277,45 +1289,47 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     if (++markers == (uint32_t)kResolvers) break;
                     continue;
                 }
-                ctl->desc[k % kDescRing] = td;
-                ctl->seq[k % kDescRing] = seq;
                 const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
                 const uint64_t left = td.n_unit - v0;
-                bool r_staged = true;
-                {
+                // A unit's last, short tile is staged too, in whole 16-byte pieces; the consumers drop what lies behind its
+                // last value.  Only behind the last value of a whole buffer there need not be anything.
+                const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
+                const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
+                // Only unchanged blocks need the receiver's cached exponents.  Where the tile one ring of stages
+                // before was dense (see kDenseValues) they are not staged: with every block changed that is 1 byte
+                // of 12 per value that need not be read.
+                const bool r_staged = FINE || k < (uint32_t)(LONG ? SW : SE) ||
+                                      ctl->agg[LONG ? (k - SW) % SR : se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
+                // what the others need of the tile (before the producer's arrival on the barrier of its weights)
+                auto describe = [&]() {
+                    ctl->desc[k % kDescRing] = td;
+                    ctl->seq[k % kDescRing] = seq;
                     const uint64_t smoff = sm_offset(td.n_unit, log2b);
                     EncodeTileInfo ti;
                     ti.sm_dst = msgs + td.msg_off + smoff + sm_bytes_of_values<DT>(v0);
                     ti.pay_dst = msgs + td.msg_off + smoff + pad16(sm_section_bytes(td.n_unit, DT));
                     ti.c_ptr = HASH ? cache + hb * 16ull : cache + td.c_off;
                     ti.w_src = weights + td.w_off;
-                    ti.nv = (uint32_t)min((uint64_t)kTileValues, left);
-                    // Only unchanged blocks need the receiver's cached exponents.  Where the tile one ring of stages
-                    // before was dense (see kDenseValues) they are not staged: with every block changed that is 1 byte
-                    // of 12 per value that need not be read.
-                    r_staged = FINE || k < (uint32_t)(LONG ? SW : SE) || ctl->agg[LONG ? (k - SW) % SR : se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
+                    ti.nv = nvt;
                     ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
-                }
-                // A unit's last, short tile is staged too, in whole 16-byte pieces; the consumers drop what lies behind its
-                // last value.  Only behind the last value of a whole buffer there need not be anything.
-                const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
-                const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
+                };
                 if (ends.has(tile, nvt)) {
+                    describe();
                     stage_buffer_end(ring_w + (size_t)sw * kWStage, weights + td.w_off, nvt * (uint32_t)VB,
                                      HASH ? nullptr : ring_e + (size_t)se * kEBytes, cache + td.c_off, nvt,
                                      STEP && r_staged ? kWBytes : 0u, tw.cache, &ctl->full_w[sw]);
-                } else if (HASH) {
-                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes);
-                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
                 } else {
-                    // all copies of the tile complete on the one barrier the consumers wait for
-                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes + e_bytes + (STEP && r_staged ? e_bytes : 0u));
+                    // all copies of the tile complete on the one barrier the consumers wait for (HASH: but the cached hashes);
+                    // they are started before the tile's addresses are worked out
+                    mbar_expect_tx(&ctl->full_w[sw], w_bytes + (HASH ? 0u : e_bytes) + (STEP && r_staged ? e_bytes : 0u));
                     bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
-                    bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, e_bytes, &ctl->full_w[sw]);
+                    if (!HASH) bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, e_bytes, &ctl->full_w[sw]);
                     if (STEP && r_staged)
                         bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, e_bytes,
                                   &ctl->full_w[sw]);
+                    describe();
+                    mbar_arrive(&ctl->full_w[sw]);
                 }
                 if constexpr (HASH) {
                     // the cached hashes of the tile's blocks (16 bytes each)
