@@ -1289,47 +1289,50 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     if (++markers == (uint32_t)kResolvers) break;
                     continue;
                 }
+                // (What the others need is written before the copies are started: the other way round the descriptor and its flags stay
+                // live across them, which no instance of 48 registers has room for.  Spill stores / loads 16 / 8 -> 36 / 16 bytes and
+                // an OLMoE-shaped layer 277 -> 296 us, bf16 sender; whole step on one tensor of 2^28 values 28 / 24 -> 100 / 76, 399 -> 415;
+                // sender with HashCache 306 -> 313.)
+                ctl->desc[k % kDescRing] = td;
+                ctl->seq[k % kDescRing] = seq;
                 const uint64_t v0 = (uint64_t)td.tile_in_unit * kTileValues;
                 const uint64_t left = td.n_unit - v0;
-                // A unit's last, short tile is staged too, in whole 16-byte pieces; the consumers drop what lies behind its
-                // last value.  Only behind the last value of a whole buffer there need not be anything.
-                const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
-                const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
-                // Only unchanged blocks need the receiver's cached exponents.  Where the tile one ring of stages
-                // before was dense (see kDenseValues) they are not staged: with every block changed that is 1 byte
-                // of 12 per value that need not be read.
-                const bool r_staged = FINE || k < (uint32_t)(LONG ? SW : SE) ||
-                                      ctl->agg[LONG ? (k - SW) % SR : se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
-                // what the others need of the tile (before the producer's arrival on the barrier of its weights)
-                auto describe = [&]() {
-                    ctl->desc[k % kDescRing] = td;
-                    ctl->seq[k % kDescRing] = seq;
+                bool r_staged = true;
+                {
                     const uint64_t smoff = sm_offset(td.n_unit, log2b);
                     EncodeTileInfo ti;
                     ti.sm_dst = msgs + td.msg_off + smoff + sm_bytes_of_values<DT>(v0);
                     ti.pay_dst = msgs + td.msg_off + smoff + pad16(sm_section_bytes(td.n_unit, DT));
                     ti.c_ptr = HASH ? cache + hb * 16ull : cache + td.c_off;
                     ti.w_src = weights + td.w_off;
-                    ti.nv = nvt;
+                    ti.nv = (uint32_t)min((uint64_t)kTileValues, left);
+                    // Only unchanged blocks need the receiver's cached exponents.  Where the tile one ring of stages
+                    // before was dense (see kDenseValues) they are not staged: with every block changed that is 1 byte
+                    // of 12 per value that need not be read.
+                    r_staged = FINE || k < (uint32_t)(LONG ? SW : SE) ||
+                               ctl->agg[LONG ? (k - SW) % SR : se] < payload_bytes_of_blocks<DT>(kDenseValues >> log2b, log2b);
                     ti.r_staged = r_staged ? 1u : 0u;
                     ctl->info[k % kDescRing] = ti;
-                };
+                }
+                // A unit's last, short tile is staged too, in whole 16-byte pieces; the consumers drop what lies behind its
+                // last value.  Only behind the last value of a whole buffer there need not be anything.
+                const uint32_t nvt = (uint32_t)min((uint64_t)kTileValues, left);
+                const uint32_t w_bytes = (nvt * (uint32_t)VB + 15u) & ~15u, e_bytes = (nvt + 15u) & ~15u;
                 if (ends.has(tile, nvt)) {
-                    describe();
                     stage_buffer_end(ring_w + (size_t)sw * kWStage, weights + td.w_off, nvt * (uint32_t)VB,
                                      HASH ? nullptr : ring_e + (size_t)se * kEBytes, cache + td.c_off, nvt,
                                      STEP && r_staged ? kWBytes : 0u, tw.cache, &ctl->full_w[sw]);
-                } else {
-                    // all copies of the tile complete on the one barrier the consumers wait for (HASH: but the cached hashes);
-                    // they are started before the tile's addresses are worked out
-                    mbar_expect_tx(&ctl->full_w[sw], w_bytes + (HASH ? 0u : e_bytes) + (STEP && r_staged ? e_bytes : 0u));
+                } else if (HASH) {
+                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes);
                     bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
-                    if (!HASH) bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, e_bytes, &ctl->full_w[sw]);
+                } else {
+                    // all copies of the tile complete on the one barrier the consumers wait for
+                    mbar_arrive_expect_tx(&ctl->full_w[sw], w_bytes + e_bytes + (STEP && r_staged ? e_bytes : 0u));
+                    bulk_load(ring_w + (size_t)sw * kWStage, weights + td.w_off, w_bytes, &ctl->full_w[sw]);
+                    bulk_load(ring_e + (size_t)se * kEBytes, cache + td.c_off, e_bytes, &ctl->full_w[sw]);
                     if (STEP && r_staged)
                         bulk_load(ring_w + (size_t)sw * kWStage + kWBytes, cache + tw.cache + td.c_off, e_bytes,
                                   &ctl->full_w[sw]);
-                    describe();
-                    mbar_arrive(&ctl->full_w[sw]);
                 }
                 if constexpr (HASH) {
                     // the cached hashes of the tile's blocks (16 bytes each)
