@@ -263,6 +263,9 @@ void count_launch();                           // launch accounting
 // A launch that may begin while the kernel before it in the stream still drains (programmatic dependent launch): blocks
 // become resident as soon as there is room, set themselves up and wait in pdl_wait() -- which every thread of such a
 // kernel calls before it touches global memory -- until the kernel before has finished and its writes are visible.
+// Only the tables of a plan's device image may be read earlier (the sender kernels do): ciera_plan_bind has waited for the
+// copy that wrote them, no kernel ever writes there, and the image stays unmodified while the plan is used.  A table that a
+// kernel fills would have to be read behind pdl_wait().
 // Sender step of 64 tiles, back to back: 8.2 -> 6.3 us; no difference where the kernels are long.
 // (early false: an ordinary launch.  For grids of a few blocks per SM that do not balance themselves: begun while a
 // persistent kernel drains, they are packed onto the SMs that it leaves first.)
