@@ -1177,13 +1177,19 @@ __global__ void __launch_bounds__(kEncodeThreads<DT, HASH>, kEncodeBlocksPerSM<D
 encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2* __restrict__ seq_runs, uint32_t n_runs,
               uint32_t spread_first, uint32_t clear_first, uint32_t log2b, const uint8_t* __restrict__ weights, uint8_t* cache, uint8_t* msgs,
               unsigned long long* wire_bytes, uint32_t* changed_blocks, void* status_words,
-              unsigned long long* groups, unsigned int* counters, int32_t* status,
+              void* scratch_a, unsigned int* scratch_b, int32_t* status,
               const void* __restrict__ per_tile, StepTwins tw, BufferEnds ends) {
     const uint32_t* const order = STEP ? static_cast<const uint32_t*>(per_tile) : nullptr;
     const unsigned long long* const tile_hash = HASH ? static_cast<const unsigned long long*>(per_tile) : nullptr;
     using Word = std::conditional_t<LONG, uint32_t, unsigned long long>;
     Word* const tile_status = static_cast<Word*>(status_words);
-    unsigned int* const blocks_done = counters + 1;
+    // What lies behind the status words.  HASH: the counters and, an argument of its own, the count of finished blocks; else the
+    // groups (LONG) and the counters.  (The instances with HashCache hold 70 to 77 registers and their time follows how the
+    // compiler deals them out: with the others' arguments an OLMoE-shaped layer takes 306.4 us in bf16 and 426.8 in fp16, like
+    // this, and with the first index into HashCache fetched together with the descriptor, 303.4 and 420.9.)
+    unsigned long long* const groups = HASH ? nullptr : static_cast<unsigned long long*>(scratch_a);
+    unsigned int* const counters = HASH ? static_cast<unsigned int*>(scratch_a) : scratch_b;
+    unsigned int* const blocks_done = HASH ? scratch_b : scratch_b + 1;
     static_assert(!(HASH && FINE), "HashCache: blocks of 16 values and more");
     static_assert(!LONG || (STEP && !FINE), "long units: the whole step with coarse blocks");
     static_assert(!(HASH && STEP), "the whole step compares with the exponent cache");
@@ -1248,9 +1254,13 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     // behind the wait / before it: one matrix of 524 288 values on 4 shards, bf16 6.68 / 6.53 us, fp32 9.21 / 8.91; one expert
     // on 16 shards 20.39 / 20.20; registers and spills of all instances are the same.
     TileDesc nxt;
+    unsigned long long hb_nxt = 0;  // HASH: index of the tile's first block in HashCache
     if (tid == 32u * (uint32_t)CW) {
         const uint32_t first = first_tile<STEP>(seq_runs, order, n_runs, spread_first, n_tiles, blockIdx.x);
-        if (first != kNoTile) nxt = load_tile_desc(tiles + first);
+        if (first != kNoTile) {
+            nxt = load_tile_desc(tiles + first);
+            if (HASH) hb_nxt = __ldg(tile_hash + first);
+        }
     }
     pdl_wait();
     __syncthreads();
@@ -1264,8 +1274,6 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             TileWalk<STEP, LONG> walk(seq_runs, order, counters, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
             uint32_t tile_nxt = walk.next(seq_nxt);  // (descriptors are fetched one tile ahead, the first one above)
-            unsigned long long hb_nxt = 0;           // HASH: index of the tile's first block in HashCache
-            if (HASH && tile_nxt != kNoTile) hb_nxt = __ldg(tile_hash + tile_nxt);
             uint32_t markers = 0;
             for (uint32_t k = 0;; ++k) {
                 const TileDesc td = nxt;
@@ -1471,7 +1479,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         uint32_t k = 0;
         // stage and phase of slot k in the rings, and of slot k - kDefer in the ring of results, kept
         // as running counters (the ring depths are no powers of two)
-        uint32_t sw = 0, pw = 0, se = 0, pe = 0, sr = 0, je = 0, pj = 0;
+        uint32_t sw = 0, pw = 0, se = 0, pe = 0, sr_own = 0, je = 0, pj = 0;
+        uint32_t& sr = LONG ? sr_own : se;  // stage of slot k in the ring of results: the ring of exponents is as long, but for LONG
         uint32_t rw = 0, rr = 0, pr = 0;  // kRebuild: stages of slot k - 1 in the rings of weights and results, phase in the latter
         // HASH: the lanes of a warp that share a block (a power of two, at most the warp) add up their terms
         const uint32_t hash_lanes_l2 = min(5u, log2b - (uint32_t)P::kLog2Values);
@@ -1627,7 +1636,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 se = 0;
                 pe ^= 1u;
             }
-            if (++sr == (uint32_t)SR) sr = 0;
+            if (LONG && ++sr == (uint32_t)SR) sr = 0;
         }
         // tiles whose changed exponents are still to be sent (when kDefer > kResolvers)
         if (!*abort && k_end != kNoTile) {
@@ -1765,6 +1774,8 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
     unsigned long long* wb = (unsigned long long*)wire_bytes_dev;
     unsigned long long* groups = (unsigned long long*)((uint8_t*)scratch + workspace_groups_offset(all_tiles));
     unsigned int* counters = (unsigned int*)((uint8_t*)scratch + workspace_sender_counters_offset(all_tiles));
+    void* scratch_a = HASH ? static_cast<void*>(counters) : groups;
+    unsigned int* scratch_b = HASH ? counters + 1 : counters;
     const void* per_tile = HASH ? static_cast<const void*>(p->tile_hash_dev) : part ? part->order : nullptr;
     const size_t smem = encode_smem_bytes<DT, FINE, HASH, STEP, LONG>(log2b);
     BufferEnds ends{p->weights_end_tile, HASH ? kNoTile : p->cache_end_tile, p->several_end_tiles};
@@ -1783,12 +1794,12 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
         // cooperative launch: the runtime starts the grid only when all of its blocks fit on the
         // GPU together, which is what the look-back between blocks relies on
         void* args[] = {&tiles, &nt, &seq_runs, &n_runs, &spread_first, &clear_first, &log2b, &w, &c, &m, &wb,
-                        &changed_blocks_dev, &scratch, &groups, &counters, &status_dev, &per_tile, &tw, &ends};
+                        &changed_blocks_dev, &scratch, &scratch_a, &scratch_b, &status_dev, &per_tile, &tw, &ends};
         e = cudaLaunchCooperativeKernel((const void*)encode_kernel<DT, FINE, HASH, STEP, LONG>, dim3(grid), dim3(kEncodeThreads<DT, HASH>), args,
                                         smem, s);
     } else {
         e = launch_after(encode_kernel<DT, FINE, HASH, STEP, LONG>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
-                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, scratch, groups, counters, status_dev, per_tile, tw, ends);
+                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, scratch, scratch_a, scratch_b, status_dev, per_tile, tw, ends);
     }
     if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
