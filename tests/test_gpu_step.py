@@ -3,6 +3,9 @@ oracle: tolerance 0.  Units end at the edges of pieces, warps, blocks and tiles;
 between thread blocks; the block changes from hardly any to every block, so that the receiver's cached exponents come
 both staged and straight from memory.  In a second pass the receiver's cache holds other exponents than the sender's:
 what comes out then shows that the receiver's part uses its own cache and not the sender's weights."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -349,17 +352,39 @@ def test_small_tables_on_several_streams_beside_a_large_one():
         assert torch.equal(codec.sender_cache, codec.receiver_cache), f"table {i}"
 
 
+def long_tiles_min():
+    """Tiles of long units from which a whole step is run by the kernel instance for them, as the library has it."""
+    src = os.path.join(os.path.dirname(__file__), "..", "paper_2609_04609_b200", "csrc", "ciera_internal.cuh")
+    with open(src) as f:
+        a, b = re.search(r"kLongTilesMin = (\d+) \* (\d+);", f.read()).groups()
+    return int(a) * int(b)
+
+
+def scratch_is_empty(codec):
+    """The sender's words and all counters are handed back empty, whatever words the call laid out there."""
+    return not codec.workspace[: 8 * codec.plan.n_tiles + 32].any()
+
+
 @pytest.mark.parametrize("block", [16, 512, 4096])
 @pytest.mark.parametrize("dtype", [0, 1, 2])
 def test_tables_of_long_units(dtype, block):
-    """Thousands of tiles in units of more than 32: units that start inside, and on the edge of, the groups of 32 tiles
-    whose words the look-back reads, ragged ends, and runs of short units beside them; hardly any, some and nearly all
-    blocks changed; once more in parts from host memory."""
+    """Thousands of tiles in units of more than 32: units that start and end inside, and on the edge of, the groups of 32
+    tiles whose words the look-back reads, ragged ends, and runs of short units beside them; hardly any, some and nearly all
+    blocks changed; steps and the three calls, whose words are others, in turn on one scratch; once more in parts from host
+    memory."""
     from paper_2609_04609_b200 import runtime
 
     tile = 8192
-    sizes = [tile * 33, tile * 1024, tile * 40 + 3, tile * 35 - 4097, tile * 1300 + 77, 100] + [tile * 5] * 240
+    shorts = [tile * 5] * 240 + [100] * 16  # (1216 tiles: the first long unit starts on the edge of a group)
+    # starts on an edge; ends on one; both; ends inside; starts and ends inside, twice; ragged; ends on an edge
+    longs = [tile * 33, tile * 63, tile * 64, tile * 35 - 4097, tile * 1024, tile * 40 + 3, tile * 2000 + 77, tile * 323]
+    sizes = longs[:3] + shorts + longs[3:]
+    tiles = [(n + tile - 1) // tile for n in longs]
+    first = 1216 + np.concatenate([[0], np.cumsum(tiles)])  # (long units come behind the short ones in the tile table)
+    assert [int(x) % 32 for x in first] == [0, 1, 0, 0, 3, 3, 12, 29, 0]
+    assert sum(tiles) >= 1.5 * long_tiles_min()
     codec = guard(runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV, slack=256))
+    assert codec.plan.n_tiles == first[-1]
     table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
     gen = wl.make_generator(17 * block + dtype, DEV)
     w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
@@ -369,21 +394,80 @@ def test_tables_of_long_units(dtype, block):
     bits = [wl.as_bits(x) for x in w]
     table.init_caches(bits[0])
     codec.init_caches(to_dev_bytes(bits[0], DEV))
-    for t in (1, 2, 3, 4):
+    for t, step in ((1, one_launch), (2, three_calls), (3, one_launch), (4, None)):
         exp = table.step(bits[t])
-        if t < 4:
-            codec.step(to_dev_bytes(bits[t], DEV))
+        if step:
+            step(codec, to_dev_bytes(bits[t], DEV))
         else:
             host = torch.from_numpy(bits[t].view(np.uint8).copy()).pin_memory()
             out = torch.zeros_like(host).pin_memory()
             codec.step_host(host, out, torch.empty(host.numel(), dtype=torch.uint8, device=DEV))
         torch.cuda.synchronize()
         codec.check_status()
+        assert scratch_is_empty(codec), f"t={t}"
         compare_step(codec, exp, bits[t], f"t={t}")
         compare_caches(codec, table, f"t={t}")
-        if t < 4:
+        if step:
             compare_recon(codec, exp, bits[t], dtype, f"t={t}")
         else:
             for u in codec.units:
                 lo, hi = (int(u["weights_off"]) + k * int(u["n_values"]) * wl.VALUE_BYTES[NAME[dtype]] for k in (0, 1))
                 assert torch.equal(out[lo:hi], host[lo:hi])
+
+
+@pytest.mark.parametrize("dtype,block", [(0, 512), (1, 64), (2, 4096)])
+def test_long_units_in_place_from_a_graph_and_on_two_streams(dtype, block):
+    """Two tables of long units stepped at once on streams of their own; then one of them replayed from a graph, and with
+    the reconstructed weights put where the weights are: what the three calls make of the same weights."""
+    from paper_2609_04609_b200 import runtime
+
+    tile, vb = 8192, wl.VALUE_BYTES[NAME[dtype]]
+    gen = wl.make_generator(29 * block + dtype, DEV)
+    jobs = []
+    for sizes in ([tile * 3000 + 5, tile * 700], [tile * 1900, 77, tile * 1750 - 9]):
+        assert sum(n // tile for n in sizes) >= 1.5 * long_tiles_min()
+        one, three = (runtime.LayerCodec.from_tensors(sizes, 1, NAME[dtype], block, DEV) for _ in range(2))
+        w = [wl.init_weights(one.weights_bytes // vb, NAME[dtype], gen)]
+        for _ in range(6):
+            w.append(wl.step_clustered(w[-1], gen, f=0.3))
+        w = [x.view(torch.uint8) for x in w]
+        for codec in (one, three):
+            codec.init_caches(w[0])
+        jobs.append((one, three, w, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def same(one, three, x, out, what):
+        torch.cuda.synchronize()
+        for codec in (one, three):
+            codec.check_status()
+        assert scratch_is_empty(one), what
+        for name in ("sender_cache", "receiver_cache", "wire_bytes", "changed_blocks"):
+            assert torch.equal(getattr(one, name), getattr(three, name)), f"{what}: {name}"
+        for u, n in zip(one.units, one.wire_bytes.tolist()):
+            lo, hi = int(u["weights_off"]), int(u["weights_off"]) + vb * int(u["n_values"])
+            assert torch.equal(out[lo:hi], x[lo:hi]), f"{what}: values from {lo}"
+            lo = int(u["msg_off"])
+            for name in ("msg_send", "msg_recv"):
+                assert torch.equal(getattr(one, name)[lo : lo + n], three.msg_send[lo : lo + n]), f"{what}: {name} from {lo}"
+
+    for t in (1, 2, 3):
+        for one, _, w, stream in jobs:
+            one.step(w[t], None, stream)
+    for one, three, w, _ in jobs:
+        for t in (1, 2, 3):
+            three_calls(three, w[t])
+        same(one, three, w[3], one.weights_out, "two streams")
+    one, three, w, _ = jobs[0]
+    x = w[4].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        one.step(x)
+    for t in (4, 5):
+        x.copy_(w[t])
+        graph.replay()
+        three_calls(three, w[t])
+        same(one, three, w[t], one.weights_out, "graph")
+    x.copy_(w[6])
+    one.step(x, x)
+    three_calls(three, w[6])
+    same(one, three, w[6], x, "in place")
