@@ -224,7 +224,8 @@ struct EncodeStepCfg<CIERA_FP32, true> {
 // 477 us, with made-up offsets 414, and 370 if in addition blocks may take tiles at their own pace).  So the exponents' ring only
 // holds the cached ones until they are compared, both caches are refreshed as soon as a tile's flags are there, its payload goes
 // out kDefer tiles later from the cache (see FromCache), tiles are drawn (see TileWalk), and the look-back reads groups: 394 us,
-// 0.90 of the copy peak.  Where offsets need no look-back, in runs of short units, the other instance stays 1 % ahead.
+// 0.90 of the copy peak.  In runs of short units, where offsets need no look-back, the other instance is as fast or faster (see
+// runs_as_long_units).
 template <int DT>
 struct EncodeLongCfg {
     static constexpr int kWStages = DT == CIERA_FP32 ? 4 : 3;
@@ -1815,7 +1816,7 @@ template <int DT>
 static int launch_encode_of(const ciera_plan* p, const void* weights_dev, void* sender_cache_dev, void* messages_dev,
                             uint64_t* wire_bytes_dev, uint32_t* changed_blocks_dev, void* scratch, int32_t* status_dev,
                             cudaStream_t s, const StepTwins* tw, const EncodePart* part) {
-    if (tw && !is_fine(p->log2b) && p->long_tiles >= kLongTilesMin)
+    if (tw && !is_fine(p->log2b) && p->long_units)
         return launch_encode<DT, false, 0, true, true>(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev,
                                                        scratch, status_dev, s, *tw, part);
     auto launch = [&](auto fine, auto step) {

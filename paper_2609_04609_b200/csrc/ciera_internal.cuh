@@ -165,10 +165,32 @@ constexpr uint32_t kEntLongSlots = 64;
 // block) and spreads everything else tile by tile over all blocks.
 constexpr uint32_t kSeqMaxTiles = 32;
 // Tiles of longer units from which a whole step with coarse blocks is run by the instance for long units: 8 to each of the 296
-// thread blocks of a B200.  With few tiles to a block the sending that is put off has nothing to hide behind.  bf16, four long
-// units, by the other instance / by this one: 1024 tiles 28.4 / 28.6 us, 2048 tiles 42.0 / 41.8, 4096 tiles 72.3 / 64.4,
-// 8192 tiles 129.4 / 112.1, 32768 tiles 476.9 / 394.5; fp32 4096 tiles 127.1 / 111.3, 16384 tiles 468.5 / 388.4.
+// thread blocks of a B200.  With few tiles to a block the sending that is put off has nothing to hide behind.  One tensor on
+// four shards, us by the other instance / by this one (fp32, of whose blocks there are 148, has its break-even at 1500 tiles):
+//   tiles   1448         2048         2435         4096           16384          32768
+//   bf16    32.7 / 34.5  41.6 / 40.9  49.2 / 46.4  71.5 / 63.3    246 / 206      477 / 396
+//   fp32    51.4 / 51.7  68.6 / 64.3  79.0 / 75.0  126.5 / 110.3  466 / 391
+//   fp16    35.2 / 37.6  45.2 / 46.1  52.4 / 52.6  77.1 / 73.7    269 / 250      523 / 485
+// Parts of a host step take the instance that the whole step would, since their status words have to be the same; they
+// have few tiles to a block, but wait for the link (2^25 bf16 values 1686 us by either, fp32 3196 and 3211 with runs 30 apart).
 constexpr uint32_t kLongTilesMin = 8 * 296;
+// Short units beside the long ones, though, are slower by that instance where their tiles are not full, in fp16, and in fp32
+// with blocks of 16 values, so it has to have as many long tiles as the weight of these:
+//                              lost by such a tile, ns        gained by a long tile, ns      weight
+//   bf16 ragged                0.6 to 1.3                     2.0 to 2.5                     1
+//   fp32 ragged                4.1 to 5.1                     3.9 to 4.6                     2
+//   fp32 all, blocks of 16     5.2                            3.0                            2
+//   fp16 full / ragged         0.3 to 0.95 / 0.9 to 8.8       0.8 to 1.1                     1 / 10
+// Units of 1024 values from 12 288 tensors beside one tensor of 2^25, by the other instance / by this one: bf16 1299 / 1522 us,
+// fp32 2026 / 3041, fp16 1869 / 2024; half an OLMoE-shaped layer beside 2^25, fp32 in blocks of 16, 676 / 790; a layer beside 2^25,
+// bf16 631 / 625, fp16 in blocks of 64 680 / 706.
+inline bool runs_as_long_units(int dtype, uint32_t log2b, uint64_t long_tiles, uint64_t short_tiles, uint64_t short_ragged_tiles) {
+    const uint64_t weight = dtype == CIERA_BF16   ? short_ragged_tiles
+                            : dtype == CIERA_FP16 ? short_tiles + 9 * short_ragged_tiles
+                            : log2b <= 4          ? 2 * short_tiles
+                                                  : 2 * short_ragged_tiles;
+    return long_tiles >= kLongTilesMin && long_tiles >= weight;
+}
 // That needs many more units than thread blocks: a table whose short units' tiles are fewer than kSpreadShare times
 // the longest of these units would leave most of the GPU idle while a few blocks work through their units, so the
 // encode kernel spreads all tiles of such a table.  197 = 2/3 of the 296 thread blocks that a B200
@@ -216,7 +238,7 @@ struct ciera_plan {
     struct SeqRun {
         uint32_t lo, hi;               // tiles [lo, hi) of the table
     };
-    uint32_t long_tiles = 0;           // tiles of the units that are spread tile by tile for their length
+    bool long_units = false;           // a whole step with coarse blocks is run by the instance for long units
     bool spread_all = false;           // the short units' tiles are spread too (kSpreadShare)
     std::vector<SeqRun> seq_runs;      // the short units' runs of tiles in the order they are handed out
     std::vector<uint32_t> unit_first;  // first tile of every unit (0xffffffff: a unit without values)

@@ -415,6 +415,34 @@ def test_tables_of_long_units(dtype, block):
                 assert torch.equal(out[lo:hi], host[lo:hi])
 
 
+@pytest.mark.parametrize("dtype,block", [(0, 16), (0, 4096), (1, 16), (2, 512)])
+def test_long_units_beside_many_short_ones(dtype, block):
+    """As many long tiles as the instance for long units asks for, but more in short units that it is slower with: the
+    other instance steps them (see test_long_units_rule.py), with the three calls in turn on one scratch."""
+    from paper_2609_04609_b200 import runtime
+
+    tile = 8192
+    codec = guard(runtime.LayerCodec.from_tensors([tile * 1300] + [1000] * 3000 + [tile * 1100 + 5], 1, NAME[dtype], block, DEV, slack=256))
+    assert long_tiles_min() <= 2401 < 3000
+    table = OracleTable(codec.units, dtype, block, codec.cache_bytes, codec.msg_bytes)
+    gen = wl.make_generator(19 * block + dtype, DEV)
+    w = [wl.init_weights(codec.weights_bytes // wl.VALUE_BYTES[NAME[dtype]], NAME[dtype], gen)]
+    for _ in range(2):
+        w.append(wl.step_clustered(w[-1], gen, f=0.3))
+    bits = [wl.as_bits(x) for x in w]
+    table.init_caches(bits[0])
+    codec.init_caches(to_dev_bytes(bits[0], DEV))
+    for t, step in ((1, one_launch), (2, three_calls), (0, one_launch)):
+        exp = table.step(bits[t])
+        step(codec, to_dev_bytes(bits[t], DEV))
+        torch.cuda.synchronize()
+        codec.check_status()
+        assert scratch_is_empty(codec), f"t={t}"
+        compare_step(codec, exp, bits[t], f"t={t}")
+        compare_caches(codec, table, f"t={t}")
+        compare_recon(codec, exp, bits[t], dtype, f"t={t}")
+
+
 @pytest.mark.parametrize("dtype,block", [(0, 512), (1, 64), (2, 4096)])
 def test_long_units_in_place_from_a_graph_and_on_two_streams(dtype, block):
     """Two tables of long units stepped at once on streams of their own; then one of them replayed from a graph, and with
