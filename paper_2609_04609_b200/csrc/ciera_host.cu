@@ -126,15 +126,18 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
     // processing order: short units by descending tile count (ties in table order), then the rest
     auto tiles_of = [&](uint32_t u) { return (uint32_t)((units_host[u].n_values + kTileValues - 1) / kTileValues); };
     std::vector<uint32_t> shorts, longs;
-    uint64_t short_tiles = 0, short_ragged_tiles = 0;
+    uint64_t short_tiles = 0, long_tiles = 0, other_ragged = 0;
     uint32_t longest_short = 0;
     for (uint32_t u = 0; u < n_units; ++u) {
         const uint32_t nt = tiles_of(u);
         if (nt == 0) continue;
         (nt <= kSeqMaxTiles ? shorts : longs).push_back(u);
+        if (nt > long_unit_tiles(dtype))
+            long_tiles += nt;
+        else
+            other_ragged += units_host[u].n_values % kTileValues != 0;
         if (nt <= kSeqMaxTiles) {
             short_tiles += nt;
-            short_ragged_tiles += units_host[u].n_values % kTileValues != 0;
             longest_short = std::max(longest_short, nt);
         }
     }
@@ -202,12 +205,8 @@ extern "C" int ciera_plan_create(const ciera_unit* units_host, uint32_t n_units,
         const uint32_t first = p->seq_first[i], end = p->seq_first[i + 1], head = head_of(end - first);
         if (first + head < end) p->seq_runs.push_back({first + head, end});
     }
-    uint64_t long_tiles = 0;
-    for (uint32_t u : longs) {
-        emit(u);
-        long_tiles += tiles_of(u);
-    }
-    p->long_units = runs_as_long_units(dtype, p->log2b, long_tiles, short_tiles, short_ragged_tiles);
+    for (uint32_t u : longs) emit(u);
+    p->long_units = runs_as_long_units(dtype, p->log2b, long_tiles, n_tiles - long_tiles, other_ragged);
     // the same tiles by address, for steps on host weights
     {
         std::vector<uint32_t> order;

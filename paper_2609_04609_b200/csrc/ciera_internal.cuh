@@ -164,18 +164,26 @@ constexpr uint32_t kEntLongSlots = 64;
 // a short unit tile after tile (the tile's place in the payload is then a running sum inside the
 // block) and spreads everything else tile by tile over all blocks.
 constexpr uint32_t kSeqMaxTiles = 32;
-// Tiles of longer units from which a whole step with coarse blocks is run by the instance for long units: 8 to each of the 296
-// thread blocks of a B200.  With few tiles to a block the sending that is put off has nothing to hide behind.  One tensor on
-// four shards, us by the other instance / by this one (fp32, of whose blocks there are 148, has its break-even at 1500 tiles):
+// Which tables a whole step with coarse blocks runs with the instance for long units.  Counted as long are the tiles of units of
+// more than 32 tiles, in fp16 of more than 128, and there have to be kLongTilesMin of them: 8 to each of the 296 thread
+// blocks of a B200, for with few tiles to a block the sending that is put off has nothing to hide behind.  One tensor on
+// four shards, us by the other instance / by this one (fp32, of whose blocks there are 148, breaks even at 1500 tiles):
 //   tiles   1448         2048         2435         4096           16384          32768
 //   bf16    32.7 / 34.5  41.6 / 40.9  49.2 / 46.4  71.5 / 63.3    246 / 206      477 / 396
 //   fp32    51.4 / 51.7  68.6 / 64.3  79.0 / 75.0  126.5 / 110.3  466 / 391
 //   fp16    35.2 / 37.6  45.2 / 46.1  52.4 / 52.6  77.1 / 73.7    269 / 250      523 / 485
+// bf16 and fp32 gain with every block size and rate of change from there on.  In fp16, whose consumers have the most to do to a
+// tile, small tables of long units lose where much changes (seven units of 400 tiles 61.7 / 65.2, 24 of 190 94.9 / 98.6, 43 of
+// 190 160.5 / 160.4), units of 34 to 100 tiles lose at any rate (240 of 34 133.5 / 139.4), and blocks of 32 and 64 values lose 3 to
+// 6 % where most change and a few, scattered, do not, as much as they gain where few change (2^28 values, four units: blocks of 64
+// 613.8 / 639.7 and 529.4 / 490.1; of 128 597.8 / 599.3, of 256 555.8 / 521.9; 28 units of 300 tiles, blocks of 16, 192.3 / 169.0).
 // Parts of a host step take the instance that the whole step would, since their status words have to be the same; they
 // have few tiles to a block, but wait for the link (2^25 bf16 values 1686 us by either, fp32 3196 and 3211 with runs 30 apart).
 constexpr uint32_t kLongTilesMin = 8 * 296;
-// Short units beside the long ones, though, are slower by that instance where their tiles are not full, in fp16, and in fp32
-// with blocks of 16 values, so it has to have as many long tiles as the weight of these:
+constexpr uint32_t kLongTilesMinFp16 = 8192;
+inline uint32_t long_unit_tiles(int dtype) { return dtype == CIERA_FP16 ? 128u : kSeqMaxTiles; }
+// Shorter units beside the long ones are slower by that instance where their tiles are not full, in fp16, and in fp32 with
+// blocks of 16 values, so there have to be as many long tiles as the weight of these:
 //                              lost by such a tile, ns        gained by a long tile, ns      weight
 //   bf16 ragged                0.6 to 1.3                     2.0 to 2.5                     1
 //   fp32 ragged                4.1 to 5.1                     3.9 to 4.6                     2
@@ -184,12 +192,11 @@ constexpr uint32_t kLongTilesMin = 8 * 296;
 // Units of 1024 values from 12 288 tensors beside one tensor of 2^25, by the other instance / by this one: bf16 1299 / 1522 us,
 // fp32 2026 / 3041, fp16 1869 / 2024; half an OLMoE-shaped layer beside 2^25, fp32 in blocks of 16, 676 / 790; a layer beside 2^25,
 // bf16 631 / 625, fp16 in blocks of 64 680 / 706.
-inline bool runs_as_long_units(int dtype, uint32_t log2b, uint64_t long_tiles, uint64_t short_tiles, uint64_t short_ragged_tiles) {
-    const uint64_t weight = dtype == CIERA_BF16   ? short_ragged_tiles
-                            : dtype == CIERA_FP16 ? short_tiles + 9 * short_ragged_tiles
-                            : log2b <= 4          ? 2 * short_tiles
-                                                  : 2 * short_ragged_tiles;
-    return long_tiles >= kLongTilesMin && long_tiles >= weight;
+inline bool runs_as_long_units(int dtype, uint32_t log2b, uint64_t long_tiles, uint64_t other_tiles, uint64_t other_ragged) {
+    if (dtype == CIERA_FP16)
+        return log2b != 5 && log2b != 6 && long_tiles >= kLongTilesMinFp16 && long_tiles >= other_tiles + 9 * other_ragged;
+    const uint64_t slow = dtype == CIERA_BF16 ? other_ragged : 2 * (log2b == 4 ? other_tiles : other_ragged);
+    return long_tiles >= kLongTilesMin && long_tiles >= slow;
 }
 // That needs many more units than thread blocks: a table whose short units' tiles are fewer than kSpreadShare times
 // the longest of these units would leave most of the GPU idle while a few blocks work through their units, so the
