@@ -52,6 +52,13 @@
 // the receiver's cached exponents while the tile is still in shared memory: 8.9 bytes.  Measured per OLMoE-shaped
 // layer, B = 512, q = 0.22: bf16 0.694 -> 0.572 ms (0.93 of the copy peak), fp32 1.436 -> 1.084 (0.94); every block
 // changed, bf16: 0.933 -> 0.724.
+//
+// Whole steps on tables of long units have an instance of their own (template flag LONG, chosen by runs_as_long_units), which
+// differs from the above in four things, explained where they stand: a block's spread tiles after the second are drawn from a
+// counter (TileWalk); the look-back reads a short word per tile and a word per group of 32 tiles (look_back); both caches are
+// refreshed as soon as a tile's flags are there, so that the exponents' ring is free once they are compared; and the payload
+// goes out six tiles later, read back from the cache (EncodeLongCfg, FromCache).  A tile's votes, flags and offset then live
+// in a ring of their own.
 #include <cstddef>
 #include <type_traits>
 
@@ -224,8 +231,9 @@ struct EncodeStepCfg<CIERA_FP32, true> {
 // 477 us, with made-up offsets 414, and 370 if in addition blocks may take tiles at their own pace).  So the exponents' ring only
 // holds the cached ones until they are compared, both caches are refreshed as soon as a tile's flags are there, its payload goes
 // out kDefer tiles later from the cache (see FromCache), tiles are drawn (see TileWalk), and the look-back reads groups: 394 us,
-// 0.90 of the copy peak.  In runs of short units, where offsets need no look-back, the other instance is as fast or faster (see
-// runs_as_long_units).
+// 0.90 of the copy peak.  Of these drawing is worth the least and not always something: given out by block number 395 us, one
+// tensor of 2^26 bf16 values 116 (drawn 112), 2^27 fp32 398 (392), 2^26 fp16 139 (132), 2^28 fp16 472 (483).  In runs of short
+// units, where offsets need no look-back, the other instance is as fast or faster (see runs_as_long_units).
 template <int DT>
 struct EncodeLongCfg {
     static constexpr int kWStages = DT == CIERA_FP32 ? 4 : 3;
@@ -1408,7 +1416,8 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                     if (lane == 0) st_status(tile_status + tile - 1, (Word)0);  // its one reader leaves the word empty again
                 }
                 run_incl = excl + agg;
-                if ((seq_bits & kSeqRunEnd) && !last && lane == 0) st_status(tile_status + tile, (LONG ? (Word)kShortPrefix : (Word)kFlagPrefix) | (Word)run_incl);
+                if ((seq_bits & kSeqRunEnd) && !last && lane == 0)
+                    st_status(tile_status + tile, (LONG ? (Word)kShortPrefix : (Word)kFlagPrefix) | (Word)run_incl);
             }
             // What the others wait for goes out before the tile's bitmap and the unit's totals: the chain votes - sums -
             // offset - sending is what small tables wait for.  The flags that are still needed are in registers by then, since
@@ -1746,8 +1755,9 @@ static int encode_grid_limit(uint32_t log2b, int* out) {
     return CIERA_OK;
 }
 
-// `scratch`: one status word per tile, then the run counter and the counter of finished blocks; all zero when
-// the kernel starts, and all zero again when it has finished without a device-side error.
+// `scratch`: the status words (and, LONG, the groups' words), then the counters of runs, of finished blocks and of spread tiles
+// (see workspace_groups_offset); all zero when the kernel starts, and all zero again when it has finished without a
+// device-side error.
 // part of a step: the tiles at places [lo, hi) of `order` (null: table order), all of them spread; the last part empties
 // the status words
 struct EncodePart {
@@ -1804,7 +1814,8 @@ static int launch_encode(const ciera_plan* p, const void* weights_dev, void* sen
                                         smem, s);
     } else {
         e = launch_after(encode_kernel<DT, FINE, HASH, STEP, LONG>, dim3(grid), kEncodeThreads<DT, HASH>, smem, s, tiles, nt, seq_runs, n_runs,
-                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, scratch, scratch_a, scratch_b, status_dev, per_tile, tw, ends);
+                         spread_first, clear_first, log2b, w, c, m, wb, changed_blocks_dev, scratch, scratch_a, scratch_b, status_dev,
+                         per_tile, tw, ends);
     }
     if (e != cudaSuccess) return record_cuda_error(e);
     count_launch();
@@ -1895,8 +1906,8 @@ extern "C" int ciera_encode(const ciera_plan* p, const void* weights_dev, void* 
     if (misaligned16(weights_dev) || misaligned16(sender_cache_dev) || misaligned16(messages_dev) ||
         misaligned16(workspace_dev) || ((uintptr_t)wire_bytes_dev & 7u) || ((uintptr_t)changed_blocks_dev & 3u))
         return CIERA_ERR_MISALIGNED;
-    // scratch = one look-back status word per tile, then two counters: all zero on entry (ciera_workspace_init,
-    // or left so by the previous call), and the kernel hands it back all zero
+    // scratch = one look-back status word per tile, then the counters: all zero on entry (ciera_workspace_init,
+    // or left so by the previous call, a step with other words among them), and the kernel hands it back all zero
     return launch_encode_any(p, weights_dev, sender_cache_dev, messages_dev, wire_bytes_dev, changed_blocks_dev,
                              workspace_dev, status_dev, s);
 }

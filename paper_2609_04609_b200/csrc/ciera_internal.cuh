@@ -146,8 +146,8 @@ constexpr uint32_t kDecodeDirectBlocks = 4096;
 //                         thread blocks (producer warps) that have drawn their last number
 //   [8 nt + 32, + 4 nt)   changed blocks before each tile of the units that go through the receiver's prefix kernel
 // Sender, transport and receiver each need their counters all zero when they start and leave them so (the last
-// thread block to finish clears them), so that no call needs a clearing launch in front of its kernel; transport
-// and receiver touch nothing of the sender's, and the per-tile counts need no initial value.
+// thread block to finish, or the last draw, clears them), so that no call needs a clearing launch in front of its kernel;
+// transport and receiver touch nothing of the sender's, and the per-tile counts need no initial value.
 __host__ __device__ inline size_t workspace_groups_offset(size_t nt) { return (nt * sizeof(uint32_t) + 7) / 8 * 8; }
 __host__ __device__ inline size_t workspace_sender_counters_offset(size_t nt) { return nt * sizeof(unsigned long long); }
 __host__ __device__ inline size_t workspace_ticket_offset(size_t nt) { return workspace_sender_counters_offset(nt) + 16; }
