@@ -1197,9 +1197,13 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
     using Word = std::conditional_t<LONG, uint32_t, unsigned long long>;
     Word* const tile_status = static_cast<Word*>(status_words);
     // What lies behind the status words.  HASH: the counters and, an argument of its own, the count of finished blocks; else the
-    // groups (LONG) and the counters.  (The instances with HashCache hold 70 to 77 registers and their time follows how the
-    // compiler deals them out: with the others' arguments an OLMoE-shaped layer takes 306.4 us in bf16 and 426.8 in fp16, like
-    // this, and with the first index into HashCache fetched together with the descriptor, 303.4 and 420.9.)
+    // groups (LONG) and the counters.  (The time of the instances with HashCache follows how the compiler deals out their
+    // registers, 70 to 77 in bf16 and fp16: with the others' arguments an OLMoE-shaped layer takes 306.4 us in bf16 and 426.8 in
+    // fp16, like this, and with the first index into HashCache fetched together with the descriptor, 303.4 and 420.9.  fp32, 48
+    // registers, fetches it later and counts the ring of results apart though it need not: half a layer in blocks of 16 657 ->
+    // 641 us, of 64 292 -> 285, 2^23 values 25.9 -> 25.6.)
+    constexpr bool kEarlyHash = HASH != 0 && DT != CIERA_FP32;
+    constexpr bool kOwnCount = LONG || (HASH != 0 && DT == CIERA_FP32);
     unsigned long long* const groups = HASH ? nullptr : static_cast<unsigned long long*>(scratch_a);
     unsigned int* const counters = HASH ? static_cast<unsigned int*>(scratch_a) : scratch_b;
     unsigned int* const blocks_done = HASH ? scratch_b : scratch_b + 1;
@@ -1272,7 +1276,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         const uint32_t first = first_tile<STEP>(seq_runs, order, n_runs, spread_first, n_tiles, blockIdx.x);
         if (first != kNoTile) {
             nxt = load_tile_desc(tiles + first);
-            if (HASH) hb_nxt = __ldg(tile_hash + first);
+            if (kEarlyHash) hb_nxt = __ldg(tile_hash + first);
         }
     }
     pdl_wait();
@@ -1287,6 +1291,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
             TileWalk<STEP, LONG> walk(seq_runs, order, counters, n_runs, spread_first, n_tiles, gridDim.x, blockIdx.x);
             uint32_t seq_nxt = 0;
             uint32_t tile_nxt = walk.next(seq_nxt);  // (descriptors are fetched one tile ahead, the first one above)
+            if (HASH && !kEarlyHash && tile_nxt != kNoTile) hb_nxt = __ldg(tile_hash + tile_nxt);
             uint32_t markers = 0;
             for (uint32_t k = 0;; ++k) {
                 const TileDesc td = nxt;
@@ -1494,7 +1499,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
         // stage and phase of slot k in the rings, and of slot k - kDefer in the ring of results, kept
         // as running counters (the ring depths are no powers of two)
         uint32_t sw = 0, pw = 0, se = 0, pe = 0, sr_own = 0, je = 0, pj = 0;
-        uint32_t& sr = LONG ? sr_own : se;  // stage of slot k in the ring of results: the ring of exponents is as long, but for LONG
+        uint32_t& sr = kOwnCount ? sr_own : se;  // stage of slot k in the ring of results: the ring of exponents is as long, but for LONG
         uint32_t rw = 0, rr = 0, pr = 0;  // kRebuild: stages of slot k - 1 in the rings of weights and results, phase in the latter
         // HASH: the lanes of a warp that share a block (a power of two, at most the warp) add up their terms
         const uint32_t hash_lanes_l2 = min(5u, log2b - (uint32_t)P::kLog2Values);
@@ -1650,7 +1655,7 @@ encode_kernel(const TileDesc* __restrict__ tiles, uint32_t n_tiles, const uint2*
                 se = 0;
                 pe ^= 1u;
             }
-            if (LONG && ++sr == (uint32_t)SR) sr = 0;
+            if (kOwnCount && ++sr == (uint32_t)SR) sr = 0;
         }
         // tiles whose changed exponents are still to be sent (when kDefer > kResolvers)
         if (!*abort && k_end != kNoTile) {
